@@ -1,6 +1,8 @@
-"""Thin ctypes binding over the C-ABI library ``libprecc.so`` (see ``include/precc.h``).
+"""Thin binding over the C-ABI library ``libprecc.so`` (see ``include/precc.h``).
 
-Argument marshalling only: every step of the path runs in the CUDA kernels behind the ABI.
+Argument marshalling only: every step of the path runs in the CUDA kernels behind the ABI.  The calls of the path go
+through a small CPython extension (``_native``, csrc/pybind.cpp; a call costs about a tenth of what ctypes takes for the
+same arguments), life cycle and size queries through ctypes.
 PyTorch is used for device memory and streams.  There is no fallback: if the library is
 missing or a call fails, a ``PreccError`` is raised.
 """
@@ -46,6 +48,7 @@ class CacheDesc(C.Structure):
 
 
 _lib = None
+_native = None
 
 
 class RopeDesc(C.Structure):
@@ -54,13 +57,20 @@ class RopeDesc(C.Structure):
 
 def load_library() -> C.CDLL:
     """dlopen the library (built in-tree by ``build.py``); raises if it is absent."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
         raise PreccError(f"{LIB_PATH} not found: build it with `python -m paper_2609_34054_b200.build` "
                          "(there is no CPU or PyTorch fallback)")
     lib = C.CDLL(LIB_PATH)
+    try:
+        from . import _native as native
+    except ImportError as e:
+        raise PreccError(f"the marshalling extension beside {LIB_PATH} does not load ({e}): "
+                         "build it with `python -m paper_2609_34054_b200.build`") from e
+    native.set_error(PreccError)
+    _native = native
     vp, i32, i64, u64, sz = C.c_void_p, C.c_int32, C.c_int64, C.c_uint64, C.c_size_t
     lib.precc_create.argtypes = [C.POINTER(vp), i32]
     lib.precc_destroy.argtypes = [vp]
@@ -174,12 +184,13 @@ class Precc:
         if rc != 0:
             raise PreccError(f"precc_create failed: {self.lib.precc_error_name(rc).decode()}")
         self.h = h
+        self._ctx = h.value             # the context's address, as the calls of the path take it (0 once closed: refused)
         self.sm_count = self.lib.precc_sm_count(h)
 
     def close(self):
         if getattr(self, "h", None):
             self.lib.precc_destroy(self.h)
-            self.h = None
+            self.h, self._ctx = None, 0
 
     def __del__(self):
         try:
@@ -251,81 +262,45 @@ class Precc:
 
     def turn_project(self, desc: LayerDesc, H: torch.Tensor, WA_packed: torch.Tensor, cache: Cache,
                      start_slot: int = 0, slot_mapping: Optional[torch.Tensor] = None, agent_mask: int = (1 << 64) - 1):
-        cd = cache.desc()
-        self._check(self.lib.precc_turn_project(self.h, C.byref(desc), _ptr(H), H.shape[0], _ptr(WA_packed),
-                                                _ptr(slot_mapping), start_slot, agent_mask & ((1 << 64) - 1),
-                                                C.byref(cd), _stream()), "precc_turn_project")
+        _native.turn_project(self._ctx, desc, H, WA_packed, cache, start_slot, slot_mapping, agent_mask)
 
     def turn_project_rows(self, desc: LayerDesc, H: torch.Tensor, WA_packed: torch.Tensor, cache: Cache,
                           slot_mapping: torch.Tensor, row_masks: torch.Tensor, lr_copy_slots: Optional[torch.Tensor] = None):
         """Fused projection with one agent mask per row (row_masks: int64 tensor holding the uint64 bit masks);
         lr_copy_slots: optional int32 [M], a second slot that also receives each row's LR rows (< 0: none)."""
-        if row_masks.dtype != torch.int64:
-            raise PreccError("row_masks must be int64 (bit patterns of uint64 masks)")
-        if lr_copy_slots is not None and lr_copy_slots.dtype != torch.int32:
-            raise PreccError("lr_copy_slots must be int32")
-        cd = cache.desc()
-        self._check(self.lib.precc_turn_project_rows(self.h, C.byref(desc), _ptr(H), H.shape[0], _ptr(WA_packed),
-                                                     _ptr(slot_mapping), _ptr(row_masks), _ptr(lr_copy_slots),
-                                                     C.byref(cd), _stream()),
-                    "precc_turn_project_rows")
+        _native.turn_project_rows(self._ctx, desc, H, WA_packed, cache, slot_mapping, row_masks, lr_copy_slots)
 
     # ------------------------------------------------------------------ the four entry points
     def lr_precompute(self, desc: LayerDesc, H: torch.Tensor, A_packed: torch.Tensor, cache: Cache,
                       start_slot: int = 0, slot_mapping: Optional[torch.Tensor] = None, agent_mask: int = (1 << 64) - 1):
-        cd = cache.desc()
-        self._check(self.lib.precc_lr_precompute(self.h, C.byref(desc), _ptr(H), H.shape[0], _ptr(A_packed),
-                                                 _ptr(slot_mapping), start_slot, agent_mask & ((1 << 64) - 1),
-                                                 C.byref(cd), _stream()), "precc_lr_precompute")
+        _native.lr_precompute(self._ctx, desc, H, A_packed, cache, start_slot, slot_mapping, agent_mask)
 
     def rebase_project(self, desc: LayerDesc, H: torch.Tensor, W_packed: torch.Tensor, cache: Cache,
                        start_slot: int = 0, slot_mapping: Optional[torch.Tensor] = None):
-        cd = cache.desc()
-        self._check(self.lib.precc_rebase_project(self.h, C.byref(desc), _ptr(H), H.shape[0], _ptr(W_packed),
-                                                  _ptr(slot_mapping), start_slot, C.byref(cd), _stream()),
-                    "precc_rebase_project")
+        _native.rebase_project(self._ctx, desc, H, W_packed, cache, start_slot, slot_mapping)
 
     # ------------------------------------------------------------------ rotary-key variant
-    @staticmethod
-    def _rope(table: torch.Tensor, positions: Optional[torch.Tensor] = None, start_pos: int = 0) -> RopeDesc:
-        if table.dtype != torch.float32 or table.dim() != 3 or table.shape[2] != 2:
-            raise PreccError("rope table must be fp32 [max_pos][hd/2][2]")
-        return RopeDesc(_ptr(table), table.shape[0], _ptr(positions), start_pos)
-
     def rebase_project_rope(self, desc: LayerDesc, H: torch.Tensor, W_packed: torch.Tensor, cache: Cache, rope: torch.Tensor,
                             start_slot: int = 0, slot_mapping: Optional[torch.Tensor] = None, start_pos: int = 0,
                             positions: Optional[torch.Tensor] = None):
-        cd, rd = cache.desc(), self._rope(rope, positions, start_pos)
-        self._check(self.lib.precc_rebase_project_rope(self.h, C.byref(desc), _ptr(H), H.shape[0], _ptr(W_packed),
-                                                       _ptr(slot_mapping), start_slot, C.byref(rd), C.byref(cd), _stream()),
-                    "precc_rebase_project_rope")
+        _native.rebase_project_rope(self._ctx, desc, H, W_packed, cache, rope, positions, start_pos, start_slot, slot_mapping)
 
     def turn_project_rope(self, desc: LayerDesc, H: torch.Tensor, WA_packed: torch.Tensor, cache: Cache, rope: torch.Tensor,
                           start_slot: int = 0, slot_mapping: Optional[torch.Tensor] = None, agent_mask: int = (1 << 64) - 1,
                           start_pos: int = 0, positions: Optional[torch.Tensor] = None):
-        cd, rd = cache.desc(), self._rope(rope, positions, start_pos)
-        self._check(self.lib.precc_turn_project_rope(self.h, C.byref(desc), _ptr(H), H.shape[0], _ptr(WA_packed),
-                                                     _ptr(slot_mapping), start_slot, agent_mask & ((1 << 64) - 1),
-                                                     C.byref(rd), C.byref(cd), _stream()), "precc_turn_project_rope")
+        _native.turn_project_rope(self._ctx, desc, H, WA_packed, cache, rope, positions, start_pos, start_slot,
+                                  slot_mapping, agent_mask)
 
     def lr_attend_decode_rope(self, desc: LayerDesc, q: torch.Tensor, agent_id: torch.Tensor, ctx_len: torch.Tensor,
                               max_ctx: int, B_k, B_v, rope: torch.Tensor, cache: Cache, out: torch.Tensor,
                               workspace: torch.Tensor, block_table: Optional[torch.Tensor] = None,
                               first_block: Optional[torch.Tensor] = None):
-        cd, rd = cache.desc(), self._rope(rope)
-        stride = block_table.shape[1] if block_table is not None else 0
-        self._check(self.lib.precc_lr_attend_decode_rope(
-            self.h, C.byref(desc), _ptr(q), q.shape[0], _ptr(agent_id), _ptr(ctx_len), _ptr(block_table), stride,
-            _ptr(first_block), max_ctx, _ptr(B_k), _ptr(B_v), C.byref(rd), C.byref(cd), _ptr(out), _ptr(workspace),
-            workspace.numel(), _stream()), "precc_lr_attend_decode_rope")
+        _native.lr_attend_decode_rope(self._ctx, desc, q, agent_id, ctx_len, max_ctx, B_k, B_v, rope, cache, out,
+                                      workspace, block_table, first_block)
 
     def lr_attend_prefill_rope(self, desc: LayerDesc, q: torch.Tensor, agent: int, ctx_len: int, B_k, B_v, rope: torch.Tensor,
                                cache: Cache, out: torch.Tensor, block_table: Optional[torch.Tensor] = None, first_block: int = 0):
-        cd, rd = cache.desc(), self._rope(rope)
-        stride = block_table.numel() if block_table is not None else 0
-        self._check(self.lib.precc_lr_attend_prefill_rope(
-            self.h, C.byref(desc), _ptr(q), q.shape[0], agent, ctx_len, _ptr(block_table), stride, first_block,
-            _ptr(B_k), _ptr(B_v), C.byref(rd), C.byref(cd), _ptr(out), _stream()), "precc_lr_attend_prefill_rope")
+        _native.lr_attend_prefill_rope(self._ctx, desc, q, agent, ctx_len, B_k, B_v, rope, cache, out, block_table, first_block)
 
     def prefill_rope_scratch_bytes(self, desc: LayerDesc, ctx_len: int, S: int) -> int:
         return int(self.lib.precc_prefill_rope_scratch_bytes(C.byref(desc), ctx_len, S))
@@ -334,12 +309,8 @@ class Precc:
                                        cache: Cache, out: torch.Tensor, key_scratch: torch.Tensor,
                                        block_table: Optional[torch.Tensor] = None, first_block: int = 0):
         """Rotary prefill through a caller-provided scratch for the sequence's adapted keys (uint8 or bf16 tensor)."""
-        cd, rd = cache.desc(), self._rope(rope)
-        stride = block_table.numel() if block_table is not None else 0
-        self._check(self.lib.precc_lr_attend_prefill_rope_scratch(
-            self.h, C.byref(desc), _ptr(q), q.shape[0], agent, ctx_len, _ptr(block_table), stride, first_block,
-            _ptr(B_k), _ptr(B_v), C.byref(rd), C.byref(cd), _ptr(out), _ptr(key_scratch),
-            key_scratch.numel() * key_scratch.element_size(), _stream()), "precc_lr_attend_prefill_rope_scratch")
+        _native.lr_attend_prefill_rope_scratch(self._ctx, desc, q, agent, ctx_len, B_k, B_v, rope, cache, out,
+                                               key_scratch, block_table, first_block)
 
     # ------------------------------------------------------------------ context-sharded decode
     def partial_record_floats(self, desc: LayerDesc) -> int:
@@ -349,19 +320,12 @@ class Precc:
                                  max_ctx: int, B_k, cache: Cache, records: torch.Tensor, workspace: torch.Tensor,
                                  block_table: Optional[torch.Tensor] = None, first_block: Optional[torch.Tensor] = None):
         """This shard's split-KV record per (request, kv head) over its local tokens: records fp32 [B][n_kv][R]."""
-        if records.dtype != torch.float32:
-            raise PreccError("records must be fp32")
-        cd = cache.desc()
-        stride = block_table.shape[1] if block_table is not None else 0
-        self._check(self.lib.precc_lr_attend_decode_partial(
-            self.h, C.byref(desc), _ptr(q), q.shape[0], _ptr(agent_id), _ptr(ctx_len), _ptr(block_table), stride,
-            _ptr(first_block), max_ctx, _ptr(B_k), C.byref(cd), _ptr(records), _ptr(workspace), workspace.numel(), _stream()),
-            "precc_lr_attend_decode_partial")
+        _native.lr_attend_decode_partial(self._ctx, desc, q, agent_id, ctx_len, max_ctx, B_k, cache, records,
+                                         workspace, block_table, first_block)
 
     def combine_partials(self, desc: LayerDesc, records: torch.Tensor, agent_id: torch.Tensor, B_v, out: torch.Tensor):
         """records fp32 [n_shards][B][n_kv][R] (as an all-gather leaves them) -> out [B][n_q][hd]."""
-        self._check(self.lib.precc_combine_partials(self.h, C.byref(desc), _ptr(records), records.shape[0], out.shape[0],
-                                                    _ptr(agent_id), _ptr(B_v), _ptr(out), _stream()), "precc_combine_partials")
+        _native.combine_partials(self._ctx, desc, records, agent_id, B_v, out)
 
     def decode_workspace(self, desc: LayerDesc, max_batch: int, max_ctx: int) -> torch.Tensor:
         n = self.lib.precc_decode_workspace_bytes(C.byref(desc), max_batch, max_ctx, self.sm_count)
@@ -374,12 +338,8 @@ class Precc:
     def lr_attend_decode(self, desc: LayerDesc, q: torch.Tensor, agent_id: torch.Tensor, ctx_len: torch.Tensor,
                          max_ctx: int, B_k, B_v, cache: Cache, out: torch.Tensor, workspace: torch.Tensor,
                          block_table: Optional[torch.Tensor] = None, first_block: Optional[torch.Tensor] = None):
-        cd = cache.desc()
-        stride = block_table.shape[1] if block_table is not None else 0
-        self._check(self.lib.precc_lr_attend_decode(
-            self.h, C.byref(desc), _ptr(q), q.shape[0], _ptr(agent_id), _ptr(ctx_len), _ptr(block_table), stride,
-            _ptr(first_block), max_ctx, _ptr(B_k), _ptr(B_v), C.byref(cd), _ptr(out), _ptr(workspace),
-            workspace.numel(), _stream()), "precc_lr_attend_decode")
+        _native.lr_attend_decode(self._ctx, desc, q, agent_id, ctx_len, max_ctx, B_k, B_v, cache, out, workspace,
+                                 block_table, first_block)
 
     def lr_attend_decode_static(self, desc: LayerDesc, q: torch.Tensor, agent_id: torch.Tensor, ctx_len: torch.Tensor,
                                 max_ctx: int, B_k, B_v, cache: Cache, out: torch.Tensor,
@@ -388,20 +348,12 @@ class Precc:
         all of HBM, code inside a stream capture, a loop that cannot afford cudaMalloc's synchronisation):
         the split-merge scratch is an array built into the library, so no workspace is passed.  All calls
         on a device share that array; do not let two of them overlap on the GPU."""
-        cd = cache.desc()
-        stride = block_table.shape[1] if block_table is not None else 0
-        self._check(self.lib.precc_lr_attend_decode_static(
-            self.h, C.byref(desc), _ptr(q), q.shape[0], _ptr(agent_id), _ptr(ctx_len), _ptr(block_table), stride,
-            _ptr(first_block), max_ctx, _ptr(B_k), _ptr(B_v), C.byref(cd), _ptr(out), _stream()),
-            "precc_lr_attend_decode_static")
+        _native.lr_attend_decode_static(self._ctx, desc, q, agent_id, ctx_len, max_ctx, B_k, B_v, cache, out,
+                                        block_table, first_block)
 
     def lr_attend_prefill(self, desc: LayerDesc, q: torch.Tensor, agent: int, ctx_len: int, B_k, B_v, cache: Cache,
                           out: torch.Tensor, block_table: Optional[torch.Tensor] = None, first_block: int = 0):
-        cd = cache.desc()
-        stride = block_table.numel() if block_table is not None else 0
-        self._check(self.lib.precc_lr_attend_prefill(
-            self.h, C.byref(desc), _ptr(q), q.shape[0], agent, ctx_len, _ptr(block_table), stride, first_block,
-            _ptr(B_k), _ptr(B_v), C.byref(cd), _ptr(out), _stream()), "precc_lr_attend_prefill")
+        _native.lr_attend_prefill(self._ctx, desc, q, agent, ctx_len, B_k, B_v, cache, out, block_table, first_block)
 
     def prefill_ws_bytes(self, desc: LayerDesc, S: int) -> int:
         return int(self.lib.precc_prefill_ws_bytes(self.h, C.byref(desc), S))
@@ -410,9 +362,5 @@ class Precc:
                              out: torch.Tensor, workspace: Optional[torch.Tensor], block_table: Optional[torch.Tensor] = None,
                              first_block: int = 0):
         """Prefill with a caller-provided workspace (uint8 tensor of prefill_ws_bytes, or None): helper blocks on idle SMs."""
-        cd = cache.desc()
-        stride = block_table.numel() if block_table is not None else 0
-        nbytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
-        self._check(self.lib.precc_lr_attend_prefill_ws(
-            self.h, C.byref(desc), _ptr(q), q.shape[0], agent, ctx_len, _ptr(block_table), stride, first_block,
-            _ptr(B_k), _ptr(B_v), C.byref(cd), _ptr(out), _ptr(workspace), nbytes, _stream()), "precc_lr_attend_prefill_ws")
+        _native.lr_attend_prefill_ws(self._ctx, desc, q, agent, ctx_len, B_k, B_v, cache, out, workspace, block_table,
+                                     first_block)
