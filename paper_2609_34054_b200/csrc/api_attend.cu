@@ -289,8 +289,8 @@ size_t precc_prefill_ws_bytes(const precc_ctx* ctx, const precc_layer_desc* desc
   const int tok_per_tile = 128 / G;
   const long long tiles = (long long)((S + tok_per_tile - 1) / tok_per_tile) * desc->n_kv_heads;
   if (tiles * 2 <= ctx->sm_count || tiles > (ctx->sm_count - tiles) * 14) return 0;   // no helper blocks for this turn length (at most 14 tiles per helper)
-  const size_t row = (size_t)((desc->head_dim + desc->rank_v + 15) / 16 * 16 + 4);
-  const size_t rec = (128 * row + 256) * 4;                                    // one partial: O' rows | m | l
+  const size_t row = (size_t)(desc->head_dim + 4);
+  const size_t rec = (128 * row + 256) * 4;                                    // one partial: O rows | m | l
   return ((size_t)tiles * 4 + 255) / 256 * 256 + (size_t)(tiles + ctx->sm_count) * rec;
 }
 

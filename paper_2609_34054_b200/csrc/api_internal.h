@@ -87,6 +87,7 @@ float softmax_scale_log2(const precc_layer_desc* d);
 int32_t make_map(precc_ctx* ctx, CUtensorMap* map, const void* base, int rows, int cols, int box_rows);
 int32_t make_map_w(precc_ctx* ctx, CUtensorMap* map, const void* base, int rows, int K, int box_rows);
 int32_t make_map2(precc_ctx* ctx, CUtensorMap* map, const void* base, long long rows, int cols, int box_rows, int box_cols);
+int32_t make_map_q(precc_ctx* ctx, CUtensorMap* map, const void* q, int S, int n_q, int hd, int box_tokens, int box_heads);
 int32_t make_map_cache4(precc_ctx* ctx, CUtensorMap* map, const void* base, long long n_blocks, int n_kv, int hd, int box_blocks);
 
 // F<HD, RK, RV>::run(ctx, args...) for the rank pair (rk, rv) of one head dimension.

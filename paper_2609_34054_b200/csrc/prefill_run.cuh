@@ -98,26 +98,28 @@ struct PrefillRun {
     const size_t kvw = (size_t)d->n_kv_heads * HD;
     const long long kv_rows = (long long)a.cache->n_blocks * d->n_kv_heads * PAGE;
     const long long lr_rows = (long long)a.cache->n_blocks * PAGE;
-    CUtensorMap mk, mv, mlk, mlv;
+    PrefillTcMaps m;
     // without a block table the pages of a 128-token stage are consecutive: whole-stage boxes (one TMA
     // instruction per 64-column slab instead of one per page)
     const bool contig = a.block_table == nullptr;
     const int box_rows = contig ? PTC_TOK : PAGE;
     const int v_box_blocks = (v_half ? PTC_TOK / 2 : PTC_TOK) / PAGE, v_box_rows = contig ? v_box_blocks * PAGE : PAGE;
-    int32_t rc = a.k_scratch ? make_map_cache4(ctx, &mk, a.k_scratch, a.k_scratch_blocks, d->n_kv_heads, HD, PTC_TOK / PAGE)
-                 : contig    ? make_map_cache4(ctx, &mk, a.cache->k_base, a.cache->n_blocks, d->n_kv_heads, HD, PTC_TOK / PAGE)
-                             : make_map2(ctx, &mk, a.cache->k_base, kv_rows, HD, PAGE, 64);
+    int32_t rc = a.k_scratch ? make_map_cache4(ctx, &m.k, a.k_scratch, a.k_scratch_blocks, d->n_kv_heads, HD, PTC_TOK / PAGE)
+                 : contig    ? make_map_cache4(ctx, &m.k, a.cache->k_base, a.cache->n_blocks, d->n_kv_heads, HD, PTC_TOK / PAGE)
+                             : make_map2(ctx, &m.k, a.cache->k_base, kv_rows, HD, PAGE, 64);
     if (rc) return rc;
-    rc = contig ? make_map_cache4(ctx, &mv, a.cache->v_base, a.cache->n_blocks, d->n_kv_heads, HD, v_box_blocks)
-                : make_map2(ctx, &mv, a.cache->v_base, kv_rows, HD, PAGE, 64);
+    rc = contig ? make_map_cache4(ctx, &m.v, a.cache->v_base, a.cache->n_blocks, d->n_kv_heads, HD, v_box_blocks)
+                : make_map2(ctx, &m.v, a.cache->v_base, kv_rows, HD, PAGE, 64);
     if (rc) return rc;
-    mlk = mk; mlv = mv;     // placeholders when a rank is zero (never dereferenced)
-    if (RK) { rc = make_map2(ctx, &mlk, (const __nv_bfloat16*)a.cache->lr_k + (size_t)a.agent * lr_rows * RK, lr_rows, RK, box_rows, C::RKP); if (rc) return rc; }
-    if (RV) { rc = make_map2(ctx, &mlv, (const __nv_bfloat16*)a.cache->lr_v + (size_t)a.agent * lr_rows * RV, lr_rows, RV, v_box_rows, 64); if (rc) return rc; }
+    m.lk = m.bk = m.k; m.lv = m.bv = m.v;     // placeholders when a rank is zero (never dereferenced)
+    rc = make_map_q(ctx, &m.q, a.q, a.S, d->n_q_heads, HD, PTC_TOK / G, G);
+    if (rc) return rc;
+    if (RK) { rc = make_map2(ctx, &m.bk, (const __nv_bfloat16*)a.B_k + (size_t)a.agent * RK * kvw, RK, (int)kvw, C::RKP, 64); if (rc) return rc; }
+    if (RV) { rc = make_map2(ctx, &m.bv, (const __nv_bfloat16*)a.B_v + (size_t)a.agent * RV * kvw, RV, (int)kvw, C::RVP, 64); if (rc) return rc; }
+    if (RK) { rc = make_map2(ctx, &m.lk, (const __nv_bfloat16*)a.cache->lr_k + (size_t)a.agent * lr_rows * RK, lr_rows, RK, box_rows, C::RKP); if (rc) return rc; }
+    if (RV) { rc = make_map2(ctx, &m.lv, (const __nv_bfloat16*)a.cache->lr_v + (size_t)a.agent * lr_rows * RV, lr_rows, RV, v_box_rows, 64); if (rc) return rc; }
     PrefillTcParams p;
-    p.q = (const __nv_bfloat16*)a.q; p.out = (__nv_bfloat16*)a.out; p.block_table = a.block_table;
-    p.B_k = RK ? (const __nv_bfloat16*)a.B_k + (size_t)a.agent * RK * kvw : nullptr;
-    p.B_v = RV ? (const __nv_bfloat16*)a.B_v + (size_t)a.agent * RV * kvw : nullptr;
+    p.out = (__nv_bfloat16*)a.out; p.block_table = a.block_table;
     p.status = ctx->status; p.n_blocks = a.cache->n_blocks;
     p.S = a.S; p.T = a.T; p.first_block = a.first_block; p.contig = contig ? 1 : 0; p.k_logical = a.k_scratch ? 1 : 0;
     p.longest_first = ctx->prefill_forward ? 0 : 1;
@@ -125,7 +127,7 @@ struct PrefillRun {
     p.scale_log2 = softmax_scale_log2(d); p.s_k = d->lora_scale_k; p.s_v = d->lora_scale_v;
     p.trace = (ctx->trace && ctx->trace_blocks >= 32) ? ctx->trace : nullptr;
     // four instantiations at most: classic / work list, whole-step / half-step value ring (the latter only where it applies)
-    using KernT = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, PrefillTcParams);
+    using KernT = void (*)(PrefillTcMaps, PrefillTcParams);
     KernT kern = lr_attend_prefill_tc_kernel<HD, RK, RV, false, false>;
     KernT kern_wl = lr_attend_prefill_tc_kernel<HD, RK, RV, true, false>;
     if constexpr (C::V_HALF_CAPABLE) {
@@ -182,7 +184,7 @@ struct PrefillRun {
         PRECC_CUDA(ctx, raise_smem_limit(ctx, kern_wl, smem));
         cudaLaunchConfig_t wc = {};
         wc.gridDim = dim3(wl.tiles + wl.helpers); wc.blockDim = dim3(PTC_THREADS); wc.dynamicSmemBytes = smem; wc.stream = a.stream;
-        PRECC_CUDA(ctx, cudaLaunchKernelEx(&wc, kern_wl, mk, mv, mlk, mlv, p));
+        PRECC_CUDA(ctx, cudaLaunchKernelEx(&wc, kern_wl, m, p));
         return PRECC_OK;
       }
     }
@@ -195,7 +197,7 @@ struct PrefillRun {
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = ns;
     cfg.attrs = attr; cfg.numAttrs = ns > 1 ? 1 : 0;
-    PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, mk, mv, mlk, mlv, p));
+    PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, m, p));
     return PRECC_OK;
   }
   // whether the tensor-memory kernel takes this call (shape, cache size, alignment, diagnostic switch)
