@@ -34,8 +34,11 @@
 // (keys are released right after S is computed, values only after O' is updated, so the two rings run
 // at different distances ahead), warp 1 = TMEM owner + Q K^T issuer, warp 2 = P V' issuer (an MMA costs
 // its issuing thread about a hundred cycles, so the two streams are issued by different threads), warps 4-11 = softmax
-// / correction / epilogue.  Registers are re-split at kernel start: 224 per softmax thread, 56 for the other four warps
-// (8 x 224 + 4 x 56 = 12 x 168).  Every mbarrier wait is bounded and falls through with PRECC_STATUS_TIMEOUT.
+// / correction / epilogue, warps 12-15 = more TMA issuers for paged caches: a copy costs its issuing warp about a hundred
+// cycles, and a step of a paged cache is up to 48 copies (two slabs and the LR rows of eight pages, keys and values), so
+// each warp takes eight of them (two issuers: 2250 cycles per step at head_dim 128; six: 1750, bound by the softmax).
+// Registers are re-split at kernel start: 208 per softmax thread, 48 for the other eight warps
+// (8 x 208 + 8 x 48 = 16 x 128).  Every mbarrier wait is bounded and falls through with PRECC_STATUS_TIMEOUT.
 //
 // Two more instantiations of the same kernel.  VH: the value ring holds units of 64 tokens instead of whole
 // steps (where one value stage fits beside two key stages but two do not), a unit being freed as soon as its
@@ -100,8 +103,9 @@ struct PrefillTcParams {
 
 constexpr int PTC_FIRST_SM_WARP = 4;                 // warps 0..3: key producer, Q K^T issuer, P V' issuer, value producer
 constexpr int PTC_SOFTMAX_WARPS = 8;                 // two warpgroups, taking alternate steps
-constexpr int PTC_THREADS = (PTC_FIRST_SM_WARP + PTC_SOFTMAX_WARPS) * 32;
-constexpr int PTC_SM_REGS = 224, PTC_CTL_REGS = 56;  // 256 x 224 + 128 x 56 = 384 x 168, the launch's registers
+constexpr int PTC_FIRST_HELPER = PTC_FIRST_SM_WARP + PTC_SOFTMAX_WARPS;   // four more TMA issuers (paged caches)
+constexpr int PTC_THREADS = (PTC_FIRST_HELPER + 4) * 32;
+constexpr int PTC_SM_REGS = 208, PTC_CTL_REGS = 48;  // 256 x 208 + 256 x 48 = 512 x 128, the launch's registers
 constexpr int PTC_SMEM_LIMIT = 232448;   // dynamic shared memory a block can opt into on this architecture
 constexpr int PTC_FIXED_BARS = 13; // barriers besides the two per ring stage
 constexpr int PTC_XCH_BYTES = 4 * 512;   // [2][128] reference maxima | [2][128] partial denominators
@@ -414,7 +418,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
     }
   };
 
-  if (warp < PTC_FIRST_SM_WARP) {
+  if (warp < PTC_FIRST_SM_WARP || warp >= PTC_FIRST_HELPER) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(PTC_CTL_REGS));
     for (int seg = 0; seg < nseg; ++seg) {
       load_piece(seg);
@@ -427,8 +431,13 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         atomicOr(p.status, StatusBits::BAD_INDEX);
         return 0;
       };
-      if (warp == 0) {
+      // helper warps copy the pages' second slab (12: keys, 13: values) and LR rows (14, 15)
+      const int role = warp < PTC_FIRST_SM_WARP ? warp : (warp & 1) ? 3 : 0;
+      const int share = warp < PTC_FIRST_SM_WARP ? 0 : 1 + ((warp - PTC_FIRST_HELPER) >> 1);
+      if (role == 0) {
         // -------------------------------------------------------------- TMA producer: query tile, B slices, keys
+        const bool whole = p.contig || p.k_logical;
+        if (share == 0) {
         const int q_rows = p.tok_per_tile * G;
         for (int i = q_rows * (HD / 8) + lane; i < 128 * (HD / 8); i += 32)    // rows no query maps to (128 not a multiple of G)
           *reinterpret_cast<uint4*>(smem + ((i % (HD / 8)) / 8) * C::SLAB_BYTES + (i / (HD / 8)) * 128 + (i % 8) * 16) = make_uint4(0, 0, 0, 0);
@@ -446,11 +455,11 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
           }
         }
         __syncwarp();
-        const bool whole = p.contig || p.k_logical;
+        }
         int ph_next = whole || lane >= PTC_TOK / PAGE ? 0 : lookup(jb * (PTC_TOK / PAGE) + lane);
-        for (int j = 0; j <= n_tiles; ++j) {
+        const int n_items = share == 0 ? (RV > 0 && n_tiles > 0 ? n_tiles + 1 : n_tiles) : whole ? 0 : n_tiles;
+        for (int j = 0; j < n_items; ++j) {
           const int s = j % KS;
-          if (j == n_tiles && (RV == 0 || n_tiles == 0)) break;
           if (j >= KS) mbar_wait(k_empty + 8 * s, ((j / KS) - 1) & 1, p.status);
           if (RK > 0 && j == KS - 1) mbar_wait(fold_done, 0, p.status);
           const uint32_t st = kring_u32 + (uint32_t)s * C::KSTAGE;
@@ -467,7 +476,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
               break;
             }
           }
-          if (lane == 0) PTC_STAMP(p, j, 8);               // stage of step j free: loads go out now
+          if (lane == 0 && share == 0) PTC_STAMP(p, j, 8); // stage of step j free: loads go out now
           if (whole) {
             // consecutive physical blocks: one box per 64-column slab covers all eight pages of the stage
             // (4-D map [block][kv head][16][hd]); blocks past the cache end arrive as zeros
@@ -482,27 +491,30 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
             continue;
           }
           const int live = min(PTC_TOK / PAGE, n_pages - (jb + j) * (PTC_TOK / PAGE));
-          if (lane == 0) mbar_expect_tx(full, live * C::K_PAGE_TX);
+          if (share == 0 && lane == 0) mbar_expect_tx(full, live * C::K_PAGE_TX);   // for all three issuers of the stage
           __syncwarp();
           if (lane < live) {
             const int ph = checked(ph_next);
             const int row_kv = (ph * p.n_kv + g) * PAGE;
 #pragma unroll
-            for (int sl = 0; sl < C::SLABS; ++sl) tma_load_2d(st + sl * C::SLAB_BYTES + lane * PAGE * 128, &maps.k, sl * 64, row_kv, full);
-            if constexpr (RK > 0) tma_load_2d(st + C::KV_BYTES + lane * PAGE * C::RKP * 2, &maps.lk, 0, ph * PAGE, full);
+            for (int sl = 0; sl < C::SLABS; ++sl)
+              if (share == sl) tma_load_2d(st + sl * C::SLAB_BYTES + lane * PAGE * 128, &maps.k, sl * 64, row_kv, full);
+            if constexpr (RK > 0)
+              if (share == 2) tma_load_2d(st + C::KV_BYTES + lane * PAGE * C::RKP * 2, &maps.lk, 0, ph * PAGE, full);
           }
           if (lane < PTC_TOK / PAGE) ph_next = lookup((jb + j + 1) * (PTC_TOK / PAGE) + lane);
           __syncwarp();
         }
-      } else if (warp == 3) {
+      } else if (role == 3) {
         // -------------------------------------------------------------- TMA producer: values, in units of a step or half a step
         constexpr int UT = VH ? PTC_TOK / 2 : PTC_TOK, UPG = UT / PAGE, UPS = PTC_TOK / UT, USLAB = UT * 128;
         int ph_next = p.contig || lane >= UPG ? 0 : lookup(UPS * jb * UPG + lane);
-        for (int u = 0; u < UPS * n_tiles; ++u) {
+        const int n_units = share > 0 && p.contig ? 0 : UPS * n_tiles;
+        for (int u = 0; u < n_units; ++u) {
           const int s = u % VS;
           if (u >= VS) mbar_wait(v_empty + 8 * s, ((u / VS) - 1) & 1, p.status);
           __syncwarp();
-          if (lane == 0) PTC_STAMP(p, u, 9);
+          if (lane == 0 && share == 0) PTC_STAMP(p, u, 9);
           const int pg0 = (UPS * jb + u) * UPG;            // first logical page of the unit
           const uint32_t st = vring_u32 + (uint32_t)s * vunit;
           const uint32_t full = v_full + 8 * s;
@@ -518,19 +530,21 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
             continue;
           }
           const int live = max(0, min(UPG, n_pages - pg0));
-          if (lane == 0) mbar_expect_tx(full, live * C::V_PAGE_TX);       // no live page: the phase completes at once
+          if (share == 0 && lane == 0) mbar_expect_tx(full, live * C::V_PAGE_TX);       // no live page: the phase completes at once
           __syncwarp();
           if (lane < live) {
             const int ph = checked(ph_next);
             const int row_kv = (ph * p.n_kv + g) * PAGE;
 #pragma unroll
-            for (int sl = 0; sl < C::SLABS; ++sl) tma_load_2d(st + sl * USLAB + lane * PAGE * 128, &maps.v, sl * 64, row_kv, full);
-            if constexpr (RV > 0) tma_load_2d(st + C::SLABS * USLAB + lane * PAGE * 128, &maps.lv, 0, ph * PAGE, full);
+            for (int sl = 0; sl < C::SLABS; ++sl)
+              if (share == sl) tma_load_2d(st + sl * USLAB + lane * PAGE * 128, &maps.v, sl * 64, row_kv, full);
+            if constexpr (RV > 0)
+              if (share == 2) tma_load_2d(st + C::SLABS * USLAB + lane * PAGE * 128, &maps.lv, 0, ph * PAGE, full);
           }
           if (lane < UPG) ph_next = lookup(pg0 + UPG + lane);
           __syncwarp();
         }
-      } else if (warp == 1) {
+      } else if (role == 1) {
         // -------------------------------------------------------------- S = Q' K'^T issuer
         // One thread issues these MMAs and another (warp 2) the P V' ones: an MMA costs its issuing thread
         // on the order of a hundred cycles, so two issue streams are needed to keep the tensor pipe fed.
