@@ -76,7 +76,7 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
   // Up to 40 rows the weight-streaming few-row kernel is the fastest (fused C3 projection: 5.8 us at 16 rows, 7.4 at
   // 32, 12.7 at 40); from there to about a thousand rows the split-K kernels (12.3 .. 23 us; the few-row kernel needs
   // 12.8 us at 41 rows and 13.7 at 64, the one-block-per-tile GEMM 27 .. 30 us throughout); the few-row kernel still
-  // takes 41..64 rows when the split does not apply (rotary epilogue, short K).
+  // takes 41..64 rows when the split does not apply (short K).
   if (M <= 40 && !ctx->force_tiled_gemm) {
     const int32_t rc = launch_small(ctx, X, M, K, Wt, n_out, gp, stream);
     if (rc >= 0) return rc;
@@ -84,7 +84,7 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
   const int m_tiles = (M + GEMM_BM - 1) / GEMM_BM;
   // A few row tiles (the tokens of a short turn): the K extent of every tile is split over a cluster.  The split
   // depends on M and K alone, so a column's summation order is the same whichever entry point produced it.
-  if (m_tiles <= 16 && !gp.rope && !ctx->no_gemm_splitk) {
+  if (m_tiles <= 16 && !ctx->no_gemm_splitk) {
     const int nkb = K / GEMM_BK;
     // planned for the width of the FUSED projection of this layer, whatever this call projects, so that the base-only,
     // LR-only and fused calls of one M take the same decision (and with it the same summation order)
@@ -114,7 +114,7 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
       const bool direct = !bulk && (ctx->gemm_direct >= 2 || (ctx->gemm_direct == 1 && M <= 64));
       const bool push = bulk || direct;
       if (nkb / ks < (ks <= GEMM_PUSH_MAX_KS ? 4 : 2)) continue;       // a coarse split of a short K is not worth a cluster
-      const int cw = ((256 + ks - 1) / ks + 7) / 8 * 8;          // planned for the widest tile, whatever this call's width
+      const int cw = ((256 + ks - 1) / ks + 15) / 16 * 16;       // planned for the widest tile and slice (rotary), whatever this call's
       const int slice = GEMM_BM * (cw + 4) * 4;
       const int dump = bulk ? 2 * (ks - 1) * slice : (direct ? (ks - 1) * slice : ks * slice);
       smem_plan = (((ring_max > dump ? ring_max : dump) + 1023) & ~1023) + (2 * SK_STAGES + 8) * 8;
@@ -125,7 +125,7 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
       plan_direct = direct; plan_push = push;
       if (cached == 0) {
         int n = 0;
-        auto kern = push ? proj_gemm_splitk_push_kernel : proj_gemm_splitk_kernel;
+        auto kern = push ? proj_gemm_splitk_push_kernel<false> : proj_gemm_splitk_kernel<false>;
         if (raise_smem_limit(ctx, kern, smem_plan) == cudaSuccess) {
           cudaLaunchConfig_t qc = {};
           qc.gridDim = dim3(ks, ctx->sm_count, 1); qc.blockDim = dim3(GEMM_THREADS); qc.dynamicSmemBytes = smem_plan;
@@ -155,7 +155,8 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
       gp.M = M; gp.N_out = n_out; gp.K = K; gp.BN = bn; gp.stages = stages; gp.tmem_cols = tmem_cols;
       gp.spread_rows = 0;
       gp.status = ctx->status;
-      auto kern = plan_push ? proj_gemm_splitk_push_kernel : proj_gemm_splitk_kernel;
+      auto kern = gp.rope ? (plan_push ? proj_gemm_splitk_push_kernel<true> : proj_gemm_splitk_kernel<true>)
+                          : (plan_push ? proj_gemm_splitk_push_kernel<false> : proj_gemm_splitk_kernel<false>);
       gp.direct_send = plan_direct ? 1 : 0;
       PRECC_CUDA(ctx, raise_smem_limit(ctx, kern, smem_plan));
       cudaLaunchConfig_t cfg = {};

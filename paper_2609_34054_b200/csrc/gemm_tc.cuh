@@ -282,12 +282,56 @@ proj_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
 }
 
 
+// Column order of a tile in the split-K merges.  The merge hands slices of neighbouring columns to the blocks of a
+// cluster; with rotary keys a key column and its partner hd/2 further on have to land in one slice, so the key columns
+// of a head are taken in the order (8 of the lower half, the 8 partners, the next 8, ...) and slices are multiples of 16
+// wide.  Everything else keeps its place.  `c`: a multiple of 8 in merge order; returns the column of the tile.
+template <bool ROPE>
+__device__ __forceinline__ int merge_col(const GemmParams& p, int n0, int c) {
+  if constexpr (ROPE) {
+    if (n0 + c < (p.n_kv << p.hd_shift)) {
+      const int u = c & (p.hd - 1);
+      return c - u + ((u & 8) ? p.hd / 2 : 0) + (u >> 4) * 8;
+    }
+  }
+  return c;
+}
+template <bool ROPE>
+__device__ __forceinline__ int merge_slice_cols(int bn, int ks) {     // columns finished by one block
+  constexpr int U = ROPE ? 16 : 8;
+  return (((bn + ks - 1) / ks) + U - 1) / U * U;
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+// sixteen columns from `c0` on, in merge order (issues the loads only)
+template <bool ROPE>
+__device__ __forceinline__ void tmem_ld_pieces(const GemmParams& p, uint32_t trow, int n0, int c0, uint32_t (&r)[16]) {
+  if constexpr (ROPE) {
+    uint32_t (&lo)[8] = *reinterpret_cast<uint32_t (*)[8]>(&r[0]);
+    uint32_t (&hi)[8] = *reinterpret_cast<uint32_t (*)[8]>(&r[8]);
+    tmem_ld8(trow + merge_col<true>(p, n0, c0), lo);
+    tmem_ld8(trow + merge_col<true>(p, n0, c0 + 8), hi);
+  } else {
+    tmem_ld16(trow + c0, r);
+  }
+}
+// position of a row in the rotary table, or -1 (reported) when it is outside
+__device__ __forceinline__ long long rope_pos(const GemmParams& p, int gm) {
+  const long long pos = p.positions ? (long long)p.positions[gm] : p.start_pos + gm;
+  if (pos >= 0 && pos < p.max_pos) return pos;
+  atomicOr(p.status, StatusBits::BAD_INDEX);
+  return -1;
+}
+
 // Reduce step of the split-K kernel: thread t of the block's 192 threads takes the 16-byte pieces t, t + 192, ...
 // of this block's slice (piece f = row * cw/4 + q), 16 / KS of them at a time, so that sixteen loads over
 // distributed shared memory are in flight per thread; consecutive lanes read consecutive pieces of a peer; the
 // peers are summed in rank order.  The odd piece of a pair hands its four columns to the even one, which
 // stores eight.
-template <int KS>
+template <int KS, bool ROPE>
 __device__ __forceinline__ void splitk_reduce(const GemmParams& p, uint32_t smem_base, int rank, int cw, int m0, int n0, int t) {
   constexpr int G = 16 / KS;
   const int XS = cw + 4, qpr = cw / 4;
@@ -317,11 +361,29 @@ __device__ __forceinline__ void splitk_reduce(const GemmParams& p, uint32_t smem
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int r = 0; r < KS; ++r) { v.x += a[g][r].x; v.y += a[g][r].y; v.z += a[g][r].z; v.w += a[g][r].w; }
+      long long pos = 0;
+      if constexpr (ROPE) {
+        // four lanes hold 8 columns of the lower half of a head and their 8 partners: rotate by the row's position
+        const float4 o = make_float4(__shfl_xor_sync(0xffffffffu, v.x, 2), __shfl_xor_sync(0xffffffffu, v.y, 2),
+                                     __shfl_xor_sync(0xffffffffu, v.z, 2), __shfl_xor_sync(0xffffffffu, v.w, 2));
+        if (f < total && m0 + row < p.M) {
+          pos = rope_pos(p, m0 + row);
+          const int cm = rank * cw + 4 * q;                    // merge order
+          if (pos >= 0 && n0 + cm < (p.n_kv << p.hd_shift)) {
+            const int pair = ((cm & (p.hd - 1)) >> 4) * 8 + (cm & 4);   // index of the first of these four pairs in the head
+            const float4* cs = p.rope + pos * (p.hd / 4) + pair / 2;
+            const float4 t0 = __ldg(cs), t1 = __ldg(cs + 1);
+            const float sg = (cm & 8) ? 1.f : -1.f;            // lower: x cos - y sin, upper: y cos + x sin
+            v.x = v.x * t0.x + sg * (o.x * t0.y); v.y = v.y * t0.z + sg * (o.y * t0.w);
+            v.z = v.z * t1.x + sg * (o.z * t1.y); v.w = v.w * t1.z + sg * (o.w * t1.w);
+          }
+        }
+      }
       const float4 hi = make_float4(__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1),
                                     __shfl_down_sync(0xffffffffu, v.z, 1), __shfl_down_sync(0xffffffffu, v.w, 1));
       if ((q & 1) == 0 && f < total) {
-        const int gm = m0 + row, c = rank * cw + 4 * q, gc = n0 + c;
-        if (gm < p.M && c < p.BN && gc < p.N_out) {
+        const int gm = m0 + row, c = rank * cw + 4 * q, gc = n0 + merge_col<ROPE>(p, n0, c);
+        if (gm < p.M && c < p.BN && gc < p.N_out && pos >= 0) {
           const long long slot = p.slot_mapping ? (long long)p.slot_mapping[gm] : p.start_slot + gm;
           if (slot < 0 || slot >= p.n_blocks * PAGE) {
             atomicOr(p.status, StatusBits::BAD_INDEX);
@@ -343,8 +405,9 @@ __device__ __forceinline__ void splitk_reduce(const GemmParams& p, uint32_t smem
 // K slice in TMEM exactly as above, writes the fp32 accumulator into its own shared memory (over the ring,
 // which is idle by then), and after a cluster barrier block r adds up columns [r*cw, (r+1)*cw) of all KS
 // partial tiles over distributed shared memory — in rank order, so the result does not depend on timing —
-// and routes them to the caches with the same epilogue.  No rotary epilogue here (a head's two halves would
-// have to land in one block's slice); rotary calls use the kernel above.
+// and routes them to the caches with the same epilogue.  ROPE: key columns are rotated on the way (200 rows of the
+// 3584 x 1280 rotary projection: 14 us against 30 on the one-block-per-tile kernel, which rotary calls used before).
+template <bool ROPE>
 __global__ void __launch_bounds__(GEMM_THREADS, 2)
 proj_gemm_splitk_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const GemmParams p) {
   // The declared alignment places the dynamic shared memory on a 1024-byte boundary (the swizzle atoms need it and
@@ -361,7 +424,7 @@ proj_gemm_splitk_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
   // [r*cw, (r+1)*cw), and finds them in every peer as one block of 128 rows x (cw + 4) floats (the 4 floats
   // of padding keep the row-per-thread dump free of bank conflicts), which it can read with consecutive lanes
   // on consecutive 16-byte pieces.
-  const int cw = (((p.BN + (int)gridDim.x - 1) / (int)gridDim.x) + 7) / 8 * 8;   // columns reduced by one block (a multiple of 8)
+  const int cw = merge_slice_cols<ROPE>(p.BN, (int)gridDim.x);  // columns reduced by one block (a multiple of 8 or 16)
   const int XS = cw + 4;                                        // row stride (floats) inside a slice
   const int ring_bytes = p.stages * stage_bytes, dump_bytes = (int)gridDim.x * GEMM_BM * XS * 4;
   const int data_bytes = ((ring_bytes > dump_bytes ? ring_bytes : dump_bytes) + 1023) & ~1023;
@@ -439,7 +502,7 @@ proj_gemm_splitk_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     for (int c0 = 0; c0 < p.BN; c0 += 16) {
       uint32_t r[16];
-      tmem_ld16(tmem_base + (static_cast<uint32_t>(lane_base) << 16) + c0, r);
+      tmem_ld_pieces<ROPE>(p, tmem_base + (static_cast<uint32_t>(lane_base) << 16), n0, c0, r);
       asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
       for (int k = 0; k < 16; k += 4) {
@@ -456,13 +519,13 @@ proj_gemm_splitk_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
   {
     const int t = threadIdx.x;                                  // the producer and MMA warps help with the merge
     switch (KS) {
-      case 8: splitk_reduce<8>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
-      case 7: splitk_reduce<7>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
-      case 6: splitk_reduce<6>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
-      case 5: splitk_reduce<5>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
-      case 4: splitk_reduce<4>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
-      case 3: splitk_reduce<3>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
-      default: splitk_reduce<2>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
+      case 8: splitk_reduce<8, ROPE>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
+      case 7: splitk_reduce<7, ROPE>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
+      case 6: splitk_reduce<6, ROPE>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
+      case 5: splitk_reduce<5, ROPE>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
+      case 4: splitk_reduce<4, ROPE>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
+      case 3: splitk_reduce<3, ROPE>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
+      default: splitk_reduce<2, ROPE>(p, smem_u32(smem), rank, cw, m0, n0, t); break;
     }
   }
   // nobody leaves while a peer may still read its partial tile
@@ -491,17 +554,12 @@ proj_gemm_splitk_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
 // sends the 16-byte pieces of its row straight from registers (st.async.v4 into the owner's receive area, which
 // alone overlays the ring), only the rows of the tile that exist; no barrier at the end either, since a send
 // carries its data with it.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-}
-
-// What the routing of a row's 16-byte pieces needs to know about the row, worked out once (no rotary keys here).
+// What the routing of a row's 16-byte pieces needs to know about the row, worked out once.
 struct RowRoute {
   bool ok;
-  long long slot, slot2, base_row;
+  long long slot, slot2, base_row, pos;
   unsigned long long mask;
+  template <bool ROPE>
   __device__ __forceinline__ void init(const GemmParams& p, int gm) {
     ok = gm < p.M;
     slot = 0; slot2 = -1;
@@ -515,6 +573,22 @@ struct RowRoute {
       if (slot2 >= p.n_blocks * PAGE) { atomicOr(p.status, StatusBits::BAD_INDEX); slot2 = -1; }
     }
     base_row = (((slot / PAGE) * p.n_kv * PAGE) + (slot % PAGE)) << p.hd_shift;
+    pos = 0;
+    if constexpr (ROPE) {
+      if (ok) { pos = rope_pos(p, gm); ok = pos >= 0; }
+    }
+  }
+  // rotates eight columns of the lower half of a key head (gc .. gc + 7) and their partners
+  __device__ __forceinline__ void rotate8(const GemmParams& p, int gc, float (&lo)[8], float (&hi)[8]) const {
+    if (!ok) return;
+    const float4* cs = p.rope + pos * (p.hd / 4) + (gc & (p.hd - 1)) / 2;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 t = __ldg(cs + k);
+      const float l0 = lo[2 * k], l1 = lo[2 * k + 1], h0 = hi[2 * k], h1 = hi[2 * k + 1];
+      lo[2 * k] = l0 * t.x - h0 * t.y; lo[2 * k + 1] = l1 * t.z - h1 * t.w;
+      hi[2 * k] = h0 * t.x + l0 * t.y; hi[2 * k + 1] = h1 * t.z + l1 * t.w;
+    }
   }
   // columns gc .. gc + 7 of the call's output (gc is the same in every lane: the branches are warp-uniform)
   __device__ __forceinline__ void store8(const GemmParams& p, int gc, const float (&v8)[8]) const {
@@ -542,6 +616,7 @@ struct RowRoute {
   }
 };
 
+template <bool ROPE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 proj_gemm_splitk_push_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const GemmParams p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -553,7 +628,7 @@ proj_gemm_splitk_push_kernel(const __grid_constant__ CUtensorMap map_x, const __
   const int KS = gridDim.x, rank = blockIdx.x;           // the cluster spans grid.x
   const int b_bytes = p.BN * GEMM_BK * 2;
   const int stage_bytes = GEMM_A_BYTES + b_bytes;
-  const int cw = (((p.BN + KS - 1) / KS) + 7) / 8 * 8;   // columns finished by one block (a multiple of 8)
+  const int cw = merge_slice_cols<ROPE>(p.BN, KS);       // columns finished by one block (a multiple of 8 or 16)
   const int XS = cw + 4;                                 // row stride (floats) inside a slice: conflict-free row-per-thread access
   const int slice_bytes = GEMM_BM * XS * 4;              // a multiple of 16
   const bool direct = p.direct_send != 0;               // the same in every block
@@ -651,7 +726,7 @@ proj_gemm_splitk_push_kernel(const __grid_constant__ CUtensorMap map_x, const __
       asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(remote) : "memory");
     }
     RowRoute route;
-    route.init(p, m0 + row);
+    route.template init<ROPE>(p, m0 + row);
     const uint32_t trow = tmem_base + (static_cast<uint32_t>(lane_base) << 16);
     // ---- the peers' slices, one after the other: TMEM (lane = row) -> shared memory fp32 [slot][128][XS] (slot = the
     //      peer's rank with the own rank left out), then one bulk copy into the peer's receive area while the next
@@ -667,8 +742,8 @@ proj_gemm_splitk_push_kernel(const __grid_constant__ CUtensorMap map_x, const __
       int c = 0;
       for (; c + 32 <= vw; c += 32) {
         uint32_t r0[16], r1[16];
-        tmem_ld16(trow + c_lo + c, r0);
-        tmem_ld16(trow + c_lo + c + 16, r1);
+        tmem_ld_pieces<ROPE>(p, trow, n0, c_lo + c, r0);
+        tmem_ld_pieces<ROPE>(p, trow, n0, c_lo + c + 16, r1);
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
         if (live) {
 #pragma unroll
@@ -680,7 +755,7 @@ proj_gemm_splitk_push_kernel(const __grid_constant__ CUtensorMap map_x, const __
       }
       for (; c + 8 <= vw; c += 8) {
         uint32_t r[8];
-        tmem_ld8(trow + c_lo + c, r);
+        tmem_ld8(trow + merge_col<ROPE>(p, n0, c_lo + c), r);
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
         if (live) {
           st_async_b32x4(dst + c * 4, r[0], r[1], r[2], r[3], bar);
@@ -695,8 +770,8 @@ proj_gemm_splitk_push_kernel(const __grid_constant__ CUtensorMap map_x, const __
       int c = 0;
       for (; c + 32 <= vw; c += 32) {
         uint32_t r0[16], r1[16];
-        tmem_ld16(trow + c_lo + c, r0);
-        tmem_ld16(trow + c_lo + c + 16, r1);
+        tmem_ld_pieces<ROPE>(p, trow, n0, c_lo + c, r0);
+        tmem_ld_pieces<ROPE>(p, trow, n0, c_lo + c + 16, r1);
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -706,7 +781,7 @@ proj_gemm_splitk_push_kernel(const __grid_constant__ CUtensorMap map_x, const __
       }
       for (; c + 8 <= vw; c += 8) {
         uint32_t r[8];
-        tmem_ld8(trow + c_lo + c, r);
+        tmem_ld8(trow + merge_col<ROPE>(p, n0, c_lo + c), r);
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
         *reinterpret_cast<uint4*>(drow + c) = make_uint4(r[0], r[1], r[2], r[3]);
         *reinterpret_cast<uint4*>(drow + c + 4) = make_uint4(r[4], r[5], r[6], r[7]);
@@ -729,54 +804,81 @@ proj_gemm_splitk_push_kernel(const __grid_constant__ CUtensorMap map_x, const __
     mbar_wait_cluster(recv_bar, 0, p.status);
     {
       const int c_lo = rank * cw, vw = min(cw, p.BN - c_lo);
-      const bool wide = KS <= GEMM_PUSH_MAX_KS;         // 16 columns at a time while the peers' pieces fit in registers
-      for (int c = 0; c + 8 <= vw; c += wide ? 16 : 8) {
-        const bool two = wide && c + 16 <= vw;          // 8 at a ragged end (the same in every lane)
+      // 16 columns at a time (8 at a ragged end), the peers' pieces of both halves in registers while that many fit
+      const bool wide = KS <= GEMM_PUSH_MAX_KS;
+      for (int c = 0; c + 8 <= vw; c += 16) {
+        const bool two = c + 16 <= vw;                  // the same in every lane
         uint32_t own[16];
         if (two) {
-          tmem_ld16(trow + c_lo + c, own);
+          tmem_ld_pieces<ROPE>(p, trow, n0, c_lo + c, own);
         } else {
           uint32_t o8[8];
-          tmem_ld8(trow + c_lo + c, o8);
+          tmem_ld8(trow + merge_col<ROPE>(p, n0, c_lo + c), o8);
 #pragma unroll
           for (int q = 0; q < 8; ++q) { own[q] = o8[q]; own[8 + q] = 0u; }
         }
-        float4 pr[GEMM_MAX_KS - 1][4];
+        float4 pr[GEMM_MAX_KS - 1][2], pr2[GEMM_PUSH_MAX_KS - 1][2];
+        auto fetch = [&](int h) {                       // the peers' eight columns of this row, half h
 #pragma unroll
-        for (int j = 0; j < GEMM_MAX_KS - 1; ++j) {
-          if (j < KS - 1) {
-            const float* src = recv + ((size_t)j * GEMM_BM + row) * XS + c;
-            pr[j][0] = *reinterpret_cast<const float4*>(src);
-            pr[j][1] = *reinterpret_cast<const float4*>(src + 4);
-            if (j < GEMM_PUSH_MAX_KS - 1) {
-              if (two) { pr[j][2] = *reinterpret_cast<const float4*>(src + 8); pr[j][3] = *reinterpret_cast<const float4*>(src + 12); }
+          for (int j = 0; j < GEMM_MAX_KS - 1; ++j) {
+            if (j < KS - 1) {
+              const float* src = recv + ((size_t)j * GEMM_BM + row) * XS + c + 8 * h;
+              pr[j][0] = *reinterpret_cast<const float4*>(src);
+              pr[j][1] = *reinterpret_cast<const float4*>(src + 4);
+            }
+          }
+        };
+        fetch(0);
+        if (wide && two) {
+#pragma unroll
+          for (int j = 0; j < GEMM_PUSH_MAX_KS - 1; ++j) {
+            if (j < KS - 1) {
+              const float* src = recv + ((size_t)j * GEMM_BM + row) * XS + c + 8;
+              pr2[j][0] = *reinterpret_cast<const float4*>(src);
+              pr2[j][1] = *reinterpret_cast<const float4*>(src + 4);
             }
           }
         }
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        float v8[2][8];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           if (h == 1 && !two) break;
-          float v8[8];
+          if (h == 1) {
+            if (wide) {
 #pragma unroll
-          for (int q = 0; q < 8; ++q) v8[q] = 0.f;
+              for (int j = 0; j < GEMM_PUSH_MAX_KS - 1; ++j) { pr[j][0] = pr2[j][0]; pr[j][1] = pr2[j][1]; }
+            } else {
+              fetch(1);
+            }
+          }
+          float (&v)[8] = v8[h];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v[q] = 0.f;
           // rank order: slot j of the receive area holds rank j (j < own rank) or j + 1, so the own slice goes in
           // just before slot `rank` (or last)
           auto add_own = [&]() {
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v8[q] += __uint_as_float(own[8 * h + q]);
+            for (int q = 0; q < 8; ++q) v[q] += __uint_as_float(own[8 * h + q]);
           };
 #pragma unroll
           for (int j = 0; j < GEMM_MAX_KS - 1; ++j) {
-            if (j < KS - 1 && (h == 0 || j < GEMM_PUSH_MAX_KS - 1)) {
+            if (j < KS - 1) {
               if (j == rank) add_own();
-              const float4 a = pr[j][h == 0 ? 0 : 2], b = pr[j][h == 0 ? 1 : 3];
-              v8[0] += a.x; v8[1] += a.y; v8[2] += a.z; v8[3] += a.w; v8[4] += b.x; v8[5] += b.y; v8[6] += b.z; v8[7] += b.w;
+              const float4 a = pr[j][0], b = pr[j][1];
+              v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w; v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
             }
           }
           if (rank == KS - 1) add_own();
-          const int gc = n0 + c_lo + c + 8 * h;
-          if (gc < p.N_out) route.store8(p, gc, v8);
+        }
+        const int gc0 = n0 + merge_col<ROPE>(p, n0, c_lo + c);
+        if constexpr (ROPE) {
+          if (n0 + c_lo + c < (p.n_kv << p.hd_shift)) route.rotate8(p, gc0, v8[0], v8[1]);   // (key slices are multiples of 16)
+        }
+        if (gc0 < p.N_out) route.store8(p, gc0, v8[0]);
+        if (two) {
+          const int gc1 = n0 + merge_col<ROPE>(p, n0, c_lo + c + 8);
+          if (gc1 < p.N_out) route.store8(p, gc1, v8[1]);
         }
       }
     }

@@ -93,6 +93,49 @@ def test_projection_rotates_keys_only(px, hd, n_kv, M):
     assert (L.cache.lr_k[0] == 0).all() and (L.cache.lr_v[0] == 0).all()
 
 
+@pytest.mark.parametrize("ks,direct,hd,n_kv,M", [
+    (8, "0", 128, 4, 130), (8, "0", 64, 3, 70), (7, "0", 128, 2, 200), (6, "0", 64, 4, 129), (5, "0", 128, 3, 257),   # pulling merge
+    (8, "1", 128, 2, 41), (7, "1", 64, 1, 64), (6, "2", 128, 1, 150),                                              # direct sends
+    (4, "1", 128, 4, 300), (3, "1", 64, 4, 200), (3, "1", 128, 1, 128), (2, "1", 128, 2, 513)])                    # bulk sends
+def test_split_projection_rotates_keys(px, monkeypatch, ks, direct, hd, n_kv, M):
+    """Rotary epilogue of the split-K projections: a head's two halves meet in one slice of the merge, at slice widths that
+    do and do not divide the tile (ks = 3, 5, 6, 7: 96, 64, 48, 48 columns).  Base-only and fused calls agree bit for bit."""
+    from paper_2609_34054_b200.binding import Precc
+    monkeypatch.setenv("PRECC_GEMM_KS_MAX", str(ks))
+    monkeypatch.setenv("PRECC_GEMM_DIRECT", direct)
+    p = Precc(0)
+    geo = I.Geometry(d_model=1088, n_q=2 * n_kv, n_kv=n_kv, hd=hd, n_agents=3, rank_k=16, rank_v=16, alpha=32.0)
+    L = Layer(p, geo, seed=13, n_blocks=(M + 15) // 16 + 1, tag="rs", fill=0.0)
+    H = I.hidden_states(M, geo, 13, "rs.H")
+    table, (cos, sin) = rope_table(2048, hd), O.rope_tables(2048, hd)
+    pos = I.uniform_int(0, 2047, M, 13, "rs.pos").to(torch.int32)
+    p.rebase_project_rope(L.desc, H.cuda(), L.W_packed, L.cache, table, 0, positions=pos.cuda())
+    p.lr_precompute(L.desc, H.cuda(), L.A_packed, L.cache, 0)
+    torch.cuda.synchronize()
+    two = [t.clone() for t in (L.cache.k_base, L.cache.v_base, L.cache.lr_k, L.cache.lr_v)]
+    # fp32 sums of d_model products of order 0.02, rotated, one bf16 rounding
+    ref = O.rope_rotate(O.base_cache(f64(H), L.w_np["W_k"]), pos.numpy(), n_kv, cos, sin)
+    assert (np.abs(base_rows(two[0])[:M] - ref) <= 2.0 ** -8 * np.abs(ref) + 2e-3).all()
+    refv = O.base_cache(f64(H), L.w_np["W_v"])
+    assert (np.abs(base_rows(two[1])[:M] - refv) <= 2.0 ** -8 * np.abs(refv) + 2e-3).all()
+    for t in (L.cache.k_base, L.cache.v_base, L.cache.lr_k, L.cache.lr_v):
+        t.zero_()
+    WA = p.pack_turn_weights(geo, *(L.w[k].cuda() for k in ("W_k", "W_v", "A_k", "A_v")))
+    p.turn_project_rope(L.desc, H.cuda(), WA, L.cache, table, 0, positions=pos.cuda())
+    torch.cuda.synchronize()
+    for a, b in zip((L.cache.k_base, L.cache.v_base, L.cache.lr_k, L.cache.lr_v), two):
+        assert torch.equal(a, b)
+    # a position outside the table: reported, that row not written
+    bad = pos.clone()
+    bad[M // 2] = 2048
+    L.cache.k_base.zero_()
+    p.rebase_project_rope(L.desc, H.cuda(), L.W_packed, L.cache, table, 0, positions=bad.cuda())
+    torch.cuda.synchronize()
+    assert p.poll_status() == 1
+    assert (base_rows(L.cache.k_base)[M // 2] == 0).all() and (base_rows(L.cache.k_base)[M // 2 - 1] != 0).any()
+    p.close()
+
+
 SHAPES = [
     # hd, n_q, n_kv, rank, T, agents
     (64, 8, 2, 16, 70, 2),
