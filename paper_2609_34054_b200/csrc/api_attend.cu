@@ -255,8 +255,14 @@ static int32_t prefill_entry(precc_ctx* ctx, const precc_layer_desc* desc, const
     long long gx = 2ll * ctx->sm_count / groups;          // two resident blocks per SM: each walks its share of the cache blocks
     if (gx < 1) gx = 1;
     if (gx > out_blocks) gx = out_blocks;
-    kern<<<dim3((unsigned)gx, (unsigned)groups), RX_THREADS, xs, (cudaStream_t)stream>>>(x);
-    PRECC_CUDA(ctx, cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)gx, (unsigned)groups); cfg.blockDim = dim3(RX_THREADS);
+    cfg.dynamicSmemBytes = xs; cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, x));
     return PRECC_OK;
   };
   int32_t xrc;

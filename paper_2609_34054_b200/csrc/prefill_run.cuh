@@ -193,10 +193,12 @@ struct PrefillRun {
     cfg.blockDim = dim3(PTC_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = a.stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = ns;
-    cfg.attrs = attr; cfg.numAttrs = ns > 1 ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = ns;
+    cfg.attrs = attr; cfg.numAttrs = ns > 1 ? 2 : 1;
     PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, m, p));
     return PRECC_OK;
   }

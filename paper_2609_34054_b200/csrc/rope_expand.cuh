@@ -129,6 +129,7 @@ rope_expand_keys_kernel(const RopeExpandParams p) {
       for (int h = 0; h < 2; ++h)
         x.cs[t][h] = __ldg(p.rope + (size_t)min(t0 + r + 8 * h, p.max_pos - 1) * (hd / 4) + (tc0 + t * 8 + q2) / 2);
   };
+  pdl_wait();                  // the kernel ahead may have written cache rows of this sequence
   In cur;
   int lb = blockIdx.x;
   if (lb < p.n_out_blocks) fetch(lb, cur);
