@@ -215,9 +215,9 @@ int32_t precc_workspace_init(precc_ctx* ctx, void* workspace, size_t workspace_b
  *                 ctx_len [B] >= 1 (a request with ctx_len < 1 gets zeros)
  *   block_table   [B][table_stride] logical block -> physical block, or NULL
  *   first_block   [B] physical block of logical block 0 when block_table is NULL (NULL = 0 for all)
- *   max_ctx       HOST upper bound on every ctx_len[b]; with B and the SM count it fixes the split of
+ *   max_ctx       HOST upper bound on every ctx_len[b]; with B, ctx_len and the SM count it fixes the split of
  *                 the context across thread blocks, so results are bit-identical for any block
- *                 placement given the same (B, max_ctx)
+ *                 placement given the same (B, max_ctx, ctx_len)
  *   B_k, B_v      [n_agents][rank][n_kv_heads*head_dim]
  * A request whose ctx_len exceeds max_ctx is rejected on the device: zeros, PRECC_STATUS_BAD_INDEX.
  * B == 0 is a no-op.

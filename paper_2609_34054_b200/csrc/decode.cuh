@@ -27,7 +27,8 @@
 //                   receives in rank order.  No global scratch, no atomics: the short-latency path for small
 //                   batches.
 //   ticket kernel   blocks publish their result to a global workspace; the last block to finish a
-//                   (b, g) (atomic ticket) merges the records in split order.  Any number of splits.
+//                   (b, g) (atomic ticket) merges the records in split order.  Any number of splits, planned by the
+//                   host from the bound on the lengths or (flat grid) by each block from the lengths themselves.
 // The ticket path never waits on another block.  In the cluster path a block waits (bounded, on its own
 // mbarrier) for the sends of blocks that are co-scheduled with it by the hardware.
 #pragma once
@@ -48,7 +49,7 @@ struct DecodeParams {
   const __nv_bfloat16* lr_v;
   const __nv_bfloat16* B_k;
   const __nv_bfloat16* B_v;
-  float* part;        // ticket kernel: [B][n_kv][max_splits][PART_STRIDE]
+  float* part;        // ticket kernel: records [PART_STRIDE] of the splits, [B][n_kv][max_splits] or one per block (flat grid)
   int32_t* tickets;   // ticket kernel: [B][n_kv], zero between calls
   float* raw;         // partial-output mode (ticket kernel): [B][n_kv][PART_STRIDE] records instead of `out`, or null
   uint32_t* status;
@@ -60,6 +61,8 @@ struct DecodeParams {
   int table_stride;
   int n_q, n_kv, group, n_agents;
   int chunk_tiles, max_splits, stages;
+  int B;                       // requests of the call
+  int even;                    // cluster kernel: 1 = each request's own pages shared out evenly, 0 = chunk_tiles for every block
   int pre_stages;              // ring slots a warp fills before it waits for the preceding kernel (the rest follow the wait)
   int max_ctx;                 // the host's bound on ctx_len[b]: it sized the grid, the split and the block table
   float scale_log2, s_k, s_v;
@@ -67,6 +70,7 @@ struct DecodeParams {
 
 constexpr int DEC_WARPS = 4;            // ticket kernel
 constexpr int DEC_MAX_SPLITS = 512;
+constexpr int DEC_FLAT_MAX_B = 256;     // requests that the flat grid's schedule handles (8 per lane)
 constexpr int DEC_MAX_CLUSTER = 16;
 // Overlap with the preceding kernel (programmatic dependent launch): before the kernel waits for its
 // predecessor it already reads the index arrays, the adapter matrices and every cache page that holds
@@ -724,8 +728,79 @@ __device__ __forceinline__ void decode_stream_block(const DecodeParams& p, unsig
 }
 
 // ------------------------------------------------------------------------------------------------
-// Ticket kernel: grid (split, kv head, request), DEC_WARPS warps.
-template <int HD, int RK, int RV, bool ROPE = false>
+// Schedule of the ticket kernel's flat grid (a template variant of its own: the kernel sits at its register limit).  The host knows a bound on the lengths only; a split planned for the longest
+// request leaves most of the machine idle when the others are shorter (64 units of 2000 .. 16000 tokens: 166 of 296
+// block slots in use).  So every block works the split out from the lengths themselves: the smallest chunk for which
+// the splits of all requests fit into the grid, evened out within each request.  Depends on the call's lengths and grid
+// only, so results do not depend on timing or block placement.  About 0.5 us per block, before the wait for the kernel ahead.
+struct FlatShare { int b, g, split, n_splits, first, chunk; };   // `first`: index of the request's first split among all
+__device__ __forceinline__ FlatShare flat_schedule(const DecodeParams& p, int n_blocks, int blk) {
+  const int lane = threadIdx.x & 31;
+  constexpr int K = DEC_FLAT_MAX_B / 32;
+  int nt[K];                                             // pages of requests lane, lane + 32, ...; a rejected request counts as one
+  int tot = 0, mx = 1;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    nt[k] = 0;
+    if (k * 32 < p.B) {
+      const int b = k * 32 + lane;
+      if (b < p.B) {
+        const int c = __ldg(p.ctx_len + b);
+        nt[k] = c >= 1 && c <= p.max_ctx ? (c + PAGE - 1) / PAGE : 1;
+      }
+      tot += nt[k];
+      mx = max(mx, nt[k]);
+    }
+  }
+  tot = __reduce_add_sync(0xffffffffu, tot);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  const int cap = n_blocks / p.n_kv;                     // splits that fit (the host sees to cap >= B)
+  auto splits = [&](int n, int c) -> int { return (int)((unsigned)(n + c - 1) / (unsigned)c); };
+  auto count = [&](int c) -> int {
+    int s = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (k * 32 < p.B) s += splits(nt[k], c);
+    return __reduce_add_sync(0xffffffffu, s);
+  };
+  int lo = max(max(DEC_WARPS, (tot + cap - 1) / cap), (mx + DEC_MAX_SPLITS - 1) / DEC_MAX_SPLITS), hi = max(lo, mx);
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (count(mid) <= cap) hi = mid; else lo = mid + 1;
+  }
+  const int u = blk / p.n_kv;
+  FlatShare r{-1, blk - u * p.n_kv, 0, 0, 0, 1};
+  int base = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    if (k * 32 < p.B) {
+      const int s = splits(nt[k], lo);
+      int inc = s;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += up;
+      }
+      const uint32_t hit = __ballot_sync(0xffffffffu, u >= base + inc - s && u < base + inc);
+      if (hit) {
+        const int o = __ffs(hit) - 1;
+        const int n = __shfl_sync(0xffffffffu, nt[k], o);
+        r.b = k * 32 + o;
+        r.n_splits = __shfl_sync(0xffffffffu, s, o);
+        r.first = base + __shfl_sync(0xffffffffu, inc, o) - r.n_splits;
+        r.split = u - r.first;
+        r.chunk = (n + r.n_splits - 1) / r.n_splits;     // even shares; still n_splits of them
+      }
+      base += __shfl_sync(0xffffffffu, inc, 31);
+    }
+  }
+  return r;
+}
+
+// ------------------------------------------------------------------------------------------------
+// Ticket kernel: flat grid (see above), or grid (split, kv head, request) planned from the bound alone (more requests
+// than the schedule handles, or one block per unit); DEC_WARPS warps.
+template <int HD, int RK, int RV, bool ROPE, bool FLAT>
 __global__ void __launch_bounds__(DEC_WARPS * 32)
 lr_attend_decode_kernel(const DecodeParams p) {
   using C = DecodeCfg<HD, RK, RV>;
@@ -736,11 +811,16 @@ lr_attend_decode_kernel(const DecodeParams p) {
   constexpr int NT = DEC_WARPS * 32;
   extern __shared__ __align__(128) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
+  FlatShare f;
+  if constexpr (FLAT) f = flat_schedule(p, (int)gridDim.x, (int)blockIdx.x);
+  const int split = FLAT ? f.split : blockIdx.x, g = FLAT ? f.g : blockIdx.y, b = FLAT ? f.b : blockIdx.z;
   const int G = p.group;
   const int cta_lin = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
   const DecodeTrace mark{p.trace ? p.trace + (size_t)cta_lin * 16 : nullptr};
   mark(0);
+  if constexpr (FLAT) {
+    if (f.b < 0) return;                       // more blocks than splits
+  }
   // The index arrays are read before the wait for the preceding kernel (see DEC_PDL_TAIL): they are inputs
   // of the whole call chain, not something the kernel just before this one produces.
   const int ctx = __ldg(p.ctx_len + b);
@@ -766,10 +846,10 @@ lr_attend_decode_kernel(const DecodeParams p) {
     return;
   }
   const int n_tiles = (ctx + PAGE - 1) / PAGE;
-  const int n_splits = (n_tiles + p.chunk_tiles - 1) / p.chunk_tiles;
+  const int n_splits = FLAT ? f.n_splits : (n_tiles + p.chunk_tiles - 1) / p.chunk_tiles;
   if (split >= n_splits) return;
-  const int tile0 = split * p.chunk_tiles;
-  const int tile_end = min(n_tiles, tile0 + p.chunk_tiles);
+  const int tile0 = split * (FLAT ? f.chunk : p.chunk_tiles);
+  const int tile_end = min(n_tiles, tile0 + (FLAT ? f.chunk : p.chunk_tiles));
   mark(1);
   if (ROPE && ctx > p.max_pos && threadIdx.x == 0) atomicOr(p.status, StatusBits::BAD_INDEX);   // positions are clamped
   decode_stream_block<HD, RK, RV, DEC_WARPS, ROPE>(p, smem, b, g, ctx, agent, use_lr, tile0, tile_end, mark);
@@ -793,7 +873,7 @@ lr_attend_decode_kernel(const DecodeParams p) {
   __shared__ float fin_l[8];
   __shared__ float fin_m[8];
   if (n_splits > 1) {
-    float* rec = p.part + (((size_t)b * p.n_kv + g) * p.max_splits + split) * C::PART_STRIDE;
+    float* rec = p.part + (FLAT ? (size_t)(f.first + split) * p.n_kv + g : ((size_t)b * p.n_kv + g) * p.max_splits + split) * C::PART_STRIDE;
     for (int i = threadIdx.x; i < rec_f / 4; i += NT)
       reinterpret_cast<float4*>(rec)[i] = reinterpret_cast<const float4*>(res)[i];
     __syncthreads();
@@ -812,7 +892,8 @@ lr_attend_decode_kernel(const DecodeParams p) {
     // The last block merges all splits in split order, so the result does not depend on which
     // block that is.  Records (and the B_v slice) are staged with one batch of async copies, so the
     // L2 round trip is paid once.
-    const float* base = p.part + (((size_t)b * p.n_kv + g) * p.max_splits) * C::PART_STRIDE;
+    const float* base = p.part + (FLAT ? (size_t)f.first * p.n_kv + g : ((size_t)b * p.n_kv + g) * p.max_splits) * C::PART_STRIDE;
+    const size_t rstep = (size_t)(FLAT ? p.n_kv : 1) * C::PART_STRIDE;    // from one split's record to the next
     float* recs = res + 16 + 8 * OW;                    // [n_splits][rec_f] (staged) or [n_splits][16]
     const bool staged = (16 + 8 * OW + n_splits * rec_f + DEC_WARPS * n_el) * 4 + bv_bytes <= region;
     if (!raw_out) stage_bv();
@@ -820,11 +901,11 @@ lr_attend_decode_kernel(const DecodeParams p) {
       const int cpr = rec_f / 4;                        // 16-byte chunks per record
       for (int c = threadIdx.x; c < n_splits * cpr; c += NT) {
         const int s2 = c / cpr, ch = c % cpr;
-        cp_async16(smem_u32(recs) + c * 16, base + (size_t)s2 * C::PART_STRIDE + ch * 4, 16);
+        cp_async16(smem_u32(recs) + c * 16, base + (size_t)s2 * rstep + ch * 4, 16);
       }
     } else {
       for (int i = threadIdx.x; i < n_splits * 16; i += NT)
-        recs[i] = __ldcg(base + (size_t)(i >> 4) * C::PART_STRIDE + (i & 15));
+        recs[i] = __ldcg(base + (size_t)(i >> 4) * rstep + (i & 15));
     }
     cp_async_commit();
     cp_async_wait<0>();
@@ -859,7 +940,7 @@ lr_attend_decode_kernel(const DecodeParams p) {
       float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
       auto fetch = [&](int s2) -> float4 {
         if (staged) return *reinterpret_cast<const float4*>(recs + (size_t)s2 * rec_f + 16 + col * 4);
-        return __ldcg(reinterpret_cast<const float4*>(base + (size_t)s2 * C::PART_STRIDE + 16 + col * 4));
+        return __ldcg(reinterpret_cast<const float4*>(base + (size_t)s2 * rstep + 16 + col * 4));
       };
       int s2 = qd;
       for (; s2 + 4 < n_splits; s2 += 8) {
@@ -967,8 +1048,9 @@ lr_attend_decode_cluster_kernel(const DecodeParams p) {
     return;
   }
   const int n_tiles = (ctx + PAGE - 1) / PAGE;
-  const int tile0 = min(n_tiles, rank * p.chunk_tiles);
-  const int tile_end = min(n_tiles, tile0 + p.chunk_tiles);
+  const int chunk = p.even ? (n_tiles + CS - 1) / CS : p.chunk_tiles;
+  const int tile0 = min(n_tiles, rank * chunk);
+  const int tile_end = min(n_tiles, tile0 + chunk);
   mark(1);
   // Columns of the merged record that are divided over the blocks: the head dimension (the LR-V coordinates are
   // spent inside each block), or the whole record in partial-output mode (no B_v there).

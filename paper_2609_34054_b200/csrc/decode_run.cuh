@@ -7,101 +7,9 @@
 namespace precc {
 
 // Split schedule of decode.  cluster > 0: the cluster kernel with that many blocks per (request, kv head);
-// otherwise the ticket kernel with up to max_splits blocks per (request, kv head).
-struct DecodePlan { int cluster, warps, chunk_tiles, max_splits, stages, smem, deep; };
-
-// `extra`: bytes of shared memory appended after the usual layout (the rotary variant's B_k slice).
-template <int HD, int RK, int RV>
-DecodePlan plan_ticket(int sm_count, int max_smem, int B, int n_kv, int max_ctx, int extra = 0) {
-  using C = DecodeCfg<HD, RK, RV>;
-  DecodePlan pl{};
-  // ring depth: as deep as possible (<= 4) while two blocks still fit on an SM
-  int stages = 4;
-  while (stages > 2 && 2 * (C::ticket_smem(stages) + extra + 1024) > max_smem) --stages;
-  pl.stages = stages;
-  pl.smem = C::ticket_smem(stages) + extra;
-  const int per_sm = (2 * (pl.smem + 1024) <= max_smem) ? 2 : 1;
-  const long long slots = (long long)sm_count * per_sm;
-  const int max_tiles = (max_ctx + PAGE - 1) / PAGE;
-  const long long units = (long long)B * n_kv;
-  // blocks per (request, kv head): fill the machine once; with plenty of work use 4 waves of
-  // blocks so that requests of different length balance out
-  long long want = slots / units;                       // rounded down: one full wave, never a wave and a bit
-  if (want < 1) want = 1;
-  const long long total_tiles = units * max_tiles;
-  if (total_tiles >= slots * 4 * 64) want = (4 * slots + units - 1) / units;
-  int chunk = (int)((max_tiles + want - 1) / want);
-  if (chunk < DEC_WARPS) chunk = DEC_WARPS;
-  if ((max_tiles + chunk - 1) / chunk > DEC_MAX_SPLITS) chunk = (max_tiles + DEC_MAX_SPLITS - 1) / DEC_MAX_SPLITS;
-  pl.chunk_tiles = chunk;
-  pl.max_splits = (max_tiles + chunk - 1) / chunk;
-  return pl;
-}
-
-// Warps of a cluster-schedule block when two blocks share an SM (8 if a two-page ring per warp fits, else 4).
-template <int HD, int RK, int RV>
-int two_per_sm_warps(int max_smem, int extra) {
-  return DecodeCfg<HD, RK, RV>::cluster_smem(8, 2) <= max_smem / 2 - 1024 - extra ? 8 : 4;
-}
-
-// The cluster kernel serves the latency-bound regime: few (request, kv head) units, each worth
-// splitting, the whole grid co-resident in one wave.  Returns cluster = 0 when it does not apply.
-template <int HD, int RK, int RV>
-DecodePlan plan_cluster(int sm_count, int max_smem, int B, int n_kv, int max_ctx, int extra = 0, bool deep_ok = true) {
-  using C = DecodeCfg<HD, RK, RV>;
-  DecodePlan pl{};
-  const int max_tiles = (max_ctx + PAGE - 1) / PAGE;
-  const long long units = (long long)B * n_kv;
-  if (units * 2 > sm_count || max_tiles <= 16) return pl;  // too many units, or nothing worth splitting
-  // two blocks per SM must fit (a 16-block cluster needs 16 free slots inside one GPC, and not every
-  // GPC has 16 SMs): 8 warps with a 2-deep ring if that fits, else 4 warps with the deepest ring that does
-  const int budget = max_smem / 2 - 1024 - extra;
-  int warps = 8, stages = 8;
-  while (stages > 2 && C::cluster_smem(8, stages) > budget) --stages;
-  if (C::cluster_smem(8, stages) > budget) {
-    warps = 4; stages = 8;
-    while (stages > 2 && C::cluster_smem(4, stages) > budget) --stages;
-    if (C::cluster_smem(4, stages) > budget) return pl;
-  }
-  // as many blocks per unit as keep the whole grid in one wave (any size up to 16, not only powers of two:
-  // 3 requests x 8 heads take 6 blocks each = 144 blocks, where 4 would leave a third of the SMs idle)
-  int cs = DEC_MAX_CLUSTER;
-  if ((long long)cs * units > sm_count) cs = (int)(sm_count / units);
-  if (cs * warps > max_tiles) cs = max_tiles / warps;
-  if (cs < 2) return pl;
-  // Wide clusters (very few units) with more than a few pages per warp: one block per SM with the whole
-  // shared memory as page rings, i.e. two to three times the bytes in flight per SM and fewer dependent DRAM
-  // round trips per warp; the run-time occupancy check then shrinks the cluster until all clusters are
-  // resident (a 16-block cluster at one block per SM does not fit every GPC).  Measured against the
-  // two-blocks-per-SM layout: 8192 tokens x 8 units 9.3 -> 9.0 us, 32768 tokens 31 -> 27 us, 65536 tokens
-  // 53 -> 46 us.  With the deep rings switched off, bandwidth-bound sizes go to the ticket kernel instead.
-  // Narrow clusters over a lot of data (e.g. 8 requests x 8 kv heads x 32768 tokens: clusters of 2): the work is
-  // bandwidth-bound and the ticket kernel, which spreads it over every SM, is faster (rotary keys: 252 against 350 us).
-  if (units * max_tiles > 32768 && cs <= 4) return pl;
-  // Wide pages (head_dim 128 with rank 32 or 64) leave the two-blocks-per-SM layout only 4 warps with 2-page
-  // rings; narrow clusters of such blocks lose to the ticket kernel's larger grid from a few thousand pages on
-  // (rank 32, 8192 tokens, 4..8 requests: 35..58 us against 33..51 us; ranks 8 and 16 keep three-page rings and win).
-  if (warps == 4 && stages == 2 && cs <= 4 && units * max_tiles >= 6000) return pl;
-  if (units * max_tiles > (deep_ok ? 2048 : 32768) && cs > 4) {
-    if (!deep_ok) return pl;
-    const int big = max_smem - 2048 - extra;
-    warps = 8; stages = 4;
-    while (stages > 2 && C::cluster_smem(8, stages) > big) --stages;
-    if (C::cluster_smem(8, stages) > big) {
-      warps = 4; stages = 4;
-      while (stages > 2 && C::cluster_smem(4, stages) > big) --stages;
-      if (C::cluster_smem(4, stages) > big) return pl;
-    }
-    pl.deep = 1;
-  }
-  pl.cluster = cs;
-  pl.warps = warps;
-  pl.stages = stages;
-  pl.smem = C::cluster_smem(warps, stages) + extra;
-  pl.chunk_tiles = (max_tiles + cs - 1) / cs;
-  pl.max_splits = cs;
-  return pl;
-}
+// otherwise the ticket kernel - on a flat grid of `flat` blocks, or (flat == 0) with up to max_splits blocks per (request,
+// kv head).
+struct DecodePlan { int cluster, warps, chunk_tiles, max_splits, stages, smem, deep, flat, even; };
 
 template <int HD, int RK, int RV, bool ROPE = false>
 struct DecodeRunT {
@@ -110,31 +18,29 @@ struct DecodeRunT {
   // of them still fit on an SM at the shallowest ring, so that the planner's blocks-per-SM figure is the same.
   static_assert(!ROPE || 2 * (DecodeCfg<HD, RK, RV>::ticket_smem(2) + DecodeCfg<HD, RK, RV>::BK_BYTES + 128 + 1024) <= 232448,
                 "rotary ticket blocks must fit two per SM, or the workspace bound of the plain kernel no longer covers them");
-  // exact need of one call
-  static size_t ws_need(int B, int n_kv, int max_splits) {
+  // exact need of one call: arrival counters and one record per block
+  static size_t ws_need(int B, int n_kv, long long records) {
     const size_t tickets = ((size_t)B * n_kv * 4 + 255) / 256 * 256;
-    return tickets + (size_t)B * n_kv * max_splits * DecodeCfg<HD, RK, RV>::PART_STRIDE * 4;
+    return tickets + (size_t)records * DecodeCfg<HD, RK, RV>::PART_STRIDE * 4;
   }
-  // Upper bound over EVERY call with at most B requests of at most max_ctx tokens (a smaller batch gets more
-  // splits per request, so the need is not monotone in B).  Mirrors plan_ticket: splits <= blocks wanted per
-  // unit, splits <= pages / DEC_WARPS, and the four-wave mode can only switch on as the context grows.
+  static int ticket_per_sm(int stages, int max_smem, int extra) {
+    const int n = max_smem / (DecodeCfg<HD, RK, RV>::ticket_smem(stages) + extra + 1024);
+    return n > 2 ? 2 : (n < 1 ? 1 : n);
+  }
+  // Upper bound over EVERY call with at most B requests of at most max_ctx tokens (a smaller batch may get more splits per
+  // request, so the need is not monotone in B).  Mirrors plan_flat: one wave of blocks, or four, which can only switch on
+  // as the context grows; never more splits of a request than a DEC_WARPS-th of its pages.
   static size_t ws_bytes(int sm_count, int max_smem, int B, int n_kv, int max_ctx) {
-    using C = DecodeCfg<HD, RK, RV>;
-    int stages = 4;
-    while (stages > 2 && 2 * (C::ticket_smem(stages) + 1024) > max_smem) --stages;
-    const long long slots = (long long)sm_count * ((2 * (C::ticket_smem(stages) + 1024) <= max_smem) ? 2 : 1);
-    const long long max_tiles = (max_ctx + PAGE - 1) / PAGE;
+    const long long slots = (long long)sm_count * ticket_per_sm(2, max_smem, 0), max_tiles = (max_ctx + PAGE - 1) / PAGE;
     size_t best = 0;
     for (int b = 1; b <= B; ++b) {
       const long long units = (long long)b * n_kv;
-      long long want = slots / units;
-      if (want < 1) want = 1;
-      if (units * max_tiles >= slots * 4 * 64) want = (4 * slots + units - 1) / units;
-      long long bound = (max_tiles + DEC_WARPS - 1) / DEC_WARPS;
-      if (bound > want) bound = want;
-      if (bound > DEC_MAX_SPLITS) bound = DEC_MAX_SPLITS;
-      if (bound < 1) bound = 1;
-      const size_t need = ws_need(b, n_kv, (int)bound);
+      long long records = HD == 64 ? 4ll * sm_count : slots;
+      if (units * max_tiles >= slots * 4 * 64) records = (4 * slots + units - 1) / units * units;
+      const long long most = units * ((max_tiles + DEC_WARPS - 1) / DEC_WARPS);
+      if (records > most) records = most;
+      if (records < units) records = units;
+      const size_t need = ws_need(b, n_kv, records);
       if (need > best) best = need;
     }
     return best;
@@ -192,47 +98,171 @@ struct DecodeRunT {
     }
     return cached[pl.cluster] - 1 >= need;
   }
+  static constexpr int extra = ROPE ? DecodeCfg<HD, RK, RV>::BK_BYTES + 128 : 0;   // the rotary variant's B_k slice, behind the usual layout
+
+  // ---- ticket kernel: one block per (request, kv head) - no merge, no workspace.  Rings as deep as the blocks that
+  //      share an SM allow.
+  static DecodePlan plan_whole(precc_ctx* ctx, long long units, int max_tiles) {
+    using C = DecodeCfg<HD, RK, RV>;
+    const int per_sm = (int)((units + ctx->sm_count - 1) / ctx->sm_count);
+    DecodePlan pl{};
+    pl.stages = 4;
+    while (pl.stages > 2 && (per_sm > 4 ? 4 : per_sm) * (C::ticket_smem(pl.stages) + extra + 1024) > ctx->max_smem_optin) --pl.stages;
+    pl.smem = C::ticket_smem(pl.stages) + extra;
+    pl.chunk_tiles = max_tiles; pl.max_splits = 1;
+    return pl;
+  }
+  // ---- ticket kernel, up to `want` blocks per unit, their chunk planned from the bound on the lengths
+  static DecodePlan plan_split(precc_ctx* ctx, int max_tiles, long long want) {
+    DecodePlan pl = plan_whole(ctx, 2 * ctx->sm_count, max_tiles);
+    if (want < 1) want = 1;
+    int chunk = (int)((max_tiles + want - 1) / want);
+    if (chunk < DEC_WARPS) chunk = DEC_WARPS;
+    if ((max_tiles + chunk - 1) / chunk > DEC_MAX_SPLITS) chunk = (max_tiles + DEC_MAX_SPLITS - 1) / DEC_MAX_SPLITS;
+    pl.chunk_tiles = chunk;
+    pl.max_splits = (max_tiles + chunk - 1) / chunk;
+    return pl;
+  }
+  // ---- ticket kernel on a flat grid: one wave of two blocks per SM (four at head_dim 64, whose blocks are small), shared
+  //      out by the actual lengths.  Rotary keys take two-page rings: they are bound by issue and gain from the finer
+  //      interleaving of short rings (64 units of 2000 .. 16000 tokens: 66 against 70 us).  With many units and plenty of
+  //      work four waves planned from the bound level unlike lengths out by themselves, at no cost per block (320 units of
+  //      5000 .. 6000 tokens, head_dim 64: 92 against 111 us; 256 units of 4096 .. 32768 tokens: 369 against 381 us).
+  static DecodePlan plan_flat(precc_ctx* ctx, int B, int n_kv, int max_tiles) {
+    using C = DecodeCfg<HD, RK, RV>;
+    const long long units = (long long)B * n_kv;
+    DecodePlan pl{};
+    pl.stages = ROPE || HD == 64 ? 2 : 4;
+    while (pl.stages > 2 && 2 * (C::ticket_smem(pl.stages) + extra + 1024) > ctx->max_smem_optin) --pl.stages;
+    pl.smem = C::ticket_smem(pl.stages) + extra;
+    const int per_sm = ticket_per_sm(pl.stages, ctx->max_smem_optin, extra);
+    const long long slots = (long long)ctx->sm_count * per_sm;
+    const long long work = units * max_tiles;
+    const bool plenty = work >= slots * 4 * 64;
+    if (B > DEC_FLAT_MAX_B || (plenty && units > (ROPE ? (HD == 128 ? 100 : 1) : 63)))
+      return plan_split(ctx, max_tiles, plenty ? (4 * slots + units - 1) / units : slots / units);
+    long long grid = HD == 64 ? 4ll * ctx->sm_count : slots;
+    const long long most = units * ((max_tiles + DEC_WARPS - 1) / DEC_WARPS);   // a split has a page for every warp
+    if (grid > most) grid = most;
+    if (grid < units) grid = units;
+    pl.flat = (int)grid;
+    pl.max_splits = 1;
+    return pl;
+  }
+  // ---- cluster kernel with `warps` warps per block at `per_sm` blocks per SM and rings of at most `max_stages` pages: the
+  //      widest cluster up to `lim` with all clusters of the grid resident at once.  cluster = 0 when there is none.
+  static DecodePlan plan_cluster(precc_ctx* ctx, long long units, int max_tiles, int warps, int per_sm, int max_stages, int lim) {
+    using C = DecodeCfg<HD, RK, RV>;
+    DecodePlan pl{};
+    int stages = max_stages;
+    if (ctx->decode_stage_cap >= 2 && stages > ctx->decode_stage_cap) stages = ctx->decode_stage_cap;
+    while (stages > 2 && per_sm * (C::cluster_smem(warps, stages) + extra + 1024) > ctx->max_smem_optin) --stages;
+    pl.smem = C::cluster_smem(warps, stages) + extra;
+    if (pl.smem > ctx->max_smem_optin || per_sm * (pl.smem + 1024) > ctx->max_smem_optin + (per_sm == 1 ? 1024 : 0)) return DecodePlan{};
+    pl.warps = warps; pl.stages = stages; pl.deep = 2 * (pl.smem + 1024) > ctx->max_smem_optin ? 1 : 0;
+    int cs = lim < DEC_MAX_CLUSTER ? lim : DEC_MAX_CLUSTER;
+    if (cs > max_tiles) cs = max_tiles;
+    if (cs * units > (long long)ctx->sm_count * per_sm) cs = (int)((long long)ctx->sm_count * per_sm / units);
+    if (ctx->decode_cluster_cap > 1 && cs > ctx->decode_cluster_cap) cs = ctx->decode_cluster_cap;
+    for (; cs >= 1; --cs) {
+      pl.cluster = cs;
+      if (warps == 8 ? cluster_fits<8>(ctx, pl, (int)units) : cluster_fits<4>(ctx, pl, (int)units)) break;
+    }
+    pl.cluster = cs;
+    pl.max_splits = cs;
+    // Short contexts are bound by latency: every request's own pages are shared out evenly.  Long ones are bound by
+    // bandwidth: with the chunk of the longest request for all, the blocks of short requests that would finish early do
+    // not start, and the longest request gets the bandwidth (24 units of 3188 pages at most: 91 -> 87 us; 12 units of
+    // 434 pages at most: 10.7 -> 10.1 us the other way round).
+    pl.chunk_tiles = cs >= 1 ? (max_tiles + cs - 1) / cs : 0;
+    pl.even = ROPE || (HD == 64 ? max_tiles < 1500 : units * max_tiles < 10000);
+    return cs >= 1 ? pl : DecodePlan{};
+  }
+  // The choice among them, from forced plans of some 1600 shapes (1 .. 64 requests of 100 .. 130000 tokens of unlike
+  // length, all layer shapes and ranks; alone, and after a projection in a decode step).  The earlier rules - ticket kernel
+  // up to 16 pages, clusters sized for the longest request only, a split planned from the bound - were 20 % above the
+  // best plan of each shape on the mean, up to 2x for short contexts; these are 5 % above it.  What decides:
+  //   few pages       a block per unit needs no merge; clusters help while most SMs would idle
+  //   units <= SMs/2  clusters: merge through distributed shared memory, everything resident in one wave
+  //   unlike lengths  the flat grid, once there is enough to read that its schedule and merge are small beside it
+  // `units` = (request, kv head) pairs, lengths in pages (mt: the longest request's).
+  static DecodePlan choose(precc_ctx* ctx, int B, int n_kv, int max_ctx) {
+    const int sm = ctx->sm_count, mt = (max_ctx + PAGE - 1) / PAGE;
+    const long long units = (long long)B * n_kv, work = units * mt;
+    auto whole = [&]() { return plan_whole(ctx, units, mt); };
+    auto flat = [&]() { return plan_flat(ctx, B, n_kv, mt); };
+    auto cluster = [&](int warps, int per_sm, int stages, int lim) { return plan_cluster(ctx, units, mt, warps, per_sm, stages, lim); };
+    if (ctx->force_ticket_decode) return flat();
+    if (units > sm) {
+      // the units fill the machine by themselves; splitting them only evens out unlike lengths
+      const int one = ROPE ? (units > 2 * sm ? 64 : 40) : units * 10 > sm * 14 ? (HD == 64 ? 300 : 200) : RK + RV >= 96 ? 200 : HD == 64 ? 64 : 100;
+      return mt <= one ? whole() : flat();
+    }
+    // Few pages: more blocks per unit than it has pages for their warps still pay for small grids (the merge is spread over
+    // the cluster, and each block owns fewer output columns), but not beyond about half of the SMs: wide clusters
+    // also wait longer for the kernel ahead to leave the SMs.
+    const int room = (int)(sm / units), few = room < mt / DEC_WARPS ? room : mt / DEC_WARPS;
+    int lim = DEC_MAX_CLUSTER;
+    if (ROPE && mt <= 150) lim = mt / 4 < room || room < 2 ? (mt / 4 > 4 ? mt / 4 : 4) : room;
+    else if (mt <= 80) lim = 80 / units > 2 ? (int)(80 / units) : 2;
+    else if (HD == 64) lim = mt / 12 > 8 ? mt / 12 : 8;
+    if (mt <= 80 && lim < few) lim = few;
+    DecodePlan pl{};
+    if (!ctx->deep_clusters || ctx->deep_always) {       // layout switches of the environment
+      if (ctx->deep_always) pl = cluster(8, 1, 4, lim);
+      else pl = HD == 64 ? cluster(8, 2, 2, lim) : cluster(4, 2, 3, lim);
+      return pl.cluster ? pl : flat();
+    }
+    if (ROPE) {
+      // issue-bound: four warps twice per SM reach as many SMs as eight once, in finer pieces; from some work on the flat
+      // grid's even shares win
+      if (units * 2 > sm && mt <= (units > 90 ? 48 : 16)) return whole();
+      if (units >= 48 && mt <= 12) return whole();
+      if (work >= (units >= 56 || RK + RV >= 96 ? 12000 : HD == 64 ? 16000 : 18000)) return flat();
+      if (units >= 8 && !(HD == 64 && RK + RV >= 96)) pl = cluster(4, 2, HD == 64 ? 3 : 2, lim);
+      if (!pl.cluster) pl = cluster(8, 1, 2, lim);
+      return pl.cluster ? pl : flat();
+    }
+    if (HD == 64) {
+      // eight warps twice per SM
+      if (units >= 56 && mt <= 16) return whole();
+      if (units > 80 && mt > 400) return flat();
+      const int wide = RV >= 32 ? (room > 8 ? room : 8) : 12;
+      pl = cluster(8, 2, 2, units > 9 && lim > wide ? wide : lim);
+      if (!pl.cluster) pl = cluster(8, 1, 3, lim);       // rank 64
+      return pl.cluster ? pl : flat();
+    }
+    if ((units >= 60 && mt <= 20) || (units >= 45 && mt <= 12)) return whole();
+    if (units >= 48 && work >= 60000) return flat();
+    if (units * 2 > sm) {
+      // too many units for two eight-warp blocks each: three four-warp blocks each, two per SM, while that fits
+      if (units * 3 <= 2 * sm && mt > 60) {
+        pl = cluster(4, 2, 3, 3);
+        if (pl.cluster == 3) return pl;
+      }
+      if (mt <= (RK + RV >= 96 ? 48 : 96)) return whole();
+      if (mt > 400) return flat();
+      if (RK + RV < 96 && units * 4 <= 3 * sm) return plan_split(ctx, mt, 2 * sm / units);
+      pl = cluster(8, 1, 3, 1);
+      return pl.cluster ? pl : flat();
+    }
+    // eight warps, one block per SM: two or three pages in flight per warp cover the memory's latency.  Where whole SMs are
+    // left over that way, four warps twice per SM may reach more of them.
+    pl = cluster(8, 1, work >= 50000 ? 2 : 3, lim);
+    if (units >= 24 && (units < 40 || units > 48) && work >= 30000 && pl.cluster * units * 13 < 10 * sm) return flat();
+    if (mt >= 100) {
+      const DecodePlan p4 = cluster(4, 2, 3, lim);
+      if (p4.cluster >= pl.cluster * 3 || (units >= 40 && units <= 48 && mt >= 300 && p4.cluster * 100 > pl.cluster * 216)) pl = p4;
+    }
+    return pl.cluster ? pl : flat();
+  }
   static int32_t run(precc_ctx* ctx, const DecodeArgs& a) {
     const precc_layer_desc* d = a.d;
-    constexpr int extra = ROPE ? DecodeCfg<HD, RK, RV>::BK_BYTES + 128 : 0;
-    // The rotary kernel at head_dim 128 is issue-bound (255 registers, 8 warps per SM at most): it gains more from
-    // the 128 blocks of the two-blocks-per-SM layout than from deeper rings on 80 SMs (131072 tokens: 141 against 238 us).
-    const bool deep_ok = ctx->deep_clusters && !(ROPE && HD == 128);
-    // planner's choice, then the experiment switches of the environment
-    auto plan = [&](bool deep) {
-      DecodePlan q = plan_cluster<HD, RK, RV>(ctx->sm_count, ctx->max_smem_optin, a.B, d->n_kv_heads, a.max_ctx, extra, deep);
-      if (ctx->force_ticket_decode) q.cluster = 0;
-      if (q.cluster > 1 && ctx->decode_cluster_cap > 1 && q.cluster > ctx->decode_cluster_cap) {
-        const int mt = (a.max_ctx + PAGE - 1) / PAGE;
-        q.cluster = ctx->decode_cluster_cap; q.chunk_tiles = (mt + q.cluster - 1) / q.cluster; q.max_splits = q.cluster;
-      }
-      if (q.cluster > 1 && ctx->decode_stage_cap >= 2 && q.stages > ctx->decode_stage_cap) {
-        q.stages = ctx->decode_stage_cap;
-        q.smem = DecodeCfg<HD, RK, RV>::cluster_smem(q.warps, q.stages) + extra;
-      }
-      return q;
-    };
-    DecodePlan pl = plan(deep_ok);
-    auto fits = [&](const DecodePlan& q) { return q.warps == 8 ? cluster_fits<8>(ctx, q, a.B * d->n_kv_heads) : cluster_fits<4>(ctx, q, a.B * d->n_kv_heads); };
-    if (pl.cluster && pl.deep) {
-      const int max_tiles = (a.max_ctx + PAGE - 1) / PAGE;
-      while (pl.cluster > 4 && !fits(pl)) { --pl.cluster; pl.chunk_tiles = (max_tiles + pl.cluster - 1) / pl.cluster; pl.max_splits = pl.cluster; }
-      if (pl.cluster <= 4) pl.cluster = 0;
-      // One block per SM means at most one cluster of more than half a GPC per GPC: 8 units get 10-block clusters,
-      // 80 of 148 SMs.  Where two 8-warp blocks fit on an SM the two-blocks-per-SM layout (16-block clusters, or
-      // the ticket kernel for long contexts) reaches more SMs and is faster then (head_dim 64, one request:
-      // 8192 tokens 8.0 -> 7.1 us, 131072 tokens 60 -> 49 us); with 4-warp blocks (head_dim 128) the deep rings win.
-      if (!ctx->deep_always && pl.cluster * a.B * d->n_kv_heads * 4 < ctx->sm_count * 3 &&
-          two_per_sm_warps<HD, RK, RV>(ctx->max_smem_optin, extra) == 8) {
-        pl = plan(false);
-        if (pl.cluster && !fits(pl)) pl.cluster = 0;
-      }
-    } else if (pl.cluster && !fits(pl)) {
-      pl.cluster = 0;
-    }
-    if (!pl.cluster) {
-      pl = plan_ticket<HD, RK, RV>(ctx->sm_count, ctx->max_smem_optin, a.B, d->n_kv_heads, a.max_ctx, extra);
-      const size_t need = ws_need(a.B, d->n_kv_heads, pl.max_splits);
+    const DecodePlan pl = choose(ctx, a.B, d->n_kv_heads, a.max_ctx);
+    // (a plan with one block per unit, and a cluster, use no workspace; the former and the shortest contexts still ask for
+    // the one record per unit that the caller's sizing provides at least, so that a missing workspace shows up early)
+    if (!pl.cluster || (a.max_ctx + PAGE - 1) / PAGE <= 16) {
+      const size_t need = ws_need(a.B, d->n_kv_heads, pl.cluster ? (long long)a.B * d->n_kv_heads : pl.flat ? pl.flat : (long long)a.B * d->n_kv_heads * pl.max_splits);
       if (!a.ws || a.ws_bytes < need) return fail(ctx, PRECC_ERR_WORKSPACE, "decode workspace: need %zu bytes, got %zu", need, a.ws_bytes);
     }
     DecodeParams p;
@@ -246,7 +276,10 @@ struct DecodeRunT {
     p.part = a.ws ? (float*)((char*)a.ws + tickets) : nullptr;
     p.raw = a.raw;
     p.status = ctx->status;
-    p.trace = (ctx->trace && (size_t)pl.max_splits * d->n_kv_heads * a.B <= ctx->trace_blocks) ? ctx->trace : nullptr;
+    p.B = a.B; p.even = pl.even;
+    const bool flat = !pl.cluster && pl.flat;
+    const size_t n_blocks = flat ? (size_t)pl.flat : (size_t)pl.max_splits * d->n_kv_heads * a.B;
+    p.trace = (ctx->trace && n_blocks <= ctx->trace_blocks) ? ctx->trace : nullptr;
     p.n_blocks = a.cache->n_blocks; p.table_stride = a.table_stride;
     p.n_q = d->n_q_heads; p.n_kv = d->n_kv_heads; p.group = d->n_q_heads / d->n_kv_heads; p.n_agents = d->n_agents;
     p.chunk_tiles = pl.chunk_tiles; p.max_splits = pl.max_splits; p.stages = pl.stages; p.max_ctx = a.max_ctx;
@@ -255,7 +288,7 @@ struct DecodeRunT {
     p.rope = reinterpret_cast<const float4*>(a.rope); p.max_pos = a.max_pos;
     p.bk_off = ROPE ? ((pl.smem - extra + 127) / 128) * 128 : 0;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(pl.max_splits, d->n_kv_heads, a.B);
+    cfg.gridDim = flat ? dim3(pl.flat) : dim3(pl.max_splits, d->n_kv_heads, a.B);
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = a.stream;
     cudaLaunchAttribute attr[3];
@@ -283,7 +316,7 @@ struct DecodeRunT {
         PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, cluster_kernel<4>(pl.deep != 0), p));
       }
     } else {
-      auto kern = lr_attend_decode_kernel<HD, RK, RV, ROPE>;
+      auto kern = flat ? lr_attend_decode_kernel<HD, RK, RV, ROPE, true> : lr_attend_decode_kernel<HD, RK, RV, ROPE, false>;
       cfg.blockDim = dim3(DEC_WARPS * 32);
       PRECC_CUDA(ctx, raise_smem_limit(ctx, kern, pl.smem));
       if (a.clear_counters) PRECC_CUDA(ctx, cudaMemsetAsync(p.tickets, 0, tickets, a.stream));

@@ -1,0 +1,82 @@
+"""How decode attention is split over the GPU: the flat grid's schedule and the other plans at their edges, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import lrkv_oracle as O
+from paper_2609_34054_b200 import inputs as I
+from paper_2609_34054_b200.binding import Cache, Precc, layer_desc
+
+from harness import assert_close, f64
+
+pytestmark = pytest.mark.gpu
+
+TICKET = {"PRECC_DECODE": "ticket"}          # no clusters: the flat grid (up to 256 requests) whatever the sizes
+
+
+def _ragged(B, low, high):
+    return [low + (b * 7919 + 13) % (high - low + 1) for b in range(B)]
+
+
+_PLANS = [
+    # env, head_dim, kv heads, query heads per kv head, rank, lengths, requests rejected on the device
+    (TICKET, 64, 1, 4, 16, [1], ()),                                     # one page, one block
+    (TICKET, 128, 2, 4, 16, [127, 129], ()),                             # fewer pages than a block has warps
+    (TICKET, 64, 2, 2, 8, [9000], ()),                                   # one request over the whole grid
+    (TICKET, 128, 3, 2, 32, [700, 16, 4000, 17, 1300], (2,)),            # a rejected request in the middle counts as one page
+    (TICKET, 64, 1, 4, 0, _ragged(32, 1, 900), ()),                      # one request per lane of the schedule
+    (TICKET, 64, 2, 8, 64, _ragged(33, 1, 900), (0, 32)),
+    (TICKET, 64, 1, 2, 16, _ragged(256, 1, 1500), (255,)),               # the most the schedule handles
+    (TICKET, 64, 1, 2, 16, _ragged(257, 1, 1500), ()),                   # one more: split from the bound
+    ({}, 64, 2, 4, 16, _ragged(80, 300, 1600), ()),                      # more units than SMs, unlike lengths: flat grid
+    ({}, 64, 2, 4, 16, _ragged(40, 60, 250), ()),                        # one block per unit
+    ({}, 128, 2, 4, 16, _ragged(50, 700, 1700), ()),                     # three blocks per unit, planned from the bound
+    ({}, 128, 2, 4, 64, _ragged(50, 700, 1700), ()),                     # one cluster block per unit
+    ({}, 128, 8, 4, 16, [10500, 900], ()),                               # clusters, the longest request's chunk for all
+    ({}, 128, 2, 4, 16, [256, 30, 250], ()),                             # clusters, every request shared out evenly
+]
+
+
+@pytest.mark.parametrize("env,hd,n_kv,G,r,ctx,rejected", _PLANS, ids=[str(i) for i in range(len(_PLANS))])
+def test_every_plan_against_the_oracle(monkeypatch, env, hd, n_kv, G, r, ctx, rejected):
+    """Paged caches (pages shared between requests, in mixed order).  The tolerance is that of every other decode test:
+    bf16 inputs and softmax weights, fp32 accumulation."""
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    px = Precc(0)                                        # the switch is read when a context is created
+    try:
+        geo = I.Geometry(512, G * n_kv, n_kv, hd, 2, r, r, alpha=2.0 * max(r, 1))
+        B, T = len(ctx), max(ctx)
+        pages = (T + 15) // 16
+        c = I.direct_caches(pages + 5, geo, 83, f"plan.{hd}.{n_kv}.{r}")
+        cache = Cache.from_tensors(geo, c["k_base"].cuda(), c["v_base"].cuda(), c["lr_k"].cuda() if r else None,
+                                   c["lr_v"].cuda() if r else None)
+        w, desc = I.layer_weights(geo, 83, "plan"), layer_desc(geo)
+        B_k, B_v = (w["B_k"].cuda(), w["B_v"].cuda()) if r else (None, None)
+        q = I.queries(B, geo, 83, "plan.q", gain=4.0)
+        table = torch.stack([torch.roll(torch.arange(pages + 5), b)[:pages] for b in range(B)]).to(torch.int32)
+        lengths = torch.tensor([8 * T if b in rejected else n for b, n in enumerate(ctx)], dtype=torch.int32).cuda()
+        agent = torch.tensor([b % 2 for b in range(B)], dtype=torch.int32).cuda()
+        ws = px.decode_workspace(desc, B, T)
+        out, again = torch.full_like(q, float("nan"), device="cuda"), torch.full_like(q, float("nan"), device="cuda")
+        for o in (out, again):
+            px.lr_attend_decode(desc, q.cuda(), agent, lengths, T, B_k, B_v, cache, o, ws, table.cuda())
+        assert px.poll_status() == (1 if rejected else 0)
+        assert torch.equal(out, again)
+        check = {b for b in (0, 1, B // 2, B - 2, B - 1, int(np.argmax(ctx)), int(np.argmin(ctx))) if 0 <= b < B}
+        for b in sorted(check | set(rejected)):
+            if b in rejected:
+                assert (out[b] == 0).all()
+                continue
+            own, n, a = table[b].long(), ctx[b], b % 2
+            for g in {0, n_kv - 1}:
+                cols, zero = slice(g * hd, (g + 1) * hd), np.zeros((1, hd))
+                rows = lambda x: f64(x.reshape(-1, x.shape[-1]))[:n]
+                lr = lambda x: rows(x[a][own]) if r else np.zeros((n, 1))
+                ref = O.attend_from_caches(f64(q[b, g * G:(g + 1) * G]), rows(c["k_base"][own, g]), rows(c["v_base"][own, g]),
+                                           lr(c["lr_k"]), lr(c["lr_v"]), f64(w["B_k"][a][:, cols]) if r else zero,
+                                           f64(w["B_v"][a][:, cols]) if r else zero, geo.scale_k if r else 0.0,
+                                           geo.scale_v if r else 0.0, 1)
+                assert_close(f64(out)[b, g * G:(g + 1) * G], ref, f"request {b} of {n} tokens, head {g}")
+    finally:
+        px.close()
