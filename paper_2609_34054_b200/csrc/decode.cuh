@@ -62,7 +62,8 @@ struct DecodeParams {
   int n_q, n_kv, group, n_agents;
   int chunk_tiles, max_splits, stages;
   int B;                       // requests of the call
-  int even;                    // cluster kernel: 1 = each request's own pages shared out evenly, 0 = chunk_tiles for every block
+  unsigned even;               // cluster kernel: 2^32 / cluster size, rounded up (each request's own pages are shared out
+                               // evenly), or 0 = chunk_tiles for every block
   int pre_stages;              // ring slots a warp fills before it waits for the preceding kernel (the rest follow the wait)
   int max_ctx;                 // the host's bound on ctx_len[b]: it sized the grid, the split and the block table
   float scale_log2, s_k, s_v;
@@ -1048,7 +1049,7 @@ lr_attend_decode_cluster_kernel(const DecodeParams p) {
     return;
   }
   const int n_tiles = (ctx + PAGE - 1) / PAGE;
-  const int chunk = p.even ? (n_tiles + CS - 1) / CS : p.chunk_tiles;
+  const int chunk = p.even ? (int)__umulhi((unsigned)(n_tiles + CS - 1), p.even) : p.chunk_tiles;
   const int tile0 = min(n_tiles, rank * chunk);
   const int tile_end = min(n_tiles, tile0 + chunk);
   mark(1);

@@ -276,7 +276,7 @@ struct DecodeRunT {
     p.part = a.ws ? (float*)((char*)a.ws + tickets) : nullptr;
     p.raw = a.raw;
     p.status = ctx->status;
-    p.B = a.B; p.even = pl.even;
+    p.B = a.B; p.even = pl.even && pl.cluster > 1 ? (unsigned)((1ull << 32) / pl.cluster + 1) : 0u;
     const bool flat = !pl.cluster && pl.flat;
     const size_t n_blocks = flat ? (size_t)pl.flat : (size_t)pl.max_splits * d->n_kv_heads * a.B;
     p.trace = (ctx->trace && n_blocks <= ctx->trace_blocks) ? ctx->trace : nullptr;
