@@ -32,11 +32,16 @@ struct PrefillRun {
     auto steps_of = [&](int x) { return (int)(((long long)T + std::min(S, (x + 1) * tok_per_tile) + PTC_TOK - 1) / PTC_TOK); };
     const int n_max = steps_of(X - 1);
     if (n_max < ctx->prefill_helper_min_steps) return best;
-    // what a record + merge costs a tile's own block, and what a piece costs a helper beyond its steps (query tile,
-    // fold, pipeline fill, record), in steps: measured at head_dim 128, rank 32 (1.3 us per step), scaled for shorter steps
+    // What a record + merge costs a tile's own block, and what a piece costs a helper beyond its steps (query tile,
+    // fold, pipeline fill, record), in steps at head_dim 128, rank 32 (1.0 us), scaled for shorter ones; and how much longer
+    // every step takes with all SMs busy instead of one per tile: at head_dim 128 the launch runs at the power cap and
+    // 35 .. 42 % of what the additional SMs add is lost to the clock; at head_dim 64 it is bound by the exponentials.  Fitted
+    // to turns of 72 .. 132 tiles over 6000 .. 48000 tokens (head_dim 128, rank 64, 112 tiles over 24000 tokens: 305 us with
+    // the helpers that a fit to slower steps chose, 275 without; 88 tiles over 48000: 448 without, 388 with).
     const int f100 = 100 * 160 / (HD + (RK + RV) / 2);
-    const int C_OWN = 14 * f100 / 100, C_PIECE = 12 * f100 / 100;
-    int best_cost = n_max - std::max(2, n_max / 12);   // a plan must win at least 8 % on paper: with every SM busy a step takes about 4 % longer
+    const int C_OWN = 14 * f100 / 100, C_PIECE = (HD == 64 ? 12 : RK + RV > 32 ? 18 : 13) * f100 / 100;
+    const int slow = HD == 64 ? 104 : 100 + (RK + RV > 32 ? 42 : 35) * H / (int)tiles;
+    int best_cost = (n_max - n_max / 25) * 100 / slow;   // a plan must win 4 % on paper
     for (int p = n_max - 1; p >= std::max(8, n_max / 2); --p) {
       if (ctx->prefill_helper_p > 0 && p != ctx->prefill_helper_p) continue;
       long long tail_sum = 0;
