@@ -5,9 +5,15 @@
 // waited for the host.  Here the same work is a few hundred nanoseconds: tensors are unpacked in place, the current
 // stream comes from c10, and the descriptor structures are built on the stack.  Nothing is kept from one call to
 // the next.  The GIL is released around the library call, as ctypes does.
+//
+// torch throws C++ exceptions (a tensor without storage, a layout without strides), which must not reach the interpreter's C
+// frames: every entry point runs inside `guarded`, dimensions are checked before a size is read, and pointers and sizes
+// are taken while the GIL is held.
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
 
 #include "../../include/precc.h"
 
@@ -61,6 +67,28 @@ struct Args {
   }
   static void* ptr(const at::Tensor* t) { return t ? t->data_ptr() : nullptr; }
   void* tptr() { return ptr(tensor()); }
+  // A required tensor of which the library wants the address and the first extent.
+  struct Rows { void* p; int32_t n; };
+  Rows rows_of(const char* name) {
+    const at::Tensor* t = required(name);
+    if (t && t->dim() < 1) { PyErr_Format(g_error, "%s has no dimensions", name); ok = false; }
+    return ok ? Rows{t->data_ptr(), static_cast<int32_t>(t->size(0))} : Rows{nullptr, 0};
+  }
+  // Block table or None: [B][stride] for decode (`per_request`), the sequence's own entries for prefill.
+  struct Table { const int32_t* p; int32_t n; };
+  Table table(bool per_request) {
+    const at::Tensor* t = tensor();
+    if (t && per_request && t->dim() < 2) bad("block_table must be [B][blocks per request]");
+    if (!ok || !t) return {nullptr, 0};
+    return {static_cast<const int32_t*>(t->data_ptr()), static_cast<int32_t>(per_request ? t->size(1) : t->numel())};
+  }
+  // Address and extent of a scratch buffer that may be None.
+  struct Buffer { void* p; size_t elements, bytes; };
+  Buffer buffer(const at::Tensor* t) {
+    if (!ok || !t) return {nullptr, 0, 0};
+    const size_t n = static_cast<size_t>(t->numel());
+    return {t->data_ptr(), n, n * t->element_size()};
+  }
 
   // LayerDesc (a ctypes structure), copied.
   precc_layer_desc desc() {
@@ -75,11 +103,9 @@ struct Args {
     return d;
   }
   void* member(PyObject* o, PyObject* name) {
-    PyObject* m = ok ? PyObject_GetAttr(o, name) : nullptr;
+    THPObjectPtr m(ok ? PyObject_GetAttr(o, name) : nullptr);   // (the cache object still holds it afterwards)
     if (!m) { ok = false; return nullptr; }
-    void* p = ptr(tensor(m));
-    Py_DECREF(m);          // the cache object still holds it
-    return p;
+    return ptr(tensor(m));
   }
   precc_cache cache() {
     precc_cache c = {};
@@ -89,10 +115,9 @@ struct Args {
     c.v_base = member(o, s_v_base);
     c.lr_k = member(o, s_lr_k);
     c.lr_v = member(o, s_lr_v);
-    PyObject* n = ok ? PyObject_GetAttr(o, s_n_blocks) : nullptr;
+    THPObjectPtr n(ok ? PyObject_GetAttr(o, s_n_blocks) : nullptr);
     if (!n) { ok = false; return c; }
     c.n_blocks = PyLong_AsLongLong(n);
-    Py_DECREF(n);
     if (c.n_blocks == -1 && PyErr_Occurred()) ok = false;
     return c;
   }
@@ -111,18 +136,20 @@ struct Args {
 };
 
 const int32_t* i32p(const at::Tensor* t) { return static_cast<const int32_t*>(Args::ptr(t)); }
-int32_t rows(const at::Tensor* t) { return static_cast<int32_t>(t->size(0)); }
-int32_t stride_of(const at::Tensor* table) { return table ? static_cast<int32_t>(table->size(1)) : 0; }
-int32_t entries(const at::Tensor* table) { return table ? static_cast<int32_t>(table->numel()) : 0; }
-size_t bytes(const at::Tensor* t) { return t ? static_cast<size_t>(t->numel()) * t->element_size() : 0; }
+
+struct GilRelease {        // (an object, so that an exception on the way leaves with the GIL held)
+  PyThreadState* state = PyEval_SaveThread();
+  ~GilRelease() { PyEval_RestoreThread(state); }
+};
 
 template <typename F>
 PyObject* finish(precc_ctx* ctx, const char* what, F&& call) {
   void* stream = c10::cuda::getCurrentCUDAStream().stream();
   int32_t rc;
-  Py_BEGIN_ALLOW_THREADS
-  rc = call(stream);
-  Py_END_ALLOW_THREADS
+  {
+    GilRelease unlocked;
+    rc = call(stream);
+  }
   if (rc == PRECC_OK) Py_RETURN_NONE;
   PyErr_Format(g_error, "%s: %s: %s", what, precc_error_name(rc), precc_last_error(ctx));
   return nullptr;
@@ -136,15 +163,15 @@ NATIVE(lr_precompute) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* H = a.required("H");
+  const Args::Rows H = a.rows_of("H");
   void* A = a.tptr();
   const precc_cache c = a.cache();
   const int64_t start = a.i64();
-  const at::Tensor* slots = a.tensor();
+  const int32_t* slots = i32p(a.tensor());
   const uint64_t mask = a.u64();
   if (!a.ok) return nullptr;
   return finish(ctx, "precc_lr_precompute", [&](void* st) {
-    return precc_lr_precompute(ctx, &d, H->data_ptr(), rows(H), A, i32p(slots), start, mask, &c, st); });
+    return precc_lr_precompute(ctx, &d, H.p, H.n, A, slots, start, mask, &c, st); });
 }
 
 NATIVE(turn_project) {
@@ -152,15 +179,15 @@ NATIVE(turn_project) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* H = a.required("H");
+  const Args::Rows H = a.rows_of("H");
   void* WA = a.tptr();
   const precc_cache c = a.cache();
   const int64_t start = a.i64();
-  const at::Tensor* slots = a.tensor();
+  const int32_t* slots = i32p(a.tensor());
   const uint64_t mask = a.u64();
   if (!a.ok) return nullptr;
   return finish(ctx, "precc_turn_project", [&](void* st) {
-    return precc_turn_project(ctx, &d, H->data_ptr(), rows(H), WA, i32p(slots), start, mask, &c, st); });
+    return precc_turn_project(ctx, &d, H.p, H.n, WA, slots, start, mask, &c, st); });
 }
 
 NATIVE(turn_project_rows) {
@@ -168,16 +195,15 @@ NATIVE(turn_project_rows) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* H = a.required("H");
+  const Args::Rows H = a.rows_of("H");
   void* WA = a.tptr();
   const precc_cache c = a.cache();
-  const at::Tensor* slots = a.tensor();
-  const at::Tensor* masks = a.typed(at::kLong, "row_masks must be int64 (bit patterns of uint64 masks)");
-  const at::Tensor* copies = a.typed(at::kInt, "lr_copy_slots must be int32");
+  const int32_t* slots = i32p(a.tensor());
+  const uint64_t* masks = static_cast<const uint64_t*>(Args::ptr(a.typed(at::kLong, "row_masks must be int64 (bit patterns of uint64 masks)")));
+  const int32_t* copies = i32p(a.typed(at::kInt, "lr_copy_slots must be int32"));
   if (!a.ok) return nullptr;
   return finish(ctx, "precc_turn_project_rows", [&](void* st) {
-    return precc_turn_project_rows(ctx, &d, H->data_ptr(), rows(H), WA, i32p(slots), static_cast<const uint64_t*>(Args::ptr(masks)),
-                                   i32p(copies), &c, st); });
+    return precc_turn_project_rows(ctx, &d, H.p, H.n, WA, slots, masks, copies, &c, st); });
 }
 
 NATIVE(rebase_project) {
@@ -185,14 +211,14 @@ NATIVE(rebase_project) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* H = a.required("H");
+  const Args::Rows H = a.rows_of("H");
   void* W = a.tptr();
   const precc_cache c = a.cache();
   const int64_t start = a.i64();
-  const at::Tensor* slots = a.tensor();
+  const int32_t* slots = i32p(a.tensor());
   if (!a.ok) return nullptr;
   return finish(ctx, "precc_rebase_project", [&](void* st) {
-    return precc_rebase_project(ctx, &d, H->data_ptr(), rows(H), W, i32p(slots), start, &c, st); });
+    return precc_rebase_project(ctx, &d, H.p, H.n, W, slots, start, &c, st); });
 }
 
 NATIVE(rebase_project_rope) {
@@ -200,15 +226,15 @@ NATIVE(rebase_project_rope) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* H = a.required("H");
+  const Args::Rows H = a.rows_of("H");
   void* W = a.tptr();
   const precc_cache c = a.cache();
   const precc_rope r = a.rope(true);
   const int64_t start = a.i64();
-  const at::Tensor* slots = a.tensor();
+  const int32_t* slots = i32p(a.tensor());
   if (!a.ok) return nullptr;
   return finish(ctx, "precc_rebase_project_rope", [&](void* st) {
-    return precc_rebase_project_rope(ctx, &d, H->data_ptr(), rows(H), W, i32p(slots), start, &r, &c, st); });
+    return precc_rebase_project_rope(ctx, &d, H.p, H.n, W, slots, start, &r, &c, st); });
 }
 
 NATIVE(turn_project_rope) {
@@ -216,16 +242,16 @@ NATIVE(turn_project_rope) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* H = a.required("H");
+  const Args::Rows H = a.rows_of("H");
   void* WA = a.tptr();
   const precc_cache c = a.cache();
   const precc_rope r = a.rope(true);
   const int64_t start = a.i64();
-  const at::Tensor* slots = a.tensor();
+  const int32_t* slots = i32p(a.tensor());
   const uint64_t mask = a.u64();
   if (!a.ok) return nullptr;
   return finish(ctx, "precc_turn_project_rope", [&](void* st) {
-    return precc_turn_project_rope(ctx, &d, H->data_ptr(), rows(H), WA, i32p(slots), start, mask, &r, &c, st); });
+    return precc_turn_project_rope(ctx, &d, H.p, H.n, WA, slots, start, mask, &r, &c, st); });
 }
 
 // ------------------------------------------------------------------------------------------------ decode
@@ -237,7 +263,7 @@ NATIVE(decode) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* q = a.required("q");
+  const Args::Rows q = a.rows_of("q");
   const int32_t* agent = i32p(a.tensor());
   const int32_t* len = i32p(a.tensor());
   const int32_t max_ctx = a.i32();
@@ -247,20 +273,20 @@ NATIVE(decode) {
   if (FORM == ROPE) r = a.rope(false);
   const precc_cache c = a.cache();
   void* out = a.tptr();
-  const at::Tensor* ws = FORM == STATIC ? nullptr : a.required("workspace");
-  const at::Tensor* table = a.tensor();
+  const Args::Buffer ws = a.buffer(FORM == STATIC ? nullptr : a.required("workspace"));
+  const Args::Table table = a.table(true);
   const int32_t* first = i32p(a.tensor());
   if (!a.ok) return nullptr;
   const char* what = FORM == ROPE ? "precc_lr_attend_decode_rope" : FORM == PLAIN ? "precc_lr_attend_decode" : "precc_lr_attend_decode_static";
   return finish(ctx, what, [&](void* st) {
     if (FORM == STATIC)
-      return precc_lr_attend_decode_static(ctx, &d, q->data_ptr(), rows(q), agent, len, i32p(table), stride_of(table), first, max_ctx,
+      return precc_lr_attend_decode_static(ctx, &d, q.p, q.n, agent, len, table.p, table.n, first, max_ctx,
                                            Bk, Bv, &c, out, st);
     if (FORM == ROPE)
-      return precc_lr_attend_decode_rope(ctx, &d, q->data_ptr(), rows(q), agent, len, i32p(table), stride_of(table), first, max_ctx,
-                                         Bk, Bv, &r, &c, out, ws->data_ptr(), static_cast<size_t>(ws->numel()), st);
-    return precc_lr_attend_decode(ctx, &d, q->data_ptr(), rows(q), agent, len, i32p(table), stride_of(table), first, max_ctx, Bk, Bv,
-                                  &c, out, ws->data_ptr(), static_cast<size_t>(ws->numel()), st); });
+      return precc_lr_attend_decode_rope(ctx, &d, q.p, q.n, agent, len, table.p, table.n, first, max_ctx,
+                                         Bk, Bv, &r, &c, out, ws.p, ws.elements, st);
+    return precc_lr_attend_decode(ctx, &d, q.p, q.n, agent, len, table.p, table.n, first, max_ctx, Bk, Bv,
+                                  &c, out, ws.p, ws.elements, st); });
 }
 
 NATIVE(decode_partial) {
@@ -268,21 +294,20 @@ NATIVE(decode_partial) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* q = a.required("q");
+  const Args::Rows q = a.rows_of("q");
   const int32_t* agent = i32p(a.tensor());
   const int32_t* len = i32p(a.tensor());
   const int32_t max_ctx = a.i32();
   void* Bk = a.tptr();
   const precc_cache c = a.cache();
-  const at::Tensor* records = a.typed(at::kFloat, "records must be fp32");
-  const at::Tensor* ws = a.required("workspace");
-  const at::Tensor* table = a.tensor();
+  float* records = static_cast<float*>(Args::ptr(a.typed(at::kFloat, "records must be fp32")));
+  const Args::Buffer ws = a.buffer(a.required("workspace"));
+  const Args::Table table = a.table(true);
   const int32_t* first = i32p(a.tensor());
   if (!a.ok) return nullptr;
   return finish(ctx, "precc_lr_attend_decode_partial", [&](void* st) {
-    return precc_lr_attend_decode_partial(ctx, &d, q->data_ptr(), rows(q), agent, len, i32p(table), stride_of(table), first, max_ctx,
-                                          Bk, &c, static_cast<float*>(Args::ptr(records)), ws->data_ptr(),
-                                          static_cast<size_t>(ws->numel()), st); });
+    return precc_lr_attend_decode_partial(ctx, &d, q.p, q.n, agent, len, table.p, table.n, first, max_ctx,
+                                          Bk, &c, records, ws.p, ws.elements, st); });
 }
 
 NATIVE(combine_partials) {
@@ -290,14 +315,13 @@ NATIVE(combine_partials) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* records = a.required("records");
+  const Args::Rows records = a.rows_of("records");
   const int32_t* agent = i32p(a.tensor());
   void* Bv = a.tptr();
-  const at::Tensor* out = a.required("out");
+  const Args::Rows out = a.rows_of("out");
   if (!a.ok) return nullptr;
   return finish(ctx, "precc_combine_partials", [&](void* st) {
-    return precc_combine_partials(ctx, &d, static_cast<const float*>(records->data_ptr()), rows(records), rows(out), agent, Bv,
-                                  out->data_ptr(), st); });
+    return precc_combine_partials(ctx, &d, static_cast<const float*>(records.p), records.n, out.n, agent, Bv, out.p, st); });
 }
 
 // ------------------------------------------------------------------------------------------------ prefill
@@ -309,7 +333,7 @@ NATIVE(prefill) {
   if (!a.ok) return nullptr;
   precc_ctx* ctx = a.ctx();
   const precc_layer_desc d = a.desc();
-  const at::Tensor* q = a.required("q");
+  const Args::Rows q = a.rows_of("q");
   const int32_t agent = a.i32(), T = a.i32();
   void* Bk = a.tptr();
   void* Bv = a.tptr();
@@ -317,25 +341,24 @@ NATIVE(prefill) {
   if (FORM == PF_ROPE || FORM == PF_SCRATCH) r = a.rope(false);
   const precc_cache c = a.cache();
   void* out = a.tptr();
-  const at::Tensor* extra = FORM == PF_WS ? a.tensor() : FORM == PF_SCRATCH ? a.required("key_scratch") : nullptr;
-  const at::Tensor* table = a.tensor();
+  const Args::Buffer extra = a.buffer(FORM == PF_WS ? a.tensor() : FORM == PF_SCRATCH ? a.required("key_scratch") : nullptr);
+  const Args::Table table = a.table(false);
   const int32_t first = a.i32();
   if (!a.ok) return nullptr;
   const char* what = FORM == PF_PLAIN ? "precc_lr_attend_prefill" : FORM == PF_WS ? "precc_lr_attend_prefill_ws" :
                      FORM == PF_ROPE ? "precc_lr_attend_prefill_rope" : "precc_lr_attend_prefill_rope_scratch";
   return finish(ctx, what, [&](void* st) {
-    const int32_t S = rows(q);
     switch (FORM) {
       case PF_WS:
-        return precc_lr_attend_prefill_ws(ctx, &d, q->data_ptr(), S, agent, T, i32p(table), entries(table), first, Bk, Bv, &c, out,
-                                          Args::ptr(extra), bytes(extra), st);
+        return precc_lr_attend_prefill_ws(ctx, &d, q.p, q.n, agent, T, table.p, table.n, first, Bk, Bv, &c, out,
+                                          extra.p, extra.bytes, st);
       case PF_ROPE:
-        return precc_lr_attend_prefill_rope(ctx, &d, q->data_ptr(), S, agent, T, i32p(table), entries(table), first, Bk, Bv, &r, &c, out, st);
+        return precc_lr_attend_prefill_rope(ctx, &d, q.p, q.n, agent, T, table.p, table.n, first, Bk, Bv, &r, &c, out, st);
       case PF_SCRATCH:
-        return precc_lr_attend_prefill_rope_scratch(ctx, &d, q->data_ptr(), S, agent, T, i32p(table), entries(table), first, Bk, Bv, &r,
-                                                    &c, out, Args::ptr(extra), bytes(extra), st);
+        return precc_lr_attend_prefill_rope_scratch(ctx, &d, q.p, q.n, agent, T, table.p, table.n, first, Bk, Bv, &r,
+                                                    &c, out, extra.p, extra.bytes, st);
       default:
-        return precc_lr_attend_prefill(ctx, &d, q->data_ptr(), S, agent, T, i32p(table), entries(table), first, Bk, Bv, &c, out, st);
+        return precc_lr_attend_prefill(ctx, &d, q.p, q.n, agent, T, table.p, table.n, first, Bk, Bv, &c, out, st);
     }
   });
 }
@@ -346,7 +369,25 @@ PyObject* set_error(PyObject*, PyObject* type) {
   Py_RETURN_NONE;
 }
 
-#define FAST(name, fn) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(fn)), METH_FASTCALL, nullptr}
+// Entry point as the interpreter sees it: C++ exceptions become Python errors (the GIL is held wherever they arrive here).
+using Entry = PyObject* (*)(PyObject*, PyObject* const*, Py_ssize_t);
+template <Entry FN>
+PyObject* guarded(PyObject* self, PyObject* const* args, Py_ssize_t nargs) {
+  try {
+    return FN(self, args, nargs);
+  } catch (python_error& e) {
+    e.restore();
+  } catch (const c10::Error& e) {
+    PyErr_SetString(g_error, e.what_without_backtrace());
+  } catch (const std::exception& e) {
+    PyErr_SetString(g_error, e.what());
+  } catch (...) {
+    PyErr_SetString(g_error, "unknown C++ exception");
+  }
+  return nullptr;
+}
+
+#define FAST(name, fn) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(&guarded<fn>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
     {"set_error", set_error, METH_O, nullptr},
     FAST("lr_precompute", lr_precompute), FAST("rebase_project", rebase_project), FAST("turn_project", turn_project),

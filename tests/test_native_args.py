@@ -30,3 +30,62 @@ def test_bad_arguments_raise(native, what):
         args.pop()
     with pytest.raises(TypeError if what == "argument count" else binding.PreccError):
         native.turn_project(*args)
+
+
+def _fake(*shape):
+    """A tensor that says it lies on a GPU and has no storage: its sizes can be read, there is nothing at its address."""
+    from torch._subclasses import FakeTensorMode
+    with FakeTensorMode():
+        return torch.empty(shape, dtype=torch.float32, device="cuda")
+
+
+_NO_CACHE = types.SimpleNamespace(k_base=None, v_base=None, lr_k=None, lr_v=None, n_blocks=1)
+
+
+def _valid(call):
+    """Arguments of `call` that pass the marshalling up to the look-up of the stream."""
+    desc, x, table = binding.layer_desc(I.C1), _fake(4, 2, 64), _fake(4, 8)
+    project = [0, desc, x, x, _NO_CACHE, 0, None, 1]
+    rope, decode = _fake(64, 32, 2), [0, desc, x, None, None, 64, None, None]
+    prefill = [0, desc, x, 0, 64, None, None]
+    return {"turn_project": project, "lr_precompute": project, "rebase_project": project[:7],
+            "turn_project_rows": [0, desc, x, x, _NO_CACHE, None, None, None],
+            "rebase_project_rope": [0, desc, x, x, _NO_CACHE, rope, None, 0, 0, None],
+            "turn_project_rope": [0, desc, x, x, _NO_CACHE, rope, None, 0, 0, None, 1],
+            "lr_attend_decode": decode + [_NO_CACHE, x, x, table, None],
+            "lr_attend_decode_rope": decode + [rope, _NO_CACHE, x, x, table, None],
+            "lr_attend_decode_static": decode + [_NO_CACHE, x, table, None],
+            "lr_attend_decode_partial": decode[:7] + [_NO_CACHE, x, x, table, None],
+            "combine_partials": [0, desc, x, None, None, x],
+            "lr_attend_prefill": prefill + [_NO_CACHE, x, table, 0],
+            "lr_attend_prefill_ws": prefill + [_NO_CACHE, x, x, table, 0],
+            "lr_attend_prefill_rope": prefill + [rope, _NO_CACHE, x, table, 0],
+            "lr_attend_prefill_rope_scratch": prefill + [rope, _NO_CACHE, x, x, table, 0]}[call]
+
+
+_CALLS = ("turn_project", "lr_precompute", "rebase_project", "turn_project_rows", "rebase_project_rope", "turn_project_rope",
+          "lr_attend_decode", "lr_attend_decode_rope", "lr_attend_decode_static", "lr_attend_decode_partial", "combine_partials",
+          "lr_attend_prefill", "lr_attend_prefill_ws", "lr_attend_prefill_rope", "lr_attend_prefill_rope_scratch")
+
+
+@pytest.mark.parametrize("call", _CALLS)
+def test_torch_exceptions_arrive_as_errors(native, call):
+    """Without a device torch throws where the stream is looked up; with one the library refuses the context."""
+    with pytest.raises(binding.PreccError):
+        getattr(native, call)(*_valid(call))
+
+
+@pytest.mark.parametrize("call", _CALLS)
+def test_no_dimension_raises(native, call):
+    args = _valid(call)
+    args[2] = _fake()
+    with pytest.raises(binding.PreccError, match="has no dimensions"):
+        getattr(native, call)(*args)
+
+
+@pytest.mark.parametrize("call", [c for c in _CALLS if "decode" in c])
+def test_flat_block_table_of_a_batch_raises(native, call):
+    args = _valid(call)
+    args[-2] = _fake(8)                     # what a prefill call takes
+    with pytest.raises(binding.PreccError, match="block_table must be"):
+        getattr(native, call)(*args)
