@@ -69,7 +69,7 @@ def load_library() -> C.CDLL:
     except ImportError as e:
         raise PreccError(f"the marshalling extension beside {LIB_PATH} does not load ({e}): "
                          "build it with `python -m paper_2609_34054_b200.build`") from e
-    native.set_error(PreccError)
+    native.set_types(PreccError, Cache)
     _native = native
     vp, i32, i64, u64, sz = C.c_void_p, C.c_int32, C.c_int64, C.c_uint64, C.c_size_t
     lib.precc_create.argtypes = [C.POINTER(vp), i32]

@@ -20,7 +20,8 @@
 namespace {
 
 PyObject* g_error = nullptr;   // binding.PreccError
-PyObject *s_k_base, *s_v_base, *s_lr_k, *s_lr_v, *s_n_blocks;
+PyObject* g_cache = nullptr;   // binding.Cache
+PyObject *s_desc, *s_k_base, *s_v_base, *s_lr_k, *s_lr_v, *s_n_blocks;
 
 // One call's arguments, taken in order; the first problem sets the Python error and makes the rest no-ops.
 struct Args {
@@ -93,24 +94,33 @@ struct Args {
   // LayerDesc (a ctypes structure), copied.
   precc_layer_desc desc() {
     precc_layer_desc d = {};
-    PyObject* o = next();
-    if (!ok) return d;
-    Py_buffer v;
-    if (PyObject_GetBuffer(o, &v, PyBUF_SIMPLE) != 0) { ok = false; return d; }
-    if (v.len == static_cast<Py_ssize_t>(sizeof(d))) memcpy(&d, v.buf, sizeof(d));
-    else bad("desc is not a LayerDesc");
-    PyBuffer_Release(&v);
+    copy(next(), &d, sizeof(d), "desc is not a LayerDesc");
     return d;
+  }
+  void copy(PyObject* o, void* to, size_t n, const char* what) {
+    Py_buffer v;
+    if (!ok) return;
+    if (PyObject_GetBuffer(o, &v, PyBUF_SIMPLE) != 0) { ok = false; return; }
+    if (v.len == static_cast<Py_ssize_t>(n)) memcpy(to, v.buf, n);
+    else bad(what);
+    PyBuffer_Release(&v);
   }
   void* member(PyObject* o, PyObject* name) {
     THPObjectPtr m(ok ? PyObject_GetAttr(o, name) : nullptr);   // (the cache object still holds it afterwards)
     if (!m) { ok = false; return nullptr; }
     return ptr(tensor(m));
   }
+  // A Cache is read member by member; any other object (a subclass, a view with a layout of its own) is asked for its desc().
   precc_cache cache() {
     precc_cache c = {};
     PyObject* o = next();
     if (!ok) return c;
+    if (reinterpret_cast<PyObject*>(Py_TYPE(o)) != g_cache) {
+      THPObjectPtr d(PyObject_CallMethodNoArgs(o, s_desc));
+      if (!d) { ok = false; return c; }
+      copy(d, &c, sizeof(c), "cache.desc() is not a CacheDesc");
+      return c;
+    }
     c.k_base = member(o, s_k_base);
     c.v_base = member(o, s_v_base);
     c.lr_k = member(o, s_lr_k);
@@ -363,9 +373,11 @@ NATIVE(prefill) {
   });
 }
 
-PyObject* set_error(PyObject*, PyObject* type) {
-  Py_INCREF(type);
-  Py_XSETREF(g_error, type);
+// (error class, cache class) of binding.py
+PyObject* set_types(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  if (n != 2) { PyErr_SetString(PyExc_TypeError, "set_types(error, cache)"); return nullptr; }
+  Py_XSETREF(g_error, Py_NewRef(args[0]));
+  Py_XSETREF(g_cache, Py_NewRef(args[1]));
   Py_RETURN_NONE;
 }
 
@@ -389,7 +401,7 @@ PyObject* guarded(PyObject* self, PyObject* const* args, Py_ssize_t nargs) {
 
 #define FAST(name, fn) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(&guarded<fn>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
-    {"set_error", set_error, METH_O, nullptr},
+    FAST("set_types", set_types),
     FAST("lr_precompute", lr_precompute), FAST("rebase_project", rebase_project), FAST("turn_project", turn_project),
     FAST("turn_project_rows", turn_project_rows), FAST("rebase_project_rope", rebase_project_rope),
     FAST("turn_project_rope", turn_project_rope),
@@ -404,6 +416,7 @@ PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_native", "Argument marshallin
 }  // namespace
 
 PyMODINIT_FUNC PyInit__native() {
+  s_desc = PyUnicode_InternFromString("desc");
   s_k_base = PyUnicode_InternFromString("k_base");
   s_v_base = PyUnicode_InternFromString("v_base");
   s_lr_k = PyUnicode_InternFromString("lr_k");

@@ -1,6 +1,4 @@
 """Argument checks of the marshalling extension (no GPU: every case is refused before the library is called)."""
-import types
-
 import pytest
 import torch
 
@@ -18,8 +16,7 @@ def native():
 @pytest.mark.parametrize("what", ["host tensor", "none where required", "not a descriptor", "not a tensor", "argument count"])
 def test_bad_arguments_raise(native, what):
     desc, H = binding.layer_desc(I.C1), torch.zeros(4, I.C1.d_model, dtype=torch.bfloat16)
-    cache = types.SimpleNamespace(k_base=None, v_base=None, lr_k=None, lr_v=None, n_blocks=1)
-    args = [0, desc, H, None, cache, 0, None, 1]
+    args = [0, desc, H, None, _NO_CACHE, 0, None, 1]
     if what == "none where required":
         args[2] = None
     elif what == "not a descriptor":
@@ -39,7 +36,8 @@ def _fake(*shape):
         return torch.empty(shape, dtype=torch.float32, device="cuda")
 
 
-_NO_CACHE = types.SimpleNamespace(k_base=None, v_base=None, lr_k=None, lr_v=None, n_blocks=1)
+_NO_CACHE = binding.Cache.__new__(binding.Cache)
+_NO_CACHE.__dict__.update(k_base=None, v_base=None, lr_k=None, lr_v=None, n_blocks=1)
 
 
 def _valid(call):
@@ -89,3 +87,27 @@ def test_flat_block_table_of_a_batch_raises(native, call):
     args[-2] = _fake(8)                     # what a prefill call takes
     with pytest.raises(binding.PreccError, match="block_table must be"):
         getattr(native, call)(*args)
+
+
+class _Window(binding.Cache):
+    """A cache with its own idea of what the library sees of it."""
+
+    def __init__(self, seen):
+        self.seen = seen
+
+    def desc(self):
+        self.seen.append(self)
+        return binding.CacheDesc(None, None, None, None, 1) if len(self.seen) < 2 else b"short"
+
+
+def test_a_cache_class_of_ones_own_is_asked_for_its_descriptor(native):
+    seen, args = [], _valid("turn_project")
+    args[4] = _Window(seen)
+    with pytest.raises(binding.PreccError):          # (the context is refused, after the descriptor has been read)
+        native.turn_project(*args)
+    assert len(seen) == 1
+    with pytest.raises(binding.PreccError, match="CacheDesc"):
+        native.turn_project(*args)
+    args[4] = object()
+    with pytest.raises(AttributeError, match="desc"):
+        native.turn_project(*args)
