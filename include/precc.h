@@ -197,9 +197,9 @@ int32_t precc_turn_project_rows(precc_ctx* ctx, const precc_layer_desc* desc, co
 
 /* Workspace size for precc_lr_attend_decode with at most max_batch requests of at most max_ctx tokens
  * on a device with `sm_count` SMs: an upper bound over every such call (a smaller batch splits each request
- * further, so the bound is taken over all batch sizes up to max_batch).  The workspace must be zeroed once (precc_workspace_init) before its
- * first use; calls leave it ready for the next call.  Two calls that may run concurrently need
- * separate workspaces. */
+ * further, so the bound is taken over all batch sizes up to max_batch).  The workspace must be zeroed once
+ * (precc_workspace_init) before its first use; calls leave it ready for the next call, of whatever batch or layer it
+ * is large enough for.  Two calls that may run concurrently need separate workspaces. */
 size_t precc_decode_workspace_bytes(const precc_layer_desc* desc, int32_t max_batch, int32_t max_ctx,
                                     int32_t sm_count);
 int32_t precc_workspace_init(precc_ctx* ctx, void* workspace, size_t workspace_bytes, void* stream);

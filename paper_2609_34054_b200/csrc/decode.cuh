@@ -50,7 +50,7 @@ struct DecodeParams {
   const __nv_bfloat16* B_k;
   const __nv_bfloat16* B_v;
   float* part;        // ticket kernel: records [PART_STRIDE] of the splits, [B][n_kv][max_splits] or one per block (flat grid)
-  int32_t* tickets;   // ticket kernel: [B][n_kv], zero between calls
+  int32_t* tickets;   // ticket kernel: counter of each split (request, kv head), zero between calls
   float* raw;         // partial-output mode (ticket kernel): [B][n_kv][PART_STRIDE] records instead of `out`, or null
   uint32_t* status;
   unsigned long long* trace;   // optional [blocks][16] phase timestamps (ns), or null

@@ -18,10 +18,17 @@ struct DecodeRunT {
   // of them still fit on an SM at the shallowest ring, so that the planner's blocks-per-SM figure is the same.
   static_assert(!ROPE || 2 * (DecodeCfg<HD, RK, RV>::ticket_smem(2) + DecodeCfg<HD, RK, RV>::BK_BYTES + 128 + 1024) <= 232448,
                 "rotary ticket blocks must fit two per SM, or the workspace bound of the plain kernel no longer covers them");
-  // exact need of one call: arrival counters and one record per block
-  static size_t ws_need(int B, int n_kv, long long records) {
-    const size_t tickets = ((size_t)B * n_kv * 4 + 255) / 256 * 256;
-    return tickets + (size_t)records * DecodeCfg<HD, RK, RV>::PART_STRIDE * 4;
+  // Workspace: arrival counters of the (request, kv head) pairs, then records.  The counters have to be zero between calls, so
+  // no call may find another one's records there: their place and size depend on the device alone, not on the batch or the
+  // layer (they used to be as many as the call had pairs, and a later call of a larger batch on the same workspace took the
+  // records behind them for counters: no block of such a pair saw itself as the last, and its output was never written).
+  // Enough for every pair that can be split: more than one block per pair takes fewer pairs than the 4 x 2 x SMs blocks
+  // that plan_split wants at most, or than the 4 x SMs of a flat grid.
+  static long long counted_units(int sm_count) { return 8ll * sm_count; }
+  static size_t counter_bytes(int sm_count) { return ((size_t)counted_units(sm_count) * 4 + 255) / 256 * 256; }
+  // need of one call: the counters if pairs are split, and the records
+  static size_t ws_need(int sm_count, bool split, long long records) {
+    return (split ? counter_bytes(sm_count) : 0) + (size_t)records * DecodeCfg<HD, RK, RV>::PART_STRIDE * 4;
   }
   static int ticket_per_sm(int stages, int max_smem, int extra) {
     const int n = max_smem / (DecodeCfg<HD, RK, RV>::ticket_smem(stages) + extra + 1024);
@@ -40,7 +47,7 @@ struct DecodeRunT {
       const long long most = units * ((max_tiles + DEC_WARPS - 1) / DEC_WARPS);
       if (records > most) records = most;
       if (records < units) records = units;
-      const size_t need = ws_need(b, n_kv, records);
+      const size_t need = ws_need(sm_count, records > units, records);
       if (need > best) best = need;
     }
     return best;
@@ -261,8 +268,10 @@ struct DecodeRunT {
     const DecodePlan pl = choose(ctx, a.B, d->n_kv_heads, a.max_ctx);
     // (a plan with one block per unit, and a cluster, use no workspace; the former and the shortest contexts still ask for
     // the one record per unit that the caller's sizing provides at least, so that a missing workspace shows up early)
+    const long long units = (long long)a.B * d->n_kv_heads, records = pl.cluster ? units : pl.flat ? pl.flat : units * pl.max_splits;
+    const bool split = records > units;                  // pairs of more than one block, which meet at the counters
     if (!pl.cluster || (a.max_ctx + PAGE - 1) / PAGE <= 16) {
-      const size_t need = ws_need(a.B, d->n_kv_heads, pl.cluster ? (long long)a.B * d->n_kv_heads : pl.flat ? pl.flat : (long long)a.B * d->n_kv_heads * pl.max_splits);
+      const size_t need = ws_need(ctx->sm_count, split, records);
       if (!a.ws || a.ws_bytes < need) return fail(ctx, PRECC_ERR_WORKSPACE, "decode workspace: need %zu bytes, got %zu", need, a.ws_bytes);
     }
     DecodeParams p;
@@ -271,14 +280,13 @@ struct DecodeRunT {
     p.k_base = (const __nv_bfloat16*)a.cache->k_base; p.v_base = (const __nv_bfloat16*)a.cache->v_base;
     p.lr_k = (const __nv_bfloat16*)a.cache->lr_k; p.lr_v = (const __nv_bfloat16*)a.cache->lr_v;
     p.B_k = (const __nv_bfloat16*)a.B_k; p.B_v = (const __nv_bfloat16*)a.B_v;
-    const size_t tickets = ((size_t)a.B * d->n_kv_heads * 4 + 255) / 256 * 256;
     p.tickets = (int32_t*)a.ws;
-    p.part = a.ws ? (float*)((char*)a.ws + tickets) : nullptr;
+    p.part = a.ws ? (float*)((char*)a.ws + counter_bytes(ctx->sm_count)) : nullptr;
     p.raw = a.raw;
     p.status = ctx->status;
     p.B = a.B; p.even = pl.even && pl.cluster > 1 ? (unsigned)((1ull << 32) / pl.cluster + 1) : 0u;
     const bool flat = !pl.cluster && pl.flat;
-    const size_t n_blocks = flat ? (size_t)pl.flat : (size_t)pl.max_splits * d->n_kv_heads * a.B;
+    const size_t n_blocks = flat ? (size_t)pl.flat : (size_t)pl.max_splits * units;
     p.trace = (ctx->trace && n_blocks <= ctx->trace_blocks) ? ctx->trace : nullptr;
     p.n_blocks = a.cache->n_blocks; p.table_stride = a.table_stride;
     p.n_q = d->n_q_heads; p.n_kv = d->n_kv_heads; p.group = d->n_q_heads / d->n_kv_heads; p.n_agents = d->n_agents;
@@ -319,7 +327,7 @@ struct DecodeRunT {
       auto kern = flat ? lr_attend_decode_kernel<HD, RK, RV, ROPE, true> : lr_attend_decode_kernel<HD, RK, RV, ROPE, false>;
       cfg.blockDim = dim3(DEC_WARPS * 32);
       PRECC_CUDA(ctx, raise_smem_limit(ctx, kern, pl.smem));
-      if (a.clear_counters) PRECC_CUDA(ctx, cudaMemsetAsync(p.tickets, 0, tickets, a.stream));
+      if (a.clear_counters && split) PRECC_CUDA(ctx, cudaMemsetAsync(p.tickets, 0, counter_bytes(ctx->sm_count), a.stream));
       PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, p));
     }
     return PRECC_OK;

@@ -80,3 +80,51 @@ def test_every_plan_against_the_oracle(monkeypatch, env, hd, n_kv, G, r, ctx, re
                 assert_close(f64(out)[b, g * G:(g + 1) * G], ref, f"request {b} of {n} tokens, head {g}")
     finally:
         px.close()
+
+
+@pytest.mark.parametrize("hd,r,rope,env", [(128, 16, False, TICKET), (64, 8, False, TICKET), (64, 64, False, TICKET), (128, 16, True, {})])
+def test_one_workspace_for_growing_batches_and_other_layers(monkeypatch, hd, r, rope, env):
+    """Split decode calls of 8 .. 256 (request, kv head) pairs, of two layer shapes, on one workspace: what a call leaves in it
+    (records) must not reach what a later call expects to be zero (arrival counters).  A first pass on a workspace
+    of its own is the reference, itself checked against the oracle."""
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    px = Precc(0)
+    try:
+        runs, need, T = [], 0, 4000
+        for n_kv in (8, 2):
+            geo = I.Geometry(512, 2 * n_kv, n_kv, hd, 2, r, r, alpha=2.0 * r)
+            desc, pages, w = layer_desc(geo), T // 16, I.layer_weights(geo, 84, "ws")
+            c = I.direct_caches(pages + 5, geo, 84, f"ws.{hd}.{n_kv}.{r}")
+            cache = Cache.from_tensors(geo, *(c[k].cuda() for k in ("k_base", "v_base", "lr_k", "lr_v")))
+            for B in (1, 8, 16, 32):
+                ctx = [T] + _ragged(B - 1, 1500, T)
+                table = torch.stack([torch.roll(torch.arange(pages + 5), b)[:pages] for b in range(B)]).to(torch.int32)
+                q = I.queries(B, geo, 84, "ws.q", gain=4.0)
+                args = [desc, q.cuda(), torch.tensor([b % 2 for b in range(B)], dtype=torch.int32).cuda(),
+                        torch.tensor(ctx, dtype=torch.int32).cuda(), T, w["B_k"].cuda(), w["B_v"].cuda()]
+                runs.append((args + ([I.rope_table(T, hd)] if rope else []) + [cache], table.cuda(), B))
+                need = max(need, px.decode_workspace(desc, 32, T).numel())
+                if not rope and B in (1, 32):
+                    own = px.decode_workspace(desc, B, T)
+                    out = torch.full_like(args[1], float("nan"))
+                    px.lr_attend_decode(*args, cache, out, own, table.cuda())
+                    b, g = B - 1, n_kv - 1
+                    pg, n, a, cols = table[b].long(), ctx[b], b % 2, slice(g * hd, (g + 1) * hd)
+                    rows = lambda x: f64(x.reshape(-1, x.shape[-1]))[:n]
+                    ref = O.attend_from_caches(f64(q[b, 2 * g:2 * g + 2]), rows(c["k_base"][pg, g]), rows(c["v_base"][pg, g]),
+                                               rows(c["lr_k"][a][pg]), rows(c["lr_v"][a][pg]), f64(w["B_k"][a][:, cols]),
+                                               f64(w["B_v"][a][:, cols]), geo.scale_k, geo.scale_v, 1)
+                    assert_close(f64(out)[b, 2 * g:2 * g + 2], ref, f"batch of {B}, {n} tokens")
+        shared = torch.zeros(need, dtype=torch.uint8, device="cuda")
+        call = px.lr_attend_decode_rope if rope else px.lr_attend_decode
+        for _ in range(2):
+            for args, table, B in runs:
+                own = px.decode_workspace(args[0], B, T)
+                want, out = (torch.full_like(args[1], float("nan")) for _ in range(2))
+                call(*args, want, own, table)
+                call(*args, out, shared, table)
+                assert not torch.isnan(out).any() and torch.equal(out, want), f"batch of {B}, {args[0].n_kv_heads} kv heads"
+        assert px.poll_status() == 0
+    finally:
+        px.close()
