@@ -26,9 +26,12 @@
 // what the warpgroups hand to each other is the row's reference maximum, one word through shared memory behind a
 // named barrier per warp pair, decided right after a step's scores are in registers.  The reference is raised
 // only when the maximum grows by more than 8 (log2 domain), so O' is rescaled a handful of times per row instead of
-// at every step; P stays below 2^8.  The denominator is summed in fp32 by the softmax threads, two values per instruction:
-// an earlier form had the P V' MMA accumulate it through a column of ones, and writing that column into every landed
-// value stage (with its proxy fence) kept the issuing warp busy for 600 cycles of each step.
+// at every step; P stays below 2^8.  The denominator is summed in fp32 by the softmax threads, two values per instruction,
+// for 0 < r_v < 64 from the rounded weights that the MMA sees (8192 over 24576: 4005 -> 4294 us; unrounded, the sum left a
+// row dominated by one token up to 2^-8 off, on top of its own rounding, and the error against float64 5 .. 15 % higher
+// where a few tokens carry a row).  Measured for the same sum and slower: a column of ones beside L_V for the P V' MMA to
+// sum - written into every landed value stage by the issuing warp it takes 600 cycles of a step, by the softmax threads 6 %
+// more time on the mean - and a warp-level mma.sync against a selection matrix, which competes with tcgen05 (5039 us).
 //
 // Warp roles: warp 0 = TMA producer of the key ring, warp 3 = TMA producer of the value ring
 // (keys are released right after S is computed, values only after O' is updated, so the two rings run
@@ -130,6 +133,9 @@ struct PrefillTcCfg {
   static constexpr int VSLABS = SLABS + (RV > 0 ? 1 : 0);     // L_V rides as one more 64-column slab (zero padded)
   static constexpr int RVP = RV == 8 ? 16 : RV;               // value-side coordinates as the MMAs see them (rank 8: zero-padded)
   static constexpr int OW = HD + RVP;                         // columns of O' in TMEM: [O | U]
+  // The denominator is the sum of the bf16 weights that the P V' MMA multiplies, so that the rounding of a dominant weight
+  // cancels; with no value adapter or rank 64 it is the sum of the unrounded ones (the accuracy these always had).
+  static constexpr bool L_ROUNDED = RV > 0 && RV < 64;
   static constexpr int VSTAGE = VSLABS * SLAB_BYTES;          // {V_base slabs | L_V slab}
   static constexpr int K_PAGE_TX = PAGE * (HD + RKP) * 2;      // bytes one page contributes to a key stage
   static constexpr int V_PAGE_TX = PAGE * VSLABS * 128;
@@ -797,8 +803,10 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
             float p0, p1;
             fma2(p0, p1, sv[c][k], sv[c][k + 1], p.scale_log2, neg_m);
             p0 = fast_exp2(p0); p1 = fast_exp2(p1);
-            add2(ls[k & 2], ls[(k & 2) + 1], p0, p1);
-            pk[c >> 1][(c & 1) * 16 + k / 2] = pack_bf16(p0, p1);
+            const uint32_t w = pack_bf16(p0, p1);
+            if constexpr (C::L_ROUNDED) add2(ls[k & 2], ls[(k & 2) + 1], __uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+            else add2(ls[k & 2], ls[(k & 2) + 1], p0, p1);
+            pk[c >> 1][(c & 1) * 16 + k / 2] = w;
           }
         l_sum += (ls[0] + ls[1]) + (ls[2] + ls[3]);
         if ((tid & 127) == 0) PTC_STAMP(p, j, 14);                 // all exponentials done

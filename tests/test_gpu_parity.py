@@ -650,6 +650,52 @@ def test_prefill_with_a_workspace_puts_helper_blocks_on_idle_sms(monkeypatch, hd
     assert p2.poll_status() == 0
 
 
+@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("r", [0, 8, 16, 32, 64])
+def test_prefill_normalises_by_the_weights_it_multiplies(px, hd, r):
+    """Rows dominated by one token of a later step, whose weight is no bf16 number (a reference maximum stays in force
+    until the maximum grows by 8 in the log2 domain).  Where the denominator is the sum of the rounded weights (0 < rank <
+    64), the weight's rounding cancels: what is left is the output's own rounding (2^-8 of the value at most) and 2^-8 / 54
+    of the first token's share, 54 = e^4.  Elsewhere the sum is of unrounded weights: 2^-8 more."""
+    from paper_2609_34054_b200.binding import Cache, layer_desc
+    geo, S, T, late = I.Geometry(512, 8, 2, hd, 2, r, r, alpha=2.0 * max(r, 1)), 64, 960, 900
+    k = torch.zeros((S + T) // 16, 2, 16, hd, dtype=torch.bfloat16)
+    k[..., 0] = -8.0                                        # next to nothing: e^-32
+    k[0, :, 0, 0], k[late // 16, :, late % 16, 0] = 0.0, 1.0
+    v = torch.zeros_like(k)
+    v[late // 16, :, late % 16] = (1.0 + I.uniform_int(0, 127, 2 * hd, 31, "peak.v").reshape(2, hd) / 128.0).to(torch.bfloat16)
+    lr = torch.zeros(2, k.shape[0], 16, r, dtype=torch.bfloat16, device="cuda") if r else None
+    B = torch.zeros(2, r, 2 * hd, dtype=torch.bfloat16, device="cuda") if r else None
+    q = torch.zeros(S, 8, hd, dtype=torch.bfloat16)
+    q[..., 0] = ((4.0 + torch.arange(S * 8).reshape(S, 8) / (S * 8) * 1.5) * hd ** 0.5).to(torch.bfloat16)
+    out = torch.full_like(q, float("nan"), device="cuda")
+    px.lr_attend_prefill(layer_desc(geo), q.cuda(), 0, T, B, B, Cache.from_tensors(geo, k.cuda(), v.cuda(), lr, lr), out)
+    weight = np.exp(f64(q[..., 0]) / hd ** 0.5)             # against the first token's 1; up to 1022 others of weight^-8 each
+    others = (T - 1 + np.arange(S)[:, None]) * weight ** -8.0
+    ref = (weight / (weight + 1.0 + others))[..., None] * f64(v[late // 16, :, late % 16]).repeat(4, axis=0)[None]
+    weight_rounding = 1.0 / 54.0 if 0 < r < 64 else 1.0
+    assert np.abs(f64(out) / ref - 1.0).max() <= 2.0 ** -8 * (1.0 + weight_rounding) + 2e-5
+
+
+@pytest.mark.parametrize("hd,r,T", [(128, 16, 300), (64, 64, 700), (128, 0, 40)])
+def test_prefill_row_that_is_not_a_number_keeps_to_itself(px, hd, r, T):
+    """A query of NaN: its head's row is NaN, every other row is what it is without it, bit for bit."""
+    from paper_2609_34054_b200.binding import Cache, layer_desc
+    geo, S = I.Geometry(512, 8, 2, hd, 2, r, r, alpha=2.0 * max(r, 1)), 70
+    c, w = I.direct_caches((S + T + 15) // 16, geo, 32, "nan"), I.layer_weights(geo, 32, "nan")
+    lr = [c[n].cuda() if r else None for n in ("lr_k", "lr_v")]
+    B = [w[n].cuda() if r else None for n in ("B_k", "B_v")]
+    cache, q = Cache.from_tensors(geo, c["k_base"].cuda(), c["v_base"].cuda(), *lr), I.queries(S, geo, 32, "nan.q").cuda()
+    clean, out = torch.empty_like(q), torch.empty_like(q)
+    px.lr_attend_prefill(layer_desc(geo), q, 1, T, *B, cache, clean)
+    bad = q.clone()
+    for i, h in ((0, 0), (13, 5), (69, 7)):
+        bad[i, h] = float("nan")
+    px.lr_attend_prefill(layer_desc(geo), bad, 1, T, *B, cache, out)
+    own = torch.isnan(bad)
+    assert torch.isnan(out[own]).all() and torch.equal(out[~own], clean[~own])
+
+
 @pytest.mark.parametrize("n", [1, 10, 100])
 def test_per_row_agent_masks_equal_two_separate_projections(px, n):
     """Double batching: adapted rows (current agent's LR rows, private slots) and adapter-free rows (the other
