@@ -446,9 +446,12 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         atomicOr(p.status, StatusBits::BAD_INDEX);
         return 0;
       };
-      // helper warps copy the pages' second slab (12: keys, 13: values) and LR rows (14, 15)
+      // helper warps copy the pages' second slab (12: keys, 13: values) and LR rows (14, 15).  One that has nothing to copy
+      // (whole-stage boxes, head_dim 64, no adapter on its side) must not walk the ring: a stage is full without it, so
+      // nothing keeps the ring from going round twice before it looks, and then its wait by parity never ends.
       const int role = warp < PTC_FIRST_SM_WARP ? warp : (warp & 1) ? 3 : 0;
       const int share = warp < PTC_FIRST_SM_WARP ? 0 : 1 + ((warp - PTC_FIRST_HELPER) >> 1);
+      auto copies = [&](bool whole, int rank) { return share == 0 || (!whole && (share == 1 ? C::SLABS > 1 : rank > 0)); };
       if (role == 0) {
         // -------------------------------------------------------------- TMA producer: query tile, B slices, keys
         const bool whole = p.contig || p.k_logical;
@@ -472,7 +475,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         __syncwarp();
         }
         int ph_next = whole || lane >= PTC_TOK / PAGE ? 0 : lookup(jb * (PTC_TOK / PAGE) + lane);
-        const int n_items = share == 0 ? (RV > 0 && n_tiles > 0 ? n_tiles + 1 : n_tiles) : whole ? 0 : n_tiles;
+        const int n_items = copies(whole, RK) ? n_tiles + (share == 0 && RV > 0 && n_tiles > 0 ? 1 : 0) : 0;
         for (int j = 0; j < n_items; ++j) {
           const int s = j % KS;
           if (j >= KS) mbar_wait(k_empty + 8 * s, ((j / KS) - 1) & 1, p.status);
@@ -524,7 +527,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         // -------------------------------------------------------------- TMA producer: values, in units of a step or half a step
         constexpr int UT = VH ? PTC_TOK / 2 : PTC_TOK, UPG = UT / PAGE, UPS = PTC_TOK / UT, USLAB = UT * 128;
         int ph_next = p.contig || lane >= UPG ? 0 : lookup(UPS * jb * UPG + lane);
-        const int n_units = share > 0 && p.contig ? 0 : UPS * n_tiles;
+        const int n_units = copies(p.contig, RV) ? UPS * n_tiles : 0;
         for (int u = 0; u < n_units; ++u) {
           const int s = u % VS;
           if (u >= VS) mbar_wait(v_empty + 8 * s, ((u / VS) - 1) & 1, p.status);

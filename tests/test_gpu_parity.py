@@ -696,6 +696,27 @@ def test_prefill_row_that_is_not_a_number_keeps_to_itself(px, hd, r, T):
     assert torch.isnan(out[own]).all() and torch.equal(out[~own], clean[~own])
 
 
+@pytest.mark.parametrize("hd,rk,rv", [(64, 0, 0), (64, 16, 16), (64, 0, 8), (128, 0, 0), (128, 0, 32), (128, 32, 32), (128, 64, 64)])
+@pytest.mark.parametrize("T,S", [(90, 30), (9001, 40)])
+def test_prefill_of_paged_caches_equals_contiguous_ones(px, hd, rk, rv, T, S):
+    """Every set of copying warps (second slab, LR rows of either side, or none), one round of the rings and many: pages
+    in mixed order give the bits of consecutive ones, and no bounded wait runs out."""
+    from paper_2609_34054_b200.binding import Cache, layer_desc
+    geo = I.Geometry(512, 8, 2, hd, 2, rk, rv, alpha=2.0 * max(rk, rv, 1))
+    n = (S + T + 15) // 16
+    c, w = I.direct_caches(n, geo, 33, "pg"), I.layer_weights(geo, 33, "pg")
+    B = [w["B_k"].cuda() if rk else None, w["B_v"].cuda() if rv else None]
+    place = lambda order: Cache.from_tensors(geo, c["k_base"][order].cuda(), c["v_base"][order].cuda(),
+                                             c["lr_k"][:, order].cuda() if rk else None, c["lr_v"][:, order].cuda() if rv else None)
+    order = (torch.arange(n) * 7 + 3) % n if n % 7 else torch.arange(n).flip(0)      # physical block i holds logical block order[i]
+    q = I.queries(S, geo, 33, "pg.q").cuda()
+    whole, paged = torch.full_like(q, float("nan")), torch.full_like(q, float("nan"))
+    px.lr_attend_prefill(layer_desc(geo), q, 1, T, *B, place(torch.arange(n)), whole)
+    px.lr_attend_prefill(layer_desc(geo), q, 1, T, *B, place(order), paged, torch.argsort(order).to(torch.int32).cuda())
+    assert px.poll_status() == 0
+    assert not torch.isnan(whole).any() and torch.equal(paged, whole)
+
+
 @pytest.mark.parametrize("n", [1, 10, 100])
 def test_per_row_agent_masks_equal_two_separate_projections(px, n):
     """Double batching: adapted rows (current agent's LR rows, private slots) and adapter-free rows (the other
