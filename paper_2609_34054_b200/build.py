@@ -32,20 +32,27 @@ def _obj(src: str) -> str:
     return os.path.join(OBJ, src[:-3] + ".o")
 
 
+def resource_log(src: str) -> str:
+    """What ptxas reported of the unit's kernels: registers, shared memory, spills."""
+    return os.path.join(OBJ, src[:-3] + ".ptxas.log")
+
+
 def _stale(src: str, hdr_time: float) -> bool:
     o = _obj(src)
-    if not os.path.exists(o):
+    if not os.path.exists(o) or not os.path.exists(resource_log(src)):
         return True
     t = os.path.getmtime(o)
     return os.path.getmtime(os.path.join(CSRC, src)) > t or hdr_time > t
 
 
-def _compile(nvcc: str, src: str, verbose: bool) -> str:
+def _compile(nvcc: str, src: str) -> str:
     extra = os.environ.get("PRECC_NVCC_FLAGS", "").split()          # e.g. -DPRECC_PF_TRACE -DPRECC_GEMM_TRACE (timeline stamps)
-    cmd = [nvcc] + NVCC_FLAGS + extra + (["-Xptxas=-v"] if verbose else []) + ["-c", os.path.join(CSRC, src), "-o", _obj(src)]
+    cmd = [nvcc] + NVCC_FLAGS + extra + ["-Xptxas=-v", "-c", os.path.join(CSRC, src), "-o", _obj(src)]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}{r.stderr}")
+    with open(resource_log(src), "w") as f:
+        f.write(r.stdout + r.stderr)
     return r.stderr
 
 
@@ -76,7 +83,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         _build_native(False)
         return LIB
     with concurrent.futures.ThreadPoolExecutor(max_workers=min(len(todo), os.cpu_count() or 1) or 1) as pool:
-        for log in pool.map(lambda s: _compile(nvcc, s, verbose), todo):
+        for log in pool.map(lambda s: _compile(nvcc, s), todo):
             if verbose:
                 sys.stderr.write(log)
     r = subprocess.run([nvcc, "-shared", "-Xlinker", "-soname=libprecc.so", "-o", LIB] + [_obj(s) for s in SOURCES], capture_output=True, text=True)

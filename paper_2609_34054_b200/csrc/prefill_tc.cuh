@@ -40,8 +40,10 @@
 // / correction / epilogue, warps 12-15 = more TMA issuers for paged caches: a copy costs its issuing warp about a hundred
 // cycles, and a step of a paged cache is up to 48 copies (two slabs and the LR rows of eight pages, keys and values), so
 // each warp takes eight of them (two issuers: 2250 cycles per step at head_dim 128; six: 1750, bound by the softmax).
-// Registers are re-split at kernel start: 208 per softmax thread, 48 for the other eight warps
-// (8 x 208 + 8 x 48 = 16 x 128).  Every mbarrier wait is bounded and falls through with PRECC_STATUS_TIMEOUT.
+// Registers are re-split at kernel start: 216 per softmax thread, 40 for the other eight warps
+// (8 x 216 + 8 x 40 = 16 x 128).  Nothing may spill in the step loop: shared memory is addressed in its own address space
+// (a base rounded up as an integer made every access a generic one with a 64-bit address: 5 % of the time of a turn), and the
+// work-list form reads its piece's data again for the epilogue.  Every mbarrier wait is bounded and falls through with PRECC_STATUS_TIMEOUT.
 //
 // Two more instantiations of the same kernel.  VH: the value ring holds units of 64 tokens instead of whole
 // steps (where one value stage fits beside two key stages but two do not), a unit being freed as soon as its
@@ -108,7 +110,7 @@ constexpr int PTC_FIRST_SM_WARP = 4;                 // warps 0..3: key producer
 constexpr int PTC_SOFTMAX_WARPS = 8;                 // two warpgroups, taking alternate steps
 constexpr int PTC_FIRST_HELPER = PTC_FIRST_SM_WARP + PTC_SOFTMAX_WARPS;   // four more TMA issuers (paged caches)
 constexpr int PTC_THREADS = (PTC_FIRST_HELPER + 4) * 32;
-constexpr int PTC_SM_REGS = 208, PTC_CTL_REGS = 48;  // 256 x 208 + 256 x 48 = 512 x 128, the launch's registers
+constexpr int PTC_SM_REGS = 216, PTC_CTL_REGS = 40;  // 256 x 216 + 256 x 40 = 512 x 128, the launch's registers
 constexpr int PTC_SMEM_LIMIT = 232448;   // dynamic shared memory a block can opt into on this architecture
 constexpr int PTC_FIXED_BARS = 13; // barriers besides the two per ring stage
 constexpr int PTC_XCH_BYTES = 4 * 512;   // [2][128] reference maxima | [2][128] partial denominators
@@ -273,7 +275,7 @@ __global__ void __launch_bounds__(PTC_THREADS, 1)
 lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __grid_constant__ PrefillTcParams p) {
   using C = PrefillTcCfg<HD, RK, RV>;
   extern __shared__ unsigned char smem_raw[];
-  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  unsigned char* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);   // (pointer arithmetic, so that it stays a shared-memory address)
   const uint32_t q_u32 = smem_u32(smem);
   const uint32_t qx_u32 = q_u32 + C::Q_BYTES;
   const uint32_t kring_u32 = qx_u32 + C::QX_BYTES;
@@ -383,7 +385,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
   // first step, `n_tiles` its number of steps (possibly zero under a context split).  Work-list launch: a short list of
   // tile pieces, taken one after the other with the block drained in between.  Loop indices are local, token
   // positions use jb + j.
-  const int nseg = WL ? tab_sc[0] : 1;
+  auto nseg = [&]() -> int { return WL ? tab_sc[0] : 1; };
   int g = 0, tok0 = 0, n_tok = 0, t_end = 0, full_vis = 0, jb = 0, n_tiles = 0;
   bool to_ws = false;                                      // work-list launch: this piece goes to a record
   int tile_u = 0, rec_id = 0, n_src = 1, src_first = 0;    // its tile, its record, and which records make up the tile
@@ -423,7 +425,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
       tc_fence_before();
       __syncwarp();
       named_sync(0, PTC_THREADS);
-      if (seg + 1 < nseg && threadIdx.x == 0) {
+      if (seg + 1 < nseg() && threadIdx.x == 0) {
         for (int i = 0; i < n_bars; ++i) asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bar0 + 8 * i) : "memory");
         init_bars();
       }
@@ -435,7 +437,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
 
   if (warp < PTC_FIRST_SM_WARP || warp >= PTC_FIRST_HELPER) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(PTC_CTL_REGS));
-    for (int seg = 0; seg < nseg; ++seg) {
+    for (int seg = 0; seg < nseg(); ++seg) {
       load_piece(seg);
       const int n_pages = (t_end + PAGE - 1) / PAGE;       // logical pages this tile may touch
       // physical block of a logical page (paged caches), fetched a step ahead of its use: the producers would otherwise sit
@@ -705,12 +707,11 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
     float* mref = xch;                                            // [2][128]: reference maximum after a step, by step parity
     float* lpart = xch + 256;                                     // [2][128]: the warpgroups' denominators
     const int bar_in = 2 + 2 * quad + (wg ^ 1), bar_out = 2 + 2 * quad + wg;   // named barriers: hand-over of the reference maximum within a warp pair
-    for (int seg = 0; seg < nseg; ++seg) {
+    for (int seg = 0; seg < nseg(); ++seg) {
       load_piece(seg);
       PTC_WL_STAMP(p, seg, 0);                                     // piece starts
-      const int i_new = tok0 + row / G, hg = row % G;
-      const bool row_ok = row < n_tok * G;
-      const int lim = row_ok ? p.T + i_new : -1;                  // last visible token of this row
+      // tokens visible to this thread's row, and to every row of the block, counted from the piece's first step
+      const int lim = (row < n_tok * G ? p.T + tok0 + row / G + 1 : 0) - jb * PTC_TOK, full = full_vis - jb * PTC_TOK;
       if constexpr (RK > 0) {
         // the folded query: fp32 product of the fold MMA, scaled and rounded to bf16, as a K-major swizzled operand
         constexpr int CPR = C::RKP / 8;
@@ -753,7 +754,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         if (lane == 0) mbar_arrive(s_free + 8 * wg);               // the S buffer may be overwritten
         if ((tid & 127) == 0) PTC_STAMP(p, j, 7);                  // scores in registers
         if constexpr (MASKED) {
-          const int nvis = lim - (jb + j) * PTC_TOK + 1;           // visible tokens of this step
+          const int nvis = lim - j * PTC_TOK;           // visible tokens of this step
 #pragma unroll
           for (int c = 0; c < 4; ++c)
 #pragma unroll
@@ -808,6 +809,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
             p0 = fast_exp2(p0); p1 = fast_exp2(p1);
             const uint32_t w = pack_bf16(p0, p1);
             if constexpr (C::L_ROUNDED) add2(ls[k & 2], ls[(k & 2) + 1], __uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+            else if constexpr (WL) { ls[k & 2] += p0; ls[(k & 2) + 1] += p1; }      // (packed, ptxas spills here)
             else add2(ls[k & 2], ls[(k & 2) + 1], p0, p1);
             pk[c >> 1][(c & 1) * 16 + k / 2] = w;
           }
@@ -830,7 +832,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         if ((tid & 127) == 0) PTC_STAMP(p, j, 6);                  // P published
       };
       for (int j = wg; j < n_tiles; j += 2) {
-        if ((jb + j) * PTC_TOK + PTC_TOK > full_vis) step(j, std::true_type{});   // only the last few steps reach the causal edge
+        if (j * PTC_TOK + PTC_TOK > full) step(j, std::true_type{});   // only the last few steps reach the causal edge
         else step(j, std::false_type{});
       }
       PTC_WL_STAMP(p, seg, 2);                                     // this warpgroup's steps done
@@ -844,6 +846,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
       }
       lpart[wg * 128 + row] = l_sum * fast_exp2(m_own - m_fin);
       named_sync(1, NSM);
+      if constexpr (WL) load_piece(seg);                           // read again rather than held in registers through the steps
       const float l_tot = lpart[row] + lpart[128 + row];
       if constexpr (RV > 0) {
         if (n_tiles > 0) {
@@ -1049,13 +1052,13 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         PTC_WL_STAMP(p, seg, 5);                                   // piece ends
       } else {
         const float inv = 1.f / l_tot;
-        __nv_bfloat16* orow = p.out + ((size_t)i_new * p.n_q + (size_t)g * G + hg) * HD;
+        __nv_bfloat16* orow = p.out + ((size_t)(tok0 + row / G) * p.n_q + (size_t)g * G + row % G) * HD;
 #pragma unroll
         for (int c = wg; c < HD / 32; c += 2) {                   // 32-column chunks: this warpgroup's half of the row
           uint32_t ov[32];
           tmem_ld32(lane_addr + C::TMEM_O + c * 32, ov);
           tmem_wait_ld();
-          if (row_ok) {
+          if (row < n_tok * G) {
 #pragma unroll
             for (int k = 0; k < 32; k += 8) {
               uint4 w;
