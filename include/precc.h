@@ -137,10 +137,11 @@ int32_t precc_selftest_wait_timeout(precc_ctx* ctx, uint32_t* done_flag, void* s
  * elements and must be packed with the dst_rows it is later used with.  Used to build the packed A (all
  * agents' down-projections side by side, Section 3.1), the packed W and the two together.  src, dst
  * device; d_model % 64 == 0.
- * Packed matrices are constants of the projection calls: a projection is a programmatic
- * dependent launch and requests its first weight boxes before it waits for the kernel ahead of it on the stream
- * (H, the slot and mask arrays and every store come after that wait).  precc_pack_kmajor itself never lets a
- * dependent launch start early, so packing and projecting back to back on one stream is ordered as usual. */
+ * Packed matrices are constants of the projection calls of up to 64 rows: such a call is a programmatic dependent
+ * launch and may request its first weight boxes before it waits for the kernel ahead of it on the stream (H, the slot
+ * and mask arrays and every store come after that wait; calls of more rows read everything after it).
+ * precc_pack_kmajor itself never lets a dependent launch start early, so packing and projecting back to back on one
+ * stream is ordered as usual. */
 int32_t precc_pack_kmajor(precc_ctx* ctx, const void* src, int32_t d_model, int32_t n_cols,
                           void* dst, int32_t dst_rows, int32_t dst_row0, void* stream);
 

@@ -207,14 +207,8 @@ proj_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_holder)), "r"(p.tmem_cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
   }
-  // the first weight boxes go out before the wait for the kernel ahead (the weights are constants); X, the slot and mask
-  // arrays and every store come after it
-  if (warp == 0 && lane == 0 && blockIdx.x < n_tiles) {
-    for (int it = 0; it < min(p.stages, nkb); ++it) {
-      mbar_expect_tx(full0 + 8 * it, stage_bytes);
-      tma_load_3d(smem_u32(smem + (size_t)it * stage_bytes) + GEMM_A_BYTES, &map_w, 0, ((int)blockIdx.x % n_tiles_n) * p.BN, it, full0 + 8 * it);
-    }
-  }
+  // The set-up above overlaps the end of the kernel ahead (programmatic dependent launch).  Everything that kernel may have
+  // written comes after the wait, the packed weights included: its writes are visible only then.
   pdl_wait();
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
@@ -227,7 +221,6 @@ proj_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
   // so the epilogue of one tile overlaps the MMAs of the next.
   if (warp == 0) {
     if (lane == 0) {
-      const int pre = min(p.stages, nkb);              // weight boxes already requested
       int it = 0;
       for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         const int m0 = row0_of(t / n_tiles_n), n0 = (t % n_tiles_n) * p.BN;
@@ -236,9 +229,9 @@ proj_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
           if (it >= p.stages) mbar_wait(empty0 + 8 * s, ((it / p.stages) - 1) & 1, p.status);
           GEMM_STAMP(p, it, 0);
           const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
-          if (it >= pre) mbar_expect_tx(full0 + 8 * s, stage_bytes);
+          mbar_expect_tx(full0 + 8 * s, stage_bytes);
           tma_load_2d(sa, &map_x, kb * GEMM_BK, m0, full0 + 8 * s);
-          if (it >= pre) tma_load_3d(sa + GEMM_A_BYTES, &map_w, 0, n0, kb, full0 + 8 * s);    // packed weights are k-blocked
+          tma_load_3d(sa + GEMM_A_BYTES, &map_w, 0, n0, kb, full0 + 8 * s);      // packed weights are k-blocked
           GEMM_STAMP(p, it, 1);
         }
       }
@@ -457,16 +450,15 @@ proj_gemm_splitk_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
     mbar_init(acc_full, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    // the ring's first fill is requested right away (this thread is the producer): its latency then overlaps the
-    // tensor-memory allocation and the block barrier below.  The weights are constants, so their boxes go out before
-    // the wait for the kernel ahead (programmatic dependent launch); X and every store come after it.
-    for (int it = 0; it < min(p.stages, nkb_s); ++it) {
-      mbar_expect_tx(full0 + 8 * it, stage_bytes);
-      tma_load_3d(smem_u32(smem + (size_t)it * stage_bytes) + GEMM_A_BYTES, &map_w, 0, n0, kb0 + it, full0 + 8 * it);
-    }
+    // the ring's first fill is requested right behind the wait for the kernel ahead (this thread is the producer): its
+    // latency then overlaps the tensor-memory allocation and the block barrier below
     pdl_wait();
-    for (int it = 0; it < min(p.stages, nkb_s); ++it)
-      tma_load_2d(smem_u32(smem + (size_t)it * stage_bytes), &map_x, (kb0 + it) * GEMM_BK, m0, full0 + 8 * it);
+    for (int it = 0; it < min(p.stages, nkb_s); ++it) {
+      const uint32_t sa = smem_u32(smem + (size_t)it * stage_bytes);
+      mbar_expect_tx(full0 + 8 * it, stage_bytes);
+      tma_load_2d(sa, &map_x, (kb0 + it) * GEMM_BK, m0, full0 + 8 * it);
+      tma_load_3d(sa + GEMM_A_BYTES, &map_w, 0, n0, kb0 + it, full0 + 8 * it);
+    }
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_holder)), "r"(p.tmem_cols) : "memory");
@@ -674,13 +666,13 @@ proj_gemm_splitk_push_kernel(const __grid_constant__ CUtensorMap map_x, const __
     mbar_expect_tx(recv_bar, direct ? (uint32_t)((KS - 1) * rows_valid * vw_own * 4) : (uint32_t)((KS - 1) * slice_bytes));
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    for (int it = 0; it < min(p.stages, nkb_s); ++it) {        // weights before the wait for the kernel ahead, as above
+    pdl_wait();                                                // then the ring's first fill, as above
+    for (int it = 0; it < min(p.stages, nkb_s); ++it) {
+      const uint32_t sa = smem_u32(smem + (size_t)it * stage_bytes);
       mbar_expect_tx(full0 + 8 * it, stage_bytes);
-      tma_load_3d(smem_u32(smem + (size_t)it * stage_bytes) + GEMM_A_BYTES, &map_w, 0, n0, kb0 + it, full0 + 8 * it);
+      tma_load_2d(sa, &map_x, (kb0 + it) * GEMM_BK, m0, full0 + 8 * it);
+      tma_load_3d(sa + GEMM_A_BYTES, &map_w, 0, n0, kb0 + it, full0 + 8 * it);
     }
-    pdl_wait();
-    for (int it = 0; it < min(p.stages, nkb_s); ++it)
-      tma_load_2d(smem_u32(smem + (size_t)it * stage_bytes), &map_x, (kb0 + it) * GEMM_BK, m0, full0 + 8 * it);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_holder)), "r"(p.tmem_cols) : "memory");

@@ -57,6 +57,7 @@ rope_expand_keys_kernel(const RopeExpandParams p) {
   const int task = blockIdx.y * RxCfg<KS>::GROUP_TASKS + warp;
   const bool has_task = task < n_tasks;
   const int tg_head = task / tasks_per_head, tc0 = (task - tg_head * tasks_per_head) * 16;
+  pdl_wait();                  // the kernel ahead may have written anything that is read below
   // ---- this warp's B^K fragments (k = rank, n = column), zero beyond the rank and beyond the last task
   uint32_t bfr[4][KS][2];
 #pragma unroll
@@ -129,7 +130,6 @@ rope_expand_keys_kernel(const RopeExpandParams p) {
       for (int h = 0; h < 2; ++h)
         x.cs[t][h] = __ldg(p.rope + (size_t)min(t0 + r + 8 * h, p.max_pos - 1) * (hd / 4) + (tc0 + t * 8 + q2) / 2);
   };
-  pdl_wait();                  // the kernel ahead may have written cache rows of this sequence
   In cur;
   int lb = blockIdx.x;
   if (lb < p.n_out_blocks) fetch(lb, cur);
