@@ -140,8 +140,9 @@ int32_t precc_selftest_wait_timeout(precc_ctx* ctx, uint32_t* done_flag, void* s
  * Packed matrices are constants of the projection calls of up to 64 rows: such a call is a programmatic dependent
  * launch and may request its first weight boxes before it waits for the kernel ahead of it on the stream (H, the slot
  * and mask arrays and every store come after that wait; calls of more rows read everything after it).
- * precc_pack_kmajor itself never lets a dependent launch start early, so packing and projecting back to back on one
- * stream is ordered as usual. */
+ * precc_pack_kmajor ends with a launch that orders its writes before such a request, so packing and projecting back
+ * to back on one stream is ordered as usual; behind any other kernel that writes a packed matrix put another launch or an
+ * event before a projection of up to 64 rows. */
 int32_t precc_pack_kmajor(precc_ctx* ctx, const void* src, int32_t d_model, int32_t n_cols,
                           void* dst, int32_t dst_rows, int32_t dst_row0, void* stream);
 

@@ -175,6 +175,8 @@ __global__ void pack_kmajor_kernel(const __nv_bfloat16* __restrict__ src, int d,
   }
 }
 
+__global__ void pack_done_kernel() {}
+
 }  // namespace
 
 }  // namespace precc
@@ -305,6 +307,11 @@ int32_t precc_pack_kmajor(precc_ctx* ctx, const void* src, int32_t d_model, int3
   if (d_model % GEMM_BK) return fail(ctx, PRECC_ERR_UNSUPPORTED, "pack_kmajor: d_model %% 64 != 0");
   dim3 grid((n_cols + 31) / 32, (d_model + 31) / 32), block(32, 8);
   pack_kmajor_kernel<<<grid, block, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)src, d_model, n_cols, (__nv_bfloat16*)dst, dst_rows, dst_row0);
+  PRECC_CUDA(ctx, cudaGetLastError());
+  // A projection of few rows requests weight boxes before it waits for the kernel ahead, and may start as soon as that
+  // kernel's blocks have left - before its writes are promised to be visible.  So the kernel ahead is not the packing: an
+  // ordinary launch starts only when everything before it has completed and is visible.
+  pack_done_kernel<<<1, 1, 0, (cudaStream_t)stream>>>();
   PRECC_CUDA(ctx, cudaGetLastError());
   return PRECC_OK;
 }

@@ -717,6 +717,29 @@ def test_prefill_of_paged_caches_equals_contiguous_ones(px, hd, rk, rv, T, S):
     assert not torch.isnan(whole).any() and torch.equal(paged, whole)
 
 
+@pytest.mark.parametrize("M", [1, 40, 64, 200, 1500])
+def test_projection_right_behind_the_packing_of_its_weights(px, M):
+    """Weights packed again and again into one buffer, each time projected with at once: the rows are those of the new
+    weights (kernels of few rows request weight boxes before they wait for the kernel ahead)."""
+    geo = I.Geometry(1024, 8, 2, 64, 2, 16, 16, alpha=32.0)
+    L = Layer(px, geo, seed=17, n_blocks=(M + 15) // 16, fill=0.0)
+    H = I.hidden_states(M, geo, 17, "pack.H").cuda()
+    sets = [[I.normal_bf16((geo.d_model, geo.kv_width), 0.02, 17, f"pack.{i}.{n}").cuda() for n in "kv"] for i in range(4)]
+    packed = [px.pack_base_weights(geo, *w) for w in sets]
+    torch.cuda.synchronize()
+    want = []
+    for W in packed:
+        px.rebase_project(L.desc, H, W, L.cache, 0)
+        torch.cuda.synchronize()
+        want.append((L.cache.k_base.clone(), L.cache.v_base.clone()))
+    for i in range(24):
+        W = px.pack_base_weights(geo, *sets[i % 4])       # (the allocator hands out the buffer of the round before)
+        px.rebase_project(L.desc, H, W, L.cache, 0)
+        got = L.cache.k_base.clone(), L.cache.v_base.clone()
+        assert torch.equal(got[0], want[i % 4][0]) and torch.equal(got[1], want[i % 4][1])
+        del W
+
+
 @pytest.mark.parametrize("n", [1, 10, 100])
 def test_per_row_agent_masks_equal_two_separate_projections(px, n):
     """Double batching: adapted rows (current agent's LR rows, private slots) and adapter-free rows (the other
