@@ -73,6 +73,7 @@ constexpr int DEC_WARPS = 4;            // ticket kernel
 constexpr int DEC_MAX_SPLITS = 512;
 constexpr int DEC_FLAT_MAX_B = 256;     // requests that the flat grid's schedule handles (8 per lane)
 constexpr int DEC_MAX_CLUSTER = 16;
+constexpr int DEC_MAX_STAGES = 4;       // pages of a warp's ring in the cluster kernel at most
 // Overlap with the preceding kernel (programmatic dependent launch): before the kernel waits for its
 // predecessor it already reads the index arrays, the adapter matrices and every cache page that holds
 // none of the request's last DEC_PDL_TAIL tokens.  The newest tokens (the in-turn append of the preceding

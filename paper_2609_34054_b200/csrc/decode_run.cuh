@@ -52,7 +52,8 @@ struct DecodeRunT {
     }
     return best;
   }
-  // Can `need` clusters of `cs` blocks be resident at once?  Asked once per (shape, warps, cluster size).
+  // Can `need` clusters of `cs` blocks be resident at once?  Asked once per (shape, warps, ring depth, cluster size): the depth
+  // decides the shared memory of a block, and an answer for another depth would make a plan depend on earlier calls.
   // The cluster kernel's shared-memory limit is only ever raised: the two ring layouts of one shape (two blocks
   // per SM / one block per SM) need different amounts, and lowering the attribute for the smaller one would
   // make a later launch of the larger one fail.
@@ -81,9 +82,9 @@ struct DecodeRunT {
   }
   template <int NW>
   static bool cluster_fits(precc_ctx* ctx, const DecodePlan& pl, int need) {
-    static int cache2[kMaxDevices][2][DEC_MAX_CLUSTER + 1] = {{{0}}};  // 0 = unknown, else max active clusters + 1
+    static int cache2[kMaxDevices][DEC_MAX_STAGES + 1][DEC_MAX_CLUSTER + 1] = {{{0}}};  // 0 = unknown, else max active clusters + 1
     std::lock_guard<std::recursive_mutex> lk(lazy_mu());
-    int* cached = cache2[ctx->device % kMaxDevices][pl.deep ? 1 : 0];
+    int* cached = cache2[ctx->device % kMaxDevices][pl.stages];
     if (cached[pl.cluster] == 0) {
       ClusterKernel kern = cluster_kernel<NW>(pl.deep != 0);
       int n = 0;
@@ -161,7 +162,7 @@ struct DecodeRunT {
   static DecodePlan plan_cluster(precc_ctx* ctx, long long units, int max_tiles, int warps, int per_sm, int max_stages, int lim) {
     using C = DecodeCfg<HD, RK, RV>;
     DecodePlan pl{};
-    int stages = max_stages;
+    int stages = max_stages < DEC_MAX_STAGES ? max_stages : DEC_MAX_STAGES;
     if (ctx->decode_stage_cap >= 2 && stages > ctx->decode_stage_cap) stages = ctx->decode_stage_cap;
     while (stages > 2 && per_sm * (C::cluster_smem(warps, stages) + extra + 1024) > ctx->max_smem_optin) --stages;
     pl.smem = C::cluster_smem(warps, stages) + extra;
