@@ -205,7 +205,7 @@ class Precc:
 
     # ------------------------------------------------------------------ plumbing
     def set_trace_buffer(self, buf: Optional[torch.Tensor]):
-        """int64 CUDA tensor [n_blocks, 8] receiving per-block phase timestamps of decode, or None."""
+        """int64 CUDA tensor [n_blocks, 16] receiving per-block phase timestamps of decode, or None."""
         if buf is None:
             self._check(self.lib.precc_set_trace_buffer(self.h, None, 0), "precc_set_trace_buffer")
         else:

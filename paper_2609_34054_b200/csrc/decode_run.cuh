@@ -193,7 +193,8 @@ struct DecodeRunT {
   //   few pages       a block per unit needs no merge; clusters help while most SMs would idle
   //   units <= SMs/2  clusters: merge through distributed shared memory, everything resident in one wave
   //   unlike lengths  the flat grid, once there is enough to read that its schedule and merge are small beside it
-  // `units` = (request, kv head) pairs, lengths in pages (mt: the longest request's).
+  // `units` = (request, kv head) pairs, lengths in pages (mt: the longest request's).  Bounds that are plain numbers of units
+  // are those of the 148 SMs that they were measured on.
   static DecodePlan choose(precc_ctx* ctx, int B, int n_kv, int max_ctx) {
     const int sm = ctx->sm_count, mt = (max_ctx + PAGE - 1) / PAGE;
     const long long units = (long long)B * n_kv, work = units * mt;
@@ -224,7 +225,8 @@ struct DecodeRunT {
     if (ROPE) {
       // issue-bound: four warps twice per SM reach as many SMs as eight once, in finer pieces; from some work on the flat
       // grid's even shares win
-      if (units * 2 > sm && mt <= (units > 90 ? 48 : 16)) return whole();
+      // (one block each: above three fifths of the SMs that is a fair share of the machine, so it pays up to more pages)
+      if (units * 2 > sm && mt <= (units * 5 > 3 * sm ? 48 : 16)) return whole();
       if (units >= 48 && mt <= 12) return whole();
       if (work >= (units >= 56 || RK + RV >= 96 ? 12000 : HD == 64 ? 16000 : 18000)) return flat();
       if (units >= 8 && !(HD == 64 && RK + RV >= 96)) pl = cluster(4, 2, HD == 64 ? 3 : 2, lim);
@@ -254,14 +256,20 @@ struct DecodeRunT {
       pl = cluster(8, 1, 3, 1);
       return pl.cluster ? pl : flat();
     }
-    // eight warps, one block per SM: two or three pages in flight per warp cover the memory's latency.  Where whole SMs are
-    // left over that way, four warps twice per SM may reach more of them.
+    // Eight warps, one block per SM: two or three pages in flight per warp cover the memory's latency.  Clusters of whole SMs
+    // do not always use them up (a cluster lives in one GPC: from 45 units on only two blocks each fit, 96 SMs); then two
+    // four-warp blocks per SM may reach more of the machine.  They take over where they have three times the blocks, or
+    // where the others leave more than a third of the SMs idle and they reach an eighth more (48 units of 320 .. 1000
+    // pages: 5 .. 16 % faster than the flat grid; where less is idle the flat grid wins: 56 units of 320 pages 22.6 against
+    // 28.1 us, 36 units of 700 pages 35.0 against 42.6).  From some work on the flat grid evens the SMs out by itself
+    // wherever clusters use less than ten thirteenths of them.
     pl = cluster(8, 1, work >= 50000 ? 2 : 3, lim);
-    if (units >= 24 && (units < 40 || units > 48) && work >= 30000 && pl.cluster * units * 13 < 10 * sm) return flat();
+    const long long reach = pl.cluster * units;          // SMs that have a block
     if (mt >= 100) {
       const DecodePlan p4 = cluster(4, 2, 3, lim);
-      if (p4.cluster >= pl.cluster * 3 || (units >= 40 && units <= 48 && mt >= 300 && p4.cluster * 100 > pl.cluster * 216)) pl = p4;
+      if (p4.cluster >= pl.cluster * 3 || (units >= 24 && mt >= 300 && reach * 3 < 2 * sm && p4.cluster * 8 >= pl.cluster * 18)) return p4.cluster ? p4 : flat();
     }
+    if (units >= 24 && work >= 30000 && reach * 13 < 10 * sm) return flat();
     return pl.cluster ? pl : flat();
   }
   static int32_t run(precc_ctx* ctx, const DecodeArgs& a) {

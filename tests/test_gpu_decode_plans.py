@@ -19,26 +19,43 @@ def _ragged(B, low, high):
 
 
 _PLANS = [
-    # env, head_dim, kv heads, query heads per kv head, rank, lengths, requests rejected on the device
-    (TICKET, 64, 1, 4, 16, [1], ()),                                     # one page, one block
-    (TICKET, 128, 2, 4, 16, [127, 129], ()),                             # fewer pages than a block has warps
-    (TICKET, 64, 2, 2, 8, [9000], ()),                                   # one request over the whole grid
-    (TICKET, 128, 3, 2, 32, [700, 16, 4000, 17, 1300], (2,)),            # a rejected request in the middle counts as one page
-    (TICKET, 64, 1, 4, 0, _ragged(32, 1, 900), ()),                      # one request per lane of the schedule
-    (TICKET, 64, 2, 8, 64, _ragged(33, 1, 900), (0, 32)),
-    (TICKET, 64, 1, 2, 16, _ragged(256, 1, 1500), (255,)),               # the most the schedule handles
-    (TICKET, 64, 1, 2, 16, _ragged(257, 1, 1500), ()),                   # one more: split from the bound
-    ({}, 64, 2, 4, 16, _ragged(80, 300, 1600), ()),                      # more units than SMs, unlike lengths: flat grid
-    ({}, 64, 2, 4, 16, _ragged(40, 60, 250), ()),                        # one block per unit
-    ({}, 128, 2, 4, 16, _ragged(50, 700, 1700), ()),                     # three blocks per unit, planned from the bound
-    ({}, 128, 2, 4, 64, _ragged(50, 700, 1700), ()),                     # one cluster block per unit
-    ({}, 128, 8, 4, 16, [10500, 900], ()),                               # clusters, the longest request's chunk for all
-    ({}, 128, 2, 4, 16, [256, 30, 250], ()),                             # clusters, every request shared out evenly
+    # plan taken, env, head_dim, kv heads, query heads per kv head, rank, lengths, requests rejected on the device
+    ("flat", TICKET, 64, 1, 4, 16, [1], ()),                                     # one page, one block
+    ("flat", TICKET, 128, 2, 4, 16, [127, 129], ()),                             # fewer pages than a block has warps
+    ("flat", TICKET, 64, 2, 2, 8, [9000], ()),                                   # one request over the whole grid
+    ("flat", TICKET, 128, 3, 2, 32, [700, 16, 4000, 17, 1300], (2,)),            # a rejected request in the middle counts as one page
+    ("flat", TICKET, 64, 1, 4, 0, _ragged(32, 1, 900), ()),                      # one request per lane of the schedule
+    ("flat", TICKET, 64, 2, 8, 64, _ragged(33, 1, 900), (0, 32)),
+    ("flat", TICKET, 64, 1, 2, 16, _ragged(256, 1, 1500), (255,)),               # the most the schedule handles
+    ("split", TICKET, 64, 1, 2, 16, _ragged(257, 1, 1500), ()),                  # one more: split from the bound (one block each)
+    ("flat", {}, 64, 2, 4, 16, _ragged(80, 300, 1600), ()),                      # more units than SMs, unlike lengths
+    ("split", {}, 64, 2, 4, 16, _ragged(40, 60, 250), ()),                       # one block per unit
+    ("split 2", {}, 128, 2, 4, 16, _ragged(50, 700, 1700), ()),                  # two blocks per unit, planned from the bound
+    ("cluster 1", {}, 128, 2, 4, 64, _ragged(50, 700, 1700), ()),                # one cluster block per unit
+    ("cluster", {}, 128, 8, 4, 16, [10500, 900], ()),                            # clusters, the longest request's chunk for all
+    ("cluster", {}, 128, 2, 4, 16, [256, 30, 250], ()),                          # clusters, every request shared out evenly
+    # where whole-SM clusters leave SMs idle: three blocks per unit, then five smaller ones while a third is idle, then the flat grid
+    ("cluster", {}, 128, 4, 4, 16, _ragged(11, 5600, 12000), ()),
+    ("cluster", {}, 128, 4, 4, 16, _ragged(12, 5600, 12000), ()),
+    ("flat", {}, 128, 4, 4, 16, _ragged(13, 5600, 12000), ()),
 ]
 
 
-@pytest.mark.parametrize("env,hd,n_kv,G,r,ctx,rejected", _PLANS, ids=[str(i) for i in range(len(_PLANS))])
-def test_every_plan_against_the_oracle(monkeypatch, env, hd, n_kv, G, r, ctx, rejected):
+def _plan_taken(px, trace, units, hd, pages):
+    """From the stamps of the last call: how many blocks it started, and whether they were clusters (only those write entry 15)."""
+    t = trace.cpu()
+    blocks, cluster = int((t[:, 0] != 0).sum()), bool((t[:, 15] != 0).any())
+    each = blocks // units
+    if cluster:
+        assert blocks == each * units
+        return {"cluster", f"cluster {each}"}
+    slots = (4 if hd == 64 else 2) * px.sm_count
+    flat = {"flat"} if blocks == max(units, min(slots, units * ((pages + 3) // 4))) else set()
+    return flat | ({"split" if each == 1 else f"split {each}"} if blocks == each * units else set())
+
+
+@pytest.mark.parametrize("plan,env,hd,n_kv,G,r,ctx,rejected", _PLANS, ids=[str(i) for i in range(len(_PLANS))])
+def test_every_plan_against_the_oracle(monkeypatch, plan, env, hd, n_kv, G, r, ctx, rejected):
     """Paged caches (pages shared between requests, in mixed order).  The tolerance is that of every other decode test:
     bf16 inputs and softmax weights, fp32 accumulation."""
     for k, v in env.items():
@@ -59,8 +76,12 @@ def test_every_plan_against_the_oracle(monkeypatch, env, hd, n_kv, G, r, ctx, re
         agent = torch.tensor([b % 2 for b in range(B)], dtype=torch.int32).cuda()
         ws = px.decode_workspace(desc, B, T)
         out, again = torch.full_like(q, float("nan"), device="cuda"), torch.full_like(q, float("nan"), device="cuda")
+        trace = torch.zeros(4096, 16, dtype=torch.int64, device="cuda")
         for o in (out, again):
             px.lr_attend_decode(desc, q.cuda(), agent, lengths, T, B_k, B_v, cache, o, ws, table.cuda())
+            px.set_trace_buffer(trace)
+        px.set_trace_buffer(None)
+        assert plan in _plan_taken(px, trace, B * n_kv, hd, pages)
         assert px.poll_status() == (1 if rejected else 0)
         assert torch.equal(out, again)
         check = {b for b in (0, 1, B // 2, B - 2, B - 1, int(np.argmax(ctx)), int(np.argmin(ctx))) if 0 <= b < B}
