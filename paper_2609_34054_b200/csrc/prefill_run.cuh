@@ -34,13 +34,13 @@ struct PrefillRun {
     if (n_max < ctx->prefill_helper_min_steps) return best;
     // What a record + merge costs a tile's own block, and what a piece costs a helper beyond its steps (query tile,
     // fold, pipeline fill, record), in steps at head_dim 128, rank 32 (1.0 us), scaled for shorter ones; and how much longer
-    // every step takes with all SMs busy instead of one per tile: at head_dim 128 the launch runs at the power cap and
-    // 35 .. 42 % of what the additional SMs add is lost to the clock; at head_dim 64 it is bound by the exponentials.  Fitted
-    // to turns of 72 .. 132 tiles over 6000 .. 48000 tokens (head_dim 128, rank 64, 112 tiles over 24000 tokens: 305 us with
-    // the helpers that a fit to slower steps chose, 275 without; 88 tiles over 48000: 448 without, 388 with).
+    // every step takes with all SMs busy instead of one per tile.  At head_dim 128 the launch runs at the power cap; steps
+    // without the sum of rounded weights are short (head_dim 64 rank 64: 0.78 us, head_dim 128 without adapter: 0.86 us for
+    // 64 KB of caches each), so that what L2 delivers to all SMs together bounds them and more SMs only stretch them.
+    // Measured on turns of 80 .. 112 tiles over 24000 and 48000 tokens, steps of the work-list launch against the plain one.
     const int f100 = 100 * 160 / (HD + (RK + RV) / 2);
     const int C_OWN = 14 * f100 / 100, C_PIECE = (HD == 64 ? 12 : RK + RV > 32 ? 18 : 13) * f100 / 100;
-    const int slow = HD == 64 ? 104 : 100 + (RK + RV > 32 ? 42 : 35) * H / (int)tiles;
+    const int slow = HD == 64 ? (RV == 64 ? 138 : RV == 0 ? 114 : 106) : RV == 0 ? 144 : RV == 64 ? 106 : 112;
     int best_cost = (n_max - n_max / 25) * 100 / slow;   // a plan must win 4 % on paper
     for (int p = n_max - 1; p >= std::max(8, n_max / 2); --p) {
       if (ctx->prefill_helper_p > 0 && p != ctx->prefill_helper_p) continue;

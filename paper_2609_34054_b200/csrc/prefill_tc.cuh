@@ -336,10 +336,11 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
     const CUtensorMap* m = &maps.k + threadIdx.x;
     asm volatile("prefetch.tensormap [%0];\n" ::"l"(m) : "memory");
   }
-  // All of the above overlaps the end of the kernel before this one (programmatic dependent launch); nothing of the
-  // caches, the queries or the block table is touched before that kernel has finished.  No early launch of the kernel
-  // behind it: the clusters of a projection placed on the SMs that this grid leaves idle keep the rest of them from
-  // fitting into one wave (301 new tokens, 80 blocks: 61.6 against 59.1 us a turn).
+  // All of the above overlaps the end of the kernel before this one (programmatic dependent launch): its whole last part
+  // behind decode, combine and few-row projections, which let a dependent launch start early, launch travel and drain behind
+  // the others.  Nothing of the caches, the queries or the block table is touched before that kernel has finished.  No early
+  // launch of the kernel behind it: the clusters of a projection placed on the SMs that this grid leaves idle keep the rest
+  // of them from fitting into one wave (301 new tokens, 80 blocks: 61.6 against 59.1 us a turn).
   pdl_wait();
   tc_fence_before();
   __syncthreads();
