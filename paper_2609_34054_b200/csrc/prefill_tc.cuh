@@ -780,9 +780,12 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         if ((tid & 127) == 0) PTC_STAMP(p, j, 5);                  // reference maximum settled
         if (j > 0 && __any_sync(0xffffffffu, m_new != m_prev)) {
           const float alpha = fast_exp2(m_prev - m_new);           // 1 for rows that keep their maximum
-          // O' is complete through step j-1.  A wait names a phase by its parity, so step j-3 has to have retired first;
-          // with one P buffer this warpgroup's previous step waited for exactly that.
-          if (C::PB == 2 && j > 2) mbar_wait(pv_done + 8 * (wg ^ 1), ((j - 3) >> 1) & 1, p.status);
+          // O' is complete through step j-1.  A wait names a phase by its parity, so it holds only on a barrier that is in that
+          // phase or the next one: step j-3, the one before on this barrier, has to have retired first.  That follows from
+          // step j-2, whose own barrier cannot be further (step j is not published); waiting for step j-3 itself
+          // would never end where step j-1 has retired already.  (With one P buffer this warpgroup's previous step
+          // waited for exactly that.)
+          if (C::PB == 2 && j > 2) mbar_wait(pv_done + 8 * wg, ((j - 2) >> 1) & 1, p.status);
           mbar_wait(pv_done + 8 * (wg ^ 1), ((j - 1) >> 1) & 1, p.status);
           tc_fence_after();
 #pragma unroll 1

@@ -740,6 +740,43 @@ def test_projection_right_behind_the_packing_of_its_weights(px, M):
         del W
 
 
+@pytest.mark.parametrize("hd,r", [(64, 0), (64, 16), (64, 64), (128, 0), (128, 32)])
+@pytest.mark.parametrize("paged", [False, True])
+def test_prefill_whose_reference_is_raised_late_and_often(px, hd, r, paged):
+    """Scores that keep growing along the context, at other rates in every row: the output is rescaled at steps of either
+    warpgroup, whatever of the steps before has retired by then.  No bounded wait may run out, every run gives the same
+    bits, and rows agree with the oracle's definition in float64."""
+    from paper_2609_34054_b200.binding import Cache, layer_desc
+    geo, S, T = I.Geometry(512, 8, 2, hd, 2, r, r, alpha=2.0 * max(r, 1)), 301, 5003
+    n = (S + T + 15) // 16
+    c, w = I.direct_caches(n, geo, 35, "grow"), I.layer_weights(geo, 35, "grow")
+    ramp = torch.linspace(0.0, 24.0, n * 16).reshape(n, 1, 16)
+    c["k_base"][..., 0] = (ramp + c["k_base"][..., 0].float()).to(torch.bfloat16)
+    q = I.queries(S, geo, 35, "grow.q", gain=3.0)
+    q[..., 0] = (torch.arange(S * 8).reshape(S, 8) % 7).to(torch.bfloat16) * 2.0
+    order = torch.randperm(n, generator=torch.Generator().manual_seed(1)) if paged else torch.arange(n)
+    lr = [c[k][:, order].cuda() if r else None for k in ("lr_k", "lr_v")]
+    B = [w[k].cuda() if r else None for k in ("B_k", "B_v")]
+    cache = Cache.from_tensors(geo, c["k_base"][order].cuda(), c["v_base"][order].cuda(), *lr)
+    table = torch.argsort(order).to(torch.int32).cuda() if paged else None
+    out, again = torch.full_like(q, float("nan"), device="cuda"), torch.empty_like(q, device="cuda")
+    px.lr_attend_prefill(layer_desc(geo), q.cuda(), 1, T, *B, cache, out, table)
+    for _ in range(30):
+        px.lr_attend_prefill(layer_desc(geo), q.cuda(), 1, T, *B, cache, again, table)
+        assert torch.equal(out, again)
+    assert px.poll_status() == 0
+    for i, h in ((0, 1), (77, 6), (150, 3), (300, 7), (299, 0)):
+        g, m = h // 4, T + i + 1
+        cols = slice(g * hd, (g + 1) * hd)
+        k, v = f64(c["k_base"][:, g].reshape(-1, hd))[:m], f64(c["v_base"][:, g].reshape(-1, hd))[:m]
+        if r:
+            k = k + geo.scale_k * f64(c["lr_k"][1].reshape(-1, r))[:m] @ f64(w["B_k"][1][:, cols])
+            v = v + geo.scale_v * f64(c["lr_v"][1].reshape(-1, r))[:m] @ f64(w["B_v"][1][:, cols])
+        z = k @ f64(q[i, h]) / hd ** 0.5
+        p = np.exp(z - z.max())
+        assert_close(f64(out)[i, h][None], ((p / p.sum()) @ v)[None], f"token {i}, head {h}")
+
+
 @pytest.mark.parametrize("n", [1, 10, 100])
 def test_per_row_agent_masks_equal_two_separate_projections(px, n):
     """Double batching: adapted rows (current agent's LR rows, private slots) and adapter-free rows (the other
