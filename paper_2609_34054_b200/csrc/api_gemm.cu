@@ -4,6 +4,7 @@
 #include "gemm_tc.cuh"
 #include "gemm_pair.cuh"
 #include "proj_small.cuh"
+#include "proj_turn.cuh"
 
 using namespace precc;
 
@@ -71,108 +72,108 @@ int32_t launch_small(precc_ctx* ctx, const void* X, int M, int K, const void* Wt
 
 int ilog2(int v) { int s = 0; while ((1 << s) < v) ++s; return s; }
 
+// How a turn's projection is cut: tiles of 128 columns x tn rows, the K extent of each over ks blocks.
+struct TurnPlan { int tn = 0, ks = 0, stages = 0; };
+
+// Clusters of `ks` blocks of the turn kernel that are resident at once (one block per SM; a cluster lives inside one GPC).
+int max_turn_clusters(precc_ctx* ctx, int ks) {
+  static int max_clusters_dev[kMaxDevices][GEMM_MAX_KS + 1] = {{0}};   // 0 = unknown, else max active clusters + 1
+  std::lock_guard<std::recursive_mutex> lk(lazy_mu());
+  int& cached = max_clusters_dev[ctx->device % kMaxDevices][ks];
+  if (cached == 0) {
+    int n = 0;
+    auto kern = proj_turn_kernel<false>;
+    if (raise_smem_limit(ctx, kern, PT_MIN_SMEM) == cudaSuccess) {
+      cudaLaunchConfig_t qc = {};
+      qc.gridDim = dim3(ks, ctx->sm_count, 1); qc.blockDim = dim3(PT_THREADS); qc.dynamicSmemBytes = PT_MIN_SMEM;
+      cudaLaunchAttribute qa[1];
+      qa[0].id = cudaLaunchAttributeClusterDimension;
+      qa[0].val.clusterDim.x = ks; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
+      qc.attrs = qa; qc.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, kern, &qc) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    } else {
+      cudaGetLastError();
+    }
+    cached = n + 1;
+  }
+  return cached - 1;
+}
+
+// The cut with the smallest predicted time among those whose clusters are all resident at once (a second wave costs more
+// than any split gains: 512 rows of the Llama-3-8B projection as 36 clusters of four, of which 33 fit, 26.9 us; as 36
+// clusters of three 17.2).  Time in us, fitted to some 450 cuts of four layers (d_model 1024 .. 4096) at 41 .. 2048 rows,
+// mean error 4 %: what a k-block costs a block, what the merge moves into one, what dumping and storing a tile takes, and the
+// cluster.  The cut it picks is within 1 % of the best one measured but for two in 36 (4 % and 11 %).
+TurnPlan plan_turn(precc_ctx* ctx, int M, int nkb, int n_fused) {
+  TurnPlan best;
+  double best_cost = 1e30;
+  const int groups = (n_fused + PT_COLS - 1) / PT_COLS;
+  const int ks_hi = (ctx->gemm_ks_max >= 2 && ctx->gemm_ks_max < GEMM_MAX_KS) ? ctx->gemm_ks_max : GEMM_MAX_KS;
+  for (int t = (M + PT_MAX_TN - 1) / PT_MAX_TN, last = 0;; ++t) {
+    const int tn = ((M + t - 1) / t + 15) / 16 * 16, tiles = (M + tn - 1) / tn;
+    if (tn < 32 || (long long)groups * tiles * ctx->gemm_ks_min > ctx->sm_count) break;
+    if (tn == last) continue;
+    last = tn;
+    for (int ks = ctx->gemm_ks_min; ks <= ks_hi && nkb / ks >= 2; ++ks) {       // at least two k-blocks per slice
+      if (groups * tiles > max_turn_clusters(ctx, ks)) continue;
+      const int kb = (nkb + ks - 1) / ks;
+      int st = kb < PT_MAX_STAGES ? kb : PT_MAX_STAGES;
+      while (st > 1 && pt_smem_bytes(tn, ks, st) > ctx->max_smem_optin) --st;
+      if (pt_smem_bytes(tn, ks, st) > ctx->max_smem_optin) continue;
+      const double cost = kb * (0.37 + 0.00036 * tn) + 0.005 * pt_share(tn, ks) * (ks - 1) + 0.0113 * tn + 0.1 * ks;
+      if (cost < best_cost) { best_cost = cost; best.tn = tn; best.ks = ks; best.stages = st; }
+    }
+  }
+  return best;
+}
+
+int32_t launch_turn(precc_ctx* ctx, const void* X, int M, int K, const void* Wt, int n_out, GemmParams gp, const TurnPlan& tp, cudaStream_t stream) {
+  int tmem_cols = 32;
+  while (tmem_cols < tp.tn) tmem_cols <<= 1;
+  CUtensorMap map_x, map_w;
+  int32_t rc = make_map(ctx, &map_x, X, M, K, tp.tn);
+  if (rc) return rc;
+  rc = make_map_w(ctx, &map_w, Wt, n_out, K, PT_COLS);
+  if (rc) return rc;
+  gp.M = M; gp.N_out = n_out; gp.K = K; gp.BN = tp.tn; gp.stages = tp.stages; gp.tmem_cols = tmem_cols;
+  gp.status = ctx->status;
+  int smem = pt_smem_bytes(tp.tn, tp.ks, tp.stages);
+  if (smem < PT_MIN_SMEM) smem = PT_MIN_SMEM;
+  auto kern = gp.rope ? proj_turn_kernel<true> : proj_turn_kernel<false>;
+  PRECC_CUDA(ctx, raise_smem_limit(ctx, kern, smem));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(tp.ks, (n_out + PT_COLS - 1) / PT_COLS, (M + tp.tn - 1) / tp.tn);
+  cfg.blockDim = dim3(PT_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = tp.ks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
+  PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, map_x, map_w, gp));
+  return PRECC_OK;
+}
+
 int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt, int n_out, GemmParams gp, cudaStream_t stream) {
   gp.hd_shift = ilog2(gp.hd); gp.rk_shift = ilog2(gp.rank_k > 0 ? gp.rank_k : 1); gp.rv_shift = ilog2(gp.rank_v > 0 ? gp.rank_v : 1);
-  // Up to 40 rows the weight-streaming few-row kernel is the fastest (fused C3 projection: 5.8 us at 16 rows, 7.4 at
-  // 32, 12.7 at 40); from there to about a thousand rows the split-K kernels (12.3 .. 23 us; the few-row kernel needs
-  // 12.8 us at 41 rows and 13.7 at 64, the one-block-per-tile GEMM 27 .. 30 us throughout); the few-row kernel still
-  // takes 41..64 rows when the split does not apply (short K).
-  if (M <= 40 && !ctx->force_tiled_gemm) {
+  // Few rows: the weight-streaming kernel (fused Llama-3-8B projection: 5.8 us at 16 rows, 7.8 at 32).  From 33 to 40 rows the
+  // turn kernel would be faster on wide layers (9.8 against 12.9 us) and slower on narrow ones (d_model 2048: 7.2 against
+  // 6.6), but rows written one by one and in one call of up to 40 have equal bits, which is worth more.  Beyond that the turn
+  // kernel, up to some two thousand rows; the few-row kernel still takes 41 .. 64 rows where the K split does not apply
+  // (short K).
+  if (M <= PS_FAST_M && !ctx->force_tiled_gemm) {
     const int32_t rc = launch_small(ctx, X, M, K, Wt, n_out, gp, stream);
     if (rc >= 0) return rc;
   }
   const int m_tiles = (M + GEMM_BM - 1) / GEMM_BM;
-  // A few row tiles (the tokens of a short turn): the K extent of every tile is split over a cluster.  The split
-  // depends on M and K alone, so a column's summation order is the same whichever entry point produced it.
+  // The tokens of a turn: 128-column tiles as wide as there are rows, the K extent of a tile split over a cluster.
   if (m_tiles <= 16 && !ctx->no_gemm_splitk) {
-    const int nkb = K / GEMM_BK;
     // planned for the width of the FUSED projection of this layer, whatever this call projects, so that the base-only,
     // LR-only and fused calls of one M take the same decision (and with it the same summation order)
-    const int n_fused = 2 * gp.n_kv * gp.hd + gp.n_agents * (gp.rank_k + gp.rank_v);
-    // 256-column tiles, one block per SM (a kernel that allocates tensor memory is given one block per SM)
-    const int bn = n_out >= 256 ? 256 : (n_out + 15) / 16 * 16;
-    const int stage_bytes = GEMM_A_BYTES + 256 * GEMM_BK * 2;
-    constexpr int SK_STAGES = 4;                          // ring depth of the split-K kernel
-    const int ring_max = SK_STAGES * stage_bytes;
-    const long long clusters = (long long)m_tiles * ((n_fused + 255) / 256);
-    // the finest split whose clusters are all resident at once (a second wave would cost more than the split gains);
-    // cluster sizes need not be powers of two: 18 clusters fit as 6-block clusters, 36 as 3-block clusters
-    bool plan_direct = false, plan_push = false;
-    int ks = (ctx->gemm_ks_max >= 2 && ctx->gemm_ks_max < GEMM_MAX_KS) ? ctx->gemm_ks_max : GEMM_MAX_KS, smem_plan = 0;
-    const int push_max = (ctx->gemm_push_max >= 0 && ctx->gemm_push_max < GEMM_PUSH_MAX_KS) ? ctx->gemm_push_max : GEMM_PUSH_MAX_KS;
-    // Clusters of 2 .. 4 blocks merge by bulk sends (proj_gemm_splitk_push_kernel), larger ones by pulling over
-    // distributed shared memory (their slices do not fit twice beside each other) or, for up to 64 rows, by direct
-    // sends.  Fused Llama-3-8B projection, graph replay over rotating weights: 384 / 512 / 640 rows (clusters of
-    // 4 / 4 / 3) 16.4 / 18.4 / 19.2 us against 19.3 / 22.1 / 22.5 us with the pulling merge; 768 / 896 / 1024 rows
-    // (clusters of 2) 22.4 / 22.6 / 23.2 us against 29.2 / 30.1 / 30.3 us on the one-block-per-tile kernel (a two-way
-    // split did not pay for a pulling merge).
-    const int ks_min = ctx->gemm_ks_min;
-    for (; ks >= ks_min; --ks) {
-      const bool bulk = ks <= push_max && ctx->gemm_direct < 2;       // whole slices by bulk copy
-      // pieces straight from registers: pays only while few rows exist (fused Llama-3-8B projection, clusters of 8:
-      // 11.7 against 12.2 us at 41 rows, 12.6 against 13.0 at 64, but 16.5 against 15.6 at 128 and 21.8 against 17.0 at 256)
-      const bool direct = !bulk && (ctx->gemm_direct >= 2 || (ctx->gemm_direct == 1 && M <= 64));
-      const bool push = bulk || direct;
-      if (nkb / ks < (ks <= GEMM_PUSH_MAX_KS ? 4 : 2)) continue;       // a coarse split of a short K is not worth a cluster
-      const int cw = ((256 + ks - 1) / ks + 15) / 16 * 16;       // planned for the widest tile and slice (rotary), whatever this call's
-      const int slice = GEMM_BM * (cw + 4) * 4;
-      const int dump = bulk ? 2 * (ks - 1) * slice : (direct ? (ks - 1) * slice : ks * slice);
-      smem_plan = (((ring_max > dump ? ring_max : dump) + 1023) & ~1023) + (2 * SK_STAGES + 8) * 8;
-      if (smem_plan > ctx->max_smem_optin) continue;
-      static int max_clusters_dev[kMaxDevices][2][GEMM_MAX_KS + 1] = {{{0}}};   // 0 = unknown, else max active clusters + 1
-      std::lock_guard<std::recursive_mutex> lk(lazy_mu());
-      int& cached = max_clusters_dev[ctx->device % kMaxDevices][push ? 1 : 0][ks];
-      plan_direct = direct; plan_push = push;
-      if (cached == 0) {
-        int n = 0;
-        auto kern = push ? proj_gemm_splitk_push_kernel<false> : proj_gemm_splitk_kernel<false>;
-        if (raise_smem_limit(ctx, kern, smem_plan) == cudaSuccess) {
-          cudaLaunchConfig_t qc = {};
-          qc.gridDim = dim3(ks, ctx->sm_count, 1); qc.blockDim = dim3(GEMM_THREADS); qc.dynamicSmemBytes = smem_plan;
-          cudaLaunchAttribute qa[1];
-          qa[0].id = cudaLaunchAttributeClusterDimension;
-          qa[0].val.clusterDim.x = ks; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
-          qc.attrs = qa; qc.numAttrs = 1;
-          if (cudaOccupancyMaxActiveClusters(&n, kern, &qc) != cudaSuccess) { cudaGetLastError(); n = 0; }
-        } else {
-          cudaGetLastError();
-        }
-        cached = n + 1;
-      }
-      if (cached - 1 >= clusters) break;
-    }
-    if (ks >= ks_min) {
-      const int n_tiles = (n_out + bn - 1) / bn;
-      int stages = SK_STAGES;
-      if (stages > nkb / ks) stages = nkb / ks;
-      int tmem_cols = 32;
-      while (tmem_cols < bn) tmem_cols <<= 1;
-      CUtensorMap map_x, map_w;
-      int32_t rc = make_map(ctx, &map_x, X, M, K, GEMM_BM);
-      if (rc) return rc;
-      rc = make_map_w(ctx, &map_w, Wt, n_out, K, bn);
-      if (rc) return rc;
-      gp.M = M; gp.N_out = n_out; gp.K = K; gp.BN = bn; gp.stages = stages; gp.tmem_cols = tmem_cols;
-      gp.spread_rows = 0;
-      gp.status = ctx->status;
-      auto kern = gp.rope ? (plan_push ? proj_gemm_splitk_push_kernel<true> : proj_gemm_splitk_kernel<true>)
-                          : (plan_push ? proj_gemm_splitk_push_kernel<false> : proj_gemm_splitk_kernel<false>);
-      gp.direct_send = plan_direct ? 1 : 0;
-      PRECC_CUDA(ctx, raise_smem_limit(ctx, kern, smem_plan));
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(ks, n_tiles, m_tiles);
-      cfg.blockDim = dim3(GEMM_THREADS);
-      cfg.dynamicSmemBytes = smem_plan;
-      cfg.stream = stream;
-      cudaLaunchAttribute attr[2];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = ks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[1].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = attr; cfg.numAttrs = 2;
-      PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, map_x, map_w, gp));
-      return PRECC_OK;
-    }
+    const TurnPlan tp = plan_turn(ctx, M, K / GEMM_BK, 2 * gp.n_kv * gp.hd + gp.n_agents * (gp.rank_k + gp.rank_v));
+    if (tp.ks > 0) return launch_turn(ctx, X, M, K, Wt, n_out, gp, tp, stream);
   }
   if (M <= PS_MAX_M && !ctx->force_tiled_gemm) {
     const int32_t rc = launch_small(ctx, X, M, K, Wt, n_out, gp, stream);

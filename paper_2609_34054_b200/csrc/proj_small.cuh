@@ -32,6 +32,7 @@ namespace precc {
 constexpr int PS_WARPS = 8;
 constexpr int PS_BK = 64;                   // k elements per step: one 128-byte swizzle row
 constexpr int PS_MAX_M = 64;
+constexpr int PS_FAST_M = 40;               // up to here it takes every call: a row has the same bits alone and among up to 39 others
 constexpr int PS_STAGES = 4;
 constexpr int PS_THREADS = (PS_WARPS + 1) * 32;       // consumer warps + one producer warp
 __host__ __device__ constexpr int ps_nt(int mt) { return mt > 1 ? 2 : 1; }               // 8-column n-tiles per warp

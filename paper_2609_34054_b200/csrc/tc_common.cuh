@@ -9,9 +9,8 @@ namespace precc {
 
 struct GemmParams {
   int M, N_out, K;
-  int BN, stages, tmem_cols;
+  int BN, stages, tmem_cols;      // BN: columns of a tile (turn kernel: rows of X in a tile)
   int spread_rows;                // 1: even row-tile spreading allowed (rows may be written twice, identically)
-  int direct_send;                // split-K merge by sends: 1 = pieces straight from registers (st.async), 0 = whole slices by bulk copy
   int mode;                       // 0 = LR caches, 1 = base caches, 2 = base columns then LR columns
   const int32_t* slot_mapping;    // [M] or null
   int64_t start_slot;
@@ -51,8 +50,7 @@ struct GemmParams {
 constexpr int GEMM_BM = 128;
 constexpr int GEMM_BK = 64;                 // 64 bf16 = one 128-byte swizzle row
 constexpr int GEMM_THREADS = 192;
-constexpr int GEMM_MAX_KS = 8;            // largest K split of the split-K kernels (cluster size)
-constexpr int GEMM_PUSH_MAX_KS = 4;       // up to this split the partial tiles are merged by bulk sends
+constexpr int GEMM_MAX_KS = 8;            // largest K split of a turn's projection (cluster size)
 constexpr int GEMM_A_BYTES = GEMM_BM * GEMM_BK * 2;
 
 // The same bounded wait for waiters that are not on the critical path (an epilogue waiting for a whole tile of

@@ -885,6 +885,42 @@ def test_short_turn_projection_split_over_a_cluster(monkeypatch, px, M, d):
     px2.close()
 
 
+@pytest.mark.parametrize("M,d,n_kv,hd,r", [(33, 1024, 1, 128, 8), (48, 512, 3, 64, 64), (255, 1024, 2, 128, 16), (257, 2048, 2, 64, 32),
+                                           (513, 1024, 1, 64, 8), (1100, 1024, 2, 128, 32)])
+def test_turn_projection_at_the_edges_of_its_tiles(px, M, d, n_kv, hd, r):
+    """Rows just below and above a tile, more than one tile with a ragged last one, fused widths that are not a multiple of the
+    128-column tile; every row with its own agent mask and every other one with a second slot for its LR rows."""
+    geo = I.Geometry(d, 2 * n_kv, n_kv, hd, 3, r, r, alpha=2.0 * r)
+    H = I.hidden_states(M, geo, seed=83, tag=f"edge.{M}.{d}")
+    nb = (2 * M + 15) // 16 + 2
+    perm = I.permutation(nb * 16, 83, f"edge.slots.{M}").to(torch.int32)
+    slots, copies = perm[:M], perm[M:2 * M].clone()
+    copies[::2] = -1
+    agent = torch.arange(M) % 3
+    masks = (torch.ones(M, dtype=torch.int64) << agent)
+    L = Layer(px, geo, seed=83, n_blocks=nb, fill=float("nan"))
+    WA = px.pack_turn_weights(geo, *(L.w[k].cuda() for k in ("W_k", "W_v", "A_k", "A_v")))
+    px.turn_project_rows(L.desc, H.cuda(), WA, L.cache, slots.cuda(), masks.cuda(), copies.cuda())
+    torch.cuda.synchronize()
+    assert px.poll_status() == 0
+    w, Hn, sl = L.w_np, f64(H), slots.long()
+    tol = lambda ref: 2.0 ** -8 * np.abs(ref) + 2e-3 * np.sqrt(d / 256)      # one bf16 rounding of an fp32 sum of d products
+    for got, ref in ((base_rows(L.cache.k_base)[sl], O.base_cache(Hn, w["W_k"])), (base_rows(L.cache.v_base)[sl], O.base_cache(Hn, w["W_v"]))):
+        assert (np.abs(got - ref) <= tol(ref)).all()
+    for cache, A in ((L.cache.lr_k, w["A_k"]), (L.cache.lr_v, w["A_v"])):
+        for a in range(3):
+            mine = (agent == a).numpy()
+            ref = O.lr_cache(Hn, A[a])[mine]
+            rows = lr_rows(cache, a)
+            assert (np.abs(rows[sl.numpy()[mine]] - ref) <= tol(ref)).all()
+            second = copies.numpy()[mine] >= 0
+            assert np.array_equal(rows[copies.numpy()[mine][second]], rows[sl.numpy()[mine][second]])
+            untouched = np.ones(nb * 16, dtype=bool)
+            untouched[sl.numpy()[mine]] = False
+            untouched[copies.numpy()[mine][second]] = False
+            assert np.isnan(rows[untouched]).all()
+
+
 @pytest.mark.parametrize("ks,M,d", [(2, 100, 1024), (2, 777, 2048), (3, 384, 4096), (3, 130, 1024), (4, 512, 2048), (4, 64, 4096), (4, 1000, 1024),
                                     (5, 200, 2048), (6, 256, 4096), (7, 41, 2048), (8, 128, 1024), (8, 77, 4096)])
 def test_split_k_merge_by_sends_equals_the_pulling_merge_bitwise(monkeypatch, ks, M, d):
