@@ -33,8 +33,10 @@ int pick_bn(int n_out, int m_tiles, int sm_count) {
 // column's summation order - and with it every output bit - is the same whichever entry point (LR only,
 // base only, fused) produced it.
 int32_t launch_small(precc_ctx* ctx, const void* X, int M, int K, const void* Wt, int n_out, GemmParams gp, cudaStream_t stream) {
+  // Slices of at least 128: with four ring slots a block then mostly has its whole slice of the weights requested before the wait
+  // for the kernel ahead, and twice the SMs take part (slices of 512 before; d_model 2048, one row: 3.8 -> 3.1 us; 1024: 3.1 -> 2.3; 3584: 8.9 -> 8.1; 32 rows: 5.4 -> 3.7, 5.0 -> 3.0, 9.9 -> 9.6).
   int cs = 8;
-  while (cs > 1 && (K / cs < 512 || K % (PS_BK * cs) != 0)) cs >>= 1;
+  while (cs > 1 && (K / cs < 128 || K % (PS_BK * cs) != 0)) cs >>= 1;
   const int k_slice = K / cs;
   const int steps = k_slice / PS_BK;
   int mt = M <= 16 ? 1 : (M <= 32 ? 2 : 4);
@@ -158,10 +160,9 @@ int32_t launch_turn(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
 
 int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt, int n_out, GemmParams gp, cudaStream_t stream) {
   gp.hd_shift = ilog2(gp.hd); gp.rk_shift = ilog2(gp.rank_k > 0 ? gp.rank_k : 1); gp.rv_shift = ilog2(gp.rank_v > 0 ? gp.rank_v : 1);
-  // Few rows: the weight-streaming kernel (fused Llama-3-8B projection: 5.8 us at 16 rows, 7.8 at 32).  From 33 to 40 rows the
-  // turn kernel would be faster on wide layers (9.8 against 12.9 us) and slower on narrow ones (d_model 2048: 7.2 against
-  // 6.6), but rows written one by one and in one call of up to 40 have equal bits, which is worth more.  Beyond that the turn
-  // kernel, up to some two thousand rows; the few-row kernel still takes 41 .. 64 rows where the K split does not apply
+  // Few rows: the weight-streaming kernel (fused Llama-3-8B projection: 6.1 us at 16 rows, 7.8 at 32, 9.8 at 40, where the turn
+  // kernel takes 9.8 too; d_model 2048, 40 rows: 4.8 against 7.3).  Rows written one by one and in one call of up to 40 have
+  // equal bits.  Beyond that the turn kernel, up to some two thousand rows; the few-row kernel still takes 41 .. 64 rows where the K split does not apply
   // (short K).
   if (M <= PS_FAST_M && !ctx->force_tiled_gemm) {
     const int32_t rc = launch_small(ctx, X, M, K, Wt, n_out, gp, stream);

@@ -8,7 +8,7 @@
 //            thread-block cluster (split-K, up to 8);
 //   loads  = TMA: per 64-deep k step one box of W rows (contiguous in memory: the packed weights are
 //            k-blocked, [K/64][n_out][64]) and one box of X rows (rows past M are zero-filled
-//            by the out-of-bounds rule) into a 4-slot ring of 128-byte-swizzled shared memory, issued by
+//            by the out-of-bounds rule) into a ring of 3 or 4 slots of 128-byte-swizzled shared memory, issued by
 //            a producer warp (full/empty mbarriers).  The ring is kept small on purpose: every cluster of
 //            the grid must be resident at once, or the launch runs in two waves;
 //   math   = mma.sync m16n8k16 (bf16 -> fp32): X rows on the M axis, a warp owns 8 (16 when M > 16)
@@ -33,14 +33,16 @@ constexpr int PS_WARPS = 8;
 constexpr int PS_BK = 64;                   // k elements per step: one 128-byte swizzle row
 constexpr int PS_MAX_M = 64;
 constexpr int PS_FAST_M = 40;               // up to here it takes every call: a row has the same bits alone and among up to 39 others
-constexpr int PS_STAGES = 4;
 constexpr int PS_THREADS = (PS_WARPS + 1) * 32;       // consumer warps + one producer warp
+// Ring depth.  Above 32 rows three slots: with four (130 KB a block) only 15 clusters of eight are resident at once and the
+// 18 of the Llama-3-8B projection ran in two waves (33 .. 40 rows: 12.8 us, now 9.7).
+__host__ __device__ constexpr int ps_stages(int mt) { return mt > 2 ? 3 : 4; }
 __host__ __device__ constexpr int ps_nt(int mt) { return mt > 1 ? 2 : 1; }               // 8-column n-tiles per warp
 __host__ __device__ constexpr int ps_cols(int mt) { return PS_WARPS * 8 * ps_nt(mt); }   // output columns per block
 __host__ __device__ constexpr int ps_step_bytes(int mt) { return (ps_cols(mt) + mt * 16) * PS_BK * 2; }
 __host__ __device__ constexpr int ps_recv_bytes(int mt) { return mt * 16 * ps_cols(mt) * 4; }   // [cluster rank][row][own columns] fp32
 __host__ __device__ constexpr int ps_smem_bytes(int mt) {
-  return PS_STAGES * ps_step_bytes(mt) + 128 + ps_recv_bytes(mt) + 1024;   // ring | mbarriers | receive area | alignment slack
+  return ps_stages(mt) * ps_step_bytes(mt) + 128 + ps_recv_bytes(mt) + 1024;   // ring | mbarriers | receive area | alignment slack
 }
 
 template <int MT>
@@ -51,6 +53,7 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   constexpr int COLS = ps_cols(MT);
   constexpr int W_BYTES = COLS * PS_BK * 2;
   constexpr int STEP_BYTES = ps_step_bytes(MT);
+  constexpr int STAGES = ps_stages(MT);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint32_t rank, CS;
@@ -61,14 +64,14 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   const int k0 = rank * k_slice;
   const int steps = k_slice / PS_BK;
   const uint32_t tiles = smem_u32(smem);
-  const uint32_t full0 = tiles + PS_STAGES * STEP_BYTES, empty0 = full0 + 8 * PS_STAGES;
-  const uint32_t recv_bar = empty0 + 8 * PS_STAGES;
+  const uint32_t full0 = tiles + STAGES * STEP_BYTES, empty0 = full0 + 8 * STAGES;
+  const uint32_t recv_bar = empty0 + 8 * STAGES;
   const uint32_t recv_u32 = full0 + 128;                // behind the barriers; never overlaid: peers send while this block computes
   const bool push = !p.rope;                            // the same in every block of the grid
   const int cpb = COLS / CS;                            // columns finished by one block (a power of two >= 8)
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < PS_STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, PS_WARPS); }
+    for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, PS_WARPS); }
     mbar_init(recv_bar, 1);
     if (push) mbar_expect_tx(recv_bar, (uint32_t)(CS * p.M * cpb * 4));   // the one arrival, and the bytes to come: rows < M of every peer
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -79,7 +82,7 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   // The weights are not the preceding kernel's to write: the first ring fill of W boxes is requested before the wait
   // for that kernel (programmatic dependent launch), so a block that is resident early has them in shared memory
   // when its predecessor ends.  X (the previous kernel's output) and every store stay behind the wait.
-  const int pre = steps < PS_STAGES ? steps : PS_STAGES;
+  const int pre = steps < STAGES ? steps : STAGES;
   if (warp == PS_WARPS && lane == 0) {
     for (int s = 0; s < pre; ++s) {
       mbar_expect_tx(full0 + 8 * s, STEP_BYTES);
@@ -101,8 +104,8 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       for (int s = 0; s < pre; ++s)                      // the X boxes of the steps whose W boxes are already on their way
         tma_load_2d(tiles + s * STEP_BYTES + W_BYTES, &map_x, k0 + s * PS_BK, 0, full0 + 8 * s);
       for (int s = pre; s < steps; ++s) {
-        const int slot = s % PS_STAGES;
-        mbar_wait(empty0 + 8 * slot, ((s / PS_STAGES) - 1) & 1, p.status);
+        const int slot = s % STAGES;
+        mbar_wait(empty0 + 8 * slot, ((s / STAGES) - 1) & 1, p.status);
         const uint32_t dst = tiles + slot * STEP_BYTES;
         mbar_expect_tx(full0 + 8 * slot, STEP_BYTES);
         tma_load_3d(dst, &map_w, 0, group * COLS, k0 / PS_BK + s, full0 + 8 * slot);   // one contiguous run of the k-blocked weights
@@ -112,8 +115,8 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   } else {
     const int mi = lane >> 3, ri = lane & 7;
     for (int s = 0; s < steps; ++s) {
-      const int slot = s % PS_STAGES;
-      mbar_wait(full0 + 8 * slot, (s / PS_STAGES) & 1, p.status);
+      const int slot = s % STAGES;
+      mbar_wait(full0 + 8 * slot, (s / STAGES) & 1, p.status);
       const uint32_t wt = tiles + slot * STEP_BYTES, xt = wt + W_BYTES;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {                      // two k steps of 16 per ldmatrix of W
@@ -160,7 +163,7 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     int it = threadIdx.x;
     int row = it / ppr, pc = it - row * ppr;              // worked out before the wait
     mbar_wait_cluster(recv_bar, 0, p.status);
-    const float* recv = reinterpret_cast<const float*>(smem + PS_STAGES * STEP_BYTES + 128);
+    const float* recv = reinterpret_cast<const float*>(smem + STAGES * STEP_BYTES + 128);
     for (; it < n_items; it += PS_THREADS, row = it / ppr, pc = it - row * ppr) {
       const int gc = group * COLS + rank * cpb + pc * 8;
       if (gc >= p.N_out) continue;
