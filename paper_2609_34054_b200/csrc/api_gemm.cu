@@ -84,7 +84,7 @@ int max_turn_clusters(precc_ctx* ctx, int ks) {
   int& cached = max_clusters_dev[ctx->device % kMaxDevices][ks];
   if (cached == 0) {
     int n = 0;
-    auto kern = proj_turn_kernel<false>;
+    auto kern = proj_turn_kernel<false, 1>;
     if (raise_smem_limit(ctx, kern, PT_MIN_SMEM) == cudaSuccess) {
       cudaLaunchConfig_t qc = {};
       qc.gridDim = dim3(ks, ctx->sm_count, 1); qc.blockDim = dim3(PT_THREADS); qc.dynamicSmemBytes = PT_MIN_SMEM;
@@ -120,8 +120,8 @@ TurnPlan plan_turn(precc_ctx* ctx, int M, int nkb, int n_fused) {
       if (groups * tiles > max_turn_clusters(ctx, ks)) continue;
       const int kb = (nkb + ks - 1) / ks;
       int st = kb < PT_MAX_STAGES ? kb : PT_MAX_STAGES;
-      while (st > 1 && pt_smem_bytes(tn, ks, st) > ctx->max_smem_optin) --st;
-      if (pt_smem_bytes(tn, ks, st) > ctx->max_smem_optin) continue;
+      while (st > 1 && pt_smem_bytes(tn, ks, st, 1) > ctx->max_smem_optin) --st;
+      if (pt_smem_bytes(tn, ks, st, 1) > ctx->max_smem_optin) continue;
       const double cost = kb * (0.37 + 0.00036 * tn) + 0.005 * pt_share(tn, ks) * (ks - 1) + 0.0113 * tn + 0.1 * ks;
       if (cost < best_cost) { best_cost = cost; best.tn = tn; best.ks = ks; best.stages = st; }
     }
@@ -129,22 +129,35 @@ TurnPlan plan_turn(precc_ctx* ctx, int M, int nkb, int n_fused) {
   return best;
 }
 
+// The turn kernel over the whole K extent (up to 256 columns): rows of a tile, or 0 where 128-row tiles are as good.  With one
+// round of those they are (9000 x 128: 28.0 against 28.5 us); from two rounds on this form wins by what they fetch twice or leave
+// idle.  Very few columns cost the tiled kernel little beside the rows, so there it has to save a fifth of them
+// (32768 x 32: 49.1 against 50.8 us for an eighth; 20000 x 32: 47.7 against 33.7 us).
+int pick_wide_rows(int M, int n_out, int sm_count) {
+  const int rt = ((M + GEMM_BM - 1) / GEMM_BM + sm_count - 1) / sm_count, rounds = (M + sm_count * PT_MAX_TN - 1) / (sm_count * PT_MAX_TN);
+  const int tn = ((M + sm_count * rounds - 1) / (sm_count * rounds) + 15) / 16 * 16;
+  if (n_out > 2 * PT_COLS || rt < 2 || (n_out <= 64 && tn * rounds * 5 > rt * GEMM_BM * 4)) return 0;
+  return tn;
+}
+
+template <int NG>
 int32_t launch_turn(precc_ctx* ctx, const void* X, int M, int K, const void* Wt, int n_out, GemmParams gp, const TurnPlan& tp, cudaStream_t stream) {
-  int tmem_cols = 32;
+  int tmem_cols = NG > 1 ? 512 : 32;
   while (tmem_cols < tp.tn) tmem_cols <<= 1;
   CUtensorMap map_x, map_w;
   int32_t rc = make_map(ctx, &map_x, X, M, K, tp.tn);
   if (rc) return rc;
-  rc = make_map_w(ctx, &map_w, Wt, n_out, K, PT_COLS);
+  rc = make_map_w(ctx, &map_w, Wt, n_out, K, NG * PT_COLS);
   if (rc) return rc;
   gp.M = M; gp.N_out = n_out; gp.K = K; gp.BN = tp.tn; gp.stages = tp.stages; gp.tmem_cols = tmem_cols;
   gp.status = ctx->status;
-  int smem = pt_smem_bytes(tp.tn, tp.ks, tp.stages);
+  int smem = pt_smem_bytes(tp.tn, tp.ks, tp.stages, NG);
   if (smem < PT_MIN_SMEM) smem = PT_MIN_SMEM;
-  auto kern = gp.rope ? proj_turn_kernel<true> : proj_turn_kernel<false>;
+  auto kern = proj_turn_kernel<false, NG>;
+  if constexpr (NG == 1) { if (gp.rope) kern = proj_turn_kernel<true, 1>; }       // (two accumulators: never with rotary keys)
   PRECC_CUDA(ctx, raise_smem_limit(ctx, kern, smem));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(tp.ks, (n_out + PT_COLS - 1) / PT_COLS, (M + tp.tn - 1) / tp.tn);
+  cfg.gridDim = dim3(tp.ks, (n_out + NG * PT_COLS - 1) / (NG * PT_COLS), (M + tp.tn - 1) / tp.tn);
   cfg.blockDim = dim3(PT_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
@@ -174,11 +187,22 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
     // planned for the width of the FUSED projection of this layer, whatever this call projects, so that the base-only,
     // LR-only and fused calls of one M take the same decision (and with it the same summation order)
     const TurnPlan tp = plan_turn(ctx, M, K / GEMM_BK, 2 * gp.n_kv * gp.hd + gp.n_agents * (gp.rank_k + gp.rank_v));
-    if (tp.ks > 0) return launch_turn(ctx, X, M, K, Wt, n_out, gp, tp, stream);
+    if (tp.ks > 0) return launch_turn<1>(ctx, X, M, K, Wt, n_out, gp, tp, stream);
   }
   if (M <= PS_MAX_M && !ctx->force_tiled_gemm) {
     const int32_t rc = launch_small(ctx, X, M, K, Wt, n_out, gp, stream);
     if (rc >= 0) return rc;
+  }
+  // Many rows, few columns: the turn kernel over the whole K extent.
+  const int wide = gp.rope || ctx->gemm_pair || ctx->force_tiled_gemm ? 0 : pick_wide_rows(M, n_out, ctx->sm_count);
+  if (wide > 0) {
+    const int ng = n_out > PT_COLS ? 2 : 1;
+    TurnPlan tp;
+    tp.tn = wide; tp.ks = 1;
+    tp.stages = K / GEMM_BK < PT_MAX_STAGES ? K / GEMM_BK : PT_MAX_STAGES;
+    while (tp.stages > 1 && pt_smem_bytes(wide, 1, tp.stages, ng) > ctx->max_smem_optin) --tp.stages;
+    if (pt_smem_bytes(wide, 1, tp.stages, ng) <= ctx->max_smem_optin)
+      return ng == 1 ? launch_turn<1>(ctx, X, M, K, Wt, n_out, gp, tp, stream) : launch_turn<2>(ctx, X, M, K, Wt, n_out, gp, tp, stream);
   }
   // Many rows: two SMs per 256 x 256 tile (each stages half of the weight tile), see gemm_pair.cuh.
   if (ctx->gemm_pair && M >= 2 * GEMM_PAIR_BM) {

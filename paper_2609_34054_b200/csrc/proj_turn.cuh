@@ -14,7 +14,11 @@
 //            while the next slice is dumped.  The receiver adds the KS slices in rank order (the result does not
 //            depend on timing) and stores 16-byte pieces, sixteen lanes on consecutive pieces of a row.  Whole heads sit in
 //            one row of the tile, so rotary keys find their partner column next to them.
-// Shared memory: [ring of {W 128 x 64 | X TN x 64} | overlaid: dump [TN][128] fp32, receive area [KS-1][tw][128] fp32]
+// NG = 2: one block takes 256 columns of its rows (two accumulators of up to 256 tensor-memory columns), KS = 1.  This is the
+// form for many rows and few columns (the LR rows of a long context), which is bound by the rows of X: cut into as many tiles
+// as there are SMs, every row is fetched once and the weights once per SM, where 128-row tiles come out as two rounds of
+// overlapping ones (32768 rows x 256 columns of d_model 4096: 71.5 -> 64.0 us; 20000 x 192: 56.6 -> 42.1; 20000 x 128, NG = 1: 53.0 -> 35.9).
+// Shared memory: [ring of {W 128 NG x 64 | X TN x 64} | overlaid: dump [TN][128] fp32, receive area [KS-1][tw][128] fp32]
 // [row table][barriers].  A block tells its peers when its ring is idle; they send only then.
 // The K split depends on M, K and the layer's fused width alone, so base-only, LR-only and fused calls agree bit for bit.
 // Measured on rotating weights from HBM, us a launch, against 128-row x 256-column tiles whose slices were pulled over
@@ -35,18 +39,18 @@ constexpr int PT_MAX_STAGES = 8;
 constexpr int PT_MIN_SMEM = 120 * 1024;                  // keeps one block per SM, so that the cluster occupancy depends on KS alone
 struct PtRow { long long slot, slot2; unsigned long long mask; int pos, ok; };   // what the routing needs to know about a row
 
-__host__ __device__ constexpr int pt_stage_bytes(int tn) { return PT_W_BYTES + tn * GEMM_BK * 2; }
+__host__ __device__ constexpr int pt_stage_bytes(int tn, int ng) { return ng * PT_W_BYTES + tn * GEMM_BK * 2; }
 __host__ __device__ constexpr int pt_share(int rows, int ks) { return ((rows + ks - 1) / ks + 7) / 8 * 8; }     // rows finished by one block
 __host__ __device__ constexpr int pt_merge_bytes(int tn, int ks) { return (tn + (ks - 1) * pt_share(tn, ks)) * PT_COLS * 4; }
-__host__ __device__ constexpr int pt_data_bytes(int tn, int ks, int stages) {
-  const int ring = stages * pt_stage_bytes(tn), merge = pt_merge_bytes(tn, ks);
+__host__ __device__ constexpr int pt_data_bytes(int tn, int ks, int stages, int ng) {
+  const int ring = stages * pt_stage_bytes(tn, ng), merge = pt_merge_bytes(tn, ks);
   return ((ring > merge ? ring : merge) + 1023) / 1024 * 1024;
 }
-__host__ __device__ constexpr int pt_smem_bytes(int tn, int ks, int stages) {
-  return pt_data_bytes(tn, ks, stages) + pt_share(tn, ks) * (int)sizeof(PtRow) + (2 * PT_MAX_STAGES + 4) * 8;
+__host__ __device__ constexpr int pt_smem_bytes(int tn, int ks, int stages, int ng) {
+  return pt_data_bytes(tn, ks, stages, ng) + pt_share(tn, ks) * (int)sizeof(PtRow) + (2 * PT_MAX_STAGES + 4) * 8;
 }
 
-template <bool ROPE>
+template <bool ROPE, int NG>
 __global__ void __launch_bounds__(PT_THREADS, 1)
 proj_turn_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const GemmParams p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -57,8 +61,8 @@ proj_turn_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
   }
   const int KS = gridDim.x, rank = blockIdx.x;           // the cluster spans grid.x
   const int TN = p.BN;
-  const int stage_bytes = pt_stage_bytes(TN);
-  PtRow* rows = reinterpret_cast<PtRow*>(smem + pt_data_bytes(TN, KS, p.stages));
+  const int stage_bytes = pt_stage_bytes(TN, NG);
+  PtRow* rows = reinterpret_cast<PtRow*>(smem + pt_data_bytes(TN, KS, p.stages, NG));
   uint64_t* bars = reinterpret_cast<uint64_t*>(rows + pt_share(TN, KS));
   // barrier map: full[stages] | empty[stages] | acc_full | ready (peers whose ring is idle) | recv (bytes received)
   const uint32_t full0 = smem_u32(bars);
@@ -71,7 +75,7 @@ proj_turn_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
   const int nkb = p.K / GEMM_BK;
   const int kb0 = (rank * nkb) / KS;
   const int nkb_s = ((rank + 1) * nkb) / KS - kb0;
-  const int m0 = blockIdx.z * TN, n0 = blockIdx.y * PT_COLS;
+  const int m0 = blockIdx.z * TN, n0 = blockIdx.y * (NG * PT_COLS);
   const int n_rows = min(TN, p.M - m0);                  // rows of this tile that exist
   const int tw = pt_share(n_rows, KS);                   // rows finished by one block (the last ones may own fewer, or none)
   auto slice_rows = [&](int r) { return max(0, min(tw, n_rows - r * tw)); };
@@ -94,7 +98,7 @@ proj_turn_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
       const uint32_t st = smem_u32(smem) + it * stage_bytes;
       mbar_expect_tx(full0 + 8 * it, stage_bytes);
       tma_load_3d(st, &map_w, 0, n0, kb0 + it, full0 + 8 * it);
-      tma_load_2d(st + PT_W_BYTES, &map_x, (kb0 + it) * GEMM_BK, m0, full0 + 8 * it);
+      tma_load_2d(st + NG * PT_W_BYTES, &map_x, (kb0 + it) * GEMM_BK, m0, full0 + 8 * it);
     }
   }
   if (warp == 1) {
@@ -117,7 +121,7 @@ proj_turn_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         const uint32_t st = smem_u32(smem) + s * stage_bytes;
         mbar_expect_tx(full0 + 8 * s, stage_bytes);
         tma_load_3d(st, &map_w, 0, n0, kb0 + it, full0 + 8 * s);
-        tma_load_2d(st + PT_W_BYTES, &map_x, (kb0 + it) * GEMM_BK, m0, full0 + 8 * s);
+        tma_load_2d(st + NG * PT_W_BYTES, &map_x, (kb0 + it) * GEMM_BK, m0, full0 + 8 * s);
       }
     }
     __syncwarp();
@@ -126,7 +130,7 @@ proj_turn_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     if (lane == 0) {
       const uint32_t idesc = umma_idesc_bf16(TN);
       const uint64_t dw0 = umma_desc_sw128(smem_u32(smem));
-      const uint64_t dx0 = umma_desc_sw128(smem_u32(smem) + PT_W_BYTES);
+      const uint64_t dx0 = umma_desc_sw128(smem_u32(smem) + NG * PT_W_BYTES);
       for (int it = 0; it < nkb_s; ++it) {
         const int s = it % p.stages;
         mbar_wait(full0 + 8 * s, (it / p.stages) & 1, p.status);
@@ -134,7 +138,9 @@ proj_turn_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         const uint64_t so = (uint64_t)((s * stage_bytes) >> 4);
 #pragma unroll
         for (int k = 0; k < GEMM_BK / 16; ++k)
-          umma_bf16(tmem_base, dw0 + so + 2 * k, dx0 + so + 2 * k, idesc, (it | k) ? 1u : 0u);
+#pragma unroll
+          for (int h = 0; h < NG; ++h)
+            umma_bf16(tmem_base + h * PT_MAX_TN, dw0 + so + h * (PT_W_BYTES >> 4) + 2 * k, dx0 + so + 2 * k, idesc, (it | k) ? 1u : 0u);
         umma_commit(empty0 + 8 * s);
       }
       umma_commit(acc_full);                       // every MMA of the slice has completed: the ring is idle too
@@ -160,113 +166,117 @@ proj_turn_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
       rows[et] = r;
     }
     const int piece = et & 15;                           // eight columns: the same ones in every pass of the reduction below
-    const int gc = n0 + piece * 8, w = p.n_kv << p.hd_shift;
-    bool live = gc < p.N_out, to_base = p.mode == 1 || (p.mode == 2 && gc < 2 * w), is_key = false;
-    __nv_bfloat16* dst0;                                 // base: [blk][n_kv][16][hd] at this head and column; LR: [slot][r] at this agent and coordinate
-    int agent = 0, sh;                                   // sh: log2 of the destination's row width
-    if (to_base) {
-      const bool is_v = gc >= w;
-      const int cc = is_v ? gc - w : gc;
-      is_key = !is_v;
-      sh = p.hd_shift;
-      dst0 = (is_v ? p.base_v : p.base_k) + ((long long)((cc >> sh) * PAGE) << sh) + (cc & (p.hd - 1));
-      if (ROPE && is_key && (cc & (p.hd - 1)) >= p.hd / 2) live = false;        // the upper half of a rotated head is written with the lower
-    } else {
-      const int n_lrk = p.rank_k > 0 ? (p.n_agents << p.rk_shift) : 0;
-      const int gl = p.mode == 2 ? gc - 2 * w : gc;
-      const bool is_v = gl >= n_lrk;
-      sh = is_v ? p.rv_shift : p.rk_shift;
-      const int cc = is_v ? gl - n_lrk : gl;
-      agent = cc >> sh;
-      dst0 = (is_v ? p.lr_v : p.lr_k) + (((long long)agent * p.n_blocks * PAGE) << sh) + (cc & ((1 << sh) - 1));
-    }
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");       // the peers' barriers are initialised
-    mbar_wait(acc_full, 0, p.status);
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    // this block's ring is idle: the peers may send into the receive area that overlays it
-    if (et < KS - 1) {
-      const int peer = et < rank ? et : et + 1;
-      asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(dsmem_addr(ready_bar, peer)) : "memory");
-    }
-    // ---- dump slice by slice, the peers' first, the own one last; a peer's slice leaves while the next is dumped
-    const uint32_t trow = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
-    float* dcol = dump + quad * 32 + lane;
-    for (int k = 1; k <= KS; ++k) {
-      const int sl = rank + k < KS ? rank + k : rank + k - KS;
-      const int c0 = sl * tw, nr = slice_rows(sl);
-      for (int c = half * 8; c < nr; c += 32) {          // two groups of eight rows in flight per warp (the last one may run up to seven rows past n_rows: inside the tile, never read)
-        uint32_t r0[8], r1[8];
-        const bool two = c + 16 < nr;
-        tmem_ld8(trow + c0 + c, r0);
-        if (two) tmem_ld8(trow + c0 + c + 16, r1);
-        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          dcol[(size_t)(c0 + c + q) * PT_COLS] = __uint_as_float(r0[q]);
-        if (two) {
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            dcol[(size_t)(c0 + c + 16 + q) * PT_COLS] = __uint_as_float(r1[q]);
-        }
-      }
-      if (k < KS) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // the copy engine reads what these threads wrote
-      asm volatile("bar.sync 1, 256;\n" ::: "memory");                            // the merging warps
-      if (k < KS && et == 0) {
-        if (k == 1) mbar_wait_cluster(ready_bar, 0, p.status);                     // every peer's ring is idle
-        if (nr > 0) {
-          const uint32_t src = smem_u32(dump) + (uint32_t)(c0 * PT_COLS * 4);
-          const uint32_t dst = dsmem_addr(smem_u32(recv) + (uint32_t)((rank < sl ? rank : rank - 1) * tw * PT_COLS * 4), sl);
-          asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-                       ::"r"(dst), "r"(src), "r"(nr * PT_COLS * 4), "r"(dsmem_addr(recv_bar, sl)) : "memory");
-        }
-      }
-    }
-    // ---- own rows + received rows, in rank order, routed to the caches: sixteen threads per row, eight columns each
-    mbar_wait_cluster(recv_bar, 0, p.status);
-    const float* own = dump + (size_t)rank * tw * PT_COLS;
-    auto gather = [&](int r, int c, float (&v)[8]) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = 0.f;
-#pragma unroll
-      for (int s = 0; s < GEMM_MAX_KS; ++s) {
-        if (s < KS) {
-          const float* src = (s == rank ? own : recv + (size_t)(s < rank ? s : s - 1) * tw * PT_COLS) + r * PT_COLS + c;
-          const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
-          v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w; v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
-        }
-      }
-    };
-    auto pack8 = [](const float (&v)[8]) {
-      return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-    };
-    for (int r = et >> 4; live && r < own_rows; r += PT_EPI_WARPS * 2) {
-      const PtRow row = rows[r];
-      if (!row.ok) continue;
-      float v[8];
-      gather(r, piece * 8, v);
+#pragma unroll 1
+    for (int h = 0; h < NG; ++h) {                       // one 128-column half after the other, through the same dump
+      const int gc = n0 + h * PT_COLS + piece * 8, w = p.n_kv << p.hd_shift;
+      bool live = gc < p.N_out, to_base = p.mode == 1 || (p.mode == 2 && gc < 2 * w), is_key = false;
+      __nv_bfloat16* dst0;                                 // base: [blk][n_kv][16][hd] at this head and column; LR: [slot][r] at this agent and coordinate
+      int agent = 0, sh;                                   // sh: log2 of the destination's row width
       if (to_base) {
-        __nv_bfloat16* dst = dst0 + (((row.slot / PAGE) * p.n_kv * PAGE + (row.slot % PAGE)) << sh);
-        if constexpr (ROPE) {
-          if (is_key) {
-            float h[8];
-            gather(r, piece * 8 + p.hd / 2, h);
-            const float4* cs = p.rope + (long long)row.pos * (p.hd / 4) + (gc & (p.hd - 1)) / 2;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const float4 t = __ldg(cs + q);
-              const float l0 = v[2 * q], l1 = v[2 * q + 1], h0 = h[2 * q], h1 = h[2 * q + 1];
-              v[2 * q] = l0 * t.x - h0 * t.y; v[2 * q + 1] = l1 * t.z - h1 * t.w;
-              h[2 * q] = h0 * t.x + l0 * t.y; h[2 * q + 1] = h1 * t.z + l1 * t.w;
-            }
-            *reinterpret_cast<uint4*>(dst + p.hd / 2) = pack8(h);
+        const bool is_v = gc >= w;
+        const int cc = is_v ? gc - w : gc;
+        is_key = !is_v;
+        sh = p.hd_shift;
+        dst0 = (is_v ? p.base_v : p.base_k) + ((long long)((cc >> sh) * PAGE) << sh) + (cc & (p.hd - 1));
+        if (ROPE && is_key && (cc & (p.hd - 1)) >= p.hd / 2) live = false;        // the upper half of a rotated head is written with the lower
+      } else {
+        const int n_lrk = p.rank_k > 0 ? (p.n_agents << p.rk_shift) : 0;
+        const int gl = p.mode == 2 ? gc - 2 * w : gc;
+        const bool is_v = gl >= n_lrk;
+        sh = is_v ? p.rv_shift : p.rk_shift;
+        const int cc = is_v ? gl - n_lrk : gl;
+        agent = cc >> sh;
+        dst0 = (is_v ? p.lr_v : p.lr_k) + (((long long)agent * p.n_blocks * PAGE) << sh) + (cc & ((1 << sh) - 1));
+      }
+      if (h == 0) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");       // the peers' barriers are initialised
+      mbar_wait(acc_full, 0, p.status);
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      // this block's ring is idle: the peers may send into the receive area that overlays it
+      if (et < KS - 1) {
+        const int peer = et < rank ? et : et + 1;
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(dsmem_addr(ready_bar, peer)) : "memory");
+      }
+      // ---- dump slice by slice, the peers' first, the own one last; a peer's slice leaves while the next is dumped
+      const uint32_t trow = tmem_base + h * PT_MAX_TN + (static_cast<uint32_t>(quad * 32) << 16);
+      float* dcol = dump + quad * 32 + lane;
+      for (int k = 1; k <= KS; ++k) {
+        const int sl = rank + k < KS ? rank + k : rank + k - KS;
+        const int c0 = sl * tw, nr = slice_rows(sl);
+        for (int c = half * 8; c < nr; c += 32) {          // two groups of eight rows in flight per warp (the last one may run up to seven rows past n_rows: inside the tile, never read)
+          uint32_t r0[8], r1[8];
+          const bool two = c + 16 < nr;
+          tmem_ld8(trow + c0 + c, r0);
+          if (two) tmem_ld8(trow + c0 + c + 16, r1);
+          asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+  #pragma unroll
+          for (int q = 0; q < 8; ++q)
+            dcol[(size_t)(c0 + c + q) * PT_COLS] = __uint_as_float(r0[q]);
+          if (two) {
+  #pragma unroll
+            for (int q = 0; q < 8; ++q)
+              dcol[(size_t)(c0 + c + 16 + q) * PT_COLS] = __uint_as_float(r1[q]);
           }
         }
-        *reinterpret_cast<uint4*>(dst) = pack8(v);
-      } else if ((row.mask >> agent) & 1ull) {
-        const uint4 o = pack8(v);
-        *reinterpret_cast<uint4*>(dst0 + (row.slot << sh)) = o;
-        if (row.slot2 >= 0) *reinterpret_cast<uint4*>(dst0 + (row.slot2 << sh)) = o;
+        if (k < KS) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // the copy engine reads what these threads wrote
+        asm volatile("bar.sync 1, 256;\n" ::: "memory");                            // the merging warps
+        if (k < KS && et == 0) {
+          if (k == 1) mbar_wait_cluster(ready_bar, 0, p.status);                     // every peer's ring is idle
+          if (nr > 0) {
+            const uint32_t src = smem_u32(dump) + (uint32_t)(c0 * PT_COLS * 4);
+            const uint32_t dst = dsmem_addr(smem_u32(recv) + (uint32_t)((rank < sl ? rank : rank - 1) * tw * PT_COLS * 4), sl);
+            asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                         ::"r"(dst), "r"(src), "r"(nr * PT_COLS * 4), "r"(dsmem_addr(recv_bar, sl)) : "memory");
+          }
+        }
       }
+      // ---- own rows + received rows, in rank order, routed to the caches: sixteen threads per row, eight columns each
+      mbar_wait_cluster(recv_bar, 0, p.status);
+      const float* own = dump + (size_t)rank * tw * PT_COLS;
+      auto gather = [&](int r, int c, float (&v)[8]) {
+  #pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = 0.f;
+  #pragma unroll
+        for (int s = 0; s < GEMM_MAX_KS; ++s) {
+          if (s < KS) {
+            const float* src = (s == rank ? own : recv + (size_t)(s < rank ? s : s - 1) * tw * PT_COLS) + r * PT_COLS + c;
+            const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
+            v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w; v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
+          }
+        }
+      };
+      auto pack8 = [](const float (&v)[8]) {
+        return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+      };
+      for (int r = et >> 4; live && r < own_rows; r += PT_EPI_WARPS * 2) {
+        const PtRow row = rows[r];
+        if (!row.ok) continue;
+        float v[8];
+        gather(r, piece * 8, v);
+        if (to_base) {
+          __nv_bfloat16* dst = dst0 + (((row.slot / PAGE) * p.n_kv * PAGE + (row.slot % PAGE)) << sh);
+          if constexpr (ROPE) {
+            if (is_key) {
+              float u[8];
+              gather(r, piece * 8 + p.hd / 2, u);
+              const float4* cs = p.rope + (long long)row.pos * (p.hd / 4) + (gc & (p.hd - 1)) / 2;
+  #pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const float4 t = __ldg(cs + q);
+                const float l0 = v[2 * q], l1 = v[2 * q + 1], h0 = u[2 * q], h1 = u[2 * q + 1];
+                v[2 * q] = l0 * t.x - h0 * t.y; v[2 * q + 1] = l1 * t.z - h1 * t.w;
+                u[2 * q] = h0 * t.x + l0 * t.y; u[2 * q + 1] = h1 * t.z + l1 * t.w;
+              }
+              *reinterpret_cast<uint4*>(dst + p.hd / 2) = pack8(u);
+            }
+          }
+          *reinterpret_cast<uint4*>(dst) = pack8(v);
+        } else if ((row.mask >> agent) & 1ull) {
+          const uint4 o = pack8(v);
+          *reinterpret_cast<uint4*>(dst0 + (row.slot << sh)) = o;
+          if (row.slot2 >= 0) *reinterpret_cast<uint4*>(dst0 + (row.slot2 << sh)) = o;
+        }
+      }
+      if (h + 1 < NG) asm volatile("bar.sync 1, 256;\n" ::: "memory");   // the dump has been read
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   }
