@@ -1,6 +1,8 @@
 // libprecc: the attention entry points (decode, its rotary, partial-record and allocation-free forms, the
 // combine step of context-sharded decode, new-turn prefill).  The kernels themselves are compiled in the
 // per-head-dimension units; this file validates arguments and forwards.
+#include <algorithm>
+
 #include "api_internal.h"
 #include "combine.cuh"
 #include "prefill.cuh"   // PF_ROWS (the size check of the prefill entry)
@@ -248,16 +250,14 @@ static int32_t prefill_entry(precc_ctx* ctx, const precc_layer_desc* desc, const
   x.n_blocks = cache->n_blocks; x.first_block = first_block; x.n_tokens = ctx_len + S;
   x.n_kv = desc->n_kv_heads; x.hd = desc->head_dim; x.rk = desc->rank_k; x.max_pos = rope->max_pos; x.s_k = desc->lora_scale_k;
   x.n_out_blocks = (int)out_blocks;
-  const int n_tasks = desc->n_kv_heads * (desc->head_dim / 32);
-  auto launch = [&](auto kern, size_t xs, int group_tasks) -> int32_t {
-    PRECC_CUDA(ctx, raise_smem_limit(ctx, kern, (int)xs));
-    const int groups = (n_tasks + group_tasks - 1) / group_tasks;
-    long long gx = 2ll * ctx->sm_count / groups;          // two resident blocks per SM: each walks its share of the cache blocks
-    if (gx < 1) gx = 1;
-    if (gx > out_blocks) gx = out_blocks;
+  // one wave: every warp walks over an equal share of the cache blocks (its B_k fragments are fetched once)
+  const int groups = (desc->n_kv_heads * (desc->head_dim / RX_COLS) + RX_WARPS - 1) / RX_WARPS;
+  auto launch = [&](auto kern, int resident) -> int32_t {
+    const long long fit = std::max(1ll, (long long)resident * ctx->sm_count / groups);
+    const long long rounds = (out_blocks + fit - 1) / fit;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)gx, (unsigned)groups); cfg.blockDim = dim3(RX_THREADS);
-    cfg.dynamicSmemBytes = xs; cfg.stream = (cudaStream_t)stream;
+    cfg.gridDim = dim3((unsigned)((out_blocks + rounds - 1) / rounds), (unsigned)groups); cfg.blockDim = dim3(RX_THREADS);
+    cfg.stream = (cudaStream_t)stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -265,10 +265,9 @@ static int32_t prefill_entry(precc_ctx* ctx, const precc_layer_desc* desc, const
     PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, x));
     return PRECC_OK;
   };
-  int32_t xrc;
-  if (desc->rank_k <= 16) xrc = launch(rope_expand_keys_kernel<1>, rope_expand_smem_bytes<1>(), RxCfg<1>::GROUP_TASKS);
-  else if (desc->rank_k == 32) xrc = launch(rope_expand_keys_kernel<2>, rope_expand_smem_bytes<2>(), RxCfg<2>::GROUP_TASKS);
-  else xrc = launch(rope_expand_keys_kernel<4>, rope_expand_smem_bytes<4>(), RxCfg<4>::GROUP_TASKS);
+  const int32_t xrc = desc->rank_k <= 16 ? launch(rope_expand_keys_kernel<1>, rx_blocks_per_sm(1))
+                    : desc->rank_k == 32 ? launch(rope_expand_keys_kernel<2>, rx_blocks_per_sm(2))
+                                         : launch(rope_expand_keys_kernel<4>, rx_blocks_per_sm(4));
   if (xrc) return xrc;
   return desc->head_dim == 64 ? prefill_run_hd64(ctx, b, 0, rv) : prefill_run_hd128(ctx, b, 0, rv);
 }

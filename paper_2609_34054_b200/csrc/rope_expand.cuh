@@ -5,7 +5,7 @@
 // with K_base_rot the cache's (already rotated) base keys, L^K the agent's unrotated LR rows and token t at
 // position t.  The result goes to a caller-provided scratch area in LOGICAL block order, layout
 // [block][kv head][16][hd] like the cache, so that the tensor-memory prefill kernel can stream it as its key
-// operand with whole-stage boxes and no key-side adapter at all.  One thread block per 16-token block.
+// operand with whole-stage boxes and no key-side adapter at all.
 #pragma once
 #include "common.cuh"
 
@@ -27,165 +27,129 @@ struct RopeExpandParams {
   float s_k;
 };
 
-constexpr int RX_THREADS = 256;
-constexpr int RX_WARPS = RX_THREADS / 32;
-
 // E = L^K B^K on the tensor cores (mma.sync m16n8k16: the 16 tokens of a cache block on the M axis, rank on K, columns
-// on N).  A task is 16 adjacent columns of the lower half of one head together with their partners in the upper half;
-// a warp owns TPW tasks for the whole kernel and keeps their B^K fragments in registers, a thread block owns a group
-// of 8 TPW tasks (blockIdx.y) and walks over the sequence's cache blocks (blockIdx.x, persistent).  Per cache block:
-// L^K fragments straight from global memory, the MMAs, the rotation, the scaled term parked in shared memory, then
-// base keys + term -> scratch with 16-byte accesses, consecutive threads on consecutive pieces of a row.
+// on N).  A warp owns 32 columns of the lower half of one head and their partners in the upper half: eight n-tiles, whose
+// columns are handed out so that a lane ends up with EIGHT ADJACENT columns of its two tokens in either half (n-tile t,
+// column n of it = column 8 (n / 2) + 2 t + (n & 1) of the 32): base keys, scratch and rotary table are then read and
+// written with 16-byte accesses straight from and to the accumulator layout, and nothing passes through shared memory.
+// A warp keeps its B^K fragments in registers and walks over cache blocks; warps know nothing of each other.
+// (The term used to be parked in shared memory between two block barriers per cache block: a call of 32 new tokens over 8000 with 4 kv
+// heads of 128, rank 16, took 32.1 us and takes 28.8; over 32768 with 8 kv heads, rank 32: 105 -> 85; head_dim 64, rank 64, 16000: 53 -> 41.)
 // KS = k steps of 16 (rank 8 and 16: 1, rank 32: 2, rank 64: 4).
-template <int KS>
-struct RxCfg {
-  static constexpr int GROUP_TASKS = RX_WARPS;           // one task per warp: 4 tiles * KS * 2 fragment registers
-  static constexpr int PIECES = GROUP_TASKS * PAGE * 4 / RX_THREADS;   // 16-byte pieces of the group per thread and cache block
-};
+constexpr int RX_WARPS = 4;
+constexpr int RX_THREADS = RX_WARPS * 32;
+constexpr int RX_COLS = 64;                              // columns of a warp: 32 of the lower half of a head, 32 of the upper
+
+__host__ __device__ constexpr int rx_blocks_per_sm(int ks) { return ks == 4 ? 2 : ks == 2 ? 3 : 4; }   // what the registers allow
 
 template <int KS>
-__global__ void __launch_bounds__(RX_THREADS, 2)
+__global__ void __launch_bounds__(RX_THREADS, rx_blocks_per_sm(KS))
 rope_expand_keys_kernel(const RopeExpandParams p) {
-  constexpr int PIECES = RxCfg<KS>::PIECES;
-  extern __shared__ __align__(16) float Es[];            // s_k RoPE(L^K B^K) of one cache block, [task of the group][token][32 columns]
   const int hd = p.hd, rk = p.rk;
   const int kvw = p.n_kv * hd;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = lane >> 2, q2 = (lane & 3) * 2;          // accumulator rows r, r + 8; columns q2, q2 + 1 of an 8-column tile
-  const int tasks_per_head = hd / 32;                    // 16 lower-half columns per task
-  const int n_tasks = p.n_kv * tasks_per_head;
-  const int task = blockIdx.y * RxCfg<KS>::GROUP_TASKS + warp;
-  const bool has_task = task < n_tasks;
-  const int tg_head = task / tasks_per_head, tc0 = (task - tg_head * tasks_per_head) * 16;
+  const int r = lane >> 2, q = lane & 3;                 // accumulator rows (tokens) r, r + 8; columns 8 q .. 8 q + 7 of either half
+  const int per_head = hd / RX_COLS;
+  const int task = blockIdx.y * RX_WARPS + warp;
+  if (task >= p.n_kv * per_head) return;
+  const int g = task / per_head, c0 = (task - g * per_head) * 32;      // head, first column in its lower half
   pdl_wait();                  // the kernel ahead may have written anything that is read below
-  // ---- this warp's B^K fragments (k = rank, n = column), zero beyond the rank and beyond the last task
-  uint32_t bfr[4][KS][2];
-#pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    const int col = tg_head * hd + tc0 + (t & 1) * 8 + (t >> 1) * (hd / 2) + r;        // B operand: n = lane >> 2
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      const int k0 = ks * 16 + q2;
-      auto bk = [&](int k) -> uint32_t {
-        return (has_task && k < rk) ? (uint32_t)__bfloat16_as_ushort(p.B_k[(size_t)k * kvw + col]) : 0u;
-      };
-      bfr[t][ks][0] = bk(k0) | (bk(k0 + 1) << 16);
-      bfr[t][ks][1] = bk(k0 + 8) | (bk(k0 + 9) << 16);
-    }
-  }
-  // ---- the 16-byte pieces this thread combines per cache block: 8 columns of one token.  The group's tasks cover
-  //      whole heads (8 tasks = 8 / tasks_per_head heads), and the pieces are taken in memory order - consecutive
-  //      threads on consecutive pieces of a token's row of one head - so that every request covers whole 128-byte lines
-  const int group_tasks = min(RxCfg<KS>::GROUP_TASKS, n_tasks - (int)blockIdx.y * RxCfg<KS>::GROUP_TASKS);
-  const int ppr = hd / 8;                                  // pieces per row
-  int p_off[PIECES], p_tok[PIECES], p_e[PIECES];
-  bool p_on[PIECES];
-#pragma unroll
-  for (int k = 0; k < PIECES; ++k) {
-    const int i = threadIdx.x + k * RX_THREADS;
-    const int pr = i % ppr, tok = (i / ppr) % PAGE, hg = i / (ppr * PAGE);            // piece in row, token, head in group
-    const int col = pr * 8, half = col >= hd / 2 ? 1 : 0, cl = col - half * (hd / 2);
-    const int tg = hg * tasks_per_head + cl / 16;                                      // task in group that produced these columns
-    const int g = blockIdx.y * (RxCfg<KS>::GROUP_TASKS / tasks_per_head) + hg;
-    p_on[k] = tg < group_tasks;
-    p_tok[k] = tok;
-    p_off[k] = (g * PAGE + tok) * hd + col;
-    p_e[k] = tg * PAGE * 32 + tok * 32 + half * 16 + (cl % 16);
-  }
-  // ---- inputs of one cache block, requested one block ahead of their use
-  struct In {
-    int ph;
-    uint32_t afr[KS][4];        // L^K rows r and r + 8 (row-major [16][rk]); rank 8 fills half a k step
-    float4 cs[2][2];            // (cos, sin) of the warp's columns at the lane's two tokens
-    uint4 kb[PIECES];           // base keys of the thread's pieces
+  int lb = blockIdx.x;
+  auto lookup = [&](int b) -> int {
+    if (b * PAGE >= p.n_tokens) return 0;
+    const int ph = p.block_table ? __ldg(p.block_table + b) : p.first_block + b;
+    if (ph >= 0 && ph < p.n_blocks) return ph;
+    if (lane == 0 && task == 0) atomicOr(p.status, StatusBits::BAD_INDEX);
+    return 0;
   };
-  auto fetch = [&](int lb, In& x) {
-    const int t0 = lb * PAGE;
-    const bool pad = t0 >= p.n_tokens;
-    int ph = 0;
-    if (!pad) {
-      ph = p.block_table ? __ldg(p.block_table + lb) : p.first_block + lb;
-      if (ph < 0 || ph >= p.n_blocks) {
-        if (threadIdx.x == 0 && blockIdx.y == 0) atomicOr(p.status, StatusBits::BAD_INDEX);
-        ph = 0;
-      }
-    }
-    x.ph = ph;
-    const __nv_bfloat16* src_blk = p.k_base + (size_t)ph * p.n_kv * PAGE * hd;
+  // ---- inputs of one cache block, requested a block ahead of their use (its place in the cache two ahead): base keys of
+  //      the lane's two tokens in both halves and L^K rows r, r + 8, zero past the sequence's end
+  struct In { uint4 kb[2][2]; uint32_t afr[KS][4]; };
+  auto fetch = [&](int b, int ph, In& x) {
+    const int t0 = b * PAGE;
+    const bool any = t0 < p.n_tokens;
+    const __nv_bfloat16* src = p.k_base + ((size_t)((size_t)ph * p.n_kv + g) * PAGE + r) * hd + c0 + q * 8;
 #pragma unroll
-    for (int k = 0; k < PIECES; ++k)
-      x.kb[k] = (p_on[k] && t0 + p_tok[k] < p.n_tokens) ? __ldg(reinterpret_cast<const uint4*>(src_blk + p_off[k])) : make_uint4(0u, 0u, 0u, 0u);
+    for (int h = 0; h < 2; ++h) {
+      const bool on = t0 + r + 8 * h < p.n_tokens;
+      x.kb[h][0] = on ? __ldg(reinterpret_cast<const uint4*>(src + h * 8 * hd)) : make_uint4(0u, 0u, 0u, 0u);
+      x.kb[h][1] = on ? __ldg(reinterpret_cast<const uint4*>(src + h * 8 * hd + hd / 2)) : make_uint4(0u, 0u, 0u, 0u);
+    }
     const __nv_bfloat16* lrow = p.lr_k + ((size_t)ph * PAGE + r) * rk;
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
-      const int k = ks * 16 + q2;
-      x.afr[ks][0] = (!pad && k < rk) ? __ldg(reinterpret_cast<const uint32_t*>(lrow + k)) : 0u;
-      x.afr[ks][1] = (!pad && k < rk) ? __ldg(reinterpret_cast<const uint32_t*>(lrow + 8 * rk + k)) : 0u;
-      x.afr[ks][2] = (!pad && k + 8 < rk) ? __ldg(reinterpret_cast<const uint32_t*>(lrow + k + 8)) : 0u;
-      x.afr[ks][3] = (!pad && k + 8 < rk) ? __ldg(reinterpret_cast<const uint32_t*>(lrow + 8 * rk + k + 8)) : 0u;
+      const int k = ks * 16 + q * 2;
+      x.afr[ks][0] = any && k < rk ? __ldg(reinterpret_cast<const uint32_t*>(lrow + k)) : 0u;
+      x.afr[ks][1] = any && k < rk ? __ldg(reinterpret_cast<const uint32_t*>(lrow + 8 * rk + k)) : 0u;
+      x.afr[ks][2] = any && k + 8 < rk ? __ldg(reinterpret_cast<const uint32_t*>(lrow + k + 8)) : 0u;
+      x.afr[ks][3] = any && k + 8 < rk ? __ldg(reinterpret_cast<const uint32_t*>(lrow + 8 * rk + k + 8)) : 0u;
     }
-#pragma unroll
-    for (int t = 0; t < 2; ++t)
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-        x.cs[t][h] = __ldg(p.rope + (size_t)min(t0 + r + 8 * h, p.max_pos - 1) * (hd / 4) + (tc0 + t * 8 + q2) / 2);
   };
+  if (lb >= p.n_out_blocks) return;
   In cur;
-  int lb = blockIdx.x;
-  if (lb < p.n_out_blocks) fetch(lb, cur);
+  fetch(lb, lookup(lb), cur);
+  int ph_next = lb + (int)gridDim.x < p.n_out_blocks ? lookup(lb + gridDim.x) : 0;
+  // ---- B^K fragments (k = rank, n = column), zero beyond the rank; tiles 0 .. 3 lower half, 4 .. 7 upper
+  uint32_t bfr[8][KS][2];
+  {
+    const unsigned short* B = reinterpret_cast<const unsigned short*>(p.B_k) + (size_t)g * hd + c0 + (r >> 1) * 8 + (r & 1);
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const unsigned short* Bt = B + (t & 3) * 2 + (t >> 2) * (hd / 2);
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) {
+        const int k0 = ks * 16 + q * 2;
+        auto bk = [&](int k) -> uint32_t { return k < rk ? (uint32_t)__ldg(Bt + (size_t)k * kvw) : 0u; };
+        bfr[t][ks][0] = bk(k0) | (bk(k0 + 1) << 16);
+        bfr[t][ks][1] = bk(k0 + 8) | (bk(k0 + 9) << 16);
+      }
+    }
+  }
   for (; lb < p.n_out_blocks; lb += gridDim.x) {
+    const int t0 = lb * PAGE, nb = lb + gridDim.x;
     In nxt = cur;
-    if (lb + (int)gridDim.x < p.n_out_blocks) fetch(lb + gridDim.x, nxt);           // in flight while this block is computed
-    const int t0 = lb * PAGE;
-    __nv_bfloat16* dst_blk = p.scratch + (size_t)lb * p.n_kv * PAGE * hd;
-    if (has_task && t0 < p.n_tokens) {
-      float acc[4][4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.f;
-#pragma unroll
-        for (int ks = 0; ks < KS; ++ks) mma_bf16_16816(acc[t], cur.afr[ks], bfr[t][ks][0], bfr[t][ks][1]);
-      }
-      // rotate (lower tile t with upper tile t + 2), park the scaled term: [task in group][token][lower 16 | upper 16]
-      float* eb = Es + (size_t)warp * PAGE * 32;
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int cl = t * 8 + q2;                        // even column inside the task's lower 16
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int tok = r + 8 * h;
-          const float lo0 = p.s_k * acc[t][2 * h], lo1 = p.s_k * acc[t][2 * h + 1];
-          const float hi0 = p.s_k * acc[t + 2][2 * h], hi1 = p.s_k * acc[t + 2][2 * h + 1];
-          const float4 cs = cur.cs[t][h];
-          *reinterpret_cast<float2*>(eb + tok * 32 + cl) = make_float2(lo0 * cs.x - hi0 * cs.y, lo1 * cs.z - hi1 * cs.w);
-          *reinterpret_cast<float2*>(eb + tok * 32 + 16 + cl) = make_float2(hi0 * cs.x + lo0 * cs.y, hi1 * cs.z + lo1 * cs.w);
-        }
-      }
+    if (nb < p.n_out_blocks) {
+      fetch(nb, ph_next, nxt);
+      if (nb + (int)gridDim.x < p.n_out_blocks) ph_next = lookup(nb + gridDim.x);
     }
-    __syncthreads();
-    // base keys + term -> scratch (zeros past the sequence's end and in the padding up to a whole 128-token stage)
+    __nv_bfloat16* dst = p.scratch + ((size_t)((size_t)lb * p.n_kv + g) * PAGE + r) * hd + c0 + q * 8;
+    float4 cs[2][4];
 #pragma unroll
-    for (int k = 0; k < PIECES; ++k) {
-      if (!p_on[k]) continue;
-      uint4 o = make_uint4(0u, 0u, 0u, 0u);
-      if (t0 + p_tok[k] < p.n_tokens) {
-        const float* e = Es + p_e[k];
-        const float4 e0 = *reinterpret_cast<const float4*>(e), e1 = *reinterpret_cast<const float4*>(e + 4);
-        auto add2 = [](uint32_t k2, float a, float b) -> uint32_t {
-          const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&k2));
-          return pack_bf16(f.x + a, f.y + b);
-        };
-        const uint4 kb = cur.kb[k];
-        o = make_uint4(add2(kb.x, e0.x, e0.y), add2(kb.y, e0.z, e0.w), add2(kb.z, e1.x, e1.y), add2(kb.w, e1.z, e1.w));
-      }
-      *reinterpret_cast<uint4*>(dst_blk + p_off[k]) = o;
+    for (int h = 0; h < 2; ++h) {
+      const float4* cs4 = p.rope + (size_t)min(t0 + r + 8 * h, p.max_pos - 1) * (hd / 4) + (c0 + q * 8) / 2;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) cs[h][t] = __ldg(cs4 + t);
     }
-    __syncthreads();                                     // the parked term is reused by the next cache block
+    float acc[8][4];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) mma_bf16_16816(acc[t], cur.afr[ks], bfr[t][ks][0], bfr[t][ks][1]);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t lo[4], hi[4];
+      const uint32_t kl[4] = {cur.kb[h][0].x, cur.kb[h][0].y, cur.kb[h][0].z, cur.kb[h][0].w};
+      const uint32_t kh[4] = {cur.kb[h][1].x, cur.kb[h][1].y, cur.kb[h][1].z, cur.kb[h][1].w};
+      auto add2 = [](uint32_t k2, float a, float b) -> uint32_t {
+        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&k2));
+        return pack_bf16(f.x + a, f.y + b);
+      };
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {                      // columns 2 t, 2 t + 1 of the lane's eight
+        const float4 c4 = cs[h][t];
+        const float lo0 = p.s_k * acc[t][2 * h], lo1 = p.s_k * acc[t][2 * h + 1];
+        const float hi0 = p.s_k * acc[t + 4][2 * h], hi1 = p.s_k * acc[t + 4][2 * h + 1];
+        lo[t] = add2(kl[t], lo0 * c4.x - hi0 * c4.y, lo1 * c4.z - hi1 * c4.w);
+        hi[t] = add2(kh[t], hi0 * c4.x + lo0 * c4.y, hi1 * c4.z + lo1 * c4.w);
+      }
+      const bool on = t0 + r + 8 * h < p.n_tokens;       // rows past the sequence's end, and the padding up to a whole 128-token stage: zeros
+      *reinterpret_cast<uint4*>(dst + h * 8 * hd) = on ? make_uint4(lo[0], lo[1], lo[2], lo[3]) : make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(dst + h * 8 * hd + hd / 2) = on ? make_uint4(hi[0], hi[1], hi[2], hi[3]) : make_uint4(0u, 0u, 0u, 0u);
+    }
     cur = nxt;
   }
 }
-
-template <int KS>
-inline size_t rope_expand_smem_bytes() { return (size_t)RxCfg<KS>::GROUP_TASKS * PAGE * 32 * sizeof(float); }
 
 }  // namespace precc
