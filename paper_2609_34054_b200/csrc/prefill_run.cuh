@@ -131,14 +131,16 @@ struct PrefillRun {
     p.n_q = d->n_q_heads; p.n_kv = d->n_kv_heads; p.group = G; p.tok_per_tile = PTC_TOK / G; p.k_stages = ks; p.v_stages = vs; p.v_half = v_half ? 1 : 0;
     p.scale_log2 = softmax_scale_log2(d); p.s_k = d->lora_scale_k; p.s_v = d->lora_scale_v;
     p.trace = (ctx->trace && ctx->trace_blocks >= 32) ? ctx->trace : nullptr;
-    // four instantiations at most: classic / work list, whole-step / half-step value ring (the latter only where it applies)
+    // the classic form, the split context and the work list, each with whole-step or (where that applies) half-step value stages
     using KernT = void (*)(PrefillTcMaps, PrefillTcParams);
     KernT kern = lr_attend_prefill_tc_kernel<HD, RK, RV, false, false>;
-    KernT kern_wl = lr_attend_prefill_tc_kernel<HD, RK, RV, true, false>;
+    KernT kern_sp = lr_attend_prefill_tc_kernel<HD, RK, RV, false, false, true>;
+    KernT kern_wl = lr_attend_prefill_tc_kernel<HD, RK, RV, true, C::V_HALF_CAPABLE>;
     if constexpr (C::V_HALF_CAPABLE) {
-      if (v_half) { kern = lr_attend_prefill_tc_kernel<HD, RK, RV, false, true>; kern_wl = lr_attend_prefill_tc_kernel<HD, RK, RV, true, true>; }
+      if (v_half) { kern = lr_attend_prefill_tc_kernel<HD, RK, RV, false, true>; kern_sp = lr_attend_prefill_tc_kernel<HD, RK, RV, false, true, true>; }
     }
     PRECC_CUDA(ctx, raise_smem_limit(ctx, kern, smem));
+    PRECC_CUDA(ctx, raise_smem_limit(ctx, kern_sp, smem));
     const int row_tiles = (a.S + p.tok_per_tile - 1) / p.tok_per_tile;
     // Short turn over a long context: too few (row tile, kv head) blocks to fill the machine, so the
     // context of each is split over a cluster of up to 8 blocks whose partial results merge over DSMEM.
@@ -164,7 +166,7 @@ struct PrefillRun {
           qa[0].val.clusterDim.x = 1; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = ns;
           qc.attrs = qa; qc.numAttrs = 1;
           int n = 0;
-          if (cudaOccupancyMaxActiveClusters(&n, kern, &qc) != cudaSuccess) { cudaGetLastError(); n = 0; }
+          if (cudaOccupancyMaxActiveClusters(&n, kern_sp, &qc) != cudaSuccess) { cudaGetLastError(); n = 0; }
           max_clusters[ns] = n + 1;
         }
         if (max_clusters[ns] - 1 >= base_blocks) break;
@@ -179,7 +181,7 @@ struct PrefillRun {
 #else
     const bool wl_ok = !p.trace;
 #endif
-    if (a.ws && ns == 1 && wl_ok) {
+    if (a.ws && ns == 1 && wl_ok && v_half == C::V_HALF_CAPABLE) {     // (the diagnostic whole-step ring has no work-list form there)
       const WorkList wl = plan_worklist(ctx, a.S, a.T, p.tok_per_tile, d->n_kv_heads);
       if (wl.p > 0 && a.ws_bytes >= worklist_ws_bytes(wl.tiles, wl.helpers)) {
         p.helper_p = wl.p; p.n_helpers = wl.helpers; p.longest_first = 0;
@@ -204,7 +206,7 @@ struct PrefillRun {
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = ns;
     cfg.attrs = attr; cfg.numAttrs = ns > 1 ? 2 : 1;
-    PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, m, p));
+    PRECC_CUDA(ctx, cudaLaunchKernelEx(&cfg, ns > 1 ? kern_sp : kern, m, p));
     return PRECC_OK;
   }
   // whether the tensor-memory kernel takes this call (shape, cache size, alignment, diagnostic switch)

@@ -26,12 +26,16 @@
 // what the warpgroups hand to each other is the row's reference maximum, one word through shared memory behind a
 // named barrier per warp pair, decided right after a step's scores are in registers.  The reference is raised
 // only when the maximum grows by more than 8 (log2 domain), so O' is rescaled a handful of times per row instead of
-// at every step; P stays below 2^8.  The denominator is summed in fp32 by the softmax threads, two values per instruction,
-// for 0 < r_v < 64 from the rounded weights that the MMA sees (8192 over 24576: 4005 -> 4294 us; unrounded, the sum left a
+// at every step; P stays below 2^8.  The denominator: for 0 < r_v < 64 the rounded weights that the MMA sees are summed, by the
+// MMA: behind each k step of P V' a second one of N = 16 multiplies the same P with a constant tile of ones (512 bytes of
+// shared memory, sixteen equal columns behind O').  The softmax threads are left with four instructions per pair of
+// scores instead of seven (8192 over 24576: 4147 -> 3895 us; 512 over 32768 with both projections: 316 -> 297).  Otherwise, and in the
+// work-list form (which would spill), they sum in fp32, two values per instruction.  (Unrounded, the sum left a
 // row dominated by one token up to 2^-8 off, on top of its own rounding, and the error against float64 5 .. 15 % higher
-// where a few tokens carry a row).  Measured for the same sum and slower: a column of ones beside L_V for the P V' MMA to
-// sum - written into every landed value stage by the issuing warp it takes 600 cycles of a step, by the softmax threads 6 %
-// more time on the mean - and a warp-level mma.sync against a selection matrix, which competes with tcgen05 (5039 us).
+// where a few tokens carry a row.)  Measured for the same sum and slower: a column of ones beside L_V in the value stage -
+// written into every landed stage by the issuing warp it takes 600 cycles of a step, by the softmax threads 6 % more time on
+// the mean -, the ones behind all eight k steps instead of between them (330 against 272 us), a warp-level mma.sync
+// against a selection matrix, which competes with tcgen05, and adds of fp32 and bf16 (turn of 512: 6 % slower).
 //
 // Warp roles: warp 0 = TMA producer of the key ring, warp 3 = TMA producer of the value ring
 // (keys are released right after S is computed, values only after O' is updated, so the two rings run
@@ -113,9 +117,10 @@ constexpr int PTC_THREADS = (PTC_FIRST_HELPER + 4) * 32;
 constexpr int PTC_SM_REGS = 216, PTC_CTL_REGS = 40;  // 256 x 216 + 256 x 40 = 512 x 128, the launch's registers
 constexpr int PTC_SMEM_LIMIT = 232448;   // dynamic shared memory a block can opt into on this architecture
 constexpr int PTC_FIXED_BARS = 13; // barriers besides the two per ring stage
-constexpr int PTC_XCH_BYTES = 4 * 512;   // [2][128] reference maxima | [2][128] partial denominators
+constexpr int PTC_XCH_BYTES = 4 * 512;   // [2][128] reference maxima | [2][128] partial denominators or the tile of ones
 constexpr int PTC_TOK = 128;      // tokens per step
 constexpr float PTC_RAISE = 8.f;  // the running maximum is raised only when it grows by more than this
+constexpr int PTC_MAX_SPLIT = 8;  // blocks of a split-context cluster at most
 constexpr int PTC_MAX_SRC = 8;    // work-list launch: pieces of one tile (its own block + helper pieces) at most
 constexpr int PTC_MAX_SEG = 16;   // work-list launch: tile pieces one helper block takes at most
 constexpr int PTC_MAX_XT = 160;   // work-list launch: row tiles at most
@@ -136,20 +141,23 @@ struct PrefillTcCfg {
   static constexpr int RVP = RV == 8 ? 16 : RV;               // value-side coordinates as the MMAs see them (rank 8: zero-padded)
   static constexpr int OW = HD + RVP;                         // columns of O' in TMEM: [O | U]
   // The denominator is the sum of the bf16 weights that the P V' MMA multiplies, so that the rounding of a dominant weight
-  // cancels; with no value adapter or rank 64 it is the sum of the unrounded ones (the accuracy these always had).
+  // cancels; with no value adapter or rank 64 (no tensor memory left beside O') it is the sum of the unrounded ones.
   static constexpr bool L_ROUNDED = RV > 0 && RV < 64;
+  static constexpr int OWL = OW + (L_ROUNDED ? 16 : 0);       // and, where the MMA sums the denominator, sixteen copies of it
   static constexpr int VSTAGE = VSLABS * SLAB_BYTES;          // {V_base slabs | L_V slab}
   static constexpr int K_PAGE_TX = PAGE * (HD + RKP) * 2;      // bytes one page contributes to a key stage
   static constexpr int V_PAGE_TX = PAGE * VSLABS * 128;
   static constexpr int UPW = RVP / 2;                         // TMEM columns of one bf16 term of s_v U
   static constexpr int BV_BYTES = RVP * HD * 2;               // the B_v slice, one more item of the key ring behind the last step
   static constexpr int SPLIT_XS = HD + 4;                     // row stride (floats) of a partial: the adapter term is added before partials are merged
-  // split-context merge area (laid over the Q tile, the folded-query tile and the rings): partial | m | l | weights | 1/l
-  static constexpr int SPLIT_BYTES = (128 * SPLIT_XS + 256 + 16 * 64 + 64) * 4;
+  // split-context merge area (laid over the Q tile, the folded-query tile and the rings): partial rows [O | m | l | - | -], then
+  // the peers' partials of the rows this block finishes (at most 6 x 19 rows, clusters of seven)
+  static constexpr int SPLIT_BYTES = (128 + 114) * SPLIT_XS * 4;
   static constexpr int REC_FLOATS = 128 * SPLIT_XS + 256;     // a tile's partial in global memory: O rows | m[128] | l[128]
   static constexpr int PB = OW <= 128 ? 2 : 1;                // P buffers
   static constexpr int TMEM_P = 2 * PTC_TOK;                  // packed bf16 P (64 columns each) after the two S buffers
   static constexpr int TMEM_O = TMEM_P + PB * (PTC_TOK / 2);  // O': at most 320 + 192 or 384 + 128 = 512
+  static_assert(TMEM_O + OWL <= 512, "tensor memory");
   __host__ __device__ static constexpr int smem_bytes(int ks, int vs, bool v_half = false) { return Q_BYTES + QX_BYTES + ks * KSTAGE + vs * (v_half ? VSTAGE / 2 : VSTAGE) + 320 + PTC_XCH_BYTES + PTC_TAB_BYTES + 1024; }
   // one whole value stage fits beside two key stages, two do not, three half-step units do (head_dim 128 with rank 64)
   static constexpr bool V_HALF_CAPABLE = smem_bytes(2, 2) > PTC_SMEM_LIMIT && smem_bytes(2, 1) <= PTC_SMEM_LIMIT && smem_bytes(2, 3, true) <= PTC_SMEM_LIMIT;
@@ -270,10 +278,15 @@ __device__ __forceinline__ bool elect_one() {
 // the classic launch carries none of its state through the step loop.
 // VH: the value ring holds units of 64 tokens (half a step) - instantiated only where shared memory has room for
 // one whole value stage but not for two.
-template <int HD, int RK, int RV, bool WL = false, bool VH = false>
+// SP: the split-context form (clusters of NS blocks, see below).  The merge has an instantiation of its own: compiled into the
+// classic form, which never takes it, it costs the step loop 6 .. 12 % through ptxas' schedule alone.
+template <int HD, int RK, int RV, bool WL = false, bool VH = false, bool SP = false>
 __global__ void __launch_bounds__(PTC_THREADS, 1)
 lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __grid_constant__ PrefillTcParams p) {
   using C = PrefillTcCfg<HD, RK, RV>;
+  // The MMA sums the denominator.  Not in the work-list form, which would spill, nor in the split-context form at head_dim 128
+  // without a key adapter (200 over 8000: 43.7 us against 40.4; 40 over 24000: 44.0 against 40.4; with one, 64 over 16384: 33.0 against 36.4).
+  constexpr bool L_MMA = C::L_ROUNDED && !WL && !(SP && RK == 0 && HD == 128);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);   // (pointer arithmetic, so that it stays a shared-memory address)
   const uint32_t q_u32 = smem_u32(smem);
@@ -290,7 +303,11 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
                  fold_done = q_full + 8, q_ready = fold_done + 8, u_full = q_ready + 8, uv_done = u_full + 8;
   const int n_bars = 2 * KS + 2 * VS + PTC_FIXED_BARS;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + n_bars);
+  const uint32_t merge_bar = bar0 + 8 * (n_bars + 1);            // SP: bytes of the peers' partials
   float* xch = reinterpret_cast<float*>(bars + n_bars + 2);      // [2][128] reference maxima (by step parity) | [2][128] partial denominators
+
+  // sixteen rows of sixteen ones, the B operand of the denominator, in the place of the partial denominators
+  uint32_t* ones = reinterpret_cast<uint32_t*>(xch + 256) + ((0u - smem_u32(xch + 256)) & 255u) / 4;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = p.group;
@@ -324,10 +341,23 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     fence_async_smem();
   };
-  if (threadIdx.x == 0) init_bars();
+  // rows of the tile that each block finishes when the context is split over a cluster
+  auto merge_share = [&](int live_rows) { return (live_rows + (int)NS - 1) / (int)NS; };
+  if (threadIdx.x == 0) {
+    if constexpr (SP) {
+      mbar_init(merge_bar, 1);
+      const int t0 = (p.longest_first ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x) * p.tok_per_tile;
+      const int live = min(p.tok_per_tile, p.S - t0) * G, R = merge_share(live);
+      mbar_expect_tx(merge_bar, (uint32_t)(((int)NS - 1) * max(0, min(R, live - (int)split * R)) * C::SPLIT_XS * 4));   // the one arrival, and the bytes to come
+    }
+    init_bars();
+  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_holder)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  if constexpr (L_MMA) {
+    if (threadIdx.x < 128) { ones[threadIdx.x] = 0x3f803f80u; fence_async_smem(); }
   }
   if constexpr (WL) {
     for (int x = threadIdx.x; x < p.row_tiles; x += blockDim.x) tab_tail[x] = max(0, steps_of(x) - p.helper_p);
@@ -629,6 +659,8 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         const uint32_t id_o = umma_idesc(C::OW, 1);
         const uint64_t vd0 = umma_desc_mnmajor(vring_u32, 128, USLAB);
         const uint32_t od = tmem_base + C::TMEM_O;
+        const uint32_t id_l = umma_idesc(16, 0);
+        const uint64_t onesd = umma_desc_kmajor(smem_u32(ones), 32);
         for (int j = 0; j < n_tiles; ++j) {
           const int n_live = min(PTC_TOK, t_end - (jb + j) * PTC_TOK);     // tokens of this step that exist
 #pragma unroll
@@ -658,10 +690,16 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
               const uint64_t so = (uint64_t)((s * vunit) >> 4);
               if (live_u == UT) {
 #pragma unroll
-                for (int ks = 0; ks < UT / 16; ++ks) umma_bf16_ts(od, a + ks * 8, vd0 + so + (uint64_t)(ks * 128), id_o, (j | part | ks) ? 1u : 0u);
+                for (int ks = 0; ks < UT / 16; ++ks) {
+                  umma_bf16_ts(od, a + ks * 8, vd0 + so + (uint64_t)(ks * 128), id_o, (j | part | ks) ? 1u : 0u);
+                  if constexpr (L_MMA) umma_bf16_ts(od + C::OW, a + ks * 8, onesd, id_l, (j | part | ks) ? 1u : 0u);
+                }
               } else {
                 const int n_ks = (live_u + 15) / 16;
-                for (int ks = 0; ks < n_ks; ++ks) umma_bf16_ts(od, a + ks * 8, vd0 + so + (uint64_t)(ks * 128), id_o, (j | part | ks) ? 1u : 0u);
+                for (int ks = 0; ks < n_ks; ++ks) {
+                  umma_bf16_ts(od, a + ks * 8, vd0 + so + (uint64_t)(ks * 128), id_o, (j | part | ks) ? 1u : 0u);
+                  if constexpr (L_MMA) umma_bf16_ts(od + C::OW, a + ks * 8, onesd, id_l, (j | part | ks) ? 1u : 0u);
+                }
               }
               umma_commit(v_empty + 8 * s);
               if (part == UPS - 1) umma_commit(pv_done + 8 * (j & 1));
@@ -693,7 +731,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         }
       }
       __syncwarp();
-      if (NS > 1) { cluster_barrier(); cluster_barrier(); }     // the softmax warps' merge of the context splits
+      if constexpr (SP) { cluster_barrier(); cluster_barrier(); }     // the softmax warps' merge of the context splits
       end_piece(seg);
     }
   } else {
@@ -789,7 +827,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
           mbar_wait(pv_done + 8 * (wg ^ 1), ((j - 1) >> 1) & 1, p.status);
           tc_fence_after();
 #pragma unroll 1
-          for (int c = 0; c < C::OW / 16; ++c) {
+          for (int c = 0; c < (L_MMA ? C::OWL : C::OW) / 16; ++c) {
             uint32_t ov[16];
             tmem_ld16(lane_addr + C::TMEM_O + c * 16, ov);
             tmem_wait_ld();
@@ -799,8 +837,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
           }
           tmem_wait_st();
         }
-        l_sum *= fast_exp2(m_own - m_new);
-        m_own = m_new;
+        if constexpr (!L_MMA) { l_sum *= fast_exp2(m_own - m_new); m_own = m_new; }
         float ls[4] = {0.f, 0.f, 0.f, 0.f};
         const float neg_m = -m_new;
         uint32_t pk[2][32];
@@ -812,12 +849,13 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
             fma2(p0, p1, sv[c][k], sv[c][k + 1], p.scale_log2, neg_m);
             p0 = fast_exp2(p0); p1 = fast_exp2(p1);
             const uint32_t w = pack_bf16(p0, p1);
-            if constexpr (C::L_ROUNDED) add2(ls[k & 2], ls[(k & 2) + 1], __uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+            if constexpr (L_MMA) { }                                  // (summed by the P V' issuer's second MMA)
+            else if constexpr (C::L_ROUNDED) add2(ls[k & 2], ls[(k & 2) + 1], __uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
             else if constexpr (WL) { ls[k & 2] += p0; ls[(k & 2) + 1] += p1; }      // (packed, ptxas spills here)
             else add2(ls[k & 2], ls[(k & 2) + 1], p0, p1);
             pk[c >> 1][(c & 1) * 16 + k / 2] = w;
           }
-        l_sum += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        if constexpr (!L_MMA) l_sum += (ls[0] + ls[1]) + (ls[2] + ls[3]);
         if ((tid & 127) == 0) PTC_STAMP(p, j, 14);                 // all exponentials done
         // the P buffer may be overwritten once the P V' that read it last has retired
         if (j >= C::PB) {
@@ -848,10 +886,22 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         mbar_wait(pv_done + 8 * ((n_tiles - 1) & 1), ((n_tiles - 1) >> 1) & 1, p.status);
         tc_fence_after();
       }
-      lpart[wg * 128 + row] = l_sum * fast_exp2(m_own - m_fin);
-      named_sync(1, NSM);
+      if constexpr (!L_MMA) {
+        lpart[wg * 128 + row] = l_sum * fast_exp2(m_own - m_fin);
+        named_sync(1, NSM);
+      }
       if constexpr (WL) load_piece(seg);                           // read again rather than held in registers through the steps
-      const float l_tot = lpart[row] + lpart[128 + row];
+      float l_tot = 0.f;
+      if constexpr (L_MMA) {
+        if (n_tiles > 0) {
+          uint32_t lv;
+          asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n" : "=r"(lv) : "r"(lane_addr + C::TMEM_O + C::OW));
+          tmem_wait_ld();
+          l_tot = __uint_as_float(lv);
+        }
+      } else {
+        l_tot = lpart[row] + lpart[128 + row];
+      }
       if constexpr (RV > 0) {
         if (n_tiles > 0) {
           // s_v U as three bf16 terms (exact to fp32's 24 bits), packed A operand in the idle S columns
@@ -884,15 +934,17 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
       }
       PTC_WL_STAMP(p, seg, 3);                                     // numerator complete
       constexpr int XS = C::SPLIT_XS;
-      if (NS > 1) {
-        // ---- split context: the partials (m, l, O) of the cluster's blocks meet over distributed shared memory; block
-        //      `split` finishes rows [split*R, (split+1)*R) of the tile
-        const int R = (128 + (int)NS - 1) / (int)NS;      // rows per block (the last block may own fewer); 2 <= NS <= 16
-        float* xo = reinterpret_cast<float*>(smem);        // the merge area starts at the Q tile: every MMA has completed
-        float* xm = xo + 128 * XS;
-        float* xl = xm + 128;
-        float* wts = xl + 128;                             // [NS][R] weights of the splits
-        float* linv = wts + 16 * 64;                       // [R]
+      if constexpr (SP) {
+        // ---- split context: block `split` of the cluster finishes rows [split R, split R + nrows) of the tile.  A block lays its
+        //      partial out by rows (O, then m and l in the padding), so that what another block finishes is one run of
+        //      memory: one bulk copy per peer into that block's receive area, counted on its merge barrier.  (Pulled with 16-byte
+        //      loads over distributed shared memory, 64 new tokens over 16384 spent 8.9 us from here to the end, now 5.2.)
+        const int live = n_tok * G, R = merge_share(live);
+        const int nrows = max(0, min(R, live - (int)split * R));
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");   // this block's rings are idle: peers may send over them
+        float* xo = reinterpret_cast<float*>(smem);               // the merge area starts at the Q tile: every MMA has completed
+        float* recv = xo + 128 * XS;                              // [NS - 1][R][XS], slot = sender's rank with the own rank left out
 #pragma unroll 1
         for (int c = wg; c < HD / 16; c += 2) {
           uint32_t ov[16];
@@ -907,55 +959,43 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
           for (int k = 0; k < 16; k += 4)
             *reinterpret_cast<uint4*>(xo + row * XS + c * 16 + k) = make_uint4(ov[k], ov[k + 1], ov[k + 2], ov[k + 3]);
         }
-        if (wg == 0) { xm[row] = m_fin; xl[row] = l_tot; }
+        if (wg == 0) *reinterpret_cast<float2*>(xo + row * XS + HD) = make_float2(m_fin, l_tot);
+        fence_async_smem();                                       // the copy engine reads what these threads wrote
         __syncwarp();
-        cluster_barrier();
-        const int r0 = (int)split * R;
-        const int nrows = max(0, min(R, 128 - r0));
-        auto peer = [&](const float* local, uint32_t s) -> uint32_t { return dsmem_addr(smem_u32(local), s); };
-        auto ld1 = [&](uint32_t a) -> float { float v; asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(a)); return v; };
-        if (tid < nrows) {
-          float ms[16], M = NEG_BIG, L = 0.f;
-#pragma unroll
-          for (uint32_t s2 = 0; s2 < 16; ++s2) { ms[s2] = s2 < NS ? ld1(peer(xm + r0 + tid, s2)) : NEG_BIG; M = fmaxf(M, ms[s2]); }
-#pragma unroll
-          for (uint32_t s2 = 0; s2 < 16; ++s2) {
-            if (s2 < NS) {
-              const float wv = fast_exp2(ms[s2] - M);
-              wts[s2 * R + tid] = wv;
-              L += wv * ld1(peer(xl + r0 + tid, s2));             // split order: deterministic
-            }
-          }
-          linv[tid] = L > 0.f ? 1.f / L : 0.f;
-        }
+        asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
         named_sync(1, NSM);
+        if (tid < (int)NS && tid != (int)split) {
+          const int n = max(0, min(R, live - tid * R));
+          const uint32_t dst = dsmem_addr(smem_u32(recv) + (uint32_t)(((int)split < tid ? (int)split : (int)split - 1) * R * XS * 4), tid);
+          if (n > 0)
+            asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                         ::"r"(dst), "r"(smem_u32(xo + tid * R * XS)), "r"(n * XS * 4), "r"(dsmem_addr(merge_bar, tid)) : "memory");
+        }
+        __syncwarp();
+        mbar_wait_cluster(merge_bar, 0, p.status);
+        __syncwarp();
+        // everything addressed to this block has arrived; a peer whose copies still read its shared memory waits for this
+        asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
         for (int it = tid; it < nrows * (HD / 8); it += NSM) {    // eight columns per item
           const int rl = it / (HD / 8), c8 = (it % (HD / 8)) * 8;
-          const int rowg = r0 + rl;
-          if (rowg >= n_tok * G) continue;
+          const int rowg = (int)split * R + rl;
+          auto src = [&](int s2) -> const float* { return s2 == (int)split ? xo + rowg * XS : recv + ((s2 < (int)split ? s2 : s2 - 1) * R + rl) * XS; };
+          float wt[PTC_MAX_SPLIT], M = NEG_BIG, L = 0.f;
+#pragma unroll
+          for (int s2 = 0; s2 < PTC_MAX_SPLIT; ++s2) { wt[s2] = s2 < (int)NS ? src(s2)[HD] : NEG_BIG; M = fmaxf(M, wt[s2]); }
           float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-          for (uint32_t s0 = 0; s0 < NS; s0 += 4) {               // eight loads in flight
-            float4 x[4][2];
 #pragma unroll
-            for (uint32_t q = 0; q < 4; ++q)
-              if (s0 + q < NS) {
-                const uint32_t a = peer(xo + rowg * XS + c8, s0 + q);
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n"
-                               : "=f"(x[q][h].x), "=f"(x[q][h].y), "=f"(x[q][h].z), "=f"(x[q][h].w) : "r"(a + h * 16));
-              }
-#pragma unroll
-            for (uint32_t q = 0; q < 4; ++q)
-              if (s0 + q < NS) {
-                const float wv = wts[(s0 + q) * R + rl];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                  o[4 * h] += wv * x[q][h].x; o[4 * h + 1] += wv * x[q][h].y; o[4 * h + 2] += wv * x[q][h].z; o[4 * h + 3] += wv * x[q][h].w;
-                }
-              }
+          for (int s2 = 0; s2 < PTC_MAX_SPLIT; ++s2) {            // split order: deterministic
+            if (s2 < (int)NS) {
+              const float* x = src(s2);
+              const float4 a = *reinterpret_cast<const float4*>(x + c8), b = *reinterpret_cast<const float4*>(x + c8 + 4);
+              const float wv = fast_exp2(wt[s2] - M);
+              L += wv * x[HD + 1];
+              o[0] += wv * a.x; o[1] += wv * a.y; o[2] += wv * a.z; o[3] += wv * a.w;
+              o[4] += wv * b.x; o[5] += wv * b.y; o[6] += wv * b.z; o[7] += wv * b.w;
+            }
           }
-          const float inv = linv[rl];
+          const float inv = L > 0.f ? 1.f / L : 0.f;
           const int i_out = tok0 + rowg / G, h_out = rowg % G;
           uint4 w;
           w.x = pack_bf16(o[0] * inv, o[1] * inv); w.y = pack_bf16(o[2] * inv, o[3] * inv);
@@ -963,7 +1003,7 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
           *reinterpret_cast<uint4*>(p.out + ((size_t)i_out * p.n_q + (size_t)g * G + h_out) * HD + c8) = w;
         }
         __syncwarp();
-        cluster_barrier();                                        // nobody leaves while a peer may still read its partial
+        asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
       } else if (WL && to_ws) {
         // ---- work-list launch: this piece's partial (m, l, O) goes to its record in global memory; the block that
         //      arrives last at the tile's ticket merges the tile's records in a fixed order and writes the output

@@ -949,6 +949,43 @@ def test_many_rows_few_columns_equal_the_tiled_kernel_bitwise(monkeypatch, px, M
     px2.close()
 
 
+@pytest.mark.parametrize("ns,hd,n_kv,G,r,S", [(2, 128, 2, 4, 32, 16), (3, 64, 3, 3, 16, 5), (4, 128, 1, 7, 8, 37), (5, 64, 2, 8, 32, 33),
+                                               (6, 128, 2, 4, 64, 3), (7, 64, 1, 5, 64, 26), (8, 128, 1, 1, 0, 2)])
+def test_split_context_merge_at_every_cluster_size(px, ns, hd, n_kv, G, r, S):
+    """A short turn over 8 ns 128-token steps and one more: clusters of ns blocks, whose partial rows are sent to the blocks that
+    finish them - fewer rows than blocks, query groups that leave rows of the tile unused, several row tiles with a ragged last one,
+    every rank of the denominator's two forms.  A late token that carries some rows.  Against the oracle, twice for determinism."""
+    from paper_2609_34054_b200.binding import Cache, layer_desc
+    geo = I.Geometry(1024, G * n_kv, n_kv, hd, 2, r, r, alpha=2.0 * max(r, 1))
+    T = ns * 8 * 128 + 70
+    nb = (T + S + 15) // 16
+    c = I.direct_caches(nb, geo, 59, f"spl.{ns}")
+    w = I.layer_weights(geo, 59, "spl")
+    q = I.queries(S, geo, 59, "spl.q", gain=3.0)
+    for g in range(n_kv):                                # the token in front of the turn answers every second query strongly
+        c["k_base"][(T - 1) // 16, g, (T - 1) % 16] = 0.5 * q[S // 2, g * G]
+    cache = Cache.from_tensors(geo, c["k_base"].cuda(), c["v_base"].cuda(), c["lr_k"].cuda() if r else None, c["lr_v"].cuda() if r else None)
+    desc = layer_desc(geo)
+    outs = []
+    for _ in range(2):
+        out = torch.full(q.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+        px.lr_attend_prefill(desc, q.cuda(), 1 if r else -1, T, w["B_k"].cuda() if r else None, w["B_v"].cuda() if r else None, cache, out)
+        torch.cuda.synchronize()
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1])
+    rows = lambda x: f64(x.reshape(-1, x.shape[-1]))
+    zero, none = np.zeros((1, hd)), np.zeros((nb * 16, 1))
+    for srow in {0, S // 2, S - 1}:
+        t = T + srow + 1
+        for g in range(n_kv):
+            cols = slice(g * hd, (g + 1) * hd)
+            ref = O.attend_from_caches(f64(q[srow, g * G:(g + 1) * G]), rows(c["k_base"][:, g])[:t], rows(c["v_base"][:, g])[:t],
+                                       rows(c["lr_k"][1])[:t] if r else none[:t], rows(c["lr_v"][1])[:t] if r else none[:t],
+                                       f64(w["B_k"][1][:, cols]) if r else zero, f64(w["B_v"][1][:, cols]) if r else zero,
+                                       geo.scale_k if r else 0.0, geo.scale_v if r else 0.0, 1)
+            assert_close(f64(outs[0])[srow, g * G:(g + 1) * G], ref, f"ns {ns} row {srow} head {g}")
+
+
 @pytest.mark.parametrize("ks,M,d", [(2, 100, 1024), (2, 777, 2048), (3, 384, 4096), (3, 130, 1024), (4, 512, 2048), (4, 64, 4096), (4, 1000, 1024),
                                     (5, 200, 2048), (6, 256, 4096), (7, 41, 2048), (8, 128, 1024), (8, 77, 4096)])
 def test_split_k_merge_by_sends_equals_the_pulling_merge_bitwise(monkeypatch, ks, M, d):
