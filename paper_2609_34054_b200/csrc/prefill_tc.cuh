@@ -284,9 +284,10 @@ template <int HD, int RK, int RV, bool WL = false, bool VH = false, bool SP = fa
 __global__ void __launch_bounds__(PTC_THREADS, 1)
 lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __grid_constant__ PrefillTcParams p) {
   using C = PrefillTcCfg<HD, RK, RV>;
-  // The MMA sums the denominator.  Not in the work-list form, which would spill, nor in the split-context form at head_dim 128
-  // without a key adapter (200 over 8000: 43.7 us against 40.4; 40 over 24000: 44.0 against 40.4; with one, 64 over 16384: 33.0 against 36.4).
-  constexpr bool L_MMA = C::L_ROUNDED && !WL && !(SP && RK == 0 && HD == 128);
+  // The MMA sums the denominator.  Not in the work-list form, which would spill.  In the split-context form at head_dim 128 only
+  // at rank 32 (64 over 16384: 33.0 us against 36.3, 30 over 60000: 69.3 against 74.0; paged, 64 over 32768: 58.9 against 56.5), not below
+  // (rank 16, 99 over 65427: 125 us against 113; rank 8, 64 over 32768: 57.5 against 55.3; no key adapter, 200 over 8000: 43.7 against 40.4).
+  constexpr bool L_MMA = C::L_ROUNDED && !WL && !(SP && HD == 128 && RK != 32);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);   // (pointer arithmetic, so that it stays a shared-memory address)
   const uint32_t q_u32 = smem_u32(smem);
