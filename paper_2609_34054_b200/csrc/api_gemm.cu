@@ -51,6 +51,7 @@ int32_t launch_small(precc_ctx* ctx, const void* X, int M, int K, const void* Wt
   rc = make_map_w(ctx, &map_w, Wt, n_out, K, cols);
   if (rc) return rc;
   const int groups = (n_out + cols - 1) / cols;
+  gp.by_rows = gp.rope || (M <= 4 && groups * cs > ctx->sm_count) ? 1 : 0;     // who finishes what, see proj_small.cuh
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(groups * cs);
   cfg.blockDim = dim3(PS_THREADS);

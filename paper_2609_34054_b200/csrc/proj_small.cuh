@@ -13,15 +13,19 @@
 //            the grid must be resident at once, or the launch runs in two waves;
 //   math   = mma.sync m16n8k16 (bf16 -> fp32): X rows on the M axis, a warp owns 8 (16 when M > 16)
 //            output columns; fragments come from shared memory with ldmatrix;
-//   reduce = every block finishes one slice of its group's columns.  The consumer threads SEND their accumulator
-//            pairs to the block that owns the column (st.async into the owner's shared memory, bytes counted on
-//            the owner's mbarrier); the owner waits for its byte count, adds the partials in rank order
-//            (deterministic) and scatters bf16 pieces into the paged caches.  No global scratch, no atomics, and
-//            no cluster barrier on the critical path (one, relaxed, at the start makes the mbarriers visible).
-//            Rotary keys keep the earlier form: partial tiles in shared memory, a cluster barrier, and each block
-//            reads its slice - and the partner half of a head - from its peers over distributed shared memory.
-// Rotary keys (GemmParams::rope): the reducing thread of the lower half of a head also gathers the partner
-// piece hd/2 columns further and writes both rotated; the block tile therefore holds whole heads.
+//   reduce = every block finishes a share of its group's tile: a slice of the columns, or (`by_rows`) some rows, all
+//            columns of them.  The consumer threads SEND their accumulator pairs to the block that owns them (st.async into the owner's
+//            shared memory, bytes counted on the owner's mbarrier); the owner waits for its byte count, adds the
+//            partials in rank order (deterministic) and scatters bf16 pieces into the paged caches.  No global scratch, no
+//            atomics, and no cluster barrier on the critical path (one, relaxed, at the start makes the mbarriers visible).
+// Rotary keys (GemmParams::rope) need `by_rows`: the thread of a piece of the lower half of a head also adds up the partner piece
+// hd/2 columns further, which is in the same row, and writes both rotated; the block tile holds whole heads.  (With columns
+// owned by blocks the halves of a head met through a cluster barrier and loads over distributed shared memory: 3584 -> 1280
+// columns, 1 / 16 / 40 rows 8.1 / 9.0 / 9.9 us, now 5.4 / 6.0 / 7.7.)  Without rotation shares of columns are the cheaper ones to send
+// from eight rows on (4096 -> 2304, 16 / 32 rows: 6.1 / 7.8 us against 6.6 / 9.1: a warp's pairs then go to one block instead of
+// eight).  Up to four rows, and where the grid puts more than one block on an SM, rows win: most blocks own nothing and leave
+// at once, which makes room for the kernel behind (one row 5.95 -> 5.70 us; 8 layers of a two-row step with their
+// attention 135.8 -> 129.8).  With one block per SM it does not (2048 -> 1152: 3.05 against 3.12).
 // The K split depends on K alone, so an output value does not depend on which entry point, which other
 // columns or how many other rows were in the call.
 #pragma once
@@ -67,18 +71,21 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   const uint32_t full0 = tiles + STAGES * STEP_BYTES, empty0 = full0 + 8 * STAGES;
   const uint32_t recv_bar = empty0 + 8 * STAGES;
   const uint32_t recv_u32 = full0 + 128;                // behind the barriers; never overlaid: peers send while this block computes
-  const bool push = !p.rope;                            // the same in every block of the grid
+  const bool by_rows = p.by_rows != 0;                  // the same in every block of the grid
   const int cpb = COLS / CS;                            // columns finished by one block (a power of two >= 8)
+  const int tw = (p.M + (int)CS - 1) / (int)CS;         // by rows: rows finished by one block (the last ones may own fewer, or none)
+  const int own = max(0, min(tw, p.M - (int)rank * tw));
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, PS_WARPS); }
     mbar_init(recv_bar, 1);
-    if (push) mbar_expect_tx(recv_bar, (uint32_t)(CS * p.M * cpb * 4));   // the one arrival, and the bytes to come: rows < M of every peer
+    // the one arrival, and the bytes to come: the own rows of every peer, or rows < M of the own columns
+    mbar_expect_tx(recv_bar, by_rows ? (uint32_t)((int)CS * own * COLS * 4) : (uint32_t)(CS * p.M * cpb * 4));
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   }
   __syncthreads();
-  if (push) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");   // waited for before the first send
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");   // waited for before the first send
   // The weights are not the preceding kernel's to write: the first ring fill of W boxes is requested before the wait
   // for that kernel (programmatic dependent launch), so a block that is resident early has them in shared memory
   // when its predecessor ends.  X (the previous kernel's output) and every store stay behind the wait.
@@ -138,7 +145,7 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(empty0 + 8 * slot) : "memory");
     }
   }
-  if (push) {
+  if (!by_rows) {
     // ---- merge by sends: accumulator pairs go straight from registers to the owner of their column
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");   // every peer's mbarrier is initialised (long since)
@@ -193,38 +200,36 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     }
     return;     // a block leaves once everything addressed to it has arrived; its own sends carry their data with them
   }
-  __syncthreads();                                     // all reads of the tiles are done; the region is reused
-
-  // ---- partial tile [MT*16][COLS] fp32 -> shared memory
-  float* part = reinterpret_cast<float*>(smem);
+  // ---- the same with rows: pairs go to the owner of their row, which has all columns of it
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
   if (warp < PS_WARPS) {
     const int r = lane >> 2, q = lane & 3;
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        const int col = (warp * NT + t) * 8 + 2 * q;
-        *reinterpret_cast<float2*>(part + (mt * 16 + r) * COLS + col) = make_float2(acc[mt][t][0], acc[mt][t][1]);
-        *reinterpret_cast<float2*>(part + (mt * 16 + r + 8) * COLS + col) = make_float2(acc[mt][t][2], acc[mt][t][3]);
+      for (int h = 0; h < 2; ++h) {
+        const int row = mt * 16 + 8 * h + r;
+        if (row >= p.M) continue;
+        const int owner = row / tw;
+        const uint32_t bar = dsmem_addr(recv_bar, owner);
+        const uint32_t dst = dsmem_addr(recv_u32 + (uint32_t)((((int)rank * tw + row - owner * tw) * COLS + warp * NT * 8 + 2 * q) * 4), owner);
+#pragma unroll
+        for (int t = 0; t < NT; ++t) st_async_f32x2(dst + t * 32, acc[mt][t][2 * h], acc[mt][t][2 * h + 1], bar);
       }
   }
-  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-
-  // ---- this block finishes columns [rank*COLS/CS, (rank+1)*COLS/CS) of its group: 8-column pieces,
-  //      all peers' values requested at once, added in rank order
-  const int pieces_per_row = COLS / 8 / CS;             // CS in {1,2,4,8}
-  const uint32_t part_u32 = smem_u32(part);
-  // eight columns [col, col+8) of one row, summed over the cluster's partial tiles
-  auto gather = [&](int row, int col, float (&v8)[8]) {
+  constexpr int PPR = COLS / 8;
+  const int n_items = own * PPR;
+  const int kw = (p.rope && p.mode != 0) ? p.n_kv * p.hd : 0;   // width of the key columns that get rotated
+  const float* recv = reinterpret_cast<const float*>(smem + STAGES * STEP_BYTES + 128);
+  auto gather = [&](int lr, int col, float (&v8)[8]) {          // columns [col, col + 8) of own row lr, summed over the cluster in rank order
     float4 x0[8], x1[8];
 #pragma unroll
-    for (uint32_t s = 0; s < 8; ++s) {
-      if (s < CS) {
-        uint32_t remote;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(remote) : "r"(part_u32 + (row * COLS + col) * 4), "r"(s));
-        asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n" : "=f"(x0[s].x), "=f"(x0[s].y), "=f"(x0[s].z), "=f"(x0[s].w) : "r"(remote));
-        asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n" : "=f"(x1[s].x), "=f"(x1[s].y), "=f"(x1[s].z), "=f"(x1[s].w) : "r"(remote + 16));
+    for (int s = 0; s < 8; ++s) {
+      if (s < (int)CS) {
+        const float* src = recv + (size_t)(s * tw + lr) * COLS + col;
+        x0[s] = *reinterpret_cast<const float4*>(src);
+        x1[s] = *reinterpret_cast<const float4*>(src + 4);
       } else {
         x0[s] = make_float4(0.f, 0.f, 0.f, 0.f); x1[s] = x0[s];
       }
@@ -237,44 +242,34 @@ proj_small_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       v8[4] += x1[s].x; v8[5] += x1[s].y; v8[6] += x1[s].z; v8[7] += x1[s].w;
     }
   };
-  const int kw = (p.rope && p.mode != 0) ? p.n_kv * p.hd : 0;   // width of the key columns that get rotated
-  for (int it = threadIdx.x; it < p.M * pieces_per_row; it += PS_THREADS) {
-    const int row = it / pieces_per_row, pc = it % pieces_per_row;
-    const int col = (rank * pieces_per_row + pc) * 8;
+  mbar_wait_cluster(recv_bar, 0, p.status);
+  for (int it = threadIdx.x; it < n_items; it += PS_THREADS) {
+    const int lr = it / PPR, col = (it % PPR) * 8, row = (int)rank * tw + lr;
     const int gc = group * COLS + col;
     if (gc >= p.N_out) continue;
-    if (gc < kw && (gc % p.hd) >= p.hd / 2) continue;   // upper half of a rotated head: written with its lower partner
-    long long slot = p.slot_mapping ? (long long)p.slot_mapping[row] : p.start_slot + row;
+    if (gc < kw && (gc & (p.hd - 1)) >= p.hd / 2) continue;   // upper half of a rotated head: written with its lower partner
+    const long long slot = p.slot_mapping ? (long long)p.slot_mapping[row] : p.start_slot + row;
     if (slot < 0 || slot >= p.n_blocks * PAGE) { atomicOr(p.status, StatusBits::BAD_INDEX); continue; }
     const unsigned long long mask = p.row_masks ? p.row_masks[row] : p.agent_mask;
     float v8[8];
-    gather(row, col, v8);
+    gather(lr, col, v8);
     if (gc < kw) {
-      // rotary keys: columns (c, c + hd/2) of a head turn by the row's position; the block tile holds whole
-      // heads (COLS % hd == 0), so the partner piece sits hd/2 columns further in the same tiles
-      long long pos = p.positions ? (long long)p.positions[row] : p.start_pos + row;
-      if (pos < 0 || pos >= p.max_pos) { atomicOr(p.status, StatusBits::BAD_INDEX); continue; }
+      const long long pos = rope_pos(p, row);
+      if (pos < 0) continue;
       float h8[8];
-      gather(row, col + p.hd / 2, h8);
-      const float4* cs = p.rope + pos * (p.hd / 4) + (gc % p.hd) / 2;
-      float lo[8], hi[8];
+      gather(lr, col + p.hd / 2, h8);
+      const float4* cs = p.rope + pos * (p.hd / 4) + (gc & (p.hd - 1)) / 2;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const float4 t4 = __ldg(cs + k);                // (cos c, sin c, cos c+1, sin c+1)
-        lo[2 * k] = v8[2 * k] * t4.x - h8[2 * k] * t4.y;
-        lo[2 * k + 1] = v8[2 * k + 1] * t4.z - h8[2 * k + 1] * t4.w;
-        hi[2 * k] = h8[2 * k] * t4.x + v8[2 * k] * t4.y;
-        hi[2 * k + 1] = h8[2 * k + 1] * t4.z + v8[2 * k + 1] * t4.w;
+        const float l0 = v8[2 * k], l1 = v8[2 * k + 1], h0 = h8[2 * k], h1 = h8[2 * k + 1];
+        v8[2 * k] = l0 * t4.x - h0 * t4.y; v8[2 * k + 1] = l1 * t4.z - h1 * t4.w;
+        h8[2 * k] = h0 * t4.x + l0 * t4.y; h8[2 * k + 1] = h1 * t4.z + l1 * t4.w;
       }
-      store_piece(p, slot / PAGE, (int)(slot % PAGE), gc, lo, mask, row);
-      store_piece(p, slot / PAGE, (int)(slot % PAGE), gc + p.hd / 2, hi, mask, row);
-      continue;
+      store_piece(p, slot / PAGE, (int)(slot % PAGE), gc + p.hd / 2, h8, mask, row);
     }
     store_piece(p, slot / PAGE, (int)(slot % PAGE), gc, v8, mask, row);
   }
-  // nobody leaves while a peer may still read its partial tile
-  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
 }  // namespace precc
