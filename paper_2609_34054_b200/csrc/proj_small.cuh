@@ -23,7 +23,7 @@
 // owned by blocks the halves of a head met through a cluster barrier and loads over distributed shared memory: 3584 -> 1280
 // columns, 1 / 16 / 40 rows 8.1 / 9.0 / 9.9 us, now 5.4 / 6.0 / 7.7.)  Without rotation shares of columns are the cheaper ones to send
 // from eight rows on (4096 -> 2304, 16 / 32 rows: 6.1 / 7.8 us against 6.6 / 9.1: a warp's pairs then go to one block instead of
-// eight).  Up to four rows, and where the grid puts more than one block on an SM, rows win: most blocks own nothing and leave
+// eight).  For up to four rows, where the grid puts more than one block on an SM, rows win: most blocks own nothing and leave
 // at once, which makes room for the kernel behind (one row 5.95 -> 5.70 us; 8 layers of a two-row step with their
 // attention 135.8 -> 129.8).  With one block per SM it does not (2048 -> 1152: 3.05 against 3.12).
 // The K split depends on K alone, so an output value does not depend on which entry point, which other
