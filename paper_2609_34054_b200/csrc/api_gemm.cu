@@ -3,6 +3,7 @@
 #include "api_internal.h"
 #include "gemm_tc.cuh"
 #include "gemm_pair.cuh"
+#include "proj_plan.h"
 #include "proj_small.cuh"
 #include "proj_turn.cuh"
 
@@ -130,17 +131,6 @@ TurnPlan plan_turn(precc_ctx* ctx, int M, int nkb, int n_fused) {
   return best;
 }
 
-// The turn kernel over the whole K extent (up to 256 columns): rows of a tile, or 0 where 128-row tiles are as good.  With one
-// round of those they are (9000 x 128: 28.0 against 28.5 us); from two rounds on this form wins by what they fetch twice or leave
-// idle.  Very few columns cost the tiled kernel little beside the rows, so there it has to save a fifth of them
-// (32768 x 32: 49.1 against 50.8 us for an eighth; 20000 x 32: 47.7 against 33.7 us).
-int pick_wide_rows(int M, int n_out, int sm_count) {
-  const int rt = ((M + GEMM_BM - 1) / GEMM_BM + sm_count - 1) / sm_count, rounds = (M + sm_count * PT_MAX_TN - 1) / (sm_count * PT_MAX_TN);
-  const int tn = ((M + sm_count * rounds - 1) / (sm_count * rounds) + 15) / 16 * 16;
-  if (n_out > 2 * PT_COLS || rt < 2 || (n_out <= 64 && tn * rounds * 5 > rt * GEMM_BM * 4)) return 0;
-  return tn;
-}
-
 template <int NG>
 int32_t launch_turn(precc_ctx* ctx, const void* X, int M, int K, const void* Wt, int n_out, GemmParams gp, const TurnPlan& tp, cudaStream_t stream) {
   int tmem_cols = NG > 1 ? 512 : 32;
@@ -195,7 +185,7 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
     if (rc >= 0) return rc;
   }
   // Many rows, few columns: the turn kernel over the whole K extent.
-  const int wide = gp.rope || ctx->gemm_pair || ctx->force_tiled_gemm ? 0 : pick_wide_rows(M, n_out, ctx->sm_count);
+  const int wide = gp.rope || ctx->gemm_pair || ctx->force_tiled_gemm ? 0 : pick_wide_rows(M, K, n_out, ctx->sm_count);
   if (wide > 0) {
     const int ng = n_out > PT_COLS ? 2 : 1;
     TurnPlan tp;

@@ -32,9 +32,7 @@ namespace precc {
 
 constexpr int PT_EPI_WARPS = 8;
 constexpr int PT_THREADS = (2 + PT_EPI_WARPS) * 32;      // producer, MMA issuer, eight merging warps
-constexpr int PT_COLS = 128;                             // output columns of a tile (the M of the MMA)
 constexpr int PT_W_BYTES = PT_COLS * GEMM_BK * 2;
-constexpr int PT_MAX_TN = 256;
 constexpr int PT_MAX_STAGES = 8;
 constexpr int PT_MIN_SMEM = 120 * 1024;                  // keeps one block per SM, so that the cluster occupancy depends on KS alone
 struct PtRow { long long slot, slot2; unsigned long long mask; int pos, ok; };   // what the routing needs to know about a row

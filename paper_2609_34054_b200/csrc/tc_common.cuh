@@ -4,6 +4,7 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "proj_plan.h"
 
 namespace precc {
 
@@ -48,8 +49,6 @@ struct GemmParams {
 #define GEMM_STAMP(p, it, slot) do { } while (0)
 #endif
 
-constexpr int GEMM_BM = 128;
-constexpr int GEMM_BK = 64;                 // 64 bf16 = one 128-byte swizzle row
 constexpr int GEMM_THREADS = 192;
 constexpr int GEMM_MAX_KS = 8;            // largest K split of a turn's projection (cluster size)
 constexpr int GEMM_A_BYTES = GEMM_BM * GEMM_BK * 2;

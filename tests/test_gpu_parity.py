@@ -949,6 +949,24 @@ def test_many_rows_few_columns_equal_the_tiled_kernel_bitwise(monkeypatch, px, M
     px2.close()
 
 
+def test_more_rows_than_a_grid_axis_has_tiles(px):
+    """16 777 217 rows onto 80 columns: more 256-row tiles than the second and third grid axes hold."""
+    M, agents, r = 65535 * 256 + 257, 5, 8
+    geo = I.Geometry(64, 2, 1, 64, agents, r, r, alpha=16.0)
+    L = Layer(px, geo, seed=86, n_blocks=(M + 15) // 16)
+    g = torch.Generator(device="cuda").manual_seed(86)
+    H = torch.empty((M, 64), dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    px.lr_precompute(L.desc, H, L.A_packed, L.cache, 0)
+    torch.cuda.synchronize()
+    assert px.poll_status() == 0
+    pick = torch.cat([torch.arange(0, 20), torch.arange(M // 2, M // 2 + 20), torch.arange(M - 300, M)])
+    for a in range(agents):
+        for cache, A in ((L.cache.lr_k, L.w_np["A_k"]), (L.cache.lr_v, L.w_np["A_v"])):
+            got = f64(cache[a].reshape(-1, r)[pick.cuda()])
+            ref = O.lr_cache(f64(H[pick.cuda()]), A[a])
+            assert (np.abs(got - ref) <= _cache_tol(ref)).all()
+
+
 @pytest.mark.parametrize("ns,hd,n_kv,G,r,S", [(2, 128, 2, 4, 32, 16), (3, 64, 3, 3, 16, 5), (4, 128, 1, 7, 8, 37), (5, 64, 2, 8, 32, 33),
                                                (6, 128, 2, 4, 64, 3), (7, 64, 1, 5, 64, 26), (8, 128, 1, 1, 0, 2)])
 def test_split_context_merge_at_every_cluster_size(px, ns, hd, n_kv, G, r, S):
