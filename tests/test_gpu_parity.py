@@ -921,31 +921,38 @@ def test_turn_projection_at_the_edges_of_its_tiles(px, M, d, n_kv, hd, r):
             assert np.isnan(rows[untouched]).all()
 
 
-@pytest.mark.parametrize("M,agents,r", [(18945, 3, 32), (19999, 4, 32), (20000, 2, 32), (21001, 2, 8), (40001, 4, 16)])
-def test_many_rows_few_columns_equal_the_tiled_kernel_bitwise(monkeypatch, px, M, agents, r):
+@pytest.mark.parametrize("M,d,agents,r", [(18945, 2048, 3, 32), (19999, 2048, 4, 32), (20000, 2048, 2, 32), (21001, 2048, 2, 8), (40001, 3072, 4, 16)])
+def test_many_rows_few_columns_equal_the_tiled_kernel_bitwise(monkeypatch, px, M, d, agents, r):
     """Up to 256 columns of more rows than one round of 128-row tiles: blocks that take as many rows as there are SMs for and two
-    128-column halves of them.  The k steps of a value are those of the tiled kernel, so the caches agree bit for bit - at one and
-    two halves, a ragged last half, scattered slots, an agent mask - and with the definition on a sample of rows."""
-    geo = I.Geometry(192, 8, 2, 64, agents, r, r, alpha=2.0 * r)
+    128-column halves of them.  The k steps of a value are those of the tiled kernel, so the caches agree bit for bit, with it and
+    with the fused projection (which has too many columns for tall tiles) - at one and two halves, one and two rounds, a
+    ragged last half, scattered slots, an agent mask - and with the definition on a sample of rows."""
+    geo = I.Geometry(d, 8, 2, 64, agents, r, r, alpha=2.0 * r)
     H = I.hidden_states(M, geo, seed=85, tag=f"wide.{M}")
     nb = (M + 15) // 16 + 3
     slots = I.permutation(nb * 16, 85, f"wide.slots.{M}")[:M].to(torch.int32)
     monkeypatch.setenv("PRECC_GEMM", "tiled")
     px2 = Precc(0)
     got = []
-    for p in (px, px2):
+    mask = ((1 << agents) - 1) & ~1
+    for p, fused in ((px, False), (px2, False), (px, True)):
         L = Layer(p, geo, seed=85, n_blocks=nb, fill=float("nan"))
-        p.lr_precompute(L.desc, H.cuda(), L.A_packed, L.cache, 0, slots.cuda(), ((1 << agents) - 1) & ~1)
+        if fused:
+            WA = p.pack_turn_weights(geo, *(L.w[k].cuda() for k in ("W_k", "W_v", "A_k", "A_v")))
+            p.turn_project(L.desc, H.cuda(), WA, L.cache, 0, slots.cuda(), mask)
+        else:
+            p.lr_precompute(L.desc, H.cuda(), L.A_packed, L.cache, 0, slots.cuda(), mask)
         torch.cuda.synchronize()
         assert p.poll_status() == 0
         got.append(L)
-    for name in ("lr_k", "lr_v"):
-        assert torch.equal(getattr(got[0].cache, name).view(torch.int16), getattr(got[1].cache, name).view(torch.int16)), name
+    for other in got[1:]:
+        for name in ("lr_k", "lr_v"):
+            assert torch.equal(getattr(got[0].cache, name).view(torch.int16), getattr(other.cache, name).view(torch.int16)), name
     assert torch.isnan(got[0].cache.lr_k[0]).all()
     pick = np.r_[0:40, M // 2:M // 2 + 40, M - 40:M]
     ref = O.lr_cache(f64(H[pick]), got[0].w_np["A_v"][agents - 1])
     rows = lr_rows(got[0].cache.lr_v, agents - 1)[slots.numpy()[pick]]
-    assert (np.abs(rows - ref) <= 2.0 ** -8 * np.abs(ref) + 2e-3).all()
+    assert (np.abs(rows - ref) <= 2.0 ** -8 * np.abs(ref) + 2e-3 * np.sqrt(d / 256)).all()      # one bf16 rounding of an fp32 sum of d products
     px2.close()
 
 
