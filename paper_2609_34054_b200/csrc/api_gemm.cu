@@ -76,9 +76,6 @@ int32_t launch_small(precc_ctx* ctx, const void* X, int M, int K, const void* Wt
 
 int ilog2(int v) { int s = 0; while ((1 << s) < v) ++s; return s; }
 
-// How a turn's projection is cut: tiles of 128 columns x tn rows, the K extent of each over ks blocks.
-struct TurnPlan { int tn = 0, ks = 0, stages = 0; };
-
 // Clusters of `ks` blocks of the turn kernel that are resident at once (one block per SM; a cluster lives inside one GPC).
 int max_turn_clusters(precc_ctx* ctx, int ks) {
   static int max_clusters_dev[kMaxDevices][GEMM_MAX_KS + 1] = {{0}};   // 0 = unknown, else max active clusters + 1
@@ -101,34 +98,6 @@ int max_turn_clusters(precc_ctx* ctx, int ks) {
     cached = n + 1;
   }
   return cached - 1;
-}
-
-// The cut with the smallest predicted time among those whose clusters are all resident at once (a second wave costs more
-// than any split gains: 512 rows of the Llama-3-8B projection as 36 clusters of four, of which 33 fit, 26.9 us; as 36
-// clusters of three 17.2).  Time in us, fitted to some 450 cuts of four layers (d_model 1024 .. 4096) at 41 .. 2048 rows,
-// mean error 4 %: what a k-block costs a block, what the merge moves into one, what dumping and storing a tile takes, and the
-// cluster.  The cut it picks is within 1 % of the best one measured but for two in 36 (4 % and 11 %).
-TurnPlan plan_turn(precc_ctx* ctx, int M, int nkb, int n_fused) {
-  TurnPlan best;
-  double best_cost = 1e30;
-  const int groups = (n_fused + PT_COLS - 1) / PT_COLS;
-  const int ks_hi = (ctx->gemm_ks_max >= 2 && ctx->gemm_ks_max < GEMM_MAX_KS) ? ctx->gemm_ks_max : GEMM_MAX_KS;
-  for (int t = (M + PT_MAX_TN - 1) / PT_MAX_TN, last = 0;; ++t) {
-    const int tn = ((M + t - 1) / t + 15) / 16 * 16, tiles = (M + tn - 1) / tn;
-    if (tn < 32 || (long long)groups * tiles * ctx->gemm_ks_min > ctx->sm_count) break;
-    if (tn == last) continue;
-    last = tn;
-    for (int ks = ctx->gemm_ks_min; ks <= ks_hi && nkb / ks >= 2; ++ks) {       // at least two k-blocks per slice
-      if (groups * tiles > max_turn_clusters(ctx, ks)) continue;
-      const int kb = (nkb + ks - 1) / ks;
-      int st = kb < PT_MAX_STAGES ? kb : PT_MAX_STAGES;
-      while (st > 1 && pt_smem_bytes(tn, ks, st, 1) > ctx->max_smem_optin) --st;
-      if (pt_smem_bytes(tn, ks, st, 1) > ctx->max_smem_optin) continue;
-      const double cost = kb * (0.37 + 0.00036 * tn) + 0.005 * pt_share(tn, ks) * (ks - 1) + 0.0113 * tn + 0.1 * ks;
-      if (cost < best_cost) { best_cost = cost; best.tn = tn; best.ks = ks; best.stages = st; }
-    }
-  }
-  return best;
 }
 
 template <int NG>
@@ -164,6 +133,7 @@ int32_t launch_turn(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
 
 int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt, int n_out, GemmParams gp, cudaStream_t stream) {
   gp.hd_shift = ilog2(gp.hd); gp.rk_shift = ilog2(gp.rank_k > 0 ? gp.rank_k : 1); gp.rv_shift = ilog2(gp.rank_v > 0 ? gp.rank_v : 1);
+  const int n_fused = 2 * gp.n_kv * gp.hd + gp.n_agents * (gp.rank_k + gp.rank_v);     // width of this layer's fused projection, whatever this call projects
   // Few rows: the weight-streaming kernel (fused Llama-3-8B projection: 6.1 us at 16 rows, 7.8 at 32, 9.8 at 40, where the turn
   // kernel takes 9.8 too; d_model 2048, 40 rows: 4.8 against 7.3).  Rows written one by one and in one call of up to 40 have
   // equal bits.  Beyond that the turn kernel, up to some two thousand rows; the few-row kernel still takes 41 .. 64 rows where the K split does not apply
@@ -175,9 +145,9 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
   const int m_tiles = (M + GEMM_BM - 1) / GEMM_BM;
   // The tokens of a turn: 128-column tiles as wide as there are rows, the K extent of a tile split over a cluster.
   if (m_tiles <= 16 && !ctx->no_gemm_splitk) {
-    // planned for the width of the FUSED projection of this layer, whatever this call projects, so that the base-only,
-    // LR-only and fused calls of one M take the same decision (and with it the same summation order)
-    const TurnPlan tp = plan_turn(ctx, M, K / GEMM_BK, 2 * gp.n_kv * gp.hd + gp.n_agents * (gp.rank_k + gp.rank_v));
+    const int ks_max = ctx->gemm_ks_max >= 2 && ctx->gemm_ks_max < GEMM_MAX_KS ? ctx->gemm_ks_max : GEMM_MAX_KS;
+    const TurnPlan tp = plan_turn(M, K / GEMM_BK, n_fused, n_out, ctx->gemm_ks_min, ks_max, ctx->sm_count, ctx->max_smem_optin,
+                                  [&](int ks) { return max_turn_clusters(ctx, ks); });
     if (tp.ks > 0) return launch_turn<1>(ctx, X, M, K, Wt, n_out, gp, tp, stream);
   }
   if (M <= PS_MAX_M && !ctx->force_tiled_gemm) {

@@ -3,12 +3,74 @@
 #pragma once
 #include <algorithm>
 
+#ifdef __CUDACC__
+#define PRECC_HD __host__ __device__
+#else
+#define PRECC_HD
+#endif
+
 namespace precc {
 
 constexpr int GEMM_BM = 128;                             // rows of a tile of the tiled kernel
 constexpr int GEMM_BK = 64;                              // 64 bf16 = one 128-byte swizzle row
 constexpr int PT_COLS = 128;                             // output columns of a tile of the turn kernel (the M of its MMA)
 constexpr int PT_MAX_TN = 256;                           // rows of X in such a tile at most
+constexpr int GEMM_MAX_KS = 8;                           // largest K split of a turn's projection (cluster size)
+constexpr int PT_W_BYTES = PT_COLS * GEMM_BK * 2;
+constexpr int PT_MAX_STAGES = 8;
+constexpr int PT_MIN_SMEM = 120 * 1024;                  // keeps one block per SM, so that the cluster occupancy depends on KS alone
+struct PtRow { long long slot, slot2; unsigned long long mask; int pos, ok; };   // what the routing needs to know about a row
+
+PRECC_HD constexpr int pt_stage_bytes(int tn, int ng) { return ng * PT_W_BYTES + tn * GEMM_BK * 2; }
+PRECC_HD constexpr int pt_share(int rows, int ks) { return ((rows + ks - 1) / ks + 7) / 8 * 8; }     // rows finished by one block
+PRECC_HD constexpr int pt_merge_bytes(int tn, int ks) { return (tn + (ks - 1) * pt_share(tn, ks)) * PT_COLS * 4; }
+PRECC_HD constexpr int pt_data_bytes(int tn, int ks, int stages, int ng) {
+  const int ring = stages * pt_stage_bytes(tn, ng), merge = pt_merge_bytes(tn, ks);
+  return ((ring > merge ? ring : merge) + 1023) / 1024 * 1024;
+}
+PRECC_HD constexpr int pt_smem_bytes(int tn, int ks, int stages, int ng) {
+  return pt_data_bytes(tn, ks, stages, ng) + pt_share(tn, ks) * (int)sizeof(PtRow) + (2 * PT_MAX_STAGES + 4) * 8;
+}
+
+// How a turn's projection is cut: tiles of 128 columns x tn rows, the K extent of each over ks blocks.
+struct TurnPlan { int tn = 0, ks = 0, stages = 0; };
+
+// The cut with the smallest predicted time among those whose clusters are all resident at once - clusters(ks) says how many of ks
+// blocks are, a cluster lives inside one GPC - (a second wave costs more than any split gains: 512 rows of the Llama-3-8B projection
+// as 36 clusters of four, of which 33 fit, 26.9 us; as 36 clusters of three 17.2).  Time in us, fitted to some 450 cuts of
+// four layers (d_model 1024 .. 4096) at 41 .. 2048 rows, mean error 4 %: what a k-block costs a block, what the merge moves into
+// one, what dumping and storing a tile takes, and the cluster.  The cut it picks is within 1 % of the best one measured but for
+// two in 36 (4 % and 11 %).
+// The K split is the one for the width of the layer's FUSED projection, whatever this call projects, so that the base-only,
+// LR-only and fused calls of one M add in the same order.  The height of the tiles changes no bit: a call of fewer columns takes lower
+// tiles on the SMs that this leaves (LR rows of two agents of rank 8, d_model 2048, 768 rows: 9.9 us in tiles of the fused
+// call's height, 8.2 in tiles of 32 rows; of three, d_model 1024, 1800 rows 8.8 -> 7.0; base rows of d_model 3584, 512 rows 12.6 -> 11.6).
+template <class Clusters>
+TurnPlan plan_turn(int M, int nkb, int n_fused, int n_out, int ks_min, int ks_max, int sm_count, int max_smem, Clusters clusters) {
+  TurnPlan best;
+  auto search = [&](int columns, int ks_lo, int ks_hi) {
+    double best_cost = 1e30;
+    const int groups = (columns + PT_COLS - 1) / PT_COLS;
+    for (int t = (M + PT_MAX_TN - 1) / PT_MAX_TN, last = 0;; ++t) {
+      const int tn = ((M + t - 1) / t + 15) / 16 * 16, tiles = (M + tn - 1) / tn;
+      if (tn < 32 || (long long)groups * tiles * ks_lo > sm_count) break;
+      if (tn == last) continue;
+      last = tn;
+      for (int ks = ks_lo; ks <= ks_hi && nkb / ks >= 2; ++ks) {       // at least two k-blocks per slice
+        if (groups * tiles > clusters(ks)) continue;
+        const int kb = (nkb + ks - 1) / ks;
+        int st = kb < PT_MAX_STAGES ? kb : PT_MAX_STAGES;
+        while (st > 1 && pt_smem_bytes(tn, ks, st, 1) > max_smem) --st;
+        if (pt_smem_bytes(tn, ks, st, 1) > max_smem) continue;
+        const double cost = kb * (0.37 + 0.00036 * tn) + 0.005 * pt_share(tn, ks) * (ks - 1) + 0.0113 * tn + 0.1 * ks;
+        if (cost < best_cost) { best_cost = cost; best.tn = tn; best.ks = ks; best.stages = st; }
+      }
+    }
+  };
+  search(n_fused, ks_min, ks_max);
+  if (best.ks > 0 && n_out < n_fused) search(n_out, best.ks, best.ks);
+  return best;
+}
 
 // The turn kernel over the whole K extent (up to 256 columns of many rows): rows of a tile, or 0 where the tiled kernel is as good.
 // The tiled kernel takes rt 128-row tiles a block; this form takes `rounds` tiles of up to 256 rows, cut so that every SM has the same

@@ -32,21 +32,6 @@ namespace precc {
 
 constexpr int PT_EPI_WARPS = 8;
 constexpr int PT_THREADS = (2 + PT_EPI_WARPS) * 32;      // producer, MMA issuer, eight merging warps
-constexpr int PT_W_BYTES = PT_COLS * GEMM_BK * 2;
-constexpr int PT_MAX_STAGES = 8;
-constexpr int PT_MIN_SMEM = 120 * 1024;                  // keeps one block per SM, so that the cluster occupancy depends on KS alone
-struct PtRow { long long slot, slot2; unsigned long long mask; int pos, ok; };   // what the routing needs to know about a row
-
-__host__ __device__ constexpr int pt_stage_bytes(int tn, int ng) { return ng * PT_W_BYTES + tn * GEMM_BK * 2; }
-__host__ __device__ constexpr int pt_share(int rows, int ks) { return ((rows + ks - 1) / ks + 7) / 8 * 8; }     // rows finished by one block
-__host__ __device__ constexpr int pt_merge_bytes(int tn, int ks) { return (tn + (ks - 1) * pt_share(tn, ks)) * PT_COLS * 4; }
-__host__ __device__ constexpr int pt_data_bytes(int tn, int ks, int stages, int ng) {
-  const int ring = stages * pt_stage_bytes(tn, ng), merge = pt_merge_bytes(tn, ks);
-  return ((ring > merge ? ring : merge) + 1023) / 1024 * 1024;
-}
-__host__ __device__ constexpr int pt_smem_bytes(int tn, int ks, int stages, int ng) {
-  return pt_data_bytes(tn, ks, stages, ng) + pt_share(tn, ks) * (int)sizeof(PtRow) + (2 * PT_MAX_STAGES + 4) * 8;
-}
 
 template <bool ROPE, int NG>
 __global__ void __launch_bounds__(PT_THREADS, 1)

@@ -50,7 +50,6 @@ struct GemmParams {
 #endif
 
 constexpr int GEMM_THREADS = 192;
-constexpr int GEMM_MAX_KS = 8;            // largest K split of a turn's projection (cluster size)
 constexpr int GEMM_A_BYTES = GEMM_BM * GEMM_BK * 2;
 
 // The same bounded wait for waiters that are not on the critical path (an epilogue waiting for a whole tile of

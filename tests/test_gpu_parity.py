@@ -845,7 +845,7 @@ def test_decode_alternating_between_ring_layouts_of_one_shape(px):
     assert px.poll_status() == 0
 
 
-@pytest.mark.parametrize("M,d", [(41, 1024), (64, 2048), (100, 1024), (129, 2048), (300, 1024), (384, 4096), (450, 2048), (512, 4096)])
+@pytest.mark.parametrize("M,d", [(41, 1024), (64, 2048), (100, 1024), (129, 2048), (300, 1024), (384, 4096), (450, 2048), (512, 4096), (769, 2048), (1791, 1024)])
 def test_short_turn_projection_split_over_a_cluster(monkeypatch, px, M, d):
     """41 to 512 rows (the tokens of a short turn): the K extent of every 128 x 256 tile is split over a cluster
     of 3 to 8 blocks (K slices need not be equal) whose partial accumulators are merged over distributed shared memory.  Against the

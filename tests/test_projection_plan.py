@@ -17,7 +17,7 @@ def plan(tmp_path_factory):
         src, exe = d / "plan.cpp", d / f"plan_{abs(hash(expr))}"
         if not exe.exists():
             src.write_text('#include <cstdio>\n#include "proj_plan.h"\nusing namespace precc;\n'
-                           f'int main() {{ int a[8]; while (scanf("%d %d %d %d", a, a + 1, a + 2, a + 3) == 4) {{ {expr} }} }}\n')
+                           f'int main() {{ int a[4]; while (scanf("%d %d %d %d", a, a + 1, a + 2, a + 3) == 4) {{ {expr} }} }}\n')
             subprocess.run(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", str(exe)], check=True)
         text = "\n".join(" ".join(map(str, (list(r) + [0] * 4)[:4])) for r in rows)
         out = subprocess.run([str(exe)], input=text, capture_output=True, text=True, check=True).stdout
@@ -55,3 +55,31 @@ def test_tall_tiles_are_taken_where_they_are_faster(plan):
     got = plan(f'printf("%d\\n", pick_wide_rows(a[0], a[1], a[2], {SMS}));', [r[:3] for r in MANY_ROWS])
     for (M, K, n, tiled, tall), (tn,) in zip(MANY_ROWS, got):
         assert (tn > 0) == (tall < tiled), (M, K, n)
+
+
+# blocks of a cluster -> clusters that are resident at once, as a B200 reports them
+CLUSTERS = {2: 74, 3: 45, 4: 33, 5: 26, 6: 22, 7: 15, 8: 15}
+SMEM = 232448
+PLAN = ("static const int fit[9] = {0, 0, %s}; " % ", ".join(str(CLUSTERS[k]) for k in range(2, 9)) +
+        f"TurnPlan p = plan_turn(a[0], a[1], a[2], a[3], 2, 8, {SMS}, {SMEM}, [&](int ks) {{ return fit[ks]; }}); "
+        'printf("%d %d %d %d\\n", p.tn, p.ks, p.stages, p.ks ? pt_smem_bytes(p.tn, p.ks, p.stages, 1) : 0);')
+
+
+def test_calls_of_a_layer_are_cut_alike_in_k_and_fill_the_chip_in_rows(plan):
+    """LR-only and base-only calls keep the K split of the fused call (the order of their sums) and take tiles that are no higher."""
+    layers = [(16, 560, 48, 512), (16, 2560, 2048, 512), (32, 1056, 32, 1024), (32, 1152, 128, 1024), (56, 1280, 256, 1024), (64, 2304, 256, 2048),
+              (64, 4096, 2048, 2048), (17, 608, 96, 512)]
+    Ms = [41, 48, 64, 65, 128, 200, 301, 512, 513, 640, 768, 1000, 1280, 1791, 2048]
+    rows = [(M, nkb, fused, n) for nkb, fused, lr, base in layers for M in Ms for n in (fused, lr, base)]
+    got = dict(zip(rows, plan(PLAN, rows)))
+    lower = 0
+    for (M, nkb, fused, n), (tn, ks, stages, smem) in got.items():
+        whole = got[M, nkb, fused, fused]
+        assert ks == whole[1] and (ks == 0 or tn <= whole[0]), (M, nkb, fused, n)
+        if ks:
+            assert tn % 16 == 0 and 32 <= tn <= 256 and stages >= 1 and smem <= SMEM
+            assert -(-n // 128) * -(-M // tn) <= CLUSTERS[ks], (M, nkb, fused, n)
+            lower += tn < whole[0]
+    assert lower > 60
+    # 768 rows onto 32 of 1056 columns: with the fused call's 256-row tiles, three clusters
+    assert got[768, 32, 1056, 32][0] <= 48 and got[1791, 16, 560, 48][0] <= 64
