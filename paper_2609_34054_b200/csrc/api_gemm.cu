@@ -134,11 +134,9 @@ int32_t launch_turn(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
 int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt, int n_out, GemmParams gp, cudaStream_t stream) {
   gp.hd_shift = ilog2(gp.hd); gp.rk_shift = ilog2(gp.rank_k > 0 ? gp.rank_k : 1); gp.rv_shift = ilog2(gp.rank_v > 0 ? gp.rank_v : 1);
   const int n_fused = 2 * gp.n_kv * gp.hd + gp.n_agents * (gp.rank_k + gp.rank_v);     // width of this layer's fused projection, whatever this call projects
-  // Few rows: the weight-streaming kernel (fused Llama-3-8B projection: 6.1 us at 16 rows, 7.8 at 32, 9.8 at 40, where the turn
-  // kernel takes 9.8 too; d_model 2048, 40 rows: 4.8 against 7.3).  Rows written one by one and in one call of up to 40 have
-  // equal bits.  Beyond that the turn kernel, up to some two thousand rows; the few-row kernel still takes 41 .. 64 rows where the K split does not apply
-  // (short K).
-  if (M <= PS_FAST_M && !ctx->force_tiled_gemm) {
+  // Few rows: the weight-streaming kernel.  Rows written one by one and in one call of up to that many have equal bits.  Beyond that the turn
+  // kernel, up to some two thousand rows; the few-row kernel still takes up to 64 rows where the K split does not apply (short K).
+  if (M <= few_row_limit(K, n_fused) && !ctx->force_tiled_gemm) {
     const int32_t rc = launch_small(ctx, X, M, K, Wt, n_out, gp, stream);
     if (rc >= 0) return rc;
   }

@@ -32,6 +32,15 @@ PRECC_HD constexpr int pt_smem_bytes(int tn, int ks, int stages, int ng) {
   return pt_data_bytes(tn, ks, stages, ng) + pt_share(tn, ks) * (int)sizeof(PtRow) + (2 * PT_MAX_STAGES + 4) * 8;
 }
 
+// Rows up to which the few-row kernel takes every call of a layer (so the same for its fused, base-only and LR-only calls).  40 of any
+// layer (fused Llama-3-8B projection: 6.1 us at 16 rows, 7.8 at 32, 9.8 at 40, where the turn kernel takes 9.8 too), all 64 that it can
+// hold where the weights are few and every column group still has its eight K slices: 64 rows onto 1280 columns of d_model 3584 6.6 us
+// against 8.7 on the turn kernel, 1152 of 2048 5.3 against 7.4, 560 of 1024 3.8 against 5.8; LR rows alone (48 columns) 3.7 against
+// 5.6; rotary keys 9.2 / 7.8 / 6.3 against 9.0 / 7.7 / 6.1.  Wider layers lose: 2304 columns of 4096 10.7 against 9.9, rotary 14.7 against 10.2;
+// 2560 of 1024 rotary 10.7 against 7.0.
+constexpr int PS_MAX_M = 64;
+inline int few_row_limit(int K, int n_fused) { return n_fused <= 1280 && K <= 4096 && K % 512 == 0 ? PS_MAX_M : 40; }
+
 // How a turn's projection is cut: tiles of 128 columns x tn rows, the K extent of each over ks blocks.
 struct TurnPlan { int tn = 0, ks = 0, stages = 0; };
 

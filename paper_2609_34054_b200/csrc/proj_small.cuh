@@ -35,8 +35,6 @@ namespace precc {
 
 constexpr int PS_WARPS = 8;
 constexpr int PS_BK = 64;                   // k elements per step: one 128-byte swizzle row
-constexpr int PS_MAX_M = 64;
-constexpr int PS_FAST_M = 40;               // up to here it takes every call: a row has the same bits alone and among up to 39 others
 constexpr int PS_THREADS = (PS_WARPS + 1) * 32;       // consumer warps + one producer warp
 // Ring depth.  Above 32 rows three slots: with four (130 KB a block) only 15 clusters of eight are resident at once and the
 // 18 of the Llama-3-8B projection ran in two waves (33 .. 40 rows: 12.8 us, now 9.7).

@@ -287,8 +287,8 @@ def test_turn_project_equals_the_two_separate_projections_bitwise(px):
         assert torch.equal(a, b), name
 
 
-@pytest.mark.parametrize("M", [1, 7, 16, 17, 33, 64])
-@pytest.mark.parametrize("d,hd,n_kv", [(192, 64, 2), (1024, 128, 2), (4096, 128, 1)])
+@pytest.mark.parametrize("M", [1, 7, 16, 17, 33, 41, 64])
+@pytest.mark.parametrize("d,hd,n_kv", [(192, 64, 2), (512, 64, 1), (1024, 128, 2), (4096, 128, 1)])
 def test_few_row_projection_kernel(px, M, d, hd, n_kv):
     """Decode-step projections (M <= 64 rows) take the weight-streaming split-K kernel: every mode against
     the definition, scattered slots, agent mask, and the fused call bit-equal to the two separate ones."""

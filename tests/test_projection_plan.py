@@ -83,3 +83,14 @@ def test_calls_of_a_layer_are_cut_alike_in_k_and_fill_the_chip_in_rows(plan):
     assert lower > 60
     # 768 rows onto 32 of 1056 columns: with the fused call's 256-row tiles, three clusters
     assert got[768, 32, 1056, 32][0] <= 48 and got[1791, 16, 560, 48][0] <= 64
+
+
+# measured at 64 rows on the few-row and the turn kernel (us): (d_model, fused width, few-row, turn)
+SIXTY_FOUR_ROWS = [(1024, 560, 3.8, 5.8), (1024, 1024, 3.9, 5.8), (2048, 1056, 5.2, 7.4), (2048, 1152, 5.3, 7.4), (3584, 1280, 6.6, 8.7),
+                   (4096, 2304, 10.7, 9.9), (4096, 4096, 15.1, 11.6)]
+
+
+def test_sixty_four_rows_run_on_the_faster_kernel(plan):
+    got = plan('printf("%d\\n", few_row_limit(a[0], a[1]));', [r[:2] for r in SIXTY_FOUR_ROWS])
+    assert [limit for limit, in got] == [64 if few < turn else 40 for _, _, few, turn in SIXTY_FOUR_ROWS]
+    assert plan('printf("%d\\n", few_row_limit(a[0], a[1]));', [(1088, 608)]) == [[40]]      # 17 k-blocks: no split, a single pass of them all
