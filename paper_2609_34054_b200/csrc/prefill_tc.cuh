@@ -940,11 +940,36 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
         //      partial out by rows (O, then m and l in the padding), so that what another block finishes is one run of
         //      memory: one bulk copy per peer into that block's receive area, counted on its merge barrier.  (Pulled with 16-byte
         //      loads over distributed shared memory, 64 new tokens over 16384 spent 8.9 us from here to the end, now 5.2.)
-        const int live = n_tok * G, R = merge_share(live);
+        // Its place in the grid, and (FRESH_SMEM) where its shared memory begins, the block reads again here, through moves that the compiler
+        // cannot merge with the ones above the step loop: carried through it, these registers change the schedule that
+        // ptxas finds for the loop.  Against the form that pulled the partials, over 36 turns of 32 .. 700 tokens on 8000 .. 65000 per pair of ranks
+        // (head_dim 128, geometric mean and slowest): ranks 16 / 16 contiguous 0.967 and 1.12 -> 0.934 and 1.00, 8 / 8 0.970 and
+        // 1.15 -> 0.936 and 1.00, 0 / 32 0.945 and 1.02 -> 0.935 and 1.00, 32 / 32 0.944 and 1.03 -> 0.924 and 0.99.  The last, and rank 64,
+        // do better with the shared-memory addresses carried (32 / 32: 1.017 otherwise, 0 / 64 1.00 instead of 0.975).
+        constexpr bool FRESH_SMEM = HD == 64 || (RK != 32 && RV != 64);
+        auto fresh = [](uint32_t x) { uint32_t y; asm volatile("mov.u32 %0, %1;\n" : "=r"(y) : "r"(x)); return y; };
+        uint32_t split, NS, bx, by, tx;
+        asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(split));
+        asm volatile("mov.u32 %0, %%cluster_nctaid.z;\n" : "=r"(NS));
+        asm volatile("mov.u32 %0, %%ctaid.x;\n" : "=r"(bx));
+        asm volatile("mov.u32 %0, %%ctaid.y;\n" : "=r"(by));
+        asm volatile("mov.u32 %0, %%tid.x;\n" : "=r"(tx));
+        const int wm = (int)(tx >> 5) - PTC_FIRST_SM_WARP, lane = tx & 31;
+        const int wg = wm >> 2, row = ((int)(tx >> 5) & 3) * 32 + lane, tid = wm * 32 + lane, g = (int)by;
+        const int tok0 = (p.longest_first ? (int)(gridDim.x - 1 - bx) : (int)bx) * p.tok_per_tile, n_tok = min(p.tok_per_tile, p.S - tok0);
+        unsigned char* area = smem;
+        uint32_t merge_u32 = merge_bar;
+        if constexpr (FRESH_SMEM) {
+          const uint32_t base = fresh(smem_u32(smem_raw)), off = (0u - base) & 1023u;
+          const int ks = (int)fresh(p.k_stages), vs = (int)fresh(p.v_stages);
+          area = smem_raw + off;
+          merge_u32 = base + off + C::Q_BYTES + C::QX_BYTES + ks * C::KSTAGE + vs * vunit + 8 * (2 * ks + 2 * vs + PTC_FIXED_BARS + 1);
+        }
+        const int live = n_tok * G, R = (live + (int)NS - 1) / (int)NS;
         const int nrows = max(0, min(R, live - (int)split * R));
         __syncwarp();
         asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");   // this block's rings are idle: peers may send over them
-        float* xo = reinterpret_cast<float*>(smem);               // the merge area starts at the Q tile: every MMA has completed
+        float* xo = reinterpret_cast<float*>(area);               // the merge area starts at the Q tile: every MMA has completed
         float* recv = xo + 128 * XS;                              // [NS - 1][R][XS], slot = sender's rank with the own rank left out
 #pragma unroll 1
         for (int c = wg; c < HD / 16; c += 2) {
@@ -970,10 +995,10 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
           const uint32_t dst = dsmem_addr(smem_u32(recv) + (uint32_t)(((int)split < tid ? (int)split : (int)split - 1) * R * XS * 4), tid);
           if (n > 0)
             asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-                         ::"r"(dst), "r"(smem_u32(xo + tid * R * XS)), "r"(n * XS * 4), "r"(dsmem_addr(merge_bar, tid)) : "memory");
+                         ::"r"(dst), "r"(smem_u32(xo + tid * R * XS)), "r"(n * XS * 4), "r"(dsmem_addr(merge_u32, tid)) : "memory");
         }
         __syncwarp();
-        mbar_wait_cluster(merge_bar, 0, p.status);
+        mbar_wait_cluster(merge_u32, 0, p.status);
         __syncwarp();
         // everything addressed to this block has arrived; a peer whose copies still read its shared memory waits for this
         asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
