@@ -288,6 +288,13 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
   // at rank 32 (64 over 16384: 33.0 us against 36.3, 30 over 60000: 69.3 against 74.0; paged, 64 over 32768: 58.9 against 56.5), not below
   // (rank 16, 99 over 65427: 125 us against 113; rank 8, 64 over 32768: 57.5 against 55.3; no key adapter, 200 over 8000: 43.7 against 40.4).
   constexpr bool L_MMA = C::L_ROUNDED && !WL && !(SP && HD == 128 && RK != 32);
+  // Running maxima over a row's 128 scores of a step (their number changes no bit).  A chain of 16 or 32 maxima keeps fewer registers than four
+  // of them beside the scores, eight keep the chain short; which one ptxas makes the faster step loop of differs by form.  Whole
+  // contexts, 80 turns of 360 .. 1400 tokens over 0 .. 40000 per pair of ranks, geometric mean and slowest against the kernel before the
+  // MMA summed the denominator, at 2 / 4 / 8: head_dim 128 ranks 0 / 32 paged 0.962, 1.03 / 1.002, 1.08 / 0.989, 1.07; 16 / 16 contiguous
+  // 0.983, 1.09 / 0.982, 1.08 / 0.958, 1.02; 32 / 32 0.952, 1.04 / 0.947, 1.05 / 0.943, 1.01; head_dim 64 ranks 0 / 64 1.003, 1.05 / 1.031,
+  // 1.17 / 1.000, 1.05; 32 / 32 0.946 / 0.932 / 0.945.
+  constexpr int N_MAX = SP || WL ? 4 : HD == 128 ? (RK > 0 ? 8 : 2) : RV == 64 ? 2 : 4;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);   // (pointer arithmetic, so that it stays a shared-memory address)
   const uint32_t q_u32 = smem_u32(smem);
@@ -801,13 +808,19 @@ lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __
             for (int k = 0; k < 32; ++k)
               if (c * 32 + k >= nvis) sv[c][k] = 0xff800000u;      // -inf: weight zero
         }
-        float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        float tm[N_MAX];
+#pragma unroll
+        for (int i = 0; i < N_MAX; ++i) tm[i] = -INFINITY;
 #pragma unroll
         for (int c = 0; c < 4; ++c)
 #pragma unroll
           for (int k = 0; k < 32; k += 2)                          // two elements per step: the three-input maximum
-            tm[(k >> 1) & 3] = fmaxf(tm[(k >> 1) & 3], fmaxf(__uint_as_float(sv[c][k]), __uint_as_float(sv[c][k + 1])));
-        const float tmax = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2;
+            tm[(k >> 1) & (N_MAX - 1)] = fmaxf(tm[(k >> 1) & (N_MAX - 1)], fmaxf(__uint_as_float(sv[c][k]), __uint_as_float(sv[c][k + 1])));
+#pragma unroll
+        for (int n = N_MAX / 2; n > 0; n /= 2)
+#pragma unroll
+          for (int i = 0; i < n; ++i) tm[i] = fmaxf(tm[i], tm[i + n]);
+        const float tmax = tm[0] * p.scale_log2;
         float m_prev = NEG_BIG;                                    // the reference in force before this step
         if (j > 0) {
           named_sync(bar_in, 64);
