@@ -847,8 +847,9 @@ def test_decode_alternating_between_ring_layouts_of_one_shape(px):
 
 @pytest.mark.parametrize("M,d", [(41, 1024), (64, 2048), (100, 1024), (129, 2048), (300, 1024), (384, 4096), (450, 2048), (512, 4096), (769, 2048), (1791, 1024)])
 def test_short_turn_projection_split_over_a_cluster(monkeypatch, px, M, d):
-    """41 to 512 rows (the tokens of a short turn): the K extent of every 128 x 256 tile is split over a cluster
-    of 3 to 8 blocks (K slices need not be equal) whose partial accumulators are merged over distributed shared memory.  Against the
+    """41 rows and more (the tokens of a turn): the K extent of every tile of 128 columns x up to 256 rows is split over a cluster of up
+    to eight blocks (K slices need not be equal) whose partial accumulators are merged by bulk sends; 41 and 64 rows of these narrow layers
+    run on the few-row kernel.  Against the
     definition, fused call bit-equal to the two separate ones, scattered slots, agent mask, untouched slots; and
     within one bf16 ulp (plus fp32 summation noise near zero) of the one-block-per-tile kernel."""
     geo = I.Geometry(d, 8, 2, 128, 3, 32, 32, alpha=64.0)
@@ -1013,44 +1014,107 @@ def test_split_context_merge_at_every_cluster_size(px, ns, hd, n_kv, G, r, S):
 
 @pytest.mark.parametrize("ks,M,d", [(2, 100, 1024), (2, 777, 2048), (3, 384, 4096), (3, 130, 1024), (4, 512, 2048), (4, 64, 4096), (4, 1000, 1024),
                                     (5, 200, 2048), (6, 256, 4096), (7, 41, 2048), (8, 128, 1024), (8, 77, 4096)])
-def test_split_k_merge_by_sends_equals_the_pulling_merge_bitwise(monkeypatch, ks, M, d):
-    """The partial tiles of a split-K cluster are merged by sends into the owner's shared memory: whole slices by bulk
-    copy (clusters of 2 to 4 blocks), or 16-byte pieces straight from registers (any cluster size; the default for
-    finer splits of up to 64 rows).  The summation order is that of the pulling merge, so all three must agree bit for bit at the
-    same split - and with the definition.  Scattered slots, agent mask, a fused width that is not a multiple of the tile."""
-    geo = I.Geometry(d, 8, 2, 128, 3, 16, 16, alpha=32.0)          # fused width 2*256 + 3*32 = 608 columns: three tiles, the last 96 wide
-    H = I.hidden_states(M, geo, seed=91, tag=f"push.{M}.{d}")
+def test_turn_projection_at_every_split(monkeypatch, ks, M, d):
+    """The K extent of a tile over a cluster of `ks` blocks (tests/test_projection_plan.py checks that these cuts are taken), slices
+    merged by bulk sends.  The fused call and the two separate ones, whose tiles are lower, agree bit for bit; the result
+    is not the unsplit kernel's, so the split ran; it is the definition's within fp32 summation and one rounding; and with small whole
+    numbers, whose sums are exact in any order, it is the definition's exactly - a slice lost, doubled or misplaced shows.  Scattered slots,
+    agent mask, a fused width that is not a multiple of the tile."""
+    geo = I.Geometry(d, 8, 2, 128, 3, 16, 16, alpha=32.0)          # fused width 2*256 + 3*32 = 608 columns: five tiles, the last 96 wide
     nb = (M + 15) // 16 + 3
     slots = I.permutation(nb * 16, 91, f"push.slots.{M}")[:M].to(torch.int32)
-    caches = []
-    for push_max, direct in (("4", "1"), ("0", "2"), ("0", "0")):       # bulk copies where they apply | direct sends | pulling
-        monkeypatch.setenv("PRECC_GEMM", "tiled")                      # keep the few-row kernel out of it
-        monkeypatch.setenv("PRECC_GEMM_KS_MAX", str(ks))
-        monkeypatch.setenv("PRECC_GEMM_KS_MIN", str(ks))
-        monkeypatch.setenv("PRECC_GEMM_PUSH_MAX", push_max)
-        monkeypatch.setenv("PRECC_GEMM_DIRECT", direct)
-        pz = Precc(0)
-        L = Layer(pz, geo, seed=91, n_blocks=nb, fill=float("nan"))
-        dev = {k: v.cuda() for k, v in L.w.items()}
-        WA = pz.pack_turn_weights(geo, dev["W_k"], dev["W_v"], dev["A_k"], dev["A_v"])
-        pz.turn_project(L.desc, H.cuda(), WA, L.cache, 0, slots.cuda(), 0b110)
+    sl, mask = slots.long(), 0b110
+    names = ("k_base", "v_base", "lr_k", "lr_v")
+
+    def project(p, H, WA):
+        L = Layer(p, geo, seed=91, n_blocks=nb, fill=float("nan"))
+        p.turn_project(L.desc, H.cuda(), WA, L.cache, 0, slots.cuda(), mask)
         torch.cuda.synchronize()
-        assert pz.poll_status() == 0
-        caches.append(L)
-        pz.close()
-    La, Lb, Lc = caches
-    for name in ("k_base", "v_base", "lr_k", "lr_v"):
-        assert torch.equal(getattr(La.cache, name).view(torch.int16), getattr(Lc.cache, name).view(torch.int16)), name
-    for name in ("k_base", "v_base", "lr_k", "lr_v"):
+        assert p.poll_status() == 0
+        return L
+
+    def against_definition(L, H, w, tol):
+        Hn = f64(H)
+        for got, ref in ((base_rows(L.cache.k_base)[sl], O.base_cache(Hn, w["W_k"])), (base_rows(L.cache.v_base)[sl], O.base_cache(Hn, w["W_v"])),
+                         (lr_rows(L.cache.lr_k, 1)[sl], O.lr_cache(Hn, w["A_k"][1])), (lr_rows(L.cache.lr_v, 2)[sl], O.lr_cache(Hn, w["A_v"][2]))):
+            assert (np.abs(got - ref) <= tol(ref)).all()
+
+    monkeypatch.setenv("PRECC_GEMM", "tiled")                       # keeps the few-row kernel out
+    monkeypatch.setenv("PRECC_GEMM_KS_MAX", str(ks))
+    monkeypatch.setenv("PRECC_GEMM_KS_MIN", str(ks))
+    pz = Precc(0)
+    monkeypatch.setenv("PRECC_GEMM_SPLITK", "0")
+    pt = Precc(0)
+    H = I.hidden_states(M, geo, seed=91, tag=f"push.{M}.{d}")
+    La = Layer(pz, geo, seed=91, n_blocks=nb, fill=float("nan"))
+    La.append(H, slot_mapping=slots.cuda(), agent_mask=mask)
+    WA = pz.pack_turn_weights(geo, *(La.w[k].cuda() for k in ("W_k", "W_v", "A_k", "A_v")))
+    Lb, Lt = project(pz, H, WA), project(pt, H, WA)
+    for name in names:
         assert torch.equal(getattr(La.cache, name).view(torch.int16), getattr(Lb.cache, name).view(torch.int16)), name
-    w, Hn, sl = La.w_np, f64(H), slots.long()
-    tol = lambda ref: 2.0 ** -8 * np.abs(ref) + 2e-3 * np.sqrt(d / 256)
-    for got, ref in ((base_rows(La.cache.k_base)[sl], O.base_cache(Hn, w["W_k"])), (base_rows(La.cache.v_base)[sl], O.base_cache(Hn, w["W_v"])),
-                     (lr_rows(La.cache.lr_k, 1)[sl], O.lr_cache(Hn, w["A_k"][1])), (lr_rows(La.cache.lr_v, 2)[sl], O.lr_cache(Hn, w["A_v"][2]))):
-        assert (np.abs(got - ref) <= tol(ref)).all()
-    assert torch.isnan(La.cache.lr_k[0]).all()                     # agent 0 is masked out
+    assert not torch.equal(Lb.cache.k_base[sl // 16, :, sl % 16], Lt.cache.k_base[sl // 16, :, sl % 16])
+    against_definition(Lb, H, Lb.w_np, lambda ref: 2.0 ** -8 * np.abs(ref) + 2e-3 * np.sqrt(d / 256))
+    assert torch.isnan(Lb.cache.lr_k[0]).all()                     # agent 0 is masked out
     untouched = torch.ones(nb * 16, dtype=torch.bool); untouched[sl] = False
-    assert torch.isnan(La.cache.k_base.permute(0, 2, 1, 3).reshape(nb * 16, -1)[untouched]).all()
+    assert torch.isnan(Lb.cache.k_base.permute(0, 2, 1, 3).reshape(nb * 16, -1)[untouched]).all()
+    whole = lambda shape, tag: I.uniform_int(-2, 2, int(np.prod(shape)), 91, tag).reshape(shape).to(torch.bfloat16)
+    w = {k: whole(tuple(v.shape), f"push.{k}.{d}") for k, v in La.w.items()}
+    Hw = whole((M, d), f"push.H.{M}.{d}")
+    Lw = project(pz, Hw, pz.pack_turn_weights(geo, *(w[k].cuda() for k in ("W_k", "W_v", "A_k", "A_v"))))
+    against_definition(Lw, Hw, {k: f64(v) for k, v in w.items()}, lambda ref: np.where(np.abs(ref) <= 256, 0.0, 2.0 ** -8 * np.abs(ref)))   # whole numbers up to 256 are bf16 values
+    pz.close(), pt.close()
+
+
+@pytest.mark.parametrize("agents,r", [(4, 32), (3, 8)])
+def test_few_rows_finished_by_rows_equal_those_finished_by_columns(px, agents, r):
+    """One to four rows of a layer whose projection puts more than one block on an SM (d_model 4096, 8 kv heads of 128): blocks of a
+    cluster of eight finish rows, most of them none.  Every row, with its own agent mask and second slot, is bit-equal to itself in a call of
+    five to eight rows, where blocks finish columns; and the definition's.  A width that is not a multiple of the tile at rank 8."""
+    d = 4096
+    geo = I.Geometry(d, 32, 8, 128, agents, r, r, alpha=2.0 * r)
+    H = I.hidden_states(8, geo, seed=43, tag="byrows").cuda()
+    nb, names = 3, ("k_base", "v_base", "lr_k", "lr_v")
+    slots = torch.tensor([5, 17, 2, 30, 8, 21, 11, 29], dtype=torch.int32).cuda()
+    copies = torch.tensor([33, -1, 40, 47, -1, 36, 38, 44], dtype=torch.int32).cuda()
+    masks = torch.tensor([1, 0b110, 0b111, 0b100, 0b011, 0b010, 0b101, 0b111], dtype=torch.int64).cuda()
+    L = Layer(px, geo, seed=43, n_blocks=nb, fill=float("nan"))
+    WA = px.pack_turn_weights(geo, *(L.w[k].cuda() for k in ("W_k", "W_v", "A_k", "A_v")))
+
+    def call(rows):
+        from paper_2609_34054_b200.binding import Cache
+        c = Cache(geo, nb, fill=float("nan"))
+        px.turn_project_rows(L.desc, H[rows].contiguous(), WA, c, slots[rows].contiguous(), masks[rows].contiguous(), copies[rows].contiguous())
+        torch.cuda.synchronize()
+        return c
+
+    bits = lambda c: [getattr(c, n).view(torch.int16).clone() for n in names]
+    for n in (5, 8):
+        whole = bits(call(list(range(n))))
+        for m in (1, 2, 3, 4):
+            nan = torch.full((1,), float("nan"), dtype=torch.bfloat16).view(torch.int16).item()
+            merged = [torch.full_like(t, nan) for t in whole]
+            for i in range(0, n, m):
+                part = bits(call(list(range(i, min(i + m, n)))))
+                for t, q in zip(merged, part):
+                    t[q != nan] = q[q != nan]
+            for name, a, b in zip(names, merged, whole):
+                assert torch.equal(a, b), (n, m, name)
+    c, Hn, sl = call([0, 1, 2, 3]), f64(H[:4]), slots[:4].cpu().long()
+    tol = lambda ref: 2.0 ** -8 * np.abs(ref) + 2e-3 * np.sqrt(d / 256)
+    for got, ref in ((base_rows(c.k_base)[sl], O.base_cache(Hn, L.w_np["W_k"])), (base_rows(c.v_base)[sl], O.base_cache(Hn, L.w_np["W_v"]))):
+        assert (np.abs(got - ref) <= tol(ref)).all()
+    for cache, A in ((c.lr_k, L.w_np["A_k"]), (c.lr_v, L.w_np["A_v"])):
+        for a in range(3):
+            ref, rows = O.lr_cache(Hn, A[a]), lr_rows(cache, a)
+            written = set()
+            for i in range(4):
+                if int(masks[i]) >> a & 1:
+                    for t in (int(slots[i]), int(copies[i])):
+                        if t >= 0:
+                            assert (np.abs(rows[t] - ref[i]) <= tol(ref[i])).all()
+                            written.add(t)
+            assert np.isnan(rows[[t for t in range(nb * 16) if t not in written]]).all()
+    assert px.poll_status() == 0
 
 
 @pytest.mark.parametrize("M,d,hd,n_kv,r", [(1000, 512, 128, 2, 32), (2125, 1024, 64, 8, 16), (640, 256, 128, 1, 8)])

@@ -46,7 +46,7 @@ def test_rope_table_matches_the_definition():
 
 
 @pytest.mark.parametrize("hd,n_kv,M", [(64, 2, 300), (128, 1, 130), (128, 4, 517),
-                                      (64, 2, 1), (128, 2, 7), (128, 1, 40), (64, 4, 64), (128, 2, 16)])   # the last five: few-row kernel
+                                      (64, 2, 1), (128, 2, 7), (128, 1, 40), (64, 4, 64), (128, 2, 16)])   # up to 40 rows: few-row kernel
 def test_projection_rotates_keys_only(px, hd, n_kv, M):
     geo = I.Geometry(d_model=256, n_q=2 * n_kv, n_kv=n_kv, hd=hd, n_agents=2, rank_k=16, rank_v=16, alpha=32.0)
     nb = (M + 15) // 16 + 2
@@ -93,16 +93,15 @@ def test_projection_rotates_keys_only(px, hd, n_kv, M):
     assert (L.cache.lr_k[0] == 0).all() and (L.cache.lr_v[0] == 0).all()
 
 
-@pytest.mark.parametrize("ks,direct,hd,n_kv,M", [
-    (8, "0", 128, 4, 130), (8, "0", 64, 3, 70), (7, "0", 128, 2, 200), (6, "0", 64, 4, 129), (5, "0", 128, 3, 257),   # pulling merge
-    (8, "1", 128, 2, 41), (7, "1", 64, 1, 64), (6, "2", 128, 1, 150),                                              # direct sends
-    (4, "1", 128, 4, 300), (3, "1", 64, 4, 200), (3, "1", 128, 1, 128), (2, "1", 128, 2, 513)])                    # bulk sends
-def test_split_projection_rotates_keys(px, monkeypatch, ks, direct, hd, n_kv, M):
-    """Rotary epilogue of the split-K projections: a head's two halves meet in one slice of the merge, at slice widths that
-    do and do not divide the tile (ks = 3, 5, 6, 7: 96, 64, 48, 48 columns).  Base-only and fused calls agree bit for bit."""
+@pytest.mark.parametrize("ks,hd,n_kv,M", [(8, 128, 4, 130), (8, 64, 3, 70), (7, 128, 2, 200), (6, 64, 4, 129), (5, 128, 3, 257), (8, 128, 2, 41),
+                                          (7, 64, 1, 64), (6, 128, 1, 150), (4, 128, 4, 300), (3, 64, 4, 200), (3, 128, 1, 128), (2, 128, 2, 513)])
+def test_split_projection_rotates_keys(px, monkeypatch, ks, hd, n_kv, M):
+    """Rotary epilogue of the split-K projections at clusters of two to eight blocks (tests/test_projection_plan.py checks that these cuts are
+    taken): a head's two halves lie in one row of the merge; K slices of unlike length (17 k-blocks), blocks that finish no rows or a ragged
+    share, several row tiles.  Base-only and fused calls agree bit for bit."""
     from paper_2609_34054_b200.binding import Precc
     monkeypatch.setenv("PRECC_GEMM_KS_MAX", str(ks))
-    monkeypatch.setenv("PRECC_GEMM_DIRECT", direct)
+    monkeypatch.setenv("PRECC_GEMM_KS_MIN", str(ks))
     p = Precc(0)
     geo = I.Geometry(d_model=1088, n_q=2 * n_kv, n_kv=n_kv, hd=hd, n_agents=3, rank_k=16, rank_v=16, alpha=32.0)
     L = Layer(p, geo, seed=13, n_blocks=(M + 15) // 16 + 1, tag="rs", fill=0.0)
@@ -134,6 +133,35 @@ def test_split_projection_rotates_keys(px, monkeypatch, ks, direct, hd, n_kv, M)
     assert p.poll_status() == 1
     assert (base_rows(L.cache.k_base)[M // 2] == 0).all() and (base_rows(L.cache.k_base)[M // 2 - 1] != 0).any()
     p.close()
+
+
+@pytest.mark.parametrize("M", [1, 5, 9, 17, 33, 40, 57, 64])
+@pytest.mark.parametrize("d,hd,n_kv", [(1024, 128, 2), (2048, 64, 3)])
+def test_few_row_projection_rotates_keys_at_eight_slices(px, M, d, hd, n_kv):
+    """Clusters of eight blocks that finish rows: fewer rows than blocks, ragged shares, every height of the tile.  Against the
+    definition; every row bit-equal to itself in a call of its own."""
+    from paper_2609_34054_b200.binding import Cache
+    geo = I.Geometry(d_model=d, n_q=2 * n_kv, n_kv=n_kv, hd=hd, n_agents=3, rank_k=8, rank_v=8, alpha=16.0)
+    L = Layer(px, geo, seed=17, n_blocks=(M + 15) // 16, tag="f8", fill=0.0)
+    H = I.hidden_states(M, geo, 17, "f8.H").cuda()
+    table, (cos, sin) = rope_table(2048, hd), O.rope_tables(2048, hd)
+    pos = I.uniform_int(0, 2047, M, 17, "f8.pos").to(torch.int32)
+    WA = px.pack_turn_weights(geo, *(L.w[k].cuda() for k in ("W_k", "W_v", "A_k", "A_v")))
+    px.turn_project_rope(L.desc, H, WA, L.cache, table, 0, positions=pos.cuda())
+    torch.cuda.synchronize()
+    tol = lambda ref: 2.0 ** -8 * np.abs(ref) + 2e-3 * np.sqrt(d / 256)
+    ref = O.rope_rotate(O.base_cache(f64(H), L.w_np["W_k"]), pos.numpy(), n_kv, cos, sin)
+    assert (np.abs(base_rows(L.cache.k_base)[:M] - ref) <= tol(ref)).all()
+    for got, ref in ((base_rows(L.cache.v_base), O.base_cache(f64(H), L.w_np["W_v"])), (L.cache.lr_k[2].reshape(-1, 8).float().cpu().numpy(), O.lr_cache(f64(H), L.w_np["A_k"][2])),
+                     (L.cache.lr_v[0].reshape(-1, 8).float().cpu().numpy(), O.lr_cache(f64(H), L.w_np["A_v"][0]))):
+        assert (np.abs(got[:M] - ref) <= tol(ref)).all()
+    one = Cache(geo, (M + 15) // 16, fill=0.0)
+    for i in range(M):
+        px.turn_project_rope(L.desc, H[i:i + 1], WA, one, table, i, positions=pos[i:i + 1].cuda())
+    torch.cuda.synchronize()
+    for name in ("k_base", "v_base", "lr_k", "lr_v"):
+        assert torch.equal(getattr(one, name).view(torch.int16), getattr(L.cache, name).view(torch.int16)), name
+    assert px.poll_status() == 0
 
 
 SHAPES = [

@@ -12,5 +12,8 @@ def test_tensor_memory_prefill_kernels_do_not_spill(src):
     build.build()
     found = re.findall(r"Compiling entry function '(\S*lr_attend_prefill_tc_kernel\S*)'.*?(\d+) bytes stack frame, (\d+) bytes spill stores,"
                        r" (\d+) bytes spill loads", open(build.resource_log(src)).read(), re.S)
-    assert len(found) >= 18                             # nine pairs of ranks, with and without helper blocks
+    # nine pairs of ranks, each for a whole context (0, 0), a context split over a cluster (0, 1) and with helper blocks (1, 0)
+    forms = [re.search(r"ILi(\d+)ELi(\d+)ELi(\d+)ELb(\d)ELb\d+ELb(\d)E", f[0]).groups() for f in found]
+    for form in (("0", "0"), ("0", "1"), ("1", "0")):
+        assert len({f[:3] for f in forms if f[3:] == form}) == 9, form
     assert [f for f in found if f[2:] != ("0", "0")] == []

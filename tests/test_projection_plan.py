@@ -85,6 +85,20 @@ def test_calls_of_a_layer_are_cut_alike_in_k_and_fill_the_chip_in_rows(plan):
     assert got[768, 32, 1056, 32][0] <= 48 and got[1791, 16, 560, 48][0] <= 64
 
 
+def test_forced_splits_of_the_gpu_tests_are_taken(plan):
+    """(blocks per cluster, rows, k-blocks, fused width) of the tests that force a split."""
+    at_every_split = [(2, 100, 16), (2, 777, 32), (3, 384, 64), (3, 130, 16), (4, 512, 32), (4, 64, 64), (4, 1000, 16), (5, 200, 32), (6, 256, 64), (7, 41, 32),
+                      (8, 128, 16), (8, 77, 64)]
+    rotary = [(8, 128, 4, 130), (8, 64, 3, 70), (7, 128, 2, 200), (6, 64, 4, 129), (5, 128, 3, 257), (8, 128, 2, 41), (7, 64, 1, 64), (6, 128, 1, 150),
+              (4, 128, 4, 300), (3, 64, 4, 200), (3, 128, 1, 128), (2, 128, 2, 513)]
+    rows = [(M, nkb, 608, ks) for ks, M, nkb in at_every_split] + [(M, 17, 2 * n_kv * hd + 96, ks) for ks, hd, n_kv, M in rotary]
+    forced = PLAN.replace("a[2], a[3], 2, 8,", "a[2], a[2], a[3], a[3],")
+    for row, (tn, ks, _, _) in zip(rows, plan(forced, rows)):
+        assert ks == row[3], row
+    shares = [((min(M, tn) + ks - 1) // ks + 7) // 8 * 8 for (M, _, _, ks), (tn, _, _, _) in zip(rows, plan(forced, rows))]
+    assert any(s * (ks - 1) >= min(M, 256) for s, (M, _, _, ks) in zip(shares, rows))     # blocks that finish no rows
+
+
 # measured at 64 rows on the few-row and the turn kernel (us): (d_model, fused width, few-row, turn)
 SIXTY_FOUR_ROWS = [(1024, 560, 3.8, 5.8), (1024, 1024, 3.9, 5.8), (2048, 1056, 5.2, 7.4), (2048, 1152, 5.3, 7.4), (3584, 1280, 6.6, 8.7),
                    (4096, 2304, 10.7, 9.9), (4096, 4096, 15.1, 11.6)]
