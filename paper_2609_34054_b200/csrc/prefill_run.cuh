@@ -2,7 +2,6 @@
 // the cluster split of short turns and the launch.  Included by one translation unit per head dimension.
 #pragma once
 #include <algorithm>
-#include <vector>
 
 #include "api_internal.h"
 #include "prefill.cuh"
@@ -13,71 +12,9 @@ namespace precc {
 template <int HD, int RK, int RV>
 struct PrefillRun {
   // ---- work-list launch of the tensor-core kernel: plan and workspace
-  struct WorkList { int p = 0, helpers = 0, tiles = 0; };
   static size_t ticket_bytes(int tiles) { return ((size_t)tiles * 4 + 255) / 256 * 256; }
   static size_t worklist_ws_bytes(int tiles, int helpers) {
     return ticket_bytes(tiles) + (size_t)(2 * tiles + helpers) * PrefillTcCfg<HD, RK, RV>::REC_FLOATS * 4;
-  }
-  // Steps of row tile x; the tail of a tile is what lies beyond the first `p` steps.  Tails are laid end to end, kv
-  // head by kv head, and cut into `helpers` equal ranges (the kernel derives the same cuts from p and helpers).
-  // The cost of a plan, in steps: the longer of a tile's own block (p + its record and possibly the merge) and a
-  // helper (its range + a drain and refill per piece).  Returns p = 0 when the classic launch is as good.
-  static WorkList plan_worklist(precc_ctx* ctx, int S, int T, int tok_per_tile, int n_kv) {
-    WorkList best;
-    if (ctx->no_prefill_helpers) return best;
-    const int X = (S + tok_per_tile - 1) / tok_per_tile;
-    const long long tiles = (long long)X * n_kv;
-    const int H = ctx->sm_count - (int)tiles;
-    if (X >= PTC_MAX_XT || tiles * 2 <= ctx->sm_count || tiles > (long long)H * (PTC_MAX_SEG - 2)) return best;
-    auto steps_of = [&](int x) { return (int)(((long long)T + std::min(S, (x + 1) * tok_per_tile) + PTC_TOK - 1) / PTC_TOK); };
-    const int n_max = steps_of(X - 1);
-    if (n_max < ctx->prefill_helper_min_steps) return best;
-    // What a record + merge costs a tile's own block, and what a piece costs a helper beyond its steps (query tile,
-    // fold, pipeline fill, record), in steps at head_dim 128, rank 32 (1.0 us), scaled for shorter ones; and how much longer
-    // every step takes with all SMs busy instead of one per tile.  At head_dim 128 the launch runs at the power cap; steps
-    // without the sum of rounded weights are short (head_dim 64 rank 64: 0.78 us, head_dim 128 without adapter: 0.86 us for
-    // 64 KB of caches each), so that what L2 delivers to all SMs together bounds them and more SMs only stretch them.
-    // Measured on turns of 80 .. 112 tiles over 24000 and 48000 tokens, steps of the work-list launch against the plain one.
-    const int f100 = 100 * 160 / (HD + (RK + RV) / 2);
-    const int C_OWN = 14 * f100 / 100, C_PIECE = (HD == 64 ? 12 : RK + RV > 32 ? 18 : 13) * f100 / 100;
-    const int slow = HD == 64 ? (RV == 64 ? 138 : RV == 0 ? 114 : 106) : RV == 0 ? 144 : RV == 64 ? 106 : 112;
-    int best_cost = (n_max - n_max / 25) * 100 / slow;   // a plan must win 4 % on paper
-    for (int p = n_max - 1; p >= std::max(8, n_max / 2); --p) {
-      if (ctx->prefill_helper_p > 0 && p != ctx->prefill_helper_p) continue;
-      long long tail_sum = 0;
-      for (int x = 0; x < X; ++x) tail_sum += std::max(0, steps_of(x) - p);
-      const long long total = tail_sum * n_kv;
-      const long long per = std::max(1ll, (total + H - 1) / H);
-      if (p + C_OWN >= best_cost && ctx->prefill_helper_p <= 0) continue;
-      // walk the tails in the kernel's order: pieces per helper and pieces per tile
-      int max_seg = 0, max_src = 0;
-      long long pos = 0;
-      for (int g = 0; g < n_kv; ++g)
-        for (int x = 0; x < X; ++x) {
-          const int tl = std::max(0, steps_of(x) - p);
-          if (tl == 0) continue;
-          const long long hf = pos / per, hl = (pos + tl - 1) / per;
-          max_src = std::max(max_src, (int)(2 + hl - hf));
-          pos += tl;
-        }
-      {
-        // pieces of helper h = tiles whose tail range meets [h per, (h+1) per)
-        std::vector<int> cnt(H, 0);
-        pos = 0;
-        for (int g = 0; g < n_kv; ++g)
-          for (int x = 0; x < X; ++x) {
-            const int tl = std::max(0, steps_of(x) - p);
-            if (tl == 0) continue;
-            for (long long h = pos / per; h <= (pos + tl - 1) / per && h < H; ++h) ++cnt[(size_t)h];
-            pos += tl;
-          }
-        for (int h = 0; h < H; ++h) max_seg = std::max(max_seg, cnt[(size_t)h]);
-      }
-      if (max_seg > PTC_MAX_SEG || max_src > PTC_MAX_SRC) continue;
-      const int cost = (int)std::max<long long>(p + C_OWN, per + (long long)C_PIECE * max_seg);
-      if (cost < best_cost || ctx->prefill_helper_p > 0) { best_cost = cost; best.p = p; best.helpers = H; best.tiles = (int)tiles; }
-    }
-    return best;
   }
   // tensor-core kernel (tcgen05 + TMEM + TMA) for the shapes it supports
   static int32_t run_tc(precc_ctx* ctx, const PrefillArgs& a) {
@@ -182,7 +119,8 @@ struct PrefillRun {
     const bool wl_ok = !p.trace;
 #endif
     if (a.ws && ns == 1 && wl_ok && v_half == C::V_HALF_CAPABLE) {     // (the diagnostic whole-step ring has no work-list form there)
-      const WorkList wl = plan_worklist(ctx, a.S, a.T, p.tok_per_tile, d->n_kv_heads);
+      const WorkList wl = ctx->no_prefill_helpers ? WorkList() : plan_worklist(HD, RK, RV, a.S, a.T, p.tok_per_tile, d->n_kv_heads, ctx->sm_count,
+                                                                               ctx->prefill_helper_min_steps, ctx->prefill_helper_p);
       if (wl.p > 0 && a.ws_bytes >= worklist_ws_bytes(wl.tiles, wl.helpers)) {
         p.helper_p = wl.p; p.n_helpers = wl.helpers; p.longest_first = 0;
         p.ws_ticket = reinterpret_cast<unsigned int*>(a.ws);

@@ -58,6 +58,7 @@
 #pragma once
 #include <type_traits>
 
+#include "prefill_plan.h"
 #include "tc_common.cuh"
 
 namespace precc {
@@ -118,12 +119,8 @@ constexpr int PTC_SM_REGS = 216, PTC_CTL_REGS = 40;  // 256 x 216 + 256 x 40 = 5
 constexpr int PTC_SMEM_LIMIT = 232448;   // dynamic shared memory a block can opt into on this architecture
 constexpr int PTC_FIXED_BARS = 13; // barriers besides the two per ring stage
 constexpr int PTC_XCH_BYTES = 4 * 512;   // [2][128] reference maxima | [2][128] partial denominators or the tile of ones
-constexpr int PTC_TOK = 128;      // tokens per step
 constexpr float PTC_RAISE = 8.f;  // the running maximum is raised only when it grows by more than this
 constexpr int PTC_MAX_SPLIT = 8;  // blocks of a split-context cluster at most
-constexpr int PTC_MAX_SRC = 8;    // work-list launch: pieces of one tile (its own block + helper pieces) at most
-constexpr int PTC_MAX_SEG = 16;   // work-list launch: tile pieces one helper block takes at most
-constexpr int PTC_MAX_XT = 160;   // work-list launch: row tiles at most
 constexpr int PTC_TAB_BYTES = (2 * PTC_MAX_XT + 8 + 4 * PTC_MAX_SEG) * 4;   // tail lengths | their prefix sums | scalars | piece list
 
 template <int HD, int RK, int RV>

@@ -1,0 +1,47 @@
+"""The rule that puts helper blocks on idle SMs, compiled from the header that the library compiles (no GPU)."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(__file__), "..", "paper_2609_34054_b200", "csrc")
+SMS, MIN_STEPS = 148, 48
+
+
+@pytest.fixture(scope="module")
+def plans(tmp_path_factory):
+    """(head_dim, rank_k, rank_v, row tiles x kv heads, tokens of the context) -> (p, helpers, tiles); eight kv heads of four query heads."""
+    d = tmp_path_factory.mktemp("plan")
+    (d / "plan.cpp").write_text('#include <cstdio>\n#include "prefill_plan.h"\nint main() { int a[5]; while (scanf("%d %d %d %d %d", a, a + 1, a + 2, a + 3, a + 4) == 5) { '
+                                f'precc::WorkList w = precc::plan_worklist(a[0], a[1], a[2], a[3] / 8 * 32 - 5, a[4], 32, 8, {SMS}, {MIN_STEPS}, 0); '
+                                'printf("%d %d %d\\n", w.p, w.helpers, w.tiles); } }\n')
+    subprocess.run(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-I", CSRC, str(d / "plan.cpp"), "-o", str(d / "plan")], check=True)
+
+    def call(rows):
+        out = subprocess.run([str(d / "plan")], input="\n".join(" ".join(map(str, r)) for r in rows), capture_output=True, text=True, check=True).stdout
+        return [tuple(map(int, line.split())) for line in out.splitlines()]
+    return call
+
+
+# turns measured without and with helper blocks: what the latter took of the former
+MEASURED = [((128, 0, 16, 104, 24000), 1.06), ((128, 0, 16, 112, 40000), 1.04), ((128, 0, 64, 96, 14000), 1.06), ((128, 0, 64, 112, 28000), 1.06),
+            ((128, 0, 64, 120, 48000), 1.05), ((128, 8, 8, 104, 24000), 1.05), ((128, 8, 8, 88, 14000), 1.06),
+            ((128, 32, 32, 80, 24000), 0.85), ((128, 32, 32, 96, 33000), 0.95), ((128, 16, 16, 88, 33000), 0.85), ((128, 8, 8, 96, 24000), 0.94),
+            ((128, 0, 16, 80, 33000), 0.85), ((128, 0, 64, 80, 33000), 0.92), ((128, 64, 64, 104, 33000), 0.92), ((64, 32, 32, 96, 33000), 0.85), ((64, 16, 16, 80, 24000), 0.82)]
+
+
+def test_helper_blocks_are_taken_where_they_are_faster(plans):
+    for (turn, share), (p, helpers, tiles) in zip(MEASURED, plans([t for t, _ in MEASURED])):
+        assert (p > 0) == (share < 1), turn
+
+
+def test_helper_block_plans_stay_inside_what_the_kernel_holds(plans):
+    rows = [(hd, rk, rv, tiles, T) for hd in (64, 128) for rk, rv in ((0, 0), (0, 8), (0, 64), (8, 8), (32, 32), (64, 64)) for tiles in range(64, 152, 8)
+            for T in (1000, 6000, 14000, 33000, 120000)]
+    taken = 0
+    for (hd, rk, rv, tiles, T), (p, helpers, n) in zip(rows, plans(rows)):
+        if p:
+            taken += 1
+            longest = -(-(T + tiles // 8 * 32 - 5) // 128)
+            assert helpers == SMS - tiles > 0 and n == tiles and longest // 2 <= p < longest and longest >= MIN_STEPS
+    assert taken > 100
