@@ -172,10 +172,11 @@ int32_t precc_rebase_project(precc_ctx* ctx, const precc_layer_desc* desc, const
  *   WA_packed  2*n_kv_heads*head_dim + n_agents*(rank_k+rank_v) packed rows: the W rows followed by the A
  *              rows (precc_pack_kmajor into one buffer of that many rows)
  *   agent_mask selects the LR caches written; the base rows are always written.
- * Results are bit-identical to precc_rebase_project followed by precc_lr_precompute with the same M (the
- * three calls pick their kernel from M, d_model and the layer's fused width alone, so they agree).  The same
+ * Results are bit-identical to precc_rebase_project followed by precc_lr_precompute with the same M: the three
+ * calls add the products of a value in an order that depends on M, d_model and the layer's fused width alone
+ * (tiles and, for many rows onto few columns, the kernel also depend on the call's own columns).  The same
  * row projected in calls of different M may differ in the last bf16 bit: few rows (a decode step), a short
- * turn and a long segment run on three kernels whose fp32 summation orders differ. */
+ * turn and a long segment run on kernels whose fp32 summation orders differ. */
 int32_t precc_turn_project(precc_ctx* ctx, const precc_layer_desc* desc, const void* H, int32_t M,
                            const void* WA_packed, const int32_t* slot_mapping, int64_t start_slot,
                            uint64_t agent_mask, const precc_cache* cache, void* stream);

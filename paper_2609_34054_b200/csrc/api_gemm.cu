@@ -182,7 +182,6 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
         rc2 = make_map_w(ctx, &map_w2, Wt, n_out, K, bn2 / 2);
         if (rc2) return rc2;
         gp.M = M; gp.N_out = n_out; gp.K = K; gp.BN = bn2; gp.stages = st2; gp.tmem_cols = tc2;
-        gp.spread_rows = 1;
         gp.status = ctx->status;
         gp.trace = (ctx->trace && ctx->trace_blocks >= 128) ? ctx->trace : nullptr;     // used by PRECC_GEMM_TRACE builds only
         PRECC_CUDA(ctx, raise_smem_limit(ctx, proj_gemm_pair_kernel, (int)smem2));
@@ -220,7 +219,6 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
   rc = make_map_w(ctx, &map_w, Wt, n_out, K, bn);
   if (rc) return rc;
   gp.M = M; gp.N_out = n_out; gp.K = K; gp.BN = bn; gp.stages = stages; gp.tmem_cols = tmem_cols;
-  gp.spread_rows = 1;
   gp.status = ctx->status;
   gp.trace = (ctx->trace && ctx->trace_blocks >= 128) ? ctx->trace : nullptr;     // used by PRECC_GEMM_TRACE builds only
   PRECC_CUDA(ctx, raise_smem_limit(ctx, proj_gemm_kernel, (int)smem));

@@ -93,7 +93,7 @@ proj_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   // of the pairs and the tiles are spread evenly over the rows (neighbours overlap by a few rows, computed twice
   // with identical results), so that every pair streams the same number of rows.
   const int m_plain = (p.M + GEMM_PAIR_BM - 1) / GEMM_PAIR_BM;
-  const bool spread = p.spread_rows && n_tiles_n == 1 && m_plain > n_pairs && p.M >= GEMM_PAIR_BM;
+  const bool spread = n_tiles_n == 1 && m_plain > n_pairs && p.M >= GEMM_PAIR_BM;
   const int m_tiles = spread ? ((m_plain + n_pairs - 1) / n_pairs) * n_pairs : m_plain;
   const int n_tiles = m_tiles * n_tiles_n;
   auto row0_of = [&](int mt) -> int {

@@ -188,7 +188,7 @@ proj_gemm_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
   // the rows: neighbours overlap by a few rows, which are computed twice with identical results (the
   // overlap is re-read from L2, not from DRAM), and every block streams the same number of rows.
   const int m_plain = (p.M + GEMM_BM - 1) / GEMM_BM;
-  const bool spread = p.spread_rows && n_tiles_n == 1 && m_plain > (int)gridDim.x && p.M >= GEMM_BM;
+  const bool spread = n_tiles_n == 1 && m_plain > (int)gridDim.x && p.M >= GEMM_BM;
   const int m_tiles = spread ? ((m_plain + (int)gridDim.x - 1) / (int)gridDim.x) * (int)gridDim.x : m_plain;
   const int n_tiles = m_tiles * n_tiles_n;
   auto row0_of = [&](int mt) -> int {

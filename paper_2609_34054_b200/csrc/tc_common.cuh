@@ -12,7 +12,6 @@ struct GemmParams {
   int M, N_out, K;
   int BN, stages, tmem_cols;      // BN: columns of a tile (turn kernel: rows of X in a tile)
   int by_rows;                    // few-row kernel: 1 = its blocks finish rows of the tile, 0 = slices of its columns
-  int spread_rows;                // 1: even row-tile spreading allowed (rows may be written twice, identically)
   int mode;                       // 0 = LR caches, 1 = base caches, 2 = base columns then LR columns
   const int32_t* slot_mapping;    // [M] or null
   int64_t start_slot;
