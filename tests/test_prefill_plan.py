@@ -45,3 +45,38 @@ def test_helper_block_plans_stay_inside_what_the_kernel_holds(plans):
             longest = -(-(T + tiles // 8 * 32 - 5) // 128)
             assert helpers == SMS - tiles > 0 and n == tiles and longest // 2 <= p < longest and longest >= MIN_STEPS
     assert taken > 100
+
+
+def _exhaustive(hd, rk, rv, tiles, T, tok=32, n_kv=8):
+    """The definition: of the p that beat the plain launch by 4 % on paper, the largest among those with the smallest cost."""
+    X, H, S = tiles // n_kv, SMS - tiles, tiles // n_kv * tok - 5
+    if X >= 160 or tiles * 2 <= SMS or tiles > H * 14:
+        return 0
+    steps = [(T + min(S, (x + 1) * tok) + 127) // 128 for x in range(X)]
+    if steps[-1] < MIN_STEPS:
+        return 0
+    f = 100 * 160 // (hd + (rk + rv) // 2)
+    own, piece = 14 * f // 100, (12 if hd == 64 else 18 if rk + rv > 32 else 13) * f // 100
+    slow = (138 if rv == 64 else 114 if rv == 0 else 106) if hd == 64 else 144 if rv == 0 else 121 if rk == 0 else 106 if rv == 64 else 115 if rk == 8 else 112
+    best, best_cost = 0, (steps[-1] - steps[-1] // 25) * 100 // slow
+    for p in range(steps[-1] - 1, max(8, steps[-1] // 2) - 1, -1):
+        tails = [max(0, s - p) for s in steps] * n_kv
+        per, pos, pieces, sources = max(1, -(-sum(tails) // H)), 0, [0] * H, 0
+        for t in tails:
+            if t:
+                first, last = pos // per, (pos + t - 1) // per
+                sources = max(sources, 2 + last - first)
+                for h in range(first, last + 1):
+                    pieces[h] += 1
+                pos += t
+        cost = max(p + own, per + piece * max(pieces))
+        if max(pieces) <= 16 and sources <= 8 and cost < best_cost:
+            best, best_cost = p, cost
+    return best
+
+
+def test_the_search_for_a_plan_misses_none(plans):
+    rows = [(hd, rk, rv, tiles, T) for hd, rk, rv in ((64, 32, 32), (64, 0, 64), (128, 8, 8), (128, 64, 64), (128, 0, 16)) for tiles in range(72, 144, 8)
+            for T in (6100, 9000, 15000, 24000, 33000, 47000)]
+    got = [p for p, _, _ in plans(rows)]
+    assert got == [_exhaustive(*r) for r in rows] and sum(p > 0 for p in got) > 60
