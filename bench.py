@@ -392,7 +392,7 @@ def extra_turn(px, T: int, S: int, seed: int = 0, cpu_seconds: float = 0.0):
     tf_pre = fl_pre / us_pre / 1e6
     pre_bytes = 2.0 * (T * geo.d_model + geo.d_model * n_lr + T * n_lr)
     attainable = min(pk["bf16_tflops_burst"], fl_pre / pre_bytes * hbm / 1e3)      # min(tensor, intensity x HBM), TFLOP/s
-    cap_pf, cap_pre = ncu_traffic("prefill_tc_c3_layer"), ncu_traffic("proj_gemm_c3_context")
+    cap_pf, cap_pre = ncu_traffic("prefill_tc_c3_layer"), ncu_traffic("proj_turn_c3_context")
     res = {"workload": f"C3 turn, one layer: d=4096 32q/8kv hd=128, N=4 r=32, T={T}, S={S}",
            "short_turn": short,
            "lr_precompute_context": {"us": us_pre, "tflops": tf_pre, "n_out": n_lr, "GBps": pre_bytes / us_pre / 1e3,
@@ -410,7 +410,7 @@ def extra_turn(px, T: int, S: int, seed: int = 0, cpu_seconds: float = 0.0):
                                 "frac": tf_attn / pk["bf16_tflops_burst"], "frac_of_sustained": tf_attn / pk["bf16_tflops_sustained"],
                                 "traffic": cap_pf["dram_bytes"] if cap_pf else None, "algorithmic_flops_per_launch": fl_attn,
                                 "avg_launch_us": us_attn},
-           "roofline_precompute": {"bound": "tensor", "kernel": "proj_gemm_kernel (mode 0, n_out 256)", "achieved": tf_pre,
+           "roofline_precompute": {"bound": "tensor", "kernel": "proj_turn_kernel<false,2> (mode 0, n_out 256)", "achieved": tf_pre,
                                    "peak": pk["bf16_tflops_burst"], "peak_kind": pk["peak_kind"] + " (burst)", "unit": "TFLOP/s",
                                    "frac": tf_pre / pk["bf16_tflops_burst"], "attainable_min_tensor_hbm": attainable,
                                    "frac_of_attainable": tf_pre / attainable,

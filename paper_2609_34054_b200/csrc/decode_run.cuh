@@ -223,7 +223,7 @@ struct DecodeRunT {
       return pl.cluster ? pl : flat();
     }
     if (ROPE) {
-      // issue-bound: four warps twice per SM reach as many SMs as eight once, in finer pieces; from some work on the flat
+      // bound by what the SMs take in from L2: four warps twice per SM reach as many SMs as eight once, in finer pieces; from some work on the flat
       // grid's even shares win
       // (one block each: above three fifths of the SMs that is a fair share of the machine, so it pays up to more pages)
       if (units * 2 > sm && mt <= (units * 5 > 3 * sm ? 48 : 16)) return whole();

@@ -29,8 +29,8 @@
 // at every step; P stays below 2^8.  The denominator: for 0 < r_v < 64 the rounded weights that the MMA sees are summed, by the
 // MMA: behind each k step of P V' a second one of N = 16 multiplies the same P with a constant tile of ones (512 bytes of
 // shared memory, sixteen equal columns behind O').  The softmax threads are left with four instructions per pair of
-// scores instead of seven (8192 over 24576: 4147 -> 3895 us; 512 over 32768 with both projections: 316 -> 297).  Otherwise, and in the
-// work-list form (which would spill), they sum in fp32, two values per instruction.  (Unrounded, the sum left a
+// scores instead of seven (8192 over 24576: 4147 -> 3895 us; 512 over 32768 with both projections: 316 -> 297).  Otherwise, in the work-list
+// form (which would spill) and in most split-context forms at head_dim 128, they sum in fp32, two values per instruction.  (Unrounded, the sum left a
 // row dominated by one token up to 2^-8 off, on top of its own rounding, and the error against float64 5 .. 15 % higher
 // where a few tokens carry a row.)  Measured for the same sum and slower: a column of ones beside L_V in the value stage -
 // written into every landed stage by the issuing warp it takes 600 cycles of a step, by the softmax threads 6 % more time on
@@ -281,9 +281,10 @@ template <int HD, int RK, int RV, bool WL = false, bool VH = false, bool SP = fa
 __global__ void __launch_bounds__(PTC_THREADS, 1)
 lr_attend_prefill_tc_kernel(const __grid_constant__ PrefillTcMaps maps, const __grid_constant__ PrefillTcParams p) {
   using C = PrefillTcCfg<HD, RK, RV>;
-  // The MMA sums the denominator.  Not in the work-list form, which would spill.  In the split-context form at head_dim 128 only
-  // at rank 32 (64 over 16384: 33.0 us against 36.3, 30 over 60000: 69.3 against 74.0; paged, 64 over 32768: 58.9 against 56.5), not below
-  // (rank 16, 99 over 65427: 125 us against 113; rank 8, 64 over 32768: 57.5 against 55.3; no key adapter, 200 over 8000: 43.7 against 40.4).
+  // The MMA sums the denominator.  Not in the work-list form, which would spill.  In the split-context form at head_dim 128 it slows the
+  // step loop that ptxas makes of the other ranks: geometric mean of 36 turns of 32 .. 700 tokens over 8000 .. 65000 per layout, against
+  // the pulling form, summed by the MMA / by the threads: ranks 32 / 32 contiguous 0.924 / 1.017, paged 0.954 / 0.945; 16 / 16 1.012 / 0.934 and
+  // 0.980 / 0.934; 8 / 8 1.006 / 0.936 and 0.979 / 0.938; 0 / 16 0.968 / 0.925 and 0.972 / 0.935; 0 / 32 0.950 / 0.935 and 0.973 / 0.945.
   constexpr bool L_MMA = C::L_ROUNDED && !WL && !(SP && HD == 128 && RK != 32);
   // Running maxima over a row's 128 scores of a step (their number changes no bit).  A chain of 16 or 32 maxima keeps fewer registers than four
   // of them beside the scores, eight keep the chain short; which one ptxas makes the faster step loop of differs by form.  Whole

@@ -20,11 +20,13 @@
 // overlapping ones (32768 rows x 256 columns of d_model 4096: 71.5 -> 64.0 us; 20000 x 192: 56.6 -> 42.1; 20000 x 128, NG = 1: 53.0 -> 35.9).
 // Shared memory: [ring of {W 128 NG x 64 | X TN x 64} | overlaid: dump [TN][128] fp32, receive area [KS-1][tw][128] fp32]
 // [row table][barriers].  A block tells its peers when its ring is idle; they send only then.
-// The K split depends on M, K and the layer's fused width alone, so base-only, LR-only and fused calls agree bit for bit.
+// The K split depends on M, K and the layer's fused width alone, so base-only, LR-only and fused calls agree bit for bit; TN, which changes no bit,
+// on the columns of the call (proj_plan.h).
 // Measured on rotating weights from HBM, us a launch, against 128-row x 256-column tiles whose slices were pulled over
 // distributed shared memory (or sent, clusters of up to four) with 128 threads: 4096 -> 2304 columns, 64 / 128 / 301 / 512 / 1024 rows:
 // 12.4 / 15.1 / 16.6 / 19.5 / 24.5 -> 10.1 / 11.3 / 15.3 / 17.2 / 20.9; 2048 -> 1152: 9.8 / 12.7 / 13.2 / 14.7 / 15.3 -> 7.5 / 7.8 / 9.1 /
 // 10.3 / 12.5; 3584 -> 1280 with rotary keys, 64 / 200 / 512: 11.6 / 15.7 / 18.4 -> 9.1 / 10.9 / 13.6; 1024 -> 560: 8.6 .. 13.8 -> 5.8 .. 8.5.
+// (Up to 64 rows the three narrower layers run on the few-row kernel, see few_row_limit.)
 #pragma once
 #include "gemm_tc.cuh"
 
