@@ -76,14 +76,15 @@ int32_t launch_small(precc_ctx* ctx, const void* X, int M, int K, const void* Wt
 
 int ilog2(int v) { int s = 0; while ((1 << s) < v) ++s; return s; }
 
-// Clusters of `ks` blocks of the turn kernel that are resident at once (one block per SM; a cluster lives inside one GPC).
-int max_turn_clusters(precc_ctx* ctx, int ks) {
-  static int max_clusters_dev[kMaxDevices][GEMM_MAX_KS + 1] = {{0}};   // 0 = unknown, else max active clusters + 1
+// Clusters of ks blocks of the turn kernel that are resident at once (one block per SM; a cluster lives inside one GPC), for every ks.
+const int* turn_clusters(precc_ctx* ctx) {
+  static int fit_dev[kMaxDevices][GEMM_MAX_KS + 1] = {{0}};       // [.][0] != 0: asked
   std::lock_guard<std::recursive_mutex> lk(lazy_mu());
-  int& cached = max_clusters_dev[ctx->device % kMaxDevices][ks];
-  if (cached == 0) {
+  int* fit = fit_dev[ctx->device % kMaxDevices];
+  if (fit[0]) return fit;
+  auto kern = proj_turn_kernel<false, 1>;
+  for (int ks = 2; ks <= GEMM_MAX_KS; ++ks) {
     int n = 0;
-    auto kern = proj_turn_kernel<false, 1>;
     if (raise_smem_limit(ctx, kern, PT_MIN_SMEM) == cudaSuccess) {
       cudaLaunchConfig_t qc = {};
       qc.gridDim = dim3(ks, ctx->sm_count, 1); qc.blockDim = dim3(PT_THREADS); qc.dynamicSmemBytes = PT_MIN_SMEM;
@@ -95,9 +96,10 @@ int max_turn_clusters(precc_ctx* ctx, int ks) {
     } else {
       cudaGetLastError();
     }
-    cached = n + 1;
+    fit[ks] = n;
   }
-  return cached - 1;
+  fit[0] = 1;
+  return fit;
 }
 
 template <int NG>
@@ -145,7 +147,7 @@ int32_t launch_gemm(precc_ctx* ctx, const void* X, int M, int K, const void* Wt,
   if (m_tiles <= 16 && !ctx->no_gemm_splitk) {
     const int ks_max = ctx->gemm_ks_max >= 2 && ctx->gemm_ks_max < GEMM_MAX_KS ? ctx->gemm_ks_max : GEMM_MAX_KS;
     const TurnPlan tp = plan_turn(M, K / GEMM_BK, n_fused, n_out, ctx->gemm_ks_min, ks_max, ctx->sm_count, ctx->max_smem_optin,
-                                  [&](int ks) { return max_turn_clusters(ctx, ks); });
+                                  turn_clusters(ctx));
     if (tp.ks > 0) return launch_turn<1>(ctx, X, M, K, Wt, n_out, gp, tp, stream);
   }
   if (M <= PS_MAX_M && !ctx->force_tiled_gemm) {

@@ -44,8 +44,8 @@ inline int few_row_limit(int K, int n_fused) { return n_fused <= 1280 && K <= 40
 // How a turn's projection is cut: tiles of 128 columns x tn rows, the K extent of each over ks blocks.
 struct TurnPlan { int tn = 0, ks = 0, stages = 0; };
 
-// The cut with the smallest predicted time among those whose clusters are all resident at once - clusters(ks) says how many of ks
-// blocks are, a cluster lives inside one GPC - (a second wave costs more than any split gains: 512 rows of the Llama-3-8B projection
+// The cut with the smallest predicted time among those whose clusters are all resident at once (a cluster lives inside one GPC;
+// a second wave costs more than any split gains: 512 rows of the Llama-3-8B projection
 // as 36 clusters of four, of which 33 fit, 26.9 us; as 36 clusters of three 17.2).  Time in us, fitted to some 450 cuts of
 // four layers (d_model 1024 .. 4096) at 41 .. 2048 rows, mean error 4 %: what a k-block costs a block, what the merge moves into
 // one, what dumping and storing a tile takes, and the cluster.  The cut it picks is within 1 % of the best one measured but for
@@ -54,30 +54,34 @@ struct TurnPlan { int tn = 0, ks = 0, stages = 0; };
 // LR-only and fused calls of one M add in the same order.  The height of the tiles changes no bit: a call of fewer columns takes lower
 // tiles on the SMs that this leaves (LR rows of two agents of rank 8, d_model 2048, 768 rows: 9.9 us in tiles of the fused
 // call's height, 8.2 in tiles of 32 rows; of three, d_model 1024, 1800 rows 8.8 -> 7.0; base rows of d_model 3584, 512 rows 12.6 -> 11.6).
-template <class Clusters>
-TurnPlan plan_turn(int M, int nkb, int n_fused, int n_out, int ks_min, int ks_max, int sm_count, int max_smem, Clusters clusters) {
+// clusters[ks]: how many clusters of ks blocks are resident at once.
+inline TurnPlan plan_turn(int M, int nkb, int n_fused, int n_out, int ks_min, int ks_max, int sm_count, int max_smem, const int* clusters) {
   TurnPlan best;
-  auto search = [&](int columns, int ks_lo, int ks_hi) {
-    double best_cost = 1e30;
-    const int groups = (columns + PT_COLS - 1) / PT_COLS;
-    for (int t = (M + PT_MAX_TN - 1) / PT_MAX_TN, last = 0;; ++t) {
-      const int tn = ((M + t - 1) / t + 15) / 16 * 16, tiles = (M + tn - 1) / tn;
-      if (tn < 32 || (long long)groups * tiles * ks_lo > sm_count) break;
-      if (tn == last) continue;
-      last = tn;
-      for (int ks = ks_lo; ks <= ks_hi && nkb / ks >= 2; ++ks) {       // at least two k-blocks per slice
-        if (groups * tiles > clusters(ks)) continue;
-        const int kb = (nkb + ks - 1) / ks;
-        int st = kb < PT_MAX_STAGES ? kb : PT_MAX_STAGES;
-        while (st > 1 && pt_smem_bytes(tn, ks, st, 1) > max_smem) --st;
-        if (pt_smem_bytes(tn, ks, st, 1) > max_smem) continue;
-        const double cost = kb * (0.37 + 0.00036 * tn) + 0.005 * pt_share(tn, ks) * (ks - 1) + 0.0113 * tn + 0.1 * ks;
-        if (cost < best_cost) { best_cost = cost; best.tn = tn; best.ks = ks; best.stages = st; }
-      }
-    }
+  double best_cost = 1e30;
+  auto ring = [&](int tn, int ks) {                    // stages that fit
+    int st = std::min((nkb + ks - 1) / ks, PT_MAX_STAGES);
+    while (st > 0 && pt_smem_bytes(tn, ks, st, 1) > max_smem) --st;
+    return st;
   };
-  search(n_fused, ks_min, ks_max);
-  if (best.ks > 0 && n_out < n_fused) search(n_out, best.ks, best.ks);
+  const int groups = (n_fused + PT_COLS - 1) / PT_COLS;
+  for (int t = (M + PT_MAX_TN - 1) / PT_MAX_TN, last = 0;; ++t) {
+    const int tn = ((M + t - 1) / t + 15) / 16 * 16, tiles = (M + tn - 1) / tn;
+    if (tn < 32 || (long long)groups * tiles * ks_min > sm_count) break;
+    if (tn == last) continue;
+    last = tn;
+    for (int ks = ks_min; ks <= ks_max && nkb / ks >= 2; ++ks) {       // at least two k-blocks per slice
+      if (groups * tiles > clusters[ks]) continue;
+      const int kb = (nkb + ks - 1) / ks, st = ring(tn, ks);
+      if (st == 0) continue;
+      const double cost = kb * (0.37 + 0.00036 * tn) + 0.005 * pt_share(tn, ks) * (ks - 1) + 0.0113 * tn + 0.1 * ks;
+      if (cost < best_cost) { best_cost = cost; best.tn = tn; best.ks = ks; best.stages = st; }
+    }
+  }
+  if (best.ks > 0 && n_out < n_fused) {                // at a given ks the lowest tiles that are all resident
+    const int tiles = clusters[best.ks] / ((n_out + PT_COLS - 1) / PT_COLS);
+    best.tn = std::max(32, ((M + tiles - 1) / tiles + 15) / 16 * 16);
+    best.stages = ring(best.tn, best.ks);
+  }
   return best;
 }
 

@@ -60,8 +60,8 @@ def test_tall_tiles_are_taken_where_they_are_faster(plan):
 # blocks of a cluster -> clusters that are resident at once, as a B200 reports them
 CLUSTERS = {2: 74, 3: 45, 4: 33, 5: 26, 6: 22, 7: 15, 8: 15}
 SMEM = 232448
-PLAN = ("static const int fit[9] = {0, 0, %s}; " % ", ".join(str(CLUSTERS[k]) for k in range(2, 9)) +
-        f"TurnPlan p = plan_turn(a[0], a[1], a[2], a[3], 2, 8, {SMS}, {SMEM}, [&](int ks) {{ return fit[ks]; }}); "
+PLAN = ("static const int fit[9] = {1, 0, %s}; " % ", ".join(str(CLUSTERS[k]) for k in range(2, 9)) +
+        f"TurnPlan p = plan_turn(a[0], a[1], a[2], a[3], 2, 8, {SMS}, {SMEM}, fit); "
         'printf("%d %d %d %d\\n", p.tn, p.ks, p.stages, p.ks ? pt_smem_bytes(p.tn, p.ks, p.stages, 1) : 0);')
 
 
